@@ -76,7 +76,7 @@ def kernel_source_hash():
     return h.hexdigest()
 
 
-KERNEL_NAMES = {1: "fwd_simt_kernel", 2: "fwd_tc_kernel", 3: "fwd_small_kernel", 4: "fwd_ws_kernel"}
+KERNEL_NAMES = {1: "fwd_simt_kernel", 2: "fwd_ws_kernel", 3: "fwd_small_kernel", 4: "fwd_ws_kernel"}
 
 
 def recorded_traffic(key):

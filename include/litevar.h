@@ -83,13 +83,13 @@ typedef struct {
 
 /* Forward kernel selection (testing / measurement). */
 enum {
-  LITEVAR_KERNEL_AUTO = 0,    /* per step: the small-step kernel where the step fits it, else a tcgen05 kernel (the one
-                                 with a softmax thread per query row on long tile lists) */
+  LITEVAR_KERNEL_AUTO = 0,    /* per step: the small-step kernel where the step fits it, else the tcgen05 kernel */
   LITEVAR_KERNEL_SIMT = 1,    /* plain CUDA-core kernel (slow; cross-check and bring-up) */
-  LITEVAR_KERNEL_TCGEN05 = 2, /* tcgen05/TMEM/TMA kernel with two softmax threads per query row, for every step */
+  LITEVAR_KERNEL_TCGEN05 = 2, /* the tcgen05/TMEM/TMA kernel for every step; reported for short tile lists (fewer than
+                                 eight key tiles per query tile on average) */
   LITEVAR_KERNEL_SMALL = 3,   /* reported by litevar_plan_step_kernel only: warp-level mma kernel for steps with one
                                  query tile, at most two raster key tiles and little work */
-  LITEVAR_KERNEL_TCGEN05_WS = 4 /* tcgen05 kernel with one softmax thread per query row, for every step */
+  LITEVAR_KERNEL_TCGEN05_WS = 4 /* the same kernel; reported for long tile lists */
 };
 
 /*
@@ -174,7 +174,7 @@ litevar_status_t litevar_attn_forward_kv8(const litevar_plan_t* plan, int32_t st
  * litevar_attn_plan keeps its tile lists in memory it gets from cudaMalloc.  A caller that may not
  * allocate (it runs inside a fixed device-memory budget, it is a plug-in that must stay away from its
  * host's allocator, or it is reached at a point where allocation is forbidden) uses this call instead:
- * it builds the tile plan of step_k on the device inside a fixed 4.2 MB array that is part of the
+ * it builds the tile plan of step_k on the device inside a fixed 4.4 MB array that is part of the
  * library image, then runs the same tensor-core forward kernel on it.  It calls no cudaMalloc, no
  * cudaFree and no allocating library routine; it launches three kernels on `stream` and returns
  * without synchronising.

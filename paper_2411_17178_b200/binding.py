@@ -305,7 +305,7 @@ class Plan:
         _check(self._lib.litevar_plan_set_kernel(self._h, int(kernel)), "litevar_plan_set_kernel")
 
     def step_kernel(self, step_k: int, batch_pairs: int = 1) -> int:
-        """KERNEL_SIMT, KERNEL_TCGEN05 or KERNEL_SMALL: what a forward of this step with that batch launches."""
+        """KERNEL_SIMT, KERNEL_SMALL, or the tcgen05 kernel: KERNEL_TCGEN05 on short, KERNEL_TCGEN05_WS on long tile lists."""
         out = ctypes.c_int32(0)
         _check(self._lib.litevar_plan_step_kernel(self._h, int(step_k), int(batch_pairs), ctypes.byref(out)),
                "litevar_plan_step_kernel")

@@ -1,35 +1,36 @@
-// Warp-specialised tensor-core forward kernel for sm_100a with register reallocation: one softmax thread owns a
-// whole query row, and the scores of the next key tile are formed while the softmax of the current one runs.
-// Used for steps with long tile lists (from eight key tiles per query tile on); the kernel of litevar_fwd_tc.cu
-// serves the shorter ones.
+// Tensor-core forward kernel for sm_100a: one query tile per CTA, two independent streams of key chunks.
 //
-// The kernel is written for NH query tiles ("halves", 128 queries each) of one (head, batch row) per CTA, walking
-// the union of their live key-tile lists; the library launches NH = 1, two CTAs per SM (see launch_forward_ws).
-//   warps 0 .. 4 NH - 1   softmax warpgroup of half h = warp / 4: thread m of the group owns query slot m (TMEM
-//                         lane m).  A key tile is taken in two passes of 64 keys through one rolled copy of the
-//                         code: 64 scores from TMEM into registers, the plan's element mask, the row maximum
-//                         without any exchange, the probabilities against a lazily updated reference maximum
-//                         (every fourth pair of exponentials on the FMA pipe by a cubic, the rest on the
-//                         exponential pipe), their sum, and P (packed bf16) into a TMEM block of its own.  The S
-//                         block is released as soon as the second pass has its scores in registers.  At the end
-//                         the thread normalises and stores its output row.
-//   warp 4 NH             TMA producer (one lane): Q of every half, then K and V of every listed key tile into two
-//                         rings of kStages tiles.
-//   warp 4 NH + 1         TMEM allocation; one lane issues S_h = Q_h K^T of the next key tile as soon as the
-//                         softmax threads have read the previous S_h.
-//   warp 4 NH + 2         one lane issues O_h += P_h V of a tile once its P is complete.  Because P does not
-//                         overlay S, the score product of tile j + 1 does not wait for the softmax of tile j and
-//                         the PV product is off the softmax's critical path.
-//   warp 4 NH + 3         idle (it completes the warpgroup that gives its registers away).
-// Registers: the kernel starts with the launch-bound count for every thread; the last warpgroup then releases
-// all but 56 per thread (setmaxnreg.dec) and the softmax warpgroups take them (setmaxnreg.inc).
-// MMA issue: four K = 16 steps per instruction sequence with immediate offsets (mma_*_x4).  Measured on B200,
-// back to back: 65 cycles per step at N = 128 (64 are pure math), 50 at N <= 64, for A in shared memory or in
-// TMEM alike; a tcgen05.commit between groups of four to eight steps adds 100 to 150 cycles of tensor-pipe time.
-// TMEM columns: S_h [128 h, +128); O_h [128 NH + 64 h, +64); P_h [192 NH + 64 h, +64).
-// Every wait on an mbarrier is bounded (2^32 cycles); on expiry the CTA raises the plan's status word, drains its
-// copies, frees its TMEM and returns.  The element mask, the tile lists and CFG sharing (second store at batch row
-// b + B) are those of the plan and of the other forward kernels (paper Sections 2 and 3).
+// A CTA owns a query tile (128 queries) of one (head, batch row) and walks the live 64-key chunks of its list (the halves of
+// the plan's 128-key tiles that hold a live entry).  Two streams share the list, chunk i going to stream i % 2; each keeps its
+// own scores, probabilities, accumulator and reference, and the two results meet at the end.  320 threads:
+//   warps 0-3, 4-7  softmax of stream 0 and 1: thread m of the group owns query slot m (TMEM lane m).  A chunk's 64 scores
+//                   come from TMEM in two halves of 32 through one rolled copy of the code: the plan's element mask, the
+//                   probabilities (every fourth pair of exponentials on the FMA pipe by a cubic, the rest on the exponential
+//                   pipe), their sum, and P (packed bf16) over the scores that have been read.
+//   warps 8, 9      the stream's copies (K and V chunks by tensor-map copies into rings of two stages) and MMAs: once P(i) is
+//                   complete, O += P(i) V(i) and S(i + 1) = Q K(i + 1) go out back to back; they execute in issue order, so
+//                   that S may overwrite P.  The warp runs converged and what it computes is uniform, so that descriptors
+//                   stay in uniform registers (a lane of its own: eight register moves per MMA); one elected lane issues.
+// Two CTAs per SM, so that every scheduler has four softmax warps of four streams that are in different phases.
+// TMEM columns: S and P of stream s at 64 s, O at 128 + 64 s.
+//
+// The reference of a row (probabilities are 2^(score * scale - reference)) needs no maximum per chunk: it starts as the
+// maximum of the first chunk; afterwards only the chunk's SUM is looked at, and when that exceeds 2^10 the reference moves by
+// whole powers of two for the next chunk (the accumulator and the sum are scaled exactly).  bf16 and fp32 have the same
+// exponent range, so P is as accurate at 2^10 as at 1.  A sum beyond 2^60, or below 2^-60 where a row meets its first live key
+// late, is out of the range in which this is safe: the CTA then redoes its list, taking every chunk's maximum first (`exact`).
+//
+// What bounds it (ncu, 2K step with the full mask): exponential pipe 78 %, tensor pipe active 50 %, issue slots 53 %; the rest
+// is the hand-off from P to the next S (arrive, issue of eight MMAs, their execution, commit, wake: 700 cycles a chunk).
+// Measured on B200, with what the kernel with one softmax thread per row and 128-key tiles took before: 2K step with the full
+// mask 5.05 ms (6.71), window 1/4 1.71 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 173 / 81 / 38 us (261 / 116 / 47),
+// 256px step 10 with 960 units 90 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
+// the way: copy look-ups off the MMA lane -4 %, 64-key streams with uniform issue code -12 %, no maxima -12 %; share of the
+// exponentials on the FMA pipe 0 / 25 / 37.5 / 50 %: 1.80 / 1.71 / 1.78 / 1.87 ms; three stages instead of two: +1 %.
+//
+// Every wait on an mbarrier is bounded; when one runs out the CTA raises the plan's status word, drains its copies, frees its
+// TMEM and returns (the softmax warps still arrive for every chunk, so that the named barriers complete).  The element mask, the
+// lists and CFG sharing (second store at batch row b + B) are those of the plan (paper Sections 2 and 3).
 #include <cstring>
 #include <mutex>
 
@@ -41,52 +42,48 @@ using namespace tc;
 
 namespace {
 
-constexpr float kRescaleThreshold = 8.f;  // log2 units: the reference maximum moves when a tile exceeds it by more
+constexpr float kRescaleThreshold = 8.f;  // log2 units: in the second pass the reference moves when a chunk exceeds it by more
+constexpr int kChunkKeys = kBlockN / 2;
+constexpr uint32_t kChunkBytes = kChunkKeys * kHeadDim * 2;
+constexpr int kStages = 2;                // K ring and V ring of a stream
+constexpr int kThreads = 320;             // two streams of four softmax warps, one issuing warp each
+constexpr uint32_t kTmemCols = 256, kColO = 128;  // S (and P over it) of stream s at 64 s, O at 128 + 64 s
 
-template <int NH>
-struct WsCfg {
-  static constexpr int kStages = NH == 2 ? 4 : 2;
-  static constexpr int kThreads = 128 * NH + 128;
-  static constexpr uint32_t kTmemCols = NH == 2 ? 512 : 256;
-  static constexpr int kMinCtas = NH == 2 ? 1 : 2;
-  static constexpr uint32_t kColO = 128 * NH;
-  static constexpr uint32_t kColP = 192 * NH;
-};
+constexpr float kMoveSum = 1024.f;        // a chunk whose probabilities sum to more moves the row's reference
+constexpr float kRedoSum = 1152921504606846976.f;  // 2^60: beyond it the reference was too far off
 
-template <int NH>
 struct WsShared {
-  static constexpr int kStages = WsCfg<NH>::kStages;
-  alignas(1024) uint8_t q[NH][kTileBytes];
-  alignas(1024) uint8_t k[kStages][kTileBytes];
-  alignas(1024) uint8_t v[kStages][kTileBytes];
+  alignas(1024) uint8_t q[kTileBytes];  // Q; at the end the output rows pass through it
+  alignas(1024) uint8_t k[2][kStages][kChunkBytes];
+  alignas(1024) uint8_t v[2][kStages][kChunkBytes];
   alignas(8) uint64_t q_full;
-  uint64_t k_full[kStages], k_free[kStages], v_full[kStages], v_free[kStages];
-  uint64_t s_full[2], s_read[2], p_full[2], pv_done[2];
+  uint64_t k_full[2][kStages], v_full[2][kStages];
+  uint64_t s_full[2], o_full[2];
   uint32_t tmem_base;
-  int abort_flag;
+  int abort_flag, redo;
 };
 
-// Instruction descriptors (kind::f16): D fp32, A/B bf16, M = 128; see the field list in the other kernel.
-constexpr uint32_t kIdescS = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBlockN >> 3) << 17) |
+// Instruction descriptors (kind::f16): D fp32, A/B bf16, M = 128, N = 64; see the field list in the other kernel.
+constexpr uint32_t kIdescS = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kChunkKeys >> 3) << 17) |
                              ((uint32_t)(kBlockM >> 4) << 24);
 constexpr uint32_t kIdescO = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(kHeadDim >> 3) << 17) |
                              ((uint32_t)(kBlockM >> 4) << 24);
 
-// 2^x for x <= 8 on the FMA pipe: x = n + f with n = round(x) and f in [-1/2, 1/2]; 2^f by a cubic fitted to it
-// (relative error 7.5e-5, far inside the bf16 rounding of P), 2^n by adding n to the exponent field.  Scores of
-// dead keys (-inf) are clamped to 2^-125.
-__device__ __forceinline__ float2 exp2_fma2(float2 x) {
-  x.x = fmaxf(x.x, -125.f);
-  x.y = fmaxf(x.y, -125.f);
-  const float2 t = __fadd2_rn(x, make_float2(12582912.f, 12582912.f));  // the integer part in the low mantissa bits
-  const float2 n = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
-  const float2 f = __fadd2_rn(x, make_float2(-n.x, -n.y));
-  float2 y = __ffma2_rn(make_float2(0.05517153441905975f, 0.05517153441905975f), f,
+// 2^x on the FMA pipe for x = score * scale - reference clamped to [-125, 125]: the caller's multiply-add saturates
+// y = (x + 125) / 250 to [0, 1] (dead keys, -inf, give 0).  x = n + f with n = round(x) and f in [-1/2, 1/2]; 2^f by a cubic
+// fitted to it (relative error 7.5e-5, far inside the bf16 rounding of P), 2^n by adding n to the exponent field.
+constexpr float kClamp = 125.f;
+__device__ __forceinline__ float2 exp2_fma2(float2 y) {
+  const float2 range = make_float2(2.f * kClamp, 2.f * kClamp);
+  const float2 t = __ffma2_rn(y, range, make_float2(12582912.f - kClamp, 12582912.f - kClamp));  // n in the low mantissa bits
+  const float2 m = __fadd2_rn(make_float2(12582912.f - kClamp, 12582912.f - kClamp), make_float2(-t.x, -t.y));  // -n - 125
+  const float2 f = __ffma2_rn(y, range, m);
+  float2 z = __ffma2_rn(make_float2(0.05517153441905975f, 0.05517153441905975f), f,
                         make_float2(0.2426111102104187f, 0.2426111102104187f));
-  y = __ffma2_rn(y, f, make_float2(0.6932610273361206f, 0.6932610273361206f));
-  y = __ffma2_rn(y, f, make_float2(0.9999280571937561f, 0.9999280571937561f));
-  return make_float2(__uint_as_float(__float_as_uint(y.x) + (__float_as_uint(t.x) << 23)),
-                     __uint_as_float(__float_as_uint(y.y) + (__float_as_uint(t.y) << 23)));
+  z = __ffma2_rn(z, f, make_float2(0.6932610273361206f, 0.6932610273361206f));
+  z = __ffma2_rn(z, f, make_float2(0.9999280571937561f, 0.9999280571937561f));
+  return make_float2(__uint_as_float(__float_as_uint(z.x) + (__float_as_uint(t.x) << 23)),
+                     __uint_as_float(__float_as_uint(z.y) + (__float_as_uint(t.y) << 23)));
 }
 
 // acc += the two bf16 halves of a packed pair: fp32 additions that take a bf16 operand as it is (no unpacking)
@@ -96,397 +93,398 @@ __device__ __forceinline__ void add_bf16_pair(float2& acc, uint32_t packed) {
       : "r"(packed));
 }
 
-template <int N>
-__device__ __forceinline__ void reg_dec() {
-  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+// One elected lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e != 0u;
 }
-template <int N>
-__device__ __forceinline__ void reg_inc() {
-  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+// mma_ts_x4 / mma_ss_x4 / mma_commit for a converged warp: one elected lane issues
+template <int kAStep, int kBStep>
+__device__ __forceinline__ void mma_ts_x4_one(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                              uint32_t accumulate_first) {
+  if (elect_one()) mma_ts_x4<kAStep, kBStep>(d_tmem, a_tmem, b_desc, idesc, accumulate_first);
+}
+template <int kAStep, int kBStep>
+__device__ __forceinline__ void mma_ss_x4_one(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                              uint32_t accumulate_first) {
+  if (elect_one()) mma_ss_x4<kAStep, kBStep>(d_tmem, a_desc, b_desc, idesc, accumulate_first);
+}
+__device__ __forceinline__ void mma_commit_one(uint64_t* bar) {
+  if (elect_one()) mma_commit(bar);
+}
+__device__ __forceinline__ KeyChunk chunk_at(const KeyChunk* c) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(c));
+  return KeyChunk{v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ void load_chunk(void* dst, const CUtensorMap* raster, const CUtensorMap* patch,
+                                           const KeyChunk& c, int h, int b, uint64_t* bar) {
+  mbar_expect_tx(bar, kChunkBytes);
+  if (c.map_slot < 0)
+    tma_load_4d(dst, raster, 0, c.row, h, b, bar);
+  else
+    tma_load_5d(dst, patch + c.map_slot, 0, c.col, c.row, h, b, bar);
 }
 
-template <int NH>
-__global__ void __launch_bounds__(WsCfg<NH>::kThreads, WsCfg<NH>::kMinCtas)
+__global__ void __launch_bounds__(kThreads, 2)
 fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ FwdParams p, int n_q_tiles) {
-  using C = WsCfg<NH>;
-  constexpr int kStages = C::kStages;
-  extern __shared__ uint8_t smem_raw[];
-  WsShared<NH>& sm = *reinterpret_cast<WsShared<NH>*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int kProducerWarp = 4 * NH, kMmaWarp = 4 * NH + 1, kPvWarp = 4 * NH + 2;
-  int pair_rank, unit;  // grouped launch order, see cta_work
-  cta_work(p, (n_q_tiles + NH - 1) / NH, pair_rank, unit);
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  WsShared& sm = *reinterpret_cast<WsShared*>(smem_raw);
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // warp-uniform
+  const int st = warp < 8 ? warp >> 2 : warp - 8;  // stream
+  int qt, unit;  // grouped launch order, see cta_work
+  cta_work(p, n_q_tiles, qt, unit);
   const int h = unit % p.n_heads, b = unit / p.n_heads;
-  const int qt0 = NH == 2 ? 2 * (p.order ? __ldg(&p.order[pair_rank]) : pair_rank) : pair_rank, qt1 = qt0 + 1;
-  const bool has1 = NH == 2 && qt1 < n_q_tiles;
   volatile int* abort_flag = &sm.abort_flag;
 
-  if (threadIdx.x == kProducerWarp * 32) {
+  if (threadIdx.x == 256) {
     mbar_init(&sm.q_full, 1);
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&sm.k_full[s], 1);
-      mbar_init(&sm.k_free[s], 1);
-      mbar_init(&sm.v_full[s], 1);
-      mbar_init(&sm.v_free[s], 1);
-    }
     for (int i = 0; i < 2; ++i) {
+      for (int s = 0; s < kStages; ++s) {
+        mbar_init(&sm.k_full[i][s], 1);
+        mbar_init(&sm.v_full[i][s], 1);
+      }
       mbar_init(&sm.s_full[i], 1);
-      mbar_init(&sm.s_read[i], 4);
-      mbar_init(&sm.p_full[i], 4);
-      mbar_init(&sm.pv_done[i], 1);
+      mbar_init(&sm.o_full[i], 1);
     }
     sm.abort_flag = 0;
+    sm.redo = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   // the next kernel of the stream may start its set-up while this grid drains; this grid's set-up ran while the
-  // previous one drained.  Nothing an earlier kernel wrote is read before the wait below.
+  // previous one drained.  Nothing an earlier kernel wrote is read before the wait below (the plan is older).
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  __syncthreads();
-  if (threadIdx.x == kProducerWarp * 32) {  // Q of every half: needs nothing from the plan
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    mbar_expect_tx(&sm.q_full, has1 ? 2 * kTileBytes : kTileBytes);
-    load_q_tile(sm.q[0], tm, p, qt0, h, b, &sm.q_full);
-    if (has1) load_q_tile(sm.q[NH - 1], tm, p, qt1, h, b, &sm.q_full);
-    if (p.first_tile_zero) {  // key tile 0 (cache rows [0,128), raster) heads every list: no look-up needed
-      mbar_expect_tx(&sm.k_full[0], kTileBytes);
-      tma_load_4d(sm.k[0], &tm.kr, 0, 0, h, b, &sm.k_full[0]);
-      mbar_expect_tx(&sm.v_full[0], kTileBytes);
-      tma_load_4d(sm.v[0], &tm.vr, 0, 0, h, b, &sm.v_full[0]);
-    }
-  }
-  if (warp == kMmaWarp) {
+  if (warp == 8) {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem_base)),
-                 "r"(C::kTmemCols)
+                 "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   const SetDesc sd = p.head_to_set ? p.sets[p.head_to_set[h]] : p.set0;
-  const int beg0 = __ldg(&sd.row_ptr[qt0]), end0 = __ldg(&sd.row_ptr[qt0 + 1]);
-  const int beg1 = end0, end1 = has1 ? __ldg(&sd.row_ptr[qt1 + 1]) : end0;
+  const int n_all = __ldg(&sd.n_chunks[qt]);
+  const int n = (n_all - st + 1) >> 1;  // this stream's chunks: st, st + 2, ...
+  const KeyChunk* chunks = sd.chunks + 2 * (size_t)__ldg(&sd.row_ptr[qt]) + st;
   tc_fence_before();
-  __syncthreads();  // TMEM address
+  __syncthreads();  // barriers, TMEM address
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
 
-  if (warp >= 4 * NH) {
-    reg_dec<56>();
-    if (warp == kProducerWarp && lane == 0 && end1 <= beg0) {
-      // nothing listed for this CTA: only the Q copies are in flight; wait for them (bounded) before leaving
-      const unsigned long long ts = global_ns();
-      while (!mbar_try(&sm.q_full, 0u))
-        if (global_ns() - ts > kWaitLimitNs) break;
-    } else if (warp == kProducerWarp && lane == 0) {
-      // ---------------------------------------------------------------- TMA producer
-      UnionWalk pw;
-      pw.init(sd.pairs, beg0, end0, beg1, end1);
-      int issued = 0;
-      if (p.first_tile_zero) {  // item 0 is already on its way
-        bool l0, l1;
-        (void)pw.next(l0, l1);
-        issued = 1;
+  bool exact = false;  // second pass over the list, every chunk's maximum taken before its probabilities
+  for (int base = 0;; base += n) {  // step counter of the pass's first chunk: barrier phases go on from pass to pass
+    const int end = base + n;
+    if (warp >= 8) {
+      // ---------------------------------------------------------------- copies and MMAs of the stream.  The whole warp runs
+      // this code (what it computes is uniform, so that descriptors and coordinates live in uniform registers); one
+      // elected lane issues.  P(i) complete is the event to wait for: PV(i) and S(i + 1) are issued back to back (they
+      // execute in issue order, so that S may overwrite P).
+      const uint64_t q_desc = make_desc(smem_u32(sm.q)), k_desc0 = make_desc(smem_u32(sm.k[st][0]));
+      const uint64_t v_desc0 = make_desc(smem_u32(sm.v[st][0]));
+      const uint32_t tS = tmem + 64 * st, tO = tmem + kColO + 64 * st;
+      auto chunk = [&](int i) { return chunk_at(chunks + 2 * min(i, n - 1)); };
+      KeyChunk c_k = {}, c_v = {};  // what the next K and V copy takes; looked up a step ahead
+      int nk = base, nv = base;     // copies issued
+      auto load_k = [&](const KeyChunk& c) {
+        if (elect_one()) load_chunk(sm.k[st][nk % kStages], &tm.kr, tm.k2, c, h, b, &sm.k_full[st][nk % kStages]);
+        ++nk;
+      };
+      auto load_v = [&](const KeyChunk& c) {
+        if (elect_one()) load_chunk(sm.v[st][nv % kStages], &tm.vr, tm.v2, c, h, b, &sm.v_full[st][nv % kStages]);
+        ++nv;
+      };
+      if (n > 0) c_k = chunk(0);
+      if (!exact) asm volatile("griddepcontrol.wait;" ::: "memory");
+      if (st == 0 && elect_one()) {
+        mbar_expect_tx(&sm.q_full, kTileBytes);
+        load_q_tile(sm.q, tm, p, qt, h, b, &sm.q_full);
       }
-      for (int i = issued; pw.has(); ++i) {
-        bool l0, l1;
-        const int kt = pw.next(l0, l1);
-        const int s = i % kStages, n = i / kStages;
-        if (n > 0 && !mbar_wait_inl(&sm.k_free[s], (uint32_t)((n - 1) & 1), abort_flag, p.status)) break;
-        mbar_expect_tx(&sm.k_full[s], kTileBytes);
-        load_kv_tile(sm.k[s], &tm.kr, tm.k2, p, kt, h, b, &sm.k_full[s]);
-        if (n > 0 && !mbar_wait_inl(&sm.v_free[s], (uint32_t)((n - 1) & 1), abort_flag, p.status)) {
-          const unsigned long long ts = global_ns();  // the K copy just issued is still in flight
-          while (!mbar_try(&sm.k_full[s], (uint32_t)(n & 1)))
-            if (global_ns() - ts > kWaitLimitNs) break;
-          break;
+      for (int i = 0; i < kStages && i < n; ++i) {
+        const KeyChunk c_next = chunk(i + 1);
+        load_k(c_k);
+        load_v(c_k);
+        c_k = c_v = c_next;
+      }
+      bool ok = mbar_wait_long(&sm.q_full, exact ? 1u : 0u, abort_flag, p.status);
+      for (int i = base - 1; i < end && n > 0; ++i) {
+        const int s = i % kStages, s1 = (i + 1) % kStages;
+        if (ok && i + 1 < end) ok = mbar_wait_long(&sm.k_full[st][s1], (uint32_t)(((i + 1) / kStages) & 1), abort_flag, p.status);
+        if (i >= base) {
+          if (ok) ok = mbar_wait_long(&sm.v_full[st][s], (uint32_t)((i / kStages) & 1), abort_flag, p.status);
+          __syncwarp();
+          asm volatile("bar.sync %0, 160;" ::"r"(5 + st) : "memory");  // P(i); the softmax warps arrive even when a wait ran out
         }
-        mbar_expect_tx(&sm.v_full[s], kTileBytes);
-        load_kv_tile(sm.v[s], &tm.vr, tm.v2, p, kt, h, b, &sm.v_full[s]);
-        issued = i + 1;
-      }
-      if (*abort_flag) {  // wait (bounded) for copies still in flight before the CTA may exit
-        const unsigned long long ts = global_ns();
-        while (!mbar_try(&sm.q_full, 0u))
-          if (global_ns() - ts > kWaitLimitNs) break;
-        for (int i = issued > kStages ? issued - kStages : 0; i < issued; ++i) {
-          const int s = i % kStages, n = i / kStages;
-          while (!(mbar_try(&sm.k_full[s], (uint32_t)(n & 1)) && mbar_try(&sm.v_full[s], (uint32_t)(n & 1))))
-            if (global_ns() - ts > 2 * kWaitLimitNs) break;
-        }
-      }
-    } else if (warp == kMmaWarp && lane == 0 && end1 > beg0) {
-      // ---------------------------------------------------------------- issuer of the score products
-      const uint64_t q_desc[2] = {make_desc(smem_u32(sm.q[0])), make_desc(smem_u32(sm.q[NH - 1]))};
-      const uint64_t k_desc0 = make_desc(smem_u32(sm.k[0]));
-      UnionWalk w;
-      w.init(sd.pairs, beg0, end0, beg1, end1);
-      bool ok = mbar_wait_inl(&sm.q_full, 0u, abort_flag, p.status);
-      int n_s[2] = {0, 0};  // products issued so far per half
-      for (int i = 0; ok && w.has(); ++i) {
-        bool live[2] = {false, false};
-        const int s = i % kStages;
-        (void)w.next(live[0], live[1]);
-        if (!(ok = mbar_wait_inl(&sm.k_full[s], (uint32_t)((i / kStages) & 1), abort_flag, p.status))) break;
-        tc_fence_after();
-        const uint64_t k_desc = k_desc0 + (uint64_t)((kTileBytes >> 4) * s);
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          if (!live[hh]) continue;
-          if (n_s[hh] > 0) {  // the softmax threads have read the previous S_hh
-            if (!(ok = mbar_wait_inl(&sm.s_read[hh], (uint32_t)((n_s[hh] - 1) & 1), abort_flag, p.status))) break;
-            tc_fence_after();
-          }
-          // 16 bf16 = 32 B per step inside the swizzle rows of Q and K
-          mma_ss_x4<2, 2>(tmem + 128 * hh, q_desc[hh], k_desc, kIdescS, 0u);
-          mma_commit(&sm.s_full[hh]);
-          ++n_s[hh];
-        }
-        if (!ok) break;
-        mma_commit(&sm.k_free[s]);
-      }
-    } else if (warp == kPvWarp && lane == 0 && end1 > beg0) {
-      // ---------------------------------------------------------------- issuer of the PV products
-      const uint64_t v_desc0 = make_desc(smem_u32(sm.v[0]));
-      UnionWalk w;
-      w.init(sd.pairs, beg0, end0, beg1, end1);
-      bool ok = true;
-      int n_pv[2] = {0, 0};
-      for (int i = 0; ok && w.has(); ++i) {
-        bool live[2] = {false, false};
-        const int s = i % kStages;
-        (void)w.next(live[0], live[1]);
-        const uint64_t v_desc = v_desc0 + (uint64_t)((kTileBytes >> 4) * s);
-        bool v_ready = false;
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          if (!live[hh]) continue;
-          if (!(ok = mbar_wait_inl(&sm.p_full[hh], (uint32_t)(n_pv[hh] & 1), abort_flag, p.status))) break;
-          if (!v_ready) {
-            if (!(ok = mbar_wait_inl(&sm.v_full[s], (uint32_t)((i / kStages) & 1), abort_flag, p.status))) break;
-            v_ready = true;
-          }
+        if (ok) {
           tc_fence_after();
-          // 16 keys per step = 16 rows of 128 B = 2048 B of V and 8 packed columns of P
-          mma_ts_x4<8, (2048 >> 4)>(tmem + C::kColO + kHeadDim * hh, tmem + C::kColP + 64 * hh, v_desc, kIdescO,
-                                    n_pv[hh] > 0 ? 1u : 0u);
-          mma_ts_x4<8, (2048 >> 4)>(tmem + C::kColO + kHeadDim * hh, tmem + C::kColP + 64 * hh + 32,
-                                    v_desc + 4 * (uint64_t)(2048 >> 4), kIdescO, 1u);
-          mma_commit(&sm.pv_done[hh]);
-          ++n_pv[hh];
+          if (i >= base) {
+            // 16 keys per step = 16 rows of 128 B = 2048 B of V and 8 packed columns of P
+            mma_ts_x4_one<8, (2048 >> 4)>(tO, tS, v_desc0 + (uint64_t)((kChunkBytes >> 4) * s), kIdescO, i > base ? 1u : 0u);
+          }
+          if (i + 1 < end) {
+            // 16 bf16 = 32 B per step inside the swizzle rows of Q and K
+            mma_ss_x4_one<2, 2>(tS, q_desc, k_desc0 + (uint64_t)((kChunkBytes >> 4) * s1), kIdescS, 0u);
+            mma_commit_one(&sm.s_full[st]);
+          } else {
+            mma_commit_one(&sm.o_full[st]);
+          }
+          // P(i) was complete, so S(i) and PV(i - 1) are: K(i + stages) and V(i - 1 + stages) go where K(i) and V(i - 1) were
+          if (i > base && nv < end) load_v(c_v);
+          if (i >= base && nk < end) {
+            load_k(c_k);
+            c_v = c_k;
+            c_k = chunk(nk - base);
+          }
+          __syncwarp();
         }
-        if (!ok) break;
-        mma_commit(&sm.v_free[s]);
       }
-    }
-  } else {
-    // ------------------------------------------------------------------ softmax + epilogue of one half
-    if constexpr (NH == 2) reg_inc<224>(); else reg_inc<200>();
-    const int hh = warp >> 2;
-    const int qt = hh ? qt1 : qt0;
-    const int pbeg = hh ? beg1 : beg0;
-    const int n_tiles = (hh ? end1 : end0) - pbeg;
-    if (n_tiles > 0) {
-      const int lane_group = warp & 3;  // TMEM lanes this warp may touch: 32 * lane_group .. + 31
+      if (*abort_flag || n <= 0) {  // wait (bounded) for copies still in flight before the CTA may exit
+        const unsigned long long ts = global_ns();
+        while (!mbar_try(&sm.q_full, exact ? 1u : 0u))
+          if (global_ns() - ts > kWaitLimitNs) break;
+        for (int i = nk > kStages ? nk - kStages : 0; i < nk; ++i)
+          while (!mbar_try(&sm.k_full[st][i % kStages], (uint32_t)((i / kStages) & 1)))
+            if (global_ns() - ts > 2 * kWaitLimitNs) break;
+        for (int i = nv > kStages ? nv - kStages : 0; i < nv; ++i)
+          while (!mbar_try(&sm.v_full[st][i % kStages], (uint32_t)((i / kStages) & 1)))
+            if (global_ns() - ts > 2 * kWaitLimitNs) break;
+      }
+    } else {
+      // ---------------------------------------------------------------- softmax + epilogue
+      const int lane_group = warp & 3;  // TMEM lanes 32 lane_group .. + 31
       const int m = lane_group * 32 + lane;
       const uint32_t tlane = tmem + ((uint32_t)(lane_group * 32) << 16);
-      const uint32_t tS = tlane + 128 * hh;
-      const uint32_t tO = tlane + C::kColO + kHeadDim * hh;
-      const uint32_t tP = tlane + C::kColP + 64 * hh;
-      bool ok = true;
+      const uint32_t tS = tlane + 64 * st, tO = tlane + kColO + 64 * st;
       const float sc = p.sm_scale * 1.4426950408889634f;
       const float2 sc2 = make_float2(sc, sc);
-      float row_max = -INFINITY;  // the score the stored probabilities refer to
-      float2 l2a = make_float2(0.f, 0.f), l2b = make_float2(0.f, 0.f);  // row sum of the probabilities
-      Pair pr = sd.pairs[pbeg];
-      uint4 mk = make_uint4(~0u, ~0u, ~0u, ~0u);
-      if (pr.mask_block >= 0) mk = __ldg(&sd.mask[(size_t)pr.mask_block * kBlockM + m]);
-      for (int j = 0; ok && j < n_tiles; ++j) {
-        Pair pr_next = pr;  // next pair's mask words travel while this tile is processed
-        uint4 mk_next = make_uint4(~0u, ~0u, ~0u, ~0u);
-        if (j + 1 < n_tiles) {
-          pr_next = sd.pairs[pbeg + j + 1];
-          if (pr_next.mask_block >= 0) mk_next = __ldg(&sd.mask[(size_t)pr_next.mask_block * kBlockM + m]);
+      const float sc_y = sc * (0.5f / kClamp);
+      // probabilities are 2^(score * sc - msc).  msc starts as the first live chunk's maximum and moves by whole powers of two
+      // when a chunk's sum gets large; it stays 0 and `none` until a live chunk has been seen.
+      float msc = 0.f;
+      bool none = true;
+      float alpha = 1.f;  // pending factor of the accumulator
+      float2 l2a = make_float2(0.f, 0.f), l2b = make_float2(0.f, 0.f);  // row sum
+      bool bad = false, ok = true;
+      const uint2* mask2 = reinterpret_cast<const uint2*>(sd.mask) + 2 * m;
+      auto mask_at = [&](int blk) {
+        return blk >= 0 ? __ldg(mask2 + (size_t)(blk >> 1) * (2 * kBlockM) + (blk & 1)) : make_uint2(~0u, ~0u);
+      };
+      const int* blocks = &chunks->mask;  // four ints per chunk, every second one is this stream's
+      int blk = n > 0 ? __ldg(blocks) : -1, blk_next = n > 1 ? __ldg(blocks + 8) : -1;
+      uint2 mk = mask_at(blk), mk_next = mask_at(blk_next);
+      // chunks without a live key for any row of the warp are skipped (uniform over the warp)
+      bool live = blk < 0 || __any_sync(0xffffffffu, (mk.x | mk.y) != 0u);
+      bool rescale = false;  // some row of the warp has a pending alpha
+      float l_seen = 0.f;     // row sum before this chunk
+      for (int j = 0; j < n; ++j) {
+        const bool partial = blk >= 0;
+        // S(j) complete; in issue order this also means that PV(j - 1) is complete
+        if (ok) ok = mbar_wait_long(&sm.s_full[st], (uint32_t)((base + j) & 1), abort_flag, p.status);
+        if (!ok) {  // the issuing warp counts on every step's arrival
+          asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
+          continue;
         }
-        const bool partial = pr.mask_block >= 0;
-        // S_hh(j) complete
-        if (!(ok = mbar_wait_inl(&sm.s_full[hh], (uint32_t)(j & 1), abort_flag, p.status))) break;
         tc_fence_after();
-        // The tile is taken in two passes of 64 keys through ONE copy of the code (the loop below is kept rolled:
-        // an unrolled 128-key body is some 30 KB of instructions, and two warps per scheduler streaming that
-        // through the instruction caches ran at a third of the speed the same arithmetic reaches in a small
-        // loop).  The probabilities refer to the running reference row_max, which a pass moves only when its own
-        // maximum exceeds it by more than the threshold.  When the second pass moves it, the P written by the
-        // first pass refers to the old reference: the tile is then simply redone (first pass without adding to
-        // the row sum, which has been rescaled with the accumulator); S stays in TMEM until the tile is finished.
-        bool pv_seen = j == 0;   // PV product of the previous tile complete: its P block is free, O_hh at rest
-        bool redo = false;
+        if (j == 0 || exact) {  // the maximum first
+          float mx = -INFINITY;
+          if (live) {
 #pragma unroll 1
-        for (int hf = 0; hf < 2; ++hf) {
-          const uint32_t w0 = hf ? mk.z : mk.x, w1 = hf ? mk.w : mk.y;
-          // keys without a live key for any row of the warp are skipped (uniform over the warp)
-          const bool live_h = !partial || __any_sync(0xffffffffu, (w0 | w1) != 0u);
-          uint32_t pk[32];
-          if (live_h) {
-            uint32_t r[64];
-            tmem_ld32(tS + 64 * hf, r);
-            tmem_ld32(tS + 64 * hf + 32, r + 32);
+            for (int hf = 0; hf < 2; ++hf) {
+              const uint32_t w = hf ? mk.y : mk.x;
+              uint32_t r[32];
+              tmem_ld32(tS + 32 * hf, r);
+              tmem_wait_ld();
+#pragma unroll
+              for (int e = 0; e < 32; ++e) mx = fmaxf(mx, (w >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
+            }
+          }
+          if (mx != -INFINITY && (none || mx * sc - msc > kRescaleThreshold)) {
+            if (!none) {
+              alpha *= fast_exp2(msc - mx * sc);
+              l2a.x *= alpha; l2a.y *= alpha; l2b.x *= alpha; l2b.y *= alpha;
+            }
+            msc = mx * sc;
+            none = false;
+          }
+          rescale = __any_sync(0xffffffffu, alpha != 1.f);
+        }
+        if (rescale) {  // the accumulator follows the reference
+#pragma unroll 1
+          for (int c = 0; c < 4; ++c) {
+            uint32_t o[16];
+            tmem_ld16(tO + 16 * c, o);
+            tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+            tmem_st16(tO + 16 * c, o);
+          }
+          alpha = 1.f;
+        }
+        if (live) {
+#pragma unroll 1
+          for (int hf = 0; hf < 2; ++hf) {
+            uint32_t r[32], pk[16];
+            tmem_ld32(tS + 32 * hf, r);
             tmem_wait_ld();
             if (partial) {  // dead scores of a partially live pair become -inf
+              const uint32_t w = hf ? mk.y : mk.x;
 #pragma unroll
-              for (int e = 0; e < 32; ++e) {
-                if (!((w0 >> e) & 1u)) r[e] = 0xff800000u;
-                if (!((w1 >> e) & 1u)) r[32 + e] = 0xff800000u;
-              }
-            }
-            if (!redo) {
-              float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-              for (int e = 0; e < 64; e += 8) {
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                  mx[u] = max3(mx[u], __uint_as_float(r[e + 2 * u]), __uint_as_float(r[e + 2 * u + 1]));
-              }
-              const float pass_max = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-              // false for pass_max = -inf (no live key in this row), true for row_max = -inf (first live key)
-              const bool moved = (pass_max - row_max) * sc > kRescaleThreshold;
-              if (__any_sync(0xffffffffu, moved)) {
-                float alpha = 1.f;
-                if (moved) {
-                  if (row_max != -INFINITY) alpha = fast_exp2((row_max - pass_max) * sc);
-                  row_max = pass_max;
-                }
-                if (__any_sync(0xffffffffu, alpha != 1.f)) {  // accumulator and row sum follow the reference
-                  if (!pv_seen) {
-                    if (!(ok = mbar_wait_inl(&sm.pv_done[hh], (uint32_t)((j - 1) & 1), abort_flag, p.status))) break;
-                    tc_fence_after();
-                    pv_seen = true;
-                  }
-                  if (j > 0) {
-#pragma unroll 1
-                    for (int c = 0; c < kHeadDim / 16; ++c) {
-                      uint32_t o[16];
-                      tmem_ld16(tO + 16 * c, o);
-                      tmem_wait_ld();
-#pragma unroll
-                      for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-                      tmem_st16(tO + 16 * c, o);
-                    }
-                  }
-                  l2a.x *= alpha; l2a.y *= alpha; l2b.x *= alpha; l2b.y *= alpha;
-                  if (hf == 1) {  // the first pass wrote P against the old reference: redo the tile
-                    redo = true;
-                    hf = -1;
-                    continue;
-                  }
-                }
-              }
-            }
-            if (hf == 1) {  // every score of the tile has been read and no redo is pending: release the S block
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(&sm.s_read[hh]);
+              for (int e = 0; e < 32; ++e)
+                if (!((w >> e) & 1u)) r[e] = 0xff800000u;
             }
             // probabilities against the reference: scale and shift (packed FMAs), 2^x, row sum, bf16
-            const float msc = row_max == -INFINITY ? 0.f : row_max * sc;
             const float2 nm2 = make_float2(-msc, -msc);
-            const bool add_sum = !(redo && hf == 0);
+            const float nm_y = fmaf(-msc, 0.5f / kClamp, 0.5f);
 #pragma unroll
-            for (int e = 0; e < 64; e += 4) {
-              const float2 xa = __ffma2_rn(make_float2(__uint_as_float(r[e + 0]), __uint_as_float(r[e + 1])), sc2, nm2);
-              const float2 xb = __ffma2_rn(make_float2(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3])), sc2, nm2);
+            for (int e = 0; e < 32; e += 4) {
+              const uint32_t* rr = r + e;
+              const float2 xa = __ffma2_rn(make_float2(__uint_as_float(rr[0]), __uint_as_float(rr[1])), sc2, nm2);
               const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
-              // every fourth pair on the FMA pipe: the exponential pipe (16 per clock and SM) is what a pass waits for
-              const float2 pb = (e & 4) ? exp2_fma2(xb) : make_float2(fast_exp2(xb.x), fast_exp2(xb.y));
+              // every fourth pair on the FMA pipe: the exponential pipe (16 per clock and SM) is the tighter of the two
+              float2 pb;
+              if (e & 4) {
+                pb = exp2_fma2(make_float2(__saturatef(fmaf(__uint_as_float(rr[2]), sc_y, nm_y)),
+                                           __saturatef(fmaf(__uint_as_float(rr[3]), sc_y, nm_y))));
+              } else {
+                const float2 xb = __ffma2_rn(make_float2(__uint_as_float(rr[2]), __uint_as_float(rr[3])), sc2, nm2);
+                pb = make_float2(fast_exp2(xb.x), fast_exp2(xb.y));
+              }
               // the row sum adds the probabilities as the PV product sees them (rounded to bf16): numerator and
               // denominator of a row then agree, and a row with one dominant key reproduces that key's V exactly
               const uint32_t ka = pack_bf16(pa.x, pa.y), kb = pack_bf16(pb.x, pb.y);
-              if (add_sum) {
-                add_bf16_pair(l2a, ka);
-                add_bf16_pair(l2b, kb);
-              }
+              add_bf16_pair(l2a, ka);
+              add_bf16_pair(l2b, kb);
               pk[(e >> 1) + 0] = ka;
               pk[(e >> 1) + 1] = kb;
             }
-          } else {
-            if (hf == 1) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(&sm.s_read[hh]);
-            }
+            tmem_st16(tS + 16 * hf, pk);  // over scores that have been read
+          }
+        } else {
+          uint32_t pk[16];
 #pragma unroll
-            for (int e = 0; e < 32; ++e) pk[e] = 0u;
-          }
-          if (!pv_seen) {
-            if (!(ok = mbar_wait_inl(&sm.pv_done[hh], (uint32_t)((j - 1) & 1), abort_flag, p.status))) break;
-            tc_fence_after();
-            pv_seen = true;
-          }
-          tmem_st32(tP + 32 * hf, pk);
+          for (int e = 0; e < 16; ++e) pk[e] = 0u;
+          tmem_st16(tS, pk);
+          tmem_st16(tS + 16, pk);
         }
-        if (!ok) break;
         tmem_wait_st();  // P and, where it was rescaled, the accumulator
         tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.p_full[hh]);
-        pr = pr_next;
-        mk = mk_next;
-      }
-      // the last PV product of this half (all earlier ones are complete by issue order)
-      if (ok && (ok = mbar_wait_inl(&sm.pv_done[hh], (uint32_t)((n_tiles - 1) & 1), abort_flag, p.status))) {
-        tc_fence_after();
-        uint32_t r[64];
-        tmem_ld32(tO, r);
-        tmem_ld32(tO + 32, r + 32);
-        tmem_wait_ld();
-        const float inv = 1.f / ((l2a.x + l2a.y) + (l2b.x + l2b.y));
-        TileGeom g = TileGeom{-1, qt * kBlockM, 0, 0};
-        if (p.q_geom != nullptr) g = p.q_geom[qt];
-        int q;  // this slot's token (-1: padding slot)
-        if (g.scale < 0) {
-          q = g.a + m;
-        } else {
-          const int qr = g.a + m / kPatchCols, qc = g.b + m % kPatchCols;
-          q = (qr < p.s_k && qc < p.s_k) ? qr * p.s_k + qc : -1;
+        asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
+        // the rest runs while the products of the next step do: the reference, which moves for the next chunk when this one
+        // exceeded it, and the next chunk's masks (the words of the one after it start travelling)
+        if (!exact) {
+          const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y), grown = l - l_seen;
+          const bool seen = blk < 0 || (mk.x | mk.y) != 0u;  // a live key in this row
+          if (!(grown <= kMoveSum) || (none && seen)) {  // (a NaN goes this way too)
+            bad |= !(grown < kRedoSum && grown > 1.f / kRedoSum);
+            none = false;
+            if (j + 1 < n) {
+              const int ex = (int)(__float_as_uint(grown) >> 23) - 127;  // floor(log2(grown))
+              alpha = __uint_as_float((uint32_t)(127 - ex) << 23);
+              msc += (float)ex;
+              l2a.x *= alpha; l2a.y *= alpha; l2b.x *= alpha; l2b.y *= alpha;
+            }
+          }
+          l_seen = (l2a.x + l2a.y) + (l2b.x + l2b.y);
         }
-        if (q >= 0 && q < p.n_k) {
-          uint16_t* dst = p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + (int64_t)q * p.o_st;
+        rescale = __any_sync(0xffffffffu, alpha != 1.f);
+        blk = blk_next;
+        mk = mk_next;
+        blk_next = j + 2 < n ? __ldg(blocks + 8 * (j + 2)) : -1;
+        live = blk < 0 || __any_sync(0xffffffffu, (mk.x | mk.y) != 0u);
+        mk_next = mask_at(blk_next);
+      }
+      if (!exact && __any_sync(0xffffffffu, bad) && lane == 0) sm.redo = 1;
+      // the last PV product (all earlier ones are complete by issue order)
+      if (ok && n > 0) ok = mbar_wait_long(&sm.o_full[st], exact ? 1u : 0u, abort_flag, p.status);
+      const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y);
+      const float own = none ? -INFINITY : msc;  // (dead keys leave traces of 2^-125 in l)
+      reinterpret_cast<float2*>(sm.k[st][0])[m] = make_float2(own, l);  // the stream's stages are idle
+      tc_fence_before();
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + lane_group) : "memory");  // the warp with the other stream of these rows
+      tc_fence_after();
+      if (ok && n_all > 0) {
+        const float2 other = reinterpret_cast<const float2*>(sm.k[st ^ 1][0])[m];
+        const float top = fmaxf(own, other.x);
+        const float f_own = fast_exp2(own - top), f_other = fast_exp2(other.x - top);
+        const float inv = 1.f / (l * f_own + other.y * f_other);
+        const float w0 = (st ? f_other : f_own) * inv, w1 = (st ? f_own : f_other) * inv;
+        // output columns [32 st, 32 st + 32) of this thread's row: both streams' accumulators, weighted (a stream
+        // without a live key has weight 0 and an accumulator that may never have been written)
+        uint32_t r[32], r1[32];
+        tmem_ld32(tlane + kColO + 32 * st, r);
+        tmem_ld32(tlane + kColO + 64 + 32 * st, r1);
+        tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < 64; e += 8) {
-            uint4 o4;
-            o4.x = pack_bf16(__uint_as_float(r[e + 0]) * inv, __uint_as_float(r[e + 1]) * inv);
-            o4.y = pack_bf16(__uint_as_float(r[e + 2]) * inv, __uint_as_float(r[e + 3]) * inv);
-            o4.z = pack_bf16(__uint_as_float(r[e + 4]) * inv, __uint_as_float(r[e + 5]) * inv);
-            o4.w = pack_bf16(__uint_as_float(r[e + 6]) * inv, __uint_as_float(r[e + 7]) * inv);
-            *reinterpret_cast<uint4*>(dst + e) = o4;
-            if (p.share_offset > 0) *reinterpret_cast<uint4*>(dst + (int64_t)p.share_offset * p.o_sb + e) = o4;
+        for (int e = 0; e < 32; ++e)
+          r[e] = __float_as_uint((w0 > 0.f ? __uint_as_float(r[e]) * w0 : 0.f) + (w1 > 0.f ? __uint_as_float(r1[e]) * w1 : 0.f));
+        // The warp's 32 rows x 64 B pass through its own 2 KB slice of the Q buffer (its last reader, the last score
+        // product, is done: every warp of both streams has seen it through o_full), so that four neighbouring lanes store one
+        // row's 64 contiguous bytes.  Chunk position XOR (row / 2) keeps both the writes and the reads free of bank conflicts.
+        uint8_t* slice = sm.q + (warp << 11);
+#pragma unroll
+        for (int e = 0; e < 32; e += 8) {
+          uint4 o4;
+          o4.x = pack_bf16(__uint_as_float(r[e + 0]), __uint_as_float(r[e + 1]));
+          o4.y = pack_bf16(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
+          o4.z = pack_bf16(__uint_as_float(r[e + 4]), __uint_as_float(r[e + 5]));
+          o4.w = pack_bf16(__uint_as_float(r[e + 6]), __uint_as_float(r[e + 7]));
+          *reinterpret_cast<uint4*>(slice + lane * 64 + ((((e >> 3) ^ (lane >> 1)) & 3) << 4)) = o4;
+        }
+        __syncwarp();
+        TileGeom tg = TileGeom{-1, qt * kBlockM, 0, 0};
+        if (p.q_geom != nullptr) tg = p.q_geom[qt];
+        uint16_t* obase = p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + 32 * st;
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+          const int rl = it * 8 + (lane >> 2), ch = lane & 3;  // row of the warp's 32, 16-byte chunk of its 64 bytes
+          const int mm = lane_group * 32 + rl;                  // query slot of that row
+          int q;                                                // its token (-1: padding slot)
+          if (tg.scale < 0) {
+            q = tg.a + mm;
+          } else {
+            const int qr = tg.a + mm / kPatchCols, qc = tg.b + mm % kPatchCols;
+            q = (qr < p.s_k && qc < p.s_k) ? qr * p.s_k + qc : -1;
+          }
+          const uint4 o4 = *reinterpret_cast<const uint4*>(slice + rl * 64 + (((ch ^ (rl >> 1)) & 3) << 4));
+          if (q >= 0 && q < p.n_k) {
+            uint16_t* dst = obase + (int64_t)q * p.o_st + 8 * ch;
+            *reinterpret_cast<uint4*>(dst) = o4;
+            if (p.share_offset > 0) *reinterpret_cast<uint4*>(dst + (int64_t)p.share_offset * p.o_sb) = o4;
           }
         }
       }
     }
+    tc_fence_before();
+    __syncwarp();
+    __syncthreads();
+    tc_fence_after();
+    if (exact || !*(volatile int*)&sm.redo || *abort_flag) break;
+    exact = true;
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // Q is copied again over the output rows
+    __syncthreads();
   }
 
   // ---------------------------------------------------------------------- teardown (all paths)
-  tc_fence_before();
-  __syncthreads();
-  if (warp == kMmaWarp) {
+  if (warp == 8) {
     __syncwarp();
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::kTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
 }
 
-template <int NH>
-litevar_status_t launch_ws_variant(const TensorMaps& tm, const FwdParams& p, int n_q_tiles, cudaStream_t stream) {
+}  // namespace
+
+litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream_t stream) {
+  TensorMaps tm;
+  if (!encode_tensor_maps(p, &tm, kChunkKeys)) return LITEVAR_ERR_INVALID_ARG;
   static std::once_flag attr_once;
   static cudaError_t attr_err = cudaSuccess;
-  constexpr int smem_bytes = (int)sizeof(WsShared<NH>) + 1024;
+  constexpr int smem_bytes = (int)sizeof(WsShared);
   std::call_once(attr_once, [] {
-    attr_err = cudaFuncSetAttribute(fwd_ws_kernel<NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    attr_err = cudaFuncSetAttribute(fwd_ws_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   });
   if (attr_err != cudaSuccess) return LITEVAR_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((n_q_tiles + NH - 1) / NH) * (unsigned)p.n_heads * (unsigned)p.batch_computed);
-  cfg.blockDim = dim3(WsCfg<NH>::kThreads);
+  cfg.gridDim = dim3((unsigned)n_q_tiles * (unsigned)p.n_heads * (unsigned)p.batch_computed);
+  cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -494,23 +492,11 @@ litevar_status_t launch_ws_variant(const TensorMaps& tm, const FwdParams& p, int
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = p.overlap_launch ? 1 : 0;
-  if (cudaLaunchKernelEx(&cfg, fwd_ws_kernel<NH>, tm, p, n_q_tiles) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, fwd_ws_kernel, tm, p, n_q_tiles) != cudaSuccess) {
     (void)cudaGetLastError();
     return LITEVAR_ERR_CUDA;
   }
   return LITEVAR_OK;
-}
-
-}  // namespace
-
-litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream_t stream) {
-  TensorMaps tm;
-  if (!encode_tensor_maps(p, &tm)) return LITEVAR_ERR_INVALID_ARG;
-  // One query tile per CTA, two CTAs per SM: measured on B200 against the two-tile build of the same kernel (one
-  // CTA per SM, K/V staged once for both tiles) it is 2 % faster on the full-mask 2K step and 4 % faster on the
-  // windowed one, where the union of two tiles' lists also executes pairs that only one of them lists.  Two
-  // independent CTAs drift apart, so that one's loads, masks and maxima fall under the other's exponentials.
-  return launch_ws_variant<1>(tm, p, n_q_tiles, stream);
 }
 
 }  // namespace litevar

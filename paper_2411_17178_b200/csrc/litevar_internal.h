@@ -47,11 +47,20 @@ struct SmallLists {
   Pair pr[2];
 };
 
+// One 64-key half of a live pair that holds a live entry: where its K and V rows are and which mask words it has.
+struct alignas(16) KeyChunk {  // read with one 16-byte load
+  int32_t row, col;   // raster (map_slot < 0): first cache row; patch: first grid row and column of a 4 x 16 half patch
+  int32_t map_slot;   // tensor maps of the key scale (patch), -1: raster
+  int32_t mask;       // 2 * mask block + half, -1: every slot pair is live
+};
+
 // Device-visible tile plan of one (step, window set).
 struct SetDesc {
   const int32_t* row_ptr;  // [n_q_tiles + 1]
   const Pair* pairs;       // [n_pairs]
   const uint4* mask;       // [n_partial][kBlockM] : 128 key bits per query slot
+  const KeyChunk* chunks;  // live halves of query tile i's pairs, from 2 * row_ptr[i] on
+  const int32_t* n_chunks; // [n_q_tiles] how many
 };
 
 struct StepSet {
@@ -60,6 +69,8 @@ struct StepSet {
   int32_t* d_row_ptr = nullptr;
   Pair* d_pairs = nullptr;
   uint4* d_mask = nullptr;
+  KeyChunk* d_chunks = nullptr;   // [2 * n_pairs]
+  int32_t* d_n_chunks = nullptr;  // [n_q_tiles]
   int2* d_bounds = nullptr;  // [k][s_k] {lo, hi} per key scale and query row/column (SQUARE)
   bool first_tile_zero = false;  // every query tile lists key tile 0 first
   int32_t* d_order = nullptr;  // [ceil(n_q_tiles / 2)] query-tile pairs, heaviest first
@@ -173,11 +184,9 @@ cudaError_t launch_forward_small_kv8(const FwdParams& p, const SmallLists& lists
                                      cudaStream_t stream);
 
 // Tensor-core path.  Returns LITEVAR_OK or an error status (tensor-map encoding can fail).
-litevar_status_t launch_forward_tcgen05(const FwdParams& p, int n_q_tiles, cudaStream_t stream);
-// The same kernel reading an 8-bit K/V cache (p.k8 ...; raster tiles only).
-litevar_status_t launch_forward_tcgen05_kv8(const FwdParams& p, int n_q_tiles, cudaStream_t stream);
-// The same path with one softmax thread per query row (register reallocation between warpgroups).
 litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream_t stream);
+// The tensor-core kernel that reads an 8-bit K/V cache (p.k8 ...; raster tiles only).
+litevar_status_t launch_forward_tcgen05_kv8(const FwdParams& p, int n_q_tiles, cudaStream_t stream);
 
 #ifdef __CUDACC__
 // 8-bit cache rows (paper Section 4): 16 int8 codes of one row -> 16 bf16 values code * s + z, as two 16-byte chunks.

@@ -258,6 +258,43 @@ __global__ void __launch_bounds__(128) mask_bits_kernel(Schedule sc, PlanGeom g,
   mask[(size_t)blk * kBlockM + threadIdx.x] = b;
 }
 
+// ------------------------------------------------------------------ A3 pass 5: live 64-key halves of every live pair
+// One warp per query tile walks its pairs: a half goes on the list when some query slot has a live key in it.
+__global__ void __launch_bounds__(128) chunk_kernel(int n_q_tiles, const TileGeom* key_geom, const int32_t* row_ptr,
+                                                    const Pair* pairs, const uint4* mask, KeyChunk* chunks,
+                                                    int32_t* n_chunks) {
+  const int qt = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (qt >= n_q_tiles) return;
+  KeyChunk* out = chunks + 2 * (size_t)row_ptr[qt];
+  int count = 0;
+  for (int i = row_ptr[qt]; i < row_ptr[qt + 1]; ++i) {
+    const Pair pr = pairs[i];
+    uint32_t any[2] = {1u, 1u};
+    if (pr.mask_block >= 0) {
+      any[0] = any[1] = 0u;
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const uint4 b = mask[(size_t)pr.mask_block * kBlockM + 32 * x + lane];
+        any[0] |= b.x | b.y;
+        any[1] |= b.z | b.w;
+      }
+    }
+    const TileGeom g = key_geom[pr.key_tile];
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      if (__any_sync(0xffffffffu, any[hf] != 0u)) {
+        if (lane == 0) {
+          const int mk = pr.mask_block < 0 ? -1 : 2 * pr.mask_block + hf;
+          out[count] = g.scale < 0 ? KeyChunk{g.a + hf * (kBlockN / 2), 0, -1, mk}
+                                   : KeyChunk{g.a + hf * (kPatchRows / 2), g.b, g.map_slot, mk};
+        }
+        ++count;
+      }
+    }
+  }
+  if (lane == 0) n_chunks[qt] = count;
+}
+
 // Launch order of the CTAs of the forward kernel (one CTA = query tiles 2u and 2u+1): heaviest first, so
 // that the light corner tiles fill the tail of the grid.  Rank sort, one thread per CTA.
 __global__ void launch_order_kernel(int n_q_tiles, const int32_t* row_ptr, int32_t* order) {
@@ -470,6 +507,7 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
         StepSet& ss = st.sets[set];
         ss.d_bounds = plan_mem.take<int2>((size_t)(k0 + 1) * st.s_k);
         ss.d_row_ptr = plan_mem.take<int32_t>((size_t)st.n_q_tiles + 1);
+        ss.d_n_chunks = plan_mem.take<int32_t>((size_t)st.n_q_tiles);
         ss.d_order = plan_mem.take<int32_t>((size_t)(st.n_q_tiles + 1) / 2);
         ss.d_pairs = plan_mem.take<Pair>(n_cand);  // room for every candidate pair; n_pairs of them are used
         SetScratch& t = scratch[(size_t)k0 * n_sets + set];
@@ -535,7 +573,7 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
   LV_TRY(cudaMemcpyAsync(totals.data(), d_totals, sizeof(SetTotals) * totals.size(), cudaMemcpyDeviceToHost, stream));
   LV_TRY(cudaGetLastError());
   LV_TRY(cudaStreamSynchronize(stream));
-  size_t mask_rows = 0;
+  size_t mask_rows = 0, n_chunks = 0;
   for (int k0 = 0; k0 < K; ++k0)
     for (int set = 0; set < n_sets; ++set) {
       const SetTotals& t = totals[(size_t)k0 * n_sets + set];
@@ -546,13 +584,16 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
       ss.n_full = t.n_full;
       ss.live_entries = (int64_t)t.live_entries;
       mask_rows += (size_t)t.n_partial * kBlockM;
+      n_chunks += 2 * (size_t)t.n_pairs;
     }
 
   // ---- A3, second pass: compaction in canonical order, element masks of the partial pairs, launch order
   void* mask_block = nullptr;
-  LV_TRY(cudaMalloc(&mask_block, (mask_rows ? mask_rows : 1) * sizeof(uint4)));
+  static_assert(sizeof(KeyChunk) == sizeof(uint4), "the chunk lists follow the mask rows in one block");
+  LV_TRY(cudaMalloc(&mask_block, (mask_rows + n_chunks + 1) * sizeof(uint4)));
   plan->allocations.push_back(mask_block);
   uint4* next_mask = static_cast<uint4*>(mask_block);
+  KeyChunk* next_chunk = reinterpret_cast<KeyChunk*>(next_mask + mask_rows);
   std::vector<SetDesc> descs((size_t)K * n_sets);
   for (int k0 = 0; k0 < K; ++k0) {
     Step& st = plan->steps[k0];
@@ -565,9 +606,13 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
       const int32_t* d_radius_row = plan->d_radius + ((size_t)set * K + k0) * K;
       ss.d_mask = next_mask;
       next_mask += (size_t)ss.n_partial * kBlockM;
+      ss.d_chunks = next_chunk;
+      next_chunk += 2 * (size_t)ss.n_pairs;
       compact_kernel<<<(unsigned)((st.n_q_tiles + 127) / 128), 128, 0, stream>>>(
           st.n_q_tiles, st.n_key_tiles, t.cls, ss.d_row_ptr, t.partial_base, ss.d_pairs, t.blk);
       mask_bits_kernel<<<grid2, 128, 0, stream>>>(sc, g, ss.d_bounds, d_radius_row, t.blk, ss.d_mask);
+      chunk_kernel<<<(unsigned)((st.n_q_tiles + 3) / 4), 128, 0, stream>>>(st.n_q_tiles, st.d_key_geom, ss.d_row_ptr, ss.d_pairs,
+                                                                       ss.d_mask, ss.d_chunks, ss.d_n_chunks);
       launch_order_kernel<<<(unsigned)(((st.n_q_tiles + 1) / 2 + 127) / 128), 128, 0, stream>>>(st.n_q_tiles,
                                                                                              ss.d_row_ptr, ss.d_order);
       first_tile_kernel<<<(unsigned)((st.n_q_tiles + 127) / 128), 128, 0, stream>>>(st.n_q_tiles, ss.d_row_ptr,
@@ -575,7 +620,7 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
       if (small_step_candidate(st.n_q_tiles, st.n_key_tiles, !st.q_patch && st.first_patch == k0 + 1) &&
           ss.n_pairs >= 1 && ss.n_pairs <= 2)
         copy_first_pairs_kernel<<<1, 32, 0, stream>>>(ss.d_pairs, &tot->n_pairs, tot->first_pairs);
-      descs[(size_t)k0 * n_sets + set] = SetDesc{ss.d_row_ptr, ss.d_pairs, ss.d_mask};
+      descs[(size_t)k0 * n_sets + set] = SetDesc{ss.d_row_ptr, ss.d_pairs, ss.d_mask, ss.d_chunks, ss.d_n_chunks};
     }
     LV_TRY(cudaMemcpyAsync(st.d_sets, &descs[(size_t)k0 * n_sets], sizeof(SetDesc) * n_sets, cudaMemcpyHostToDevice,
                            stream));
@@ -600,11 +645,9 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
   return LITEVAR_OK;
 }
 
-// Which of the two tcgen05 kernels runs a step that is not a small one.  The kernel with one softmax thread per
-// query row pays off on long tile lists (measured on B200: 5 to 8 % faster from about eight key tiles per query
-// tile on, i.e. the last steps of the 512px schedule and the 2K step; 5 % slower on the two-to-six-tile lists of
-// the 256px schedule, where the set-up of its longer pipeline is not written off).
-bool use_row_kernel(const litevar_plan_t* plan, const Step& st) {
+// Length class of a step that is not a small one, as litevar_plan_step_kernel reports it.  Both classes run the same kernel:
+// it is the faster one from two key tiles per query tile to 268 (measured on B200).
+bool long_lists(const litevar_plan_t* plan, const Step& st) {
   if (plan->kernel == LITEVAR_KERNEL_TCGEN05_WS) return true;
   if (plan->kernel != LITEVAR_KERNEL_AUTO) return false;
   return (st.sets[0].n_pairs + st.n_q_tiles - 1) / st.n_q_tiles >= 8;
@@ -682,7 +725,7 @@ static void fill_step_params(const litevar_plan_t* plan, const Step& st, int32_t
   memset(&p, 0, sizeof(p));
   p.sets = st.d_sets;
   p.head_to_set = plan->n_sets > 1 ? plan->d_head_to_set : nullptr;
-  p.set0 = SetDesc{st.sets[0].d_row_ptr, st.sets[0].d_pairs, st.sets[0].d_mask};
+  p.set0 = SetDesc{st.sets[0].d_row_ptr, st.sets[0].d_pairs, st.sets[0].d_mask, st.sets[0].d_chunks, st.sets[0].d_n_chunks};
   p.order = st.sets[0].d_order;
   p.n_k = st.n_k;
   p.L_k = st.L_k;
@@ -746,8 +789,7 @@ litevar_status_t litevar_attn_forward(const litevar_plan_t* plan, int32_t step_k
     }
     return LITEVAR_OK;
   }
-  if (use_row_kernel(plan, st)) return launch_forward_ws(p, st.n_q_tiles, stream);
-  return launch_forward_tcgen05(p, st.n_q_tiles, stream);
+  return launch_forward_ws(p, st.n_q_tiles, stream);
 }
 
 litevar_status_t litevar_attn_forward_kv8(const litevar_plan_t* plan, int32_t step_k, int32_t batch_pairs,
@@ -885,7 +927,7 @@ litevar_status_t litevar_plan_materialize_mask(const litevar_plan_t* plan, int32
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   size_t words = (size_t)((st.L_k + 31) / 32);
   LV_CUDA(cudaMemsetAsync(dev_bits, 0, sizeof(uint32_t) * words * st.n_k, stream));
-  SetDesc sd{ss.d_row_ptr, ss.d_pairs, ss.d_mask};
+  SetDesc sd{ss.d_row_ptr, ss.d_pairs, ss.d_mask, ss.d_chunks, ss.d_n_chunks};
   PlanGeom g{step_k - 1, st.s_k, st.n_k, st.L_k, st.n_key_tiles, plan->shape, st.raster_len, st.d_q_geom, st.d_key_geom};
   materialize_kernel<<<(unsigned)st.n_q_tiles, 128, 0, stream>>>(sd, plan->sched, g, static_cast<uint32_t*>(dev_bits));
   LV_CUDA(cudaGetLastError());
@@ -917,7 +959,7 @@ litevar_status_t litevar_plan_step_kernel(const litevar_plan_t* plan, int32_t st
   const long long units = (long long)plan->n_heads * (st.share ? batch_pairs : 2 * batch_pairs);
   *kernel = plan->kernel == LITEVAR_KERNEL_SIMT ? LITEVAR_KERNEL_SIMT
             : small_mode(plan, st, units)       ? LITEVAR_KERNEL_SMALL
-            : use_row_kernel(plan, st)          ? LITEVAR_KERNEL_TCGEN05_WS
+            : long_lists(plan, st)              ? LITEVAR_KERNEL_TCGEN05_WS
                                                 : LITEVAR_KERNEL_TCGEN05;
   return LITEVAR_OK;
 }

@@ -30,11 +30,13 @@ struct StaticPlan {
   int32_t pad[9];
   int32_t row_ptr[kStaticMaxPairs + 1];
   Pair pairs[kStaticMaxPairs];
+  int32_t n_chunks[kStaticMaxPairs];
+  KeyChunk chunks[2 * kStaticMaxPairs];
   uint8_t cls[kStaticMaxPairs];
   uint4 mask[(size_t)kStaticMaxPairs * kBlockM];
 };
 
-// 4.2 MB per GPU.  In host code this name is only a handle for cudaGetSymbolAddress: it is not a device
+// 4.4 MB per GPU.  In host code this name is only a handle for cudaGetSymbolAddress: it is not a device
 // address and must never be passed to a kernel.  Device code below names it directly.
 static __device__ __align__(256) unsigned char litevar_static_scratch[sizeof(StaticPlan)];
 
@@ -104,11 +106,11 @@ __global__ void __launch_bounds__(kBlockM) static_classify_kernel(Schedule sc, S
     }
   }
   const int cnt = __popc(w[0]) + __popc(w[1]) + __popc(w[2]) + __popc(w[3]);
-  const int any = __syncthreads_or(cnt != 0);
+  const int any0 = __syncthreads_or((w[0] | w[1]) != 0u), any1 = __syncthreads_or((w[2] | w[3]) != 0u);
   const int all = __syncthreads_and(!valid || cnt == kBlockN);
   const int cand = qt * a.n_key_tiles + kt;
   sp->mask[(size_t)cand * kBlockM + m] = make_uint4(w[0], w[1], w[2], w[3]);
-  if (m == 0) sp->cls[cand] = any ? (all ? 2 : 1) : 0;
+  if (m == 0) sp->cls[cand] = (any0 || any1) ? ((all ? 2 : 1) | (any0 ? 4 : 0) | (any1 ? 8 : 0)) : 0;
 }
 
 // One block: per query tile count the live pairs, scan, write the CSR list in canonical order
@@ -132,20 +134,27 @@ __global__ void static_compact_kernel(int n_q_tiles, int n_key_tiles) {
     sp->set.row_ptr = sp->row_ptr;
     sp->set.pairs = sp->pairs;
     sp->set.mask = sp->mask;
+    sp->set.chunks = sp->chunks;
+    sp->set.n_chunks = sp->n_chunks;
     sp->status = 0;
   }
   __syncthreads();
   for (int qt = threadIdx.x; qt < n_q_tiles; qt += blockDim.x) {
-    int o = sp->row_ptr[qt];
+    int o = sp->row_ptr[qt], n_chunks = 0;
+    KeyChunk* chunks = sp->chunks + 2 * o;
     for (int kt = 0; kt < n_key_tiles; ++kt) {
       const int cand = qt * n_key_tiles + kt;
       const int c = sp->cls[cand];
       if (c != 0) {
         sp->pairs[o].key_tile = kt;
-        sp->pairs[o].mask_block = c == 1 ? cand : -1;
+        const bool partial = (c & 3) == 1;
+        sp->pairs[o].mask_block = partial ? cand : -1;
         ++o;
+        for (int hf = 0; hf < 2; ++hf)
+          if (c & (4 << hf)) chunks[n_chunks++] = KeyChunk{kt * kBlockN + hf * (kBlockN / 2), 0, -1, partial ? 2 * cand + hf : -1};
       }
     }
+    sp->n_chunks[qt] = n_chunks;
   }
 }
 
@@ -251,7 +260,7 @@ extern "C" litevar_status_t litevar_attn_forward_static(
   FwdParams p;
   p.sets = &sp->set;
   p.head_to_set = nullptr;
-  p.set0 = SetDesc{sp->row_ptr, sp->pairs, sp->mask};  // device addresses inside the fixed array
+  p.set0 = SetDesc{sp->row_ptr, sp->pairs, sp->mask, sp->chunks, sp->n_chunks};  // device addresses inside the fixed array
   p.order = nullptr;
   p.q = static_cast<const uint16_t*>(Q);
   p.k = static_cast<const uint16_t*>(Kc);
@@ -280,5 +289,5 @@ extern "C" litevar_status_t litevar_attn_forward_static(
   p.units_per_group = units_per_l2_group(p.L_k, p.n_heads * p.batch_computed);
   p.first_tile_zero = 0;
   p.overlap_launch = 0;  // the plan is written by the two kernels launched just above
-  return launch_forward_tcgen05(p, a.n_q_tiles, stream);
+  return launch_forward_ws(p, a.n_q_tiles, stream);
 }

@@ -423,3 +423,34 @@ def test_small_step_kernel_shape_extremes(scales, n_global, share):
         if share:
             assert torch.equal(out[:B].view(torch.int16), out[B:].view(torch.int16))
     plan.close()
+
+
+@pytest.mark.parametrize("kind", ["late-huge", "rising", "all-low"])
+@pytest.mark.parametrize("tiling", TILINGS, ids=lambda t: TNAME[t])
+def test_row_reference_moves_and_redo(kind, tiling):
+    """The tcgen05 kernel's reference of a row moves by a chunk's sum, and the list is redone when a score is out of
+    its range: scores that rise from chunk to chunk by less than 2^60, a late key far above everything before it, and rows
+    whose first live key comes late with every score far below 0."""
+    lib_ready()
+    scales, H, B = (1, 2, 3, 4, 6, 9, 13), 2, 1
+    n_global = 0 if kind == "all-low" else 3
+    tab = orc.window_table(scales, n_global_scales=n_global)
+    if kind == "all-low":       # the lower scales are dead but for the co-located key: whole chunks are dead for a row
+        tab[6, 3:6] = 0
+    w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=94)
+    Q = wl.make_q(w, 0, 7).float()
+    Kc, Vc = (t.float() for t in wl.make_kv(w, 0))
+    L = Kc.shape[2]
+    if kind == "late-huge":     # two keys of the current scale with scores in the thousands, of either sign per row
+        Kc[:, :, L - 40] *= 300
+        Kc[:, :, 150] *= -250
+    elif kind == "rising":      # up to 2^50 between neighbouring chunks
+        Kc *= torch.linspace(0.2, 9, L).view(1, 1, L, 1)
+    else:                       # q . k = -64 * 49 / 8 for every pair, plus noise
+        Q, Kc = 7 + 0.02 * Q, -7 + 0.02 * Kc
+    Q, Kc, Vc = Q.bfloat16(), Kc.bfloat16(), Vc.bfloat16()
+    plan = binding.Plan(scales, n_heads=H, radius=tab, tiling=tiling)
+    got, _ = run_forward(plan, 7, B, Q, Kc, Vc, binding.KERNEL_TCGEN05)
+    ref = orc.attention_step(scales, 7, tab[6], Q, Kc, Vc)
+    assert_close(got, ref, kind)
+    plan.close()
