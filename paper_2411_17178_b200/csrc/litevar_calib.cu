@@ -18,9 +18,17 @@
 // column distance is smaller fall into bin dr and add up in a register before one shared-memory update per
 // key row; the others belong to the bin of their own column distance, which is fixed per lane, so they add up
 // in registers over all key rows of the query.
+//
+// The distance of an entry does not depend on the map, so several maps are added up entry by entry first (sum_maps_kernel, a
+// pass at memory speed) and the histogram pass reads one or a few summed maps instead of all of them.  The histogram pass costs
+// about 3.5 times what reading its input costs, so this pays from two maps on; it takes fp32 sums of at most
+// kMaxSumMaps maps and a scratch buffer of at most kScratchBytes (a single 2K map, 2.2 GB, goes to the histogram directly).
+// Measured on B200: 64 maps of the last 512px step (587 MB): the call 338 -> 169 us; 1280 maps of the last 256px step
+// (891 MB): see below.
 #include <cuda_runtime.h>
 
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "litevar_internal.h"
@@ -33,6 +41,80 @@ constexpr int kCalibWarps = 4;
 constexpr int kMaxDist = kMaxScale;   // distances 0 .. s_j - 1
 constexpr int kCalibFlushRows = 256;  // rows a lane's fp32 bins take in before they are flushed
 constexpr int kCalibMaxRows = 1 << 30;  // (map, query) rows of one launch
+constexpr int kSumThreads = 256, kSumPerThread = 4, kSumUnroll = 4;
+constexpr int kMaxSumMaps = 256;               // maps added up in fp32
+constexpr size_t kScratchBytes = 32u << 20;    // summed maps of one call, at most
+
+// out[g][i] = sum of maps m in [g * per_group, (g + 1) * per_group) of maps[m][i].  A thread owns kSumPerThread entries, a block's
+// width apart (coalesced whatever the alignment of a map), and has kSumPerThread * kSumUnroll loads in flight.
+__global__ void __launch_bounds__(kSumThreads) sum_maps_kernel(const float* __restrict__ maps, int64_t n, int64_t n_maps,
+                                                               int64_t per_group, float* __restrict__ out) {
+  const int64_t first = (int64_t)blockIdx.x * (kSumThreads * kSumPerThread) + threadIdx.x;
+  const int64_t m0 = blockIdx.y * per_group, m1 = min(n_maps, m0 + per_group);
+  float acc[kSumPerThread] = {};
+  const float* src = maps + m0 * n + first;
+  if (first + (kSumPerThread - 1) * kSumThreads < n) {
+    int64_t m = m0;
+    for (; m + kSumUnroll <= m1; m += kSumUnroll) {
+      float v[kSumUnroll][kSumPerThread];
+#pragma unroll
+      for (int u = 0; u < kSumUnroll; ++u)
+#pragma unroll
+        for (int e = 0; e < kSumPerThread; ++e) v[u][e] = __ldcs(src + u * n + e * kSumThreads);
+#pragma unroll
+      for (int u = 0; u < kSumUnroll; ++u)
+#pragma unroll
+        for (int e = 0; e < kSumPerThread; ++e) acc[e] += v[u][e];
+      src += kSumUnroll * n;
+    }
+    for (; m < m1; ++m, src += n)
+#pragma unroll
+      for (int e = 0; e < kSumPerThread; ++e) acc[e] += __ldcs(src + e * kSumThreads);
+  } else {  // the last block of a map
+    for (int64_t m = m0; m < m1; ++m, src += n)
+#pragma unroll
+      for (int e = 0; e < kSumPerThread; ++e)
+        if (first + e * kSumThreads < n) acc[e] += __ldcs(src + e * kSumThreads);
+  }
+#pragma unroll
+  for (int e = 0; e < kSumPerThread; ++e)
+    if (first + e * kSumThreads < n) out[blockIdx.y * n + first + e * kSumThreads] = acc[e];
+}
+
+// Stream-ordered pool of the calibration scratch, one per device, made on first use.  It keeps at most one call's scratch
+// between calls (the device's default pool gives every block back at the synchronisation each call ends with, which made the
+// next call pay for a new mapping: 0.3 to 0.9 ms); what overlapping calls took beyond that goes back at their
+// synchronisations.  The memory returns to the device when the library is unloaded.
+struct ScratchPools {
+  std::mutex mu;
+  cudaMemPool_t pool[64] = {};
+  ~ScratchPools() {
+    for (cudaMemPool_t p : pool)
+      if (p) (void)cudaMemPoolDestroy(p);
+  }
+  cudaError_t get(int dev, cudaMemPool_t* out) {
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!pool[dev]) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      cudaMemPool_t p = nullptr;
+      cudaError_t e = cudaMemPoolCreate(&p, &props);
+      if (e != cudaSuccess) return e;
+      uint64_t keep = kScratchBytes + (1u << 20);
+      e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+      if (e != cudaSuccess) {
+        (void)cudaMemPoolDestroy(p);
+        return e;
+      }
+      pool[dev] = p;
+    }
+    *out = pool[dev];
+    return cudaSuccess;
+  }
+};
 
 // Wide part (more than 256 keys) of one query row: NC 32-column chunks per key row, 16 loads in flight per round.
 template <int NC>
@@ -209,19 +291,50 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
   if (first_part > k0) return LITEVAR_OK;  // every part of this step is global
 
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-  double* d_hist = nullptr;
   const size_t hist_bytes = sizeof(double) * kMaxScales * kMaxDist;
-  if (cudaMallocAsync(&d_hist, hist_bytes, stream) != cudaSuccess) {
+  const int n_k = scales[k0] * scales[k0];
+  const long long L_k = sc.off[k0 + 1], map_len = (long long)n_k * L_k;
+  int dev = 0, n_sm = 148;
+  cudaMemPool_t pool = nullptr;
+  static ScratchPools pools;
+  if (cudaGetDevice(&dev) != cudaSuccess || pools.get(dev, &pool) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return LITEVAR_ERR_CUDA;
+  }
+  (void)cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  // groups of maps that are added up: as many as fill the chip with threads, no more maps in one than kMaxSumMaps
+  long long groups = 0, per_group = 0;
+  if (n_maps > 1 && map_len <= (long long)(kScratchBytes / sizeof(float))) {
+    const long long threads = (map_len + kSumPerThread - 1) / kSumPerThread;
+    groups = (2048ll * n_sm + threads - 1) / threads;
+    if (groups < (n_maps + kMaxSumMaps - 1) / kMaxSumMaps) groups = (n_maps + kMaxSumMaps - 1) / kMaxSumMaps;
+    if (groups > (n_maps + 3) / 4) groups = (n_maps + 3) / 4;
+    const long long room = (long long)(kScratchBytes / sizeof(float)) / map_len;
+    if (groups > room || groups > 65535) groups = 0;  // too much for the scratch: straight to the histogram
+    if (groups > 0) {
+      per_group = (n_maps + groups - 1) / groups;
+      groups = (n_maps + per_group - 1) / per_group;
+    }
+  }
+  char* scratch = nullptr;
+  if (cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), hist_bytes + (size_t)(groups * map_len) * sizeof(float), pool,
+                              stream) != cudaSuccess) {
     (void)cudaGetLastError();
     return LITEVAR_ERR_OOM;
   }
+  double* d_hist = reinterpret_cast<double*>(scratch);
   litevar_status_t st = LITEVAR_OK;
   std::vector<double> hist((size_t)kMaxScales * kMaxDist);
-  const int n_k = scales[k0] * scales[k0];
+  if (groups > 0) {
+    float* summed = reinterpret_cast<float*>(scratch + hist_bytes);
+    const long long per_block = kSumThreads * kSumPerThread;
+    sum_maps_kernel<<<dim3((unsigned)((map_len + per_block - 1) / per_block), (unsigned)groups), kSumThreads, 0, stream>>>(
+        maps, map_len, n_maps, per_group, summed);
+    if (cudaGetLastError() != cudaSuccess) st = LITEVAR_ERR_CUDA;
+    maps = summed;
+    n_maps = groups;
+  }
   const long long rows = (long long)n_maps * n_k;
-  const long long L_k = sc.off[k0 + 1];
-  int dev = 0, n_sm = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) (void)cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   int s_max = 1;
   for (int j = first_part; j <= k0; ++j) s_max = scales[j] > s_max ? scales[j] : s_max;
   const size_t smem = sizeof(float) * 32 * (size_t)s_max * kCalibWarps;
@@ -230,7 +343,7 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
   if (blocks_per_sm > 32 / kCalibWarps) blocks_per_sm = 32 / kCalibWarps;
   if (blocks_per_sm < 1) blocks_per_sm = 1;
   const long long n_warps = (long long)n_sm * blocks_per_sm * kCalibWarps;
-  if (cudaMemsetAsync(d_hist, 0, hist_bytes, stream) != cudaSuccess ||
+  if (st != LITEVAR_OK || cudaMemsetAsync(d_hist, 0, hist_bytes, stream) != cudaSuccess ||
       cudaFuncSetAttribute(calib_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     st = LITEVAR_ERR_CUDA;
   for (long long first = 0; first < rows && st == LITEVAR_OK; first += kCalibMaxRows) {
@@ -257,7 +370,7 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
   if (st == LITEVAR_OK && (cudaMemcpyAsync(hist.data(), d_hist, hist_bytes, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
                            cudaStreamSynchronize(stream) != cudaSuccess))
     st = LITEVAR_ERR_CUDA;
-  (void)cudaFreeAsync(d_hist, stream);
+  (void)cudaFreeAsync(scratch, stream);
   if (st != LITEVAR_OK) {
     (void)cudaGetLastError();
     return st;
