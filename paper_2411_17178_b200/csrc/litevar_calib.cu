@@ -172,7 +172,7 @@ calib_hist_kernel(Schedule sc, int k0, int first_part, int s_max, const float* _
   const int n_warps = gridDim.x * kCalibWarps;
   const int flush_every = max(1, kCalibFlushRows / rows_per_batch);
 
-  for (int j = first_part; j <= k0; ++j) {
+  for (int j = first_part + blockIdx.y; j <= k0; j += gridDim.y) {  // few rows: the parts go to blocks of their own
     const int s_j = sc.scale[j];
     const int n_j = s_j * s_j;
     const int n_chunks = (n_j + 31) >> 5;
@@ -363,11 +363,12 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
     const long long n_batches = ((long long)n_rows + rows_per_batch - 1) / rows_per_batch;
     long long blocks = (n_batches + kCalibWarps - 1) / kCalibWarps;
     if (blocks > (long long)n_sm * blocks_per_sm) blocks = (long long)n_sm * blocks_per_sm;
-    calib_hist_kernel<<<(unsigned)blocks, kCalibWarps * 32, smem, stream>>>(
+    const unsigned parts = (unsigned)(k0 + 1 - first_part);
+    calib_hist_kernel<<<dim3((unsigned)blocks, n_batches <= 2 * n_warps ? parts : 1u), kCalibWarps * 32, smem, stream>>>(
         sc, k0, first_part, s_max, maps + first * L_k, n_rows, (int)(first % n_k), rows_per_batch, d_hist);
     if (cudaGetLastError() != cudaSuccess) st = LITEVAR_ERR_CUDA;
   }
-  if (st == LITEVAR_OK && (cudaMemcpyAsync(hist.data(), d_hist, hist_bytes, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+  if (st == LITEVAR_OK && (cudaMemcpyAsync(hist.data(), d_hist, sizeof(double) * kMaxDist * (size_t)step_k, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
                            cudaStreamSynchronize(stream) != cudaSuccess))
     st = LITEVAR_ERR_CUDA;
   (void)cudaFreeAsync(scratch, stream);

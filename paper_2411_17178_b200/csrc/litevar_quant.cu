@@ -14,7 +14,6 @@
 //
 // The integer decision is taken in fp32 with one IEEE operation at a time (no contraction into fused
 // multiply-adds), so that it can be reproduced exactly.
-#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include "litevar_internal.h"
@@ -25,128 +24,175 @@ namespace {
 
 constexpr int kQuantThreads = 256;
 
+// Division of an unsigned 31-bit number by a fixed one: multiply and shift (host-computed).
+struct FastDiv {
+  uint32_t d, mul, shift;
+};
+FastDiv fast_div(uint32_t d) {
+  uint32_t l = 0;
+  while (l < 31 && (1u << l) < d) ++l;  // 2^l >= d
+  // floor(n / d) = (n mul) >> (31 + l) for n < 2^31 with mul = floor(2^(31 + l) / d) + 1: the error n (mul d - 2^(31 + l)) is
+  // at most n d < 2^(31 + l)
+  return FastDiv{d, (uint32_t)((1ull << (31 + l)) / d + 1), 31 + l};
+}
+__device__ __forceinline__ uint32_t div_by(uint32_t n, const FastDiv& f) {
+  return (uint32_t)(((uint64_t)n * f.mul) >> f.shift);
+}
+
 // One tensor of a launch: rows [first_row, first_row + batch * n_heads * n_tokens) of the launch's row space.
 struct QuantTensor {
   const uint16_t* x;
   uint16_t* dq;  // nullptr: no dequantised output
   int64_t x_sb, x_sh, x_st, d_sb, d_sh, d_st;
-  int32_t n_tokens;
+  FastDiv n_tokens;
   long long first_row;
 };
 struct QuantArgs {
   QuantTensor t[3];
-  int32_t n_tensors, n_heads;
+  int32_t n_tensors;
+  FastDiv n_heads;
   long long n_rows;
-  float levels, lo, hi;
+  float levels, hi;
   int8_t* codes;  // outputs of the first tensor only
   float* scale;
   float* zero;
 };
 
+__device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+__device__ __forceinline__ float lo_bf16(uint32_t v) { return __uint_as_float(v << 16); }
+__device__ __forceinline__ float hi_bf16(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+
 // kQuantRowsPerGroup rows per 8-thread group: that many 16-byte loads in flight per thread.  Four for large
 // tensors (bandwidth), one for the few rows of a single step (more threads, shorter latency chain).
 template <int kQuantRowsPerGroup>
-__global__ void __launch_bounds__(kQuantThreads, 4) quant_rows_kernel(QuantArgs a) {
+__global__ void __launch_bounds__(kQuantThreads, 4) quant_rows_kernel(const __grid_constant__ QuantArgs a) {
   // the rows were written by earlier work of the stream; a launch with programmatic serialisation starts early
   asm volatile("griddepcontrol.launch_dependents;");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  constexpr int R = kQuantRowsPerGroup;
+  constexpr float kMagic = 12582912.f;  // 1.5 * 2^23: a float in [2^23, 2^24) holds an integer in its low mantissa bits
   const int part = threadIdx.x & 7;  // 16-byte column of the row
   // rows [R * group, R * group + R) per eight threads, no loop: the grid covers the rows (fewer than 2^31,
   // checked on the host).  Slots past the last row redo the last row and store nothing, so that every lane
   // joins the shuffles.
   const unsigned group = blockIdx.x * (unsigned)(kQuantThreads / 8) + (threadIdx.x >> 3);
-  bool valid[kQuantRowsPerGroup];
-  unsigned row[kQuantRowsPerGroup];
-  int ti[kQuantRowsPerGroup];
-  int64_t x_off[kQuantRowsPerGroup], d_off[kQuantRowsPerGroup];
-  uint4 raw[kQuantRowsPerGroup];
+  int ti[R];
+  int64_t x_off[R], d_off[R];
+  uint4 raw[R];
 #pragma unroll
-  for (int g = 0; g < kQuantRowsPerGroup; ++g) {
-    const unsigned slot = group * kQuantRowsPerGroup + g;
-    valid[g] = slot < (unsigned)a.n_rows;
-    row[g] = valid[g] ? slot : (unsigned)a.n_rows - 1u;
+  for (int g = 0; g < R; ++g) {
+    const unsigned row = min(group * R + g, (unsigned)a.n_rows - 1u);
     ti[g] = 0;
-    if (a.n_tensors > 1 && row[g] >= (unsigned)a.t[1].first_row) ti[g] = 1;
-    if (a.n_tensors > 2 && row[g] >= (unsigned)a.t[2].first_row) ti[g] = 2;
+    if (R == 1) {  // (launches of several tensors take one row per group)
+      if (a.n_tensors > 1 && row >= (unsigned)a.t[1].first_row) ti[g] = 1;
+      if (a.n_tensors > 2 && row >= (unsigned)a.t[2].first_row) ti[g] = 2;
+    }
     const QuantTensor& tn = a.t[ti[g]];
-    const unsigned local = row[g] - (unsigned)tn.first_row;
-    const unsigned bh = local / (unsigned)tn.n_tokens;
-    const int t = (int)(local - bh * (unsigned)tn.n_tokens);
-    const unsigned b = bh / (unsigned)a.n_heads;
-    const int h = (int)(bh - b * (unsigned)a.n_heads);
-    x_off[g] = b * tn.x_sb + h * tn.x_sh + (int64_t)t * tn.x_st + part * 8;
-    d_off[g] = b * tn.d_sb + h * tn.d_sh + (int64_t)t * tn.d_st + part * 8;
-    raw[g] = *reinterpret_cast<const uint4*>(tn.x + x_off[g]);
+    const unsigned local = row - (unsigned)tn.first_row;
+    const unsigned bh = div_by(local, tn.n_tokens);
+    const unsigned t = local - bh * tn.n_tokens.d;
+    const unsigned b = div_by(bh, a.n_heads);
+    const unsigned h = bh - b * a.n_heads.d;
+    x_off[g] = b * tn.x_sb + h * tn.x_sh + t * tn.x_st + part * 8;
+    d_off[g] = b * tn.d_sb + h * tn.d_sh + t * tn.d_st + part * 8;
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+#pragma unroll
+  for (int g = 0; g < R; ++g) raw[g] = *reinterpret_cast<const uint4*>(a.t[ti[g]].x + x_off[g]);
+
+  // the row's maximum and minimum: packed bf16 maxima of x and -x (exact), then (max, -min) as one pair through three
+  // shuffles; the eight threads of a row are adjacent lanes
+  uint32_t top[R];
+#pragma unroll
+  for (int g = 0; g < R; ++g) {
+    const uint4 r = raw[g];
+    const uint32_t mx = bf16x2_max(bf16x2_max(r.x, r.y), bf16x2_max(r.z, r.w));
+    const uint32_t mn = bf16x2_max(bf16x2_max(r.x ^ 0x80008000u, r.y ^ 0x80008000u),
+                                   bf16x2_max(r.z ^ 0x80008000u, r.w ^ 0x80008000u));
+    top[g] = bf16x2_max(__byte_perm(mx, mn, 0x5410), __byte_perm(mx, mn, 0x7632));
   }
 #pragma unroll
-  for (int g = 0; g < kQuantRowsPerGroup; ++g) {
-    const QuantTensor& tn = a.t[ti[g]];
-    const uint32_t u[4] = {raw[g].x, raw[g].y, raw[g].z, raw[g].w};
-    float v[8];
+  for (int o = 1; o < 8; o <<= 1)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      v[2 * i] = __uint_as_float(u[i] << 16);
-      v[2 * i + 1] = __uint_as_float(u[i] & 0xffff0000u);
-    }
-    float mx = v[0], mn = v[0];
+    for (int g = 0; g < R; ++g) top[g] = bf16x2_max(top[g], __shfl_xor_sync(0xffffffffu, top[g], o));
+  // step and its reciprocal, one row per thread (two divisions are a tenth of a thread's work otherwise)
+  float s_row[R], r_row[R], z_row[R];
+  {
+    uint32_t mine = top[0];
 #pragma unroll
-    for (int i = 1; i < 8; ++i) {
-      mx = fmaxf(mx, v[i]);
-      mn = fminf(mn, v[i]);
-    }
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {  // the eight threads of a row are adjacent lanes
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-    }
-    const float z = __fmul_rn(__fadd_rn(mx, mn), 0.5f);
+    for (int g = 1; g < R; ++g)
+      if ((part & (R - 1)) == g) mine = top[g];
+    const float mx = lo_bf16(mine), mn = -hi_bf16(mine);
     const float s = __fdiv_rn(__fsub_rn(mx, mn), a.levels);
-    const float s1 = s > 0.f ? s : 1.f;
-    const float r = __fdiv_rn(1.f, s1);  // one division per row; the elements multiply, see below
-    float c[8];
-    uint32_t packed[4];
-    // round to nearest even without the conversion pipe: adding and subtracting 1.5 * 2^23 is exact rounding
-    // to an integer for |y| < 2^22, and |y| stays near 2^(B-1) here.  The estimate y = (x - z) * (1 / s) is within
+    const float r = __fdiv_rn(1.f, s > 0.f ? s : 1.f);
+    const float z = __fmul_rn(__fadd_rn(mx, mn), 0.5f);
+    const unsigned row = group * R + (part & (R - 1));
+    if (part < R && row < (unsigned)a.n_rows && (R > 1 || ti[0] == 0)) {
+      if (a.scale != nullptr) a.scale[row] = s;
+      if (a.zero != nullptr) a.zero[row] = z;
+    }
+#pragma unroll
+    for (int g = 0; g < R; ++g) {
+      const int from = (threadIdx.x & 24) + g;
+      s_row[g] = R == 1 ? s : __shfl_sync(0xffffffffu, s, from);
+      r_row[g] = R == 1 ? r : __shfl_sync(0xffffffffu, r, from);
+      z_row[g] = __fmul_rn(__fadd_rn(lo_bf16(top[g]), -hi_bf16(top[g])), 0.5f);
+    }
+  }
+#pragma unroll
+  for (int g = 0; g < R; ++g) {
+    const QuantTensor& tn = a.t[ti[g]];
+    const bool valid = group * R + g < (unsigned)a.n_rows;
+    const uint32_t u[4] = {raw[g].x, raw[g].y, raw[g].z, raw[g].w};
+    const float s = s_row[g], r = r_row[g], z = z_row[g];
+    const float2 nz2 = make_float2(-z, -z), r2 = make_float2(r, r);
+    const float2 magic2 = make_float2(kMagic, kMagic), nmagic2 = make_float2(-kMagic, -kMagic);
+    // Round to nearest even without the conversion pipe: adding 1.5 * 2^23 leaves the integer in the low mantissa bits (|y|
+    // stays near 2^(B-1) here), subtracting it again gives it as a float.  The estimate y = (x - z) * (1 / s) is within
     // |y| * 2^-23 < 2^-15.9 of the true quotient and the correctly rounded quotient within 2^-17 of it, so an
     // estimate farther than 2^-14 from a half-integer rounds as the IEEE quotient does; a thread with an estimate
     // closer than that redoes its eight values with the division.  So does every thread of a row whose step is so
-    // small that its reciprocal is not a normal number.
-    bool divide = !(s1 > 1e-30f);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float y = __fmul_rn(__fsub_rn(v[i], z), r);
-      const float n = __fsub_rn(__fadd_rn(y, 12582912.f), 12582912.f);
-      divide |= fabsf(__fsub_rn(y, n)) > 0.5f - 0.00006103515625f;
-      c[i] = n;
-    }
-    if (divide) {  // rare (one thread-row in a thousand): all eight values again, with the IEEE division
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        c[i] = __fsub_rn(__fadd_rn(__fdiv_rn(__fsub_rn(v[i], z), s1), 12582912.f), 12582912.f);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) c[i] = s > 0.f ? fminf(fmaxf(c[i], a.lo), a.hi) : 0.f;
+    // small that its reciprocal is not a normal number.  (s = 0: x = z for every element, code 0.)
+    float2 t[4];  // 1.5 * 2^23 + code
+    float far = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const __nv_bfloat162 d2 = __floats2bfloat162_rn(__fadd_rn(__fmul_rn(c[2 * i], s), z),
-                                                      __fadd_rn(__fmul_rn(c[2 * i + 1], s), z));
-      packed[i] = *reinterpret_cast<const uint32_t*>(&d2);
+      const float2 y = __fmul2_rn(__fadd2_rn(make_float2(lo_bf16(u[i]), hi_bf16(u[i])), nz2), r2);
+      t[i] = __fadd2_rn(y, magic2);
+      const float2 n = __fadd2_rn(t[i], nmagic2);
+      const float2 d = __fadd2_rn(y, make_float2(-n.x, -n.y));
+      asm("max.f32 %0, %0, %1, %2;" : "+f"(far) : "f"(fabsf(d.x)), "f"(fabsf(d.y)));
     }
-    if (valid[g] && tn.dq != nullptr)
-      *reinterpret_cast<uint4*>(tn.dq + d_off[g]) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-    if (valid[g] && ti[g] == 0) {
-      if (a.codes != nullptr) {
-        uint32_t w[2];
+    if (far > 0.5f - 0.00006103515625f || !((s > 0.f ? s : 1.f) > 1e-30f)) {  // rare (one thread-row in a thousand)
+      const float s1 = s > 0.f ? s : 1.f;
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
-          w[i] = ((uint32_t)(int)c[4 * i] & 0xffu) | (((uint32_t)(int)c[4 * i + 1] & 0xffu) << 8) |
-                 (((uint32_t)(int)c[4 * i + 2] & 0xffu) << 16) | (((uint32_t)(int)c[4 * i + 3] & 0xffu) << 24);
-        *reinterpret_cast<uint2*>(a.codes + (size_t)row[g] * kHeadDim + part * 8) = make_uint2(w[0], w[1]);
-      }
-      if (part == 0) {
-        if (a.scale != nullptr) a.scale[row[g]] = s;
-        if (a.zero != nullptr) a.zero[row[g]] = z;
-      }
+      for (int i = 0; i < 4; ++i)
+        t[i] = make_float2(__fadd_rn(__fdiv_rn(__fsub_rn(lo_bf16(u[i]), z), s1), kMagic),
+                           __fadd_rn(__fdiv_rn(__fsub_rn(hi_bf16(u[i]), z), s1), kMagic));
+    }
+    // the upper clamp (a row's extremes are at +-(2^B - 1) / 2, which rounds to 2^(B-1) or below: -2^(B-1) needs no clamp)
+    uint32_t packed[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      t[i].x = fminf(t[i].x, a.hi);
+      t[i].y = fminf(t[i].y, a.hi);
+      const float2 c = __fadd2_rn(t[i], nmagic2);
+      // two roundings: the packed product and sum were contracted into one multiply-add (measured: other bf16 values)
+      const float2 d = make_float2(__fadd_rn(__fmul_rn(c.x, s), z), __fadd_rn(__fmul_rn(c.y, s), z));
+      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(packed[i]) : "f"(d.y), "f"(d.x));
+    }
+    if (valid && tn.dq != nullptr)
+      *reinterpret_cast<uint4*>(tn.dq + d_off[g]) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+    if (valid && ti[g] == 0 && a.codes != nullptr) {
+      uint32_t w[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)  // the low bytes of four codes
+        w[i] = __byte_perm(__byte_perm(__float_as_uint(t[2 * i].x), __float_as_uint(t[2 * i].y), 0x0040),
+                           __byte_perm(__float_as_uint(t[2 * i + 1].x), __float_as_uint(t[2 * i + 1].y), 0x0040), 0x5410);
+      *reinterpret_cast<uint2*>(a.codes + (size_t)(group * R + g) * kHeadDim + part * 8) = make_uint2(w[0], w[1]);
     }
   }
 }
@@ -158,10 +204,9 @@ bool quant_strides_ok(const litevar_strides_t* s) {
 
 litevar_status_t launch_quant(QuantArgs& a, int bits, bool overlap, cudaStream_t stream) {
   a.levels = (float)((1 << bits) - 1);
-  a.lo = -(float)(1 << (bits - 1));
-  a.hi = (float)((1 << (bits - 1)) - 1);
+  a.hi = 12582912.f + (float)((1 << (bits - 1)) - 1);
   if (a.n_rows >= (1LL << 31)) return LITEVAR_ERR_UNSUPPORTED;  // 2^31 rows of 128 bytes do not fit the device
-  const bool large = a.n_rows >= (1LL << 20);
+  const bool large = a.n_tensors == 1 && a.n_rows >= (1LL << 20);
   const long long rows_per_block = (kQuantThreads / 8) * (large ? 4 : 1);
   const long long blocks = (a.n_rows + rows_per_block - 1) / rows_per_block;
   cudaLaunchConfig_t cfg = {};
@@ -203,10 +248,10 @@ extern "C" litevar_status_t litevar_quantize_rows(const void* x, const litevar_s
   a.t[0].dq = static_cast<uint16_t*>(x_dq);
   a.t[0].x_sb = sx->batch; a.t[0].x_sh = sx->head; a.t[0].x_st = sx->token;
   if (x_dq) { a.t[0].d_sb = sdq->batch; a.t[0].d_sh = sdq->head; a.t[0].d_st = sdq->token; }
-  a.t[0].n_tokens = n_tokens;
+  a.t[0].n_tokens = fast_div((uint32_t)n_tokens);
   a.t[0].first_row = 0;
   a.n_tensors = 1;
-  a.n_heads = n_heads;
+  a.n_heads = fast_div((uint32_t)n_heads);
   a.n_rows = (long long)batch * n_heads * n_tokens;
   a.codes = codes; a.scale = scale; a.zero = zero;
   return launch_quant(a, bits, false, static_cast<cudaStream_t>(stream_));
@@ -232,12 +277,12 @@ extern "C" litevar_status_t litevar_quantize_qkv(void* q, const litevar_strides_
     a.t[i].x_sb = a.t[i].d_sb = st[i]->batch;
     a.t[i].x_sh = a.t[i].d_sh = st[i]->head;
     a.t[i].x_st = a.t[i].d_st = st[i]->token;
-    a.t[i].n_tokens = tokens[i];
+    a.t[i].n_tokens = fast_div((uint32_t)tokens[i]);
     a.t[i].first_row = first;
     first += (long long)batch * n_heads * tokens[i];
   }
   a.n_tensors = 3;
-  a.n_heads = n_heads;
+  a.n_heads = fast_div((uint32_t)n_heads);
   a.n_rows = first;
   return launch_quant(a, bits, true, static_cast<cudaStream_t>(stream_));
 }
