@@ -70,7 +70,7 @@ def peaks():
 def kernel_source_hash():
     import hashlib
     h = hashlib.sha256()
-    for f in ("litevar_fwd_tc.cu", "litevar_fwd_ws.cu", "litevar_tc_ptx.h", "litevar_fwd_small.cu", "litevar_plan.cu",
+    for f in ("litevar_maps.cu", "litevar_fwd_ws.cu", "litevar_tc_ptx.h", "litevar_fwd_small.cu", "litevar_plan.cu",
               "litevar_internal.h"):
         h.update(open(os.path.join(ROOT, "paper_2411_17178_b200", "csrc", f), "rb").read())
     return h.hexdigest()

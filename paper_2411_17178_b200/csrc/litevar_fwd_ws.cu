@@ -52,7 +52,22 @@ constexpr uint32_t kTmemCols = 256, kColO = 128;  // S (and P over it) of stream
 constexpr float kMoveSum = 1024.f;        // a chunk whose probabilities sum to more moves the row's reference
 constexpr float kRedoSum = 1152921504606846976.f;  // 2^60: beyond it the reference was too far off
 
-struct WsShared {
+// 8-bit cache build: the codes of a chunk (64 rows of 64 bytes, as the tensor-map copy delivers them, no swizzle) and its rows'
+// scales and shifted zero points, on their way into the bf16 stages (empty in the bf16 build).
+constexpr uint32_t kCodeBytes = kChunkKeys * kHeadDim;
+template <bool KV8>
+struct CodeStage {};
+template <>
+struct CodeStage<true> {
+  alignas(128) uint8_t kc[2][2][kCodeBytes];  // [stream][chunk % 2]
+  alignas(128) uint8_t vc[2][kCodeBytes];
+  float k_sz[2][2][2][kChunkKeys];  // [stream][chunk % 2][scale, shifted zero point][row]
+  float v_sz[2][2][kChunkKeys];
+  uint64_t kc_full[2][2], vc_full[2];
+};
+
+template <bool KV8>
+struct WsShared : CodeStage<KV8> {
   alignas(1024) uint8_t q[kTileBytes];  // Q; at the end the output rows pass through it
   alignas(1024) uint8_t k[2][kStages][kChunkBytes];
   alignas(1024) uint8_t v[2][kStages][kChunkBytes];
@@ -126,10 +141,50 @@ __device__ __forceinline__ void load_chunk(void* dst, const CUtensorMap* raster,
     tma_load_5d(dst, patch + c.map_slot, 0, c.col, c.row, h, b, bar);
 }
 
+// One chunk of codes -> bf16 rows in the 128-byte swizzle the tensor-map copies of the bf16 path produce (16-byte piece c of row m
+// at position c ^ (m & 7)).  Paper Section 4 (8-bit Q/K/V): a row enters the attention as code * s + z, rounded to bf16; the
+// arithmetic is widen_codes16's.  128 threads, two pieces of 16 codes each; consecutive threads take consecutive pieces.
+__device__ __forceinline__ void widen_chunk(const uint8_t* codes, const float (&sz)[2][kChunkKeys], uint8_t* stage, int t) {
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const int id = t + 128 * it, m = id >> 2, c = id & 3;
+    const uint4 q = *reinterpret_cast<const uint4*>(codes + id * 16);
+    uint4 lo, hi;
+    widen_codes16(q, sz[0][m], sz[1][m], lo, hi);
+    uint8_t* row = stage + m * 128;
+    *reinterpret_cast<uint4*>(row + (((2 * c) ^ (m & 7)) << 4)) = lo;
+    *reinterpret_cast<uint4*>(row + (((2 * c + 1) ^ (m & 7)) << 4)) = hi;
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> the tensor pipe's reads
+}
+
+// Scales and zero points of a chunk's rows lane and lane + 32 (rows past L_k: 0 and 0; their codes arrive as zeros).
+struct RowScales {
+  float s[2], z[2];
+};
+__device__ __forceinline__ RowScales row_scales(const float* scale, const float* zero, int row, int L_k, int lane) {
+  RowScales r;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int at = row + lane + 32 * i;
+    r.s[i] = at < L_k ? __ldg(scale + at) : 0.f;
+    r.z[i] = at < L_k ? __ldg(zero + at) : 0.f;
+  }
+  return r;
+}
+__device__ __forceinline__ void put_scales(float (&sz)[2][kChunkKeys], const RowScales& r, int lane) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    sz[0][lane + 32 * i] = r.s[i];
+    sz[1][lane + 32 * i] = shifted_zero_point(r.z[i], r.s[i]);
+  }
+}
+
+template <bool KV8>
 __global__ void __launch_bounds__(kThreads, 2)
 fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ FwdParams p, int n_q_tiles) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  WsShared& sm = *reinterpret_cast<WsShared*>(smem_raw);
+  WsShared<KV8>& sm = *reinterpret_cast<WsShared<KV8>*>(smem_raw);
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // warp-uniform
   const int st = warp < 8 ? warp >> 2 : warp - 8;  // stream
   int qt, unit;  // grouped launch order, see cta_work
@@ -141,8 +196,13 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
     mbar_init(&sm.q_full, 1);
     for (int i = 0; i < 2; ++i) {
       for (int s = 0; s < kStages; ++s) {
-        mbar_init(&sm.k_full[i][s], 1);
-        mbar_init(&sm.v_full[i][s], 1);
+        mbar_init(&sm.k_full[i][s], KV8 ? 4 : 1);  // 8-bit cache: every softmax warp of the stream arrives
+        mbar_init(&sm.v_full[i][s], KV8 ? 4 : 1);
+      }
+      if constexpr (KV8) {
+        mbar_init(&sm.kc_full[i][0], 1);
+        mbar_init(&sm.kc_full[i][1], 1);
+        mbar_init(&sm.vc_full[i], 1);
       }
       mbar_init(&sm.s_full[i], 1);
       mbar_init(&sm.o_full[i], 1);
@@ -193,24 +253,88 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         if (elect_one()) load_chunk(sm.v[st][nv % kStages], &tm.vr, tm.v2, c, h, b, &sm.v_full[st][nv % kStages]);
         ++nv;
       };
+      // 8-bit cache: the copies bring codes, and the warp puts the rows' scales beside them (looked up a step ahead)
+      RowScales rs_k = {}, rs_v = {};
+      const float* scales[4] = {};
+      if constexpr (KV8) {
+        const int64_t at = (int64_t)b * p.z_sb + (int64_t)h * p.z_sh;
+        scales[0] = p.k_scale + at;
+        scales[1] = p.k_zero + at;
+        scales[2] = p.v_scale + at;
+        scales[3] = p.v_zero + at;
+      }
+      auto load_kc = [&](const KeyChunk& c) {
+        if constexpr (KV8) {
+          const int s = nk & 1;
+          put_scales(sm.k_sz[st][s], rs_k, lane);
+          __syncwarp();
+          if (elect_one()) {
+            mbar_expect_tx(&sm.kc_full[st][s], kCodeBytes);
+            tma_load_4d(sm.kc[st][s], &tm.kr, 0, c.row, h, b, &sm.kc_full[st][s]);
+          }
+          ++nk;
+        }
+      };
+      auto load_vc = [&](const KeyChunk& c) {
+        if constexpr (KV8) {
+          put_scales(sm.v_sz[st], rs_v, lane);
+          __syncwarp();
+          if (elect_one()) {
+            mbar_expect_tx(&sm.vc_full[st], kCodeBytes);
+            tma_load_4d(sm.vc[st], &tm.vr, 0, c.row, h, b, &sm.vc_full[st]);
+          }
+          ++nv;
+        }
+      };
       if (n > 0) c_k = chunk(0);
       if (!exact) asm volatile("griddepcontrol.wait;" ::: "memory");
       if (st == 0 && elect_one()) {
         mbar_expect_tx(&sm.q_full, kTileBytes);
         load_q_tile(sm.q, tm, p, qt, h, b, &sm.q_full);
       }
-      for (int i = 0; i < kStages && i < n; ++i) {
-        const KeyChunk c_next = chunk(i + 1);
-        load_k(c_k);
-        load_v(c_k);
-        c_k = c_v = c_next;
+      if constexpr (KV8) {
+        if (n > 0) {
+          c_v = chunk(1);
+          rs_k = row_scales(scales[0], scales[1], c_k.row, p.L_k, lane);
+          rs_v = row_scales(scales[2], scales[3], c_k.row, p.L_k, lane);
+          const RowScales rs_k1 = row_scales(scales[0], scales[1], c_v.row, p.L_k, lane);
+          load_kc(c_k);
+          load_vc(c_k);
+          rs_k = rs_k1;
+          if (n > 1) load_kc(c_v);
+          c_k = chunk(2);
+          rs_k = row_scales(scales[0], scales[1], c_k.row, p.L_k, lane);
+          rs_v = row_scales(scales[2], scales[3], c_v.row, p.L_k, lane);
+        }
+      } else {
+        for (int i = 0; i < kStages && i < n; ++i) {
+          const KeyChunk c_next = chunk(i + 1);
+          load_k(c_k);
+          load_v(c_k);
+          c_k = c_v = c_next;
+        }
       }
       bool ok = mbar_wait_long(&sm.q_full, exact ? 1u : 0u, abort_flag, p.status);
       for (int i = base - 1; i < end && n > 0; ++i) {
         const int s = i % kStages, s1 = (i + 1) % kStages;
         if (ok && i + 1 < end) ok = mbar_wait_long(&sm.k_full[st][s1], (uint32_t)(((i + 1) / kStages) & 1), abort_flag, p.status);
+        if (i >= base && ok) ok = mbar_wait_long(&sm.v_full[st][s], (uint32_t)((i / kStages) & 1), abort_flag, p.status);
+        if constexpr (KV8) {  // K(i + 1) and V(i) are widened: their code buffers take K(i + 3) and V(i + 1)
+          if (ok) {
+            const KeyChunk c = c_k;
+            if (i >= base && nv < end) {
+              load_vc(c_v);
+              c_v = chunk(nv - base);
+              rs_v = row_scales(scales[2], scales[3], c_v.row, p.L_k, lane);
+            }
+            if (nk < end) {
+              load_kc(c);
+              c_k = chunk(nk - base);
+              rs_k = row_scales(scales[0], scales[1], c_k.row, p.L_k, lane);
+            }
+          }
+        }
         if (i >= base) {
-          if (ok) ok = mbar_wait_long(&sm.v_full[st][s], (uint32_t)((i / kStages) & 1), abort_flag, p.status);
           __syncwarp();
           asm volatile("bar.sync %0, 160;" ::"r"(5 + st) : "memory");  // P(i); the softmax warps arrive even when a wait ran out
         }
@@ -228,11 +352,13 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
             mma_commit_one(&sm.o_full[st]);
           }
           // P(i) was complete, so S(i) and PV(i - 1) are: K(i + stages) and V(i - 1 + stages) go where K(i) and V(i - 1) were
-          if (i > base && nv < end) load_v(c_v);
-          if (i >= base && nk < end) {
-            load_k(c_k);
-            c_v = c_k;
-            c_k = chunk(nk - base);
+          if constexpr (!KV8) {
+            if (i > base && nv < end) load_v(c_v);
+            if (i >= base && nk < end) {
+              load_k(c_k);
+              c_v = c_k;
+              c_k = chunk(nk - base);
+            }
           }
           __syncwarp();
         }
@@ -241,12 +367,20 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         const unsigned long long ts = global_ns();
         while (!mbar_try(&sm.q_full, exact ? 1u : 0u))
           if (global_ns() - ts > kWaitLimitNs) break;
-        for (int i = nk > kStages ? nk - kStages : 0; i < nk; ++i)
-          while (!mbar_try(&sm.k_full[st][i % kStages], (uint32_t)((i / kStages) & 1)))
+        if constexpr (KV8) {
+          for (int i = nk > 2 ? nk - 2 : 0; i < nk; ++i)
+            while (!mbar_try(&sm.kc_full[st][i & 1], (uint32_t)((i >> 1) & 1)))
+              if (global_ns() - ts > 2 * kWaitLimitNs) break;
+          while (nv > 0 && !mbar_try(&sm.vc_full[st], (uint32_t)((nv - 1) & 1)))
             if (global_ns() - ts > 2 * kWaitLimitNs) break;
-        for (int i = nv > kStages ? nv - kStages : 0; i < nv; ++i)
-          while (!mbar_try(&sm.v_full[st][i % kStages], (uint32_t)((i / kStages) & 1)))
-            if (global_ns() - ts > 2 * kWaitLimitNs) break;
+        } else {
+          for (int i = nk > kStages ? nk - kStages : 0; i < nk; ++i)
+            while (!mbar_try(&sm.k_full[st][i % kStages], (uint32_t)((i / kStages) & 1)))
+              if (global_ns() - ts > 2 * kWaitLimitNs) break;
+          for (int i = nv > kStages ? nv - kStages : 0; i < nv; ++i)
+            while (!mbar_try(&sm.v_full[st][i % kStages], (uint32_t)((i / kStages) & 1)))
+              if (global_ns() - ts > 2 * kWaitLimitNs) break;
+        }
       }
     } else {
       // ---------------------------------------------------------------- softmax + epilogue
@@ -275,6 +409,29 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       bool live = blk < 0 || __any_sync(0xffffffffu, (mk.x | mk.y) != 0u);
       bool rescale = false;  // some row of the warp has a pending alpha
       float l_seen = 0.f;     // row sum before this chunk
+      // 8-bit cache: the stream's softmax threads widen its chunks, K(i + 2) and V(i + 1) while the products after P(i) run
+      const int t = threadIdx.x & 127;
+      auto widen_k = [&](int i) {
+        if constexpr (KV8) {
+          if (ok && i < end && (ok = mbar_wait_long(&sm.kc_full[st][i & 1], (uint32_t)((i >> 1) & 1), abort_flag, p.status))) {
+            widen_chunk(sm.kc[st][i & 1], sm.k_sz[st][i & 1], sm.k[st][i % kStages], t);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.k_full[st][i % kStages]);
+          }
+        }
+      };
+      auto widen_v = [&](int i) {
+        if constexpr (KV8) {
+          if (ok && i < end && (ok = mbar_wait_long(&sm.vc_full[st], (uint32_t)(i & 1), abort_flag, p.status))) {
+            widen_chunk(sm.vc[st], sm.v_sz[st], sm.v[st][i % kStages], t);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.v_full[st][i % kStages]);
+          }
+        }
+      };
+      widen_k(base);
+      widen_v(base);
+      widen_k(base + 1);
       for (int j = 0; j < n; ++j) {
         const bool partial = blk >= 0;
         // S(j) complete; in issue order this also means that PV(j - 1) is complete
@@ -386,6 +543,8 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           l_seen = (l2a.x + l2a.y) + (l2b.x + l2b.y);
         }
         rescale = __any_sync(0xffffffffu, alpha != 1.f);
+        widen_v(base + j + 1);
+        widen_k(base + j + 2);
         blk = blk_next;
         mk = mk_next;
         blk_next = j + 2 < n ? __ldg(blocks + 8 * (j + 2)) : -1;
@@ -470,16 +629,14 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
   }
 }
 
-}  // namespace
-
-litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream_t stream) {
-  TensorMaps tm;
-  if (!encode_tensor_maps(p, &tm, kChunkKeys)) return LITEVAR_ERR_INVALID_ARG;
+template <bool KV8>
+litevar_status_t launch_variant(const TensorMaps& tm, const FwdParams& p, int n_q_tiles, cudaStream_t stream) {
   static std::once_flag attr_once;
   static cudaError_t attr_err = cudaSuccess;
-  constexpr int smem_bytes = (int)sizeof(WsShared);
+  constexpr int smem_bytes = (int)sizeof(WsShared<KV8>);
+  static_assert(smem_bytes <= 115712, "two CTAs per SM");
   std::call_once(attr_once, [] {
-    attr_err = cudaFuncSetAttribute(fwd_ws_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    attr_err = cudaFuncSetAttribute(fwd_ws_kernel<KV8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   });
   if (attr_err != cudaSuccess) return LITEVAR_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
@@ -491,12 +648,26 @@ litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = p.overlap_launch ? 1 : 0;
-  if (cudaLaunchKernelEx(&cfg, fwd_ws_kernel, tm, p, n_q_tiles) != cudaSuccess) {
+  cfg.numAttrs = p.overlap_launch ? 1 : 0;  // off when an earlier kernel of the stream writes what the set-up reads
+  if (cudaLaunchKernelEx(&cfg, fwd_ws_kernel<KV8>, tm, p, n_q_tiles) != cudaSuccess) {
     (void)cudaGetLastError();
     return LITEVAR_ERR_CUDA;
   }
   return LITEVAR_OK;
+}
+
+}  // namespace
+
+litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream_t stream) {
+  TensorMaps tm;
+  if (!encode_tensor_maps(p, &tm, kChunkKeys)) return LITEVAR_ERR_INVALID_ARG;
+  return launch_variant<false>(tm, p, n_q_tiles, stream);
+}
+
+litevar_status_t launch_forward_ws_kv8(const FwdParams& p, int n_q_tiles, cudaStream_t stream) {
+  TensorMaps tm;
+  if (!encode_code_maps(p, &tm, kChunkKeys)) return LITEVAR_ERR_INVALID_ARG;
+  return launch_variant<true>(tm, p, n_q_tiles, stream);
 }
 
 }  // namespace litevar

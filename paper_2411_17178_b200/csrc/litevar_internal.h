@@ -185,8 +185,8 @@ cudaError_t launch_forward_small_kv8(const FwdParams& p, const SmallLists& lists
 
 // Tensor-core path.  Returns LITEVAR_OK or an error status (tensor-map encoding can fail).
 litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream_t stream);
-// The tensor-core kernel that reads an 8-bit K/V cache (p.k8 ...; raster tiles only).
-litevar_status_t launch_forward_tcgen05_kv8(const FwdParams& p, int n_q_tiles, cudaStream_t stream);
+// The same kernel reading an 8-bit K/V cache (p.k8 ...; raster tiles only).
+litevar_status_t launch_forward_ws_kv8(const FwdParams& p, int n_q_tiles, cudaStream_t stream);
 
 #ifdef __CUDACC__
 // 8-bit cache rows (paper Section 4): 16 int8 codes of one row -> 16 bf16 values code * s + z, as two 16-byte chunks.

@@ -828,7 +828,7 @@ litevar_status_t litevar_attn_forward_kv8(const litevar_plan_t* plan, int32_t st
     }
     return LITEVAR_OK;
   }
-  return launch_forward_tcgen05_kv8(p, st.n_q_tiles, stream);
+  return launch_forward_ws_kv8(p, st.n_q_tiles, stream);
 }
 
 static litevar_status_t check_step_set(const litevar_plan_t* plan, int32_t step_k, int32_t set) {

@@ -14,7 +14,6 @@ namespace tc {
 
 constexpr uint32_t kTileBytes = kBlockN * kHeadDim * 2;  // 16 KB: 128 rows of 128 B
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
-constexpr int kNoTile = 0x7fffffff;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -26,13 +25,6 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
   return (uint64_t)((saddr >> 4) & 0x3FFFu) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
          (2ull << 61);
 }
-// MN-major operand wider than one 64-element block: the leading-dimension byte offset (bits 16-29)
-// is the distance from the first block of N columns to the next one.
-__device__ __forceinline__ uint64_t make_desc_mn(uint32_t saddr, uint32_t next_block_bytes) {
-  return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)((next_block_bytes >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
@@ -60,34 +52,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// Bounded wait.  Returns false when another role gave up or the time limit passed; the caller then
-// leaves its loop and falls through to the common teardown.
-__device__ __forceinline__ bool mbar_wait_loop(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                               int32_t* status) {
-  const unsigned long long t0 = global_ns();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try(bar, parity)) return true;
-    if ((it & 63u) == 0u) {
-      if (*abort_flag) return false;
-      if (global_ns() - t0 > kWaitLimitNs) {
-        *abort_flag = 1;
-        atomicExch(status, 1);
-        return false;
-      }
-    }
-  }
-}
-static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                                   int32_t* status) {
-  return mbar_wait_loop(bar, parity, abort_flag, status);
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                          int32_t* status) {
-  if (mbar_try(bar, parity)) return true;
-  if (mbar_try(bar, parity)) return true;
-  return mbar_wait_slow(bar, parity, abort_flag, status);
-}
-// The same wait for the roles of a pipeline, which wait often: the polls carry a suspend-time hint (1 ms), so that a waiting
+// Bounded wait of a pipeline's role.  Returns false when another role gave up or the time limit passed; the caller then falls
+// through to the common teardown. the polls carry a suspend-time hint (1 ms), so that a waiting
 // warp leaves its issue slots to the others (measured on the 2K step: 2.5 % against polls without the hint, although a poll
 // takes 112 cycles instead of 74), and the clock is the SM's cycle counter (the global timer costs hundreds of cycles
 // per read).  The limit is 2^32 cycles, two seconds or more at any clock the part runs at.
@@ -152,35 +118,6 @@ __device__ __forceinline__ void load_q_tile(void* dst, const TensorMaps& tm, con
     tma_load_4d(dst, &tm.q, 0, g.a, h, b, bar);
   else
     tma_load_5d(dst, &tm.q, 0, g.b, g.a, h, b, bar);
-}
-__device__ __forceinline__ void load_kv_tile(void* dst, const CUtensorMap* raster, const CUtensorMap* patch,
-                                             const FwdParams& p, int kt, int h, int b, uint64_t* bar) {
-  if (p.key_geom == nullptr) {
-    tma_load_4d(dst, raster, 0, kt * kBlockN, h, b, bar);
-    return;
-  }
-  const TileGeom g = p.key_geom[kt];
-  if (g.scale < 0)
-    tma_load_4d(dst, raster, 0, g.a, h, b, bar);
-  else
-    tma_load_5d(dst, patch + g.map_slot, 0, g.b, g.a, h, b, bar);
-}
-
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
 }
 // Four consecutive K = 16 steps of one product in a single instruction sequence: step i reads A at
 // a_tmem + i * kAStep (TMEM columns) and B at b_desc + i * kBStep (descriptor units of 16 bytes); the first step
@@ -320,34 +257,11 @@ __device__ __forceinline__ void cta_work(const FwdParams& p, int n_ranks, int& r
   unit = group * g_units + (r - rank * here);
 }
 
-// Walk of the union of two ascending key-tile lists (the two halves of the CTA).
-struct UnionWalk {
-  const Pair* pairs;
-  int i0, e0, i1, e1;
-  int kt0, kt1;  // heads of the two lists (kNoTile when exhausted)
-  __device__ __forceinline__ void init(const Pair* p, int b0, int end0, int b1, int end1) {
-    pairs = p;
-    i0 = b0; e0 = end0; i1 = b1; e1 = end1;
-    kt0 = i0 < e0 ? __ldg(&pairs[i0].key_tile) : kNoTile;
-    kt1 = i1 < e1 ? __ldg(&pairs[i1].key_tile) : kNoTile;
-  }
-  __device__ __forceinline__ bool has() const { return kt0 != kNoTile || kt1 != kNoTile; }
-  // Next key tile and which halves list it; heads are refilled at once so that the loads overlap
-  // the caller's waits.
-  __device__ __forceinline__ int next(bool& live0, bool& live1) {
-    const int kt = min(kt0, kt1);
-    live0 = kt0 == kt;
-    live1 = kt1 == kt;
-    if (live0) kt0 = ++i0 < e0 ? __ldg(&pairs[i0].key_tile) : kNoTile;
-    if (live1) kt1 = ++i1 < e1 ? __ldg(&pairs[i1].key_tile) : kNoTile;
-    return kt;
-  }
-};
-
 }  // namespace tc
 
-// Fills the tensor maps of a launch from its parameters (host); K and V boxes of `key_rows` rows (128, or 64: half tiles).
-// False when an encoding fails.
-bool encode_tensor_maps(const FwdParams& p, tc::TensorMaps* tm, int key_rows = kBlockN);
+// Fills the tensor maps of a launch from its parameters (host); K and V boxes of `key_rows` rows.  encode_code_maps: kr and vr
+// cover the tensors of 8-bit codes (raster tiles only).  False when an encoding fails.
+bool encode_tensor_maps(const FwdParams& p, tc::TensorMaps* tm, int key_rows);
+bool encode_code_maps(const FwdParams& p, tc::TensorMaps* tm, int key_rows);
 
 }  // namespace litevar
