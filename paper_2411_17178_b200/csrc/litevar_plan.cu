@@ -491,18 +491,25 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
   SetTotals* d_totals = nullptr;
   int32_t* d_user = nullptr;
   Arena plan_mem, tmp_mem;
+  size_t geom_begin = 0, geom_end = 0, sets_end = 0;
   auto lay_out = [&]() {
     plan->d_status = plan_mem.take<int32_t>(1);
     plan->d_radius = plan_mem.take<int32_t>((size_t)n_sets * K * K);
     plan->d_head_to_set = plan->head_to_set.empty() ? nullptr : plan_mem.take<int32_t>((size_t)n_heads);
     d_totals = tmp_mem.take<SetTotals>((size_t)K * n_sets);
+    // what the host fills in comes first, so that it travels in two copies for all steps: tile geometry, set descriptors
+    geom_begin = plan_mem.used;
+    for (Step& st : plan->steps) {
+      st.d_q_geom = plan_mem.take<TileGeom>(st.q_geom.size());
+      st.d_key_geom = plan_mem.take<TileGeom>(st.key_geom.size());
+    }
+    geom_end = plan_mem.used;
+    for (Step& st : plan->steps) st.d_sets = plan_mem.take<SetDesc>((size_t)n_sets);
+    sets_end = plan_mem.used;
     d_user = window->radius ? tmp_mem.take<int32_t>((size_t)n_sets * K * K) : nullptr;
     for (int k0 = 0; k0 < K; ++k0) {
       Step& st = plan->steps[k0];
       const size_t n_cand = (size_t)st.n_q_tiles * st.n_key_tiles;
-      st.d_q_geom = plan_mem.take<TileGeom>(st.q_geom.size());
-      st.d_key_geom = plan_mem.take<TileGeom>(st.key_geom.size());
-      st.d_sets = plan_mem.take<SetDesc>((size_t)n_sets);
       for (int set = 0; set < n_sets; ++set) {
         StepSet& ss = st.sets[set];
         ss.d_bounds = plan_mem.take<int2>((size_t)(k0 + 1) * st.s_k);
@@ -547,13 +554,18 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
     LV_TRY(cudaMemcpyAsync(plan->d_head_to_set, plan->head_to_set.data(), sizeof(int32_t) * n_heads,
                            cudaMemcpyHostToDevice, stream));
 
+  std::vector<char> host_fill(sets_end - geom_begin);  // alive until the synchronisations below
+  auto host_at = [&](const void* d) { return host_fill.data() + (static_cast<const char*>(d) - (static_cast<char*>(plan_block) + geom_begin)); };
+  for (const Step& st : plan->steps) {
+    memcpy(host_at(st.d_q_geom), st.q_geom.data(), sizeof(TileGeom) * st.q_geom.size());
+    memcpy(host_at(st.d_key_geom), st.key_geom.data(), sizeof(TileGeom) * st.key_geom.size());
+  }
+  LV_TRY(cudaMemcpyAsync(static_cast<char*>(plan_block) + geom_begin, host_fill.data(), geom_end - geom_begin,
+                         cudaMemcpyHostToDevice, stream));
+
   // ---- A2 + A3, counting pass: bounds, classification of every candidate pair, per-tile counts and offsets
   for (int k0 = 0; k0 < K; ++k0) {
     Step& st = plan->steps[k0];
-    LV_TRY(cudaMemcpyAsync(st.d_q_geom, st.q_geom.data(), sizeof(TileGeom) * st.q_geom.size(), cudaMemcpyHostToDevice,
-                           stream));
-    LV_TRY(cudaMemcpyAsync(st.d_key_geom, st.key_geom.data(), sizeof(TileGeom) * st.key_geom.size(),
-                           cudaMemcpyHostToDevice, stream));
     const PlanGeom g{k0, st.s_k, st.n_k, st.L_k, st.n_key_tiles, plan->shape, st.raster_len, st.d_q_geom, st.d_key_geom};
     const dim3 grid2((unsigned)st.n_key_tiles, (unsigned)st.n_q_tiles);
     const int threads = st.n_q_tiles < 32 ? 32 : (st.n_q_tiles > 512 ? 512 : ((st.n_q_tiles + 31) / 32) * 32);
@@ -594,7 +606,6 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
   plan->allocations.push_back(mask_block);
   uint4* next_mask = static_cast<uint4*>(mask_block);
   KeyChunk* next_chunk = reinterpret_cast<KeyChunk*>(next_mask + mask_rows);
-  std::vector<SetDesc> descs((size_t)K * n_sets);
   for (int k0 = 0; k0 < K; ++k0) {
     Step& st = plan->steps[k0];
     const PlanGeom g{k0, st.s_k, st.n_k, st.L_k, st.n_key_tiles, plan->shape, st.raster_len, st.d_q_geom, st.d_key_geom};
@@ -620,11 +631,12 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
       if (small_step_candidate(st.n_q_tiles, st.n_key_tiles, !st.q_patch && st.first_patch == k0 + 1) &&
           ss.n_pairs >= 1 && ss.n_pairs <= 2)
         copy_first_pairs_kernel<<<1, 32, 0, stream>>>(ss.d_pairs, &tot->n_pairs, tot->first_pairs);
-      descs[(size_t)k0 * n_sets + set] = SetDesc{ss.d_row_ptr, ss.d_pairs, ss.d_mask, ss.d_chunks, ss.d_n_chunks};
+      const SetDesc desc{ss.d_row_ptr, ss.d_pairs, ss.d_mask, ss.d_chunks, ss.d_n_chunks};
+      memcpy(host_at(st.d_sets + set), &desc, sizeof(desc));
     }
-    LV_TRY(cudaMemcpyAsync(st.d_sets, &descs[(size_t)k0 * n_sets], sizeof(SetDesc) * n_sets, cudaMemcpyHostToDevice,
-                           stream));
   }
+  LV_TRY(cudaMemcpyAsync(static_cast<char*>(plan_block) + geom_end, host_fill.data() + (geom_end - geom_begin),
+                         sets_end - geom_end, cudaMemcpyHostToDevice, stream));
   LV_TRY(cudaMemcpyAsync(totals.data(), d_totals, sizeof(SetTotals) * totals.size(), cudaMemcpyDeviceToHost, stream));
   LV_TRY(cudaGetLastError());
   LV_TRY(cudaStreamSynchronize(stream));  // the scratch block is freed on return
@@ -696,16 +708,17 @@ litevar_status_t litevar_attn_plan(const int32_t* scales, int32_t n_scales, int3
   if (head_dim != kHeadDim) return LITEVAR_ERR_UNSUPPORTED;
 
   int dev = 0;
-  cudaDeviceProp prop;
+  int major = 0, n_sm = 0;  // (two attribute queries: the whole property structure takes a millisecond)
   LV_CUDA(cudaGetDevice(&dev));
-  LV_CUDA(cudaGetDeviceProperties(&prop, dev));
-  if (prop.major != 10) return LITEVAR_ERR_ARCH;
+  LV_CUDA(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+  LV_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+  if (major != 10) return LITEVAR_ERR_ARCH;
 
   litevar_plan* plan = new (std::nothrow) litevar_plan();
   if (!plan) return LITEVAR_ERR_OOM;
   litevar_status_t result = LITEVAR_ERR_OOM;
   try {
-    result = build_plan(plan, scales, n_scales, n_heads, sm_scale, window, share, dev, prop.multiProcessorCount,
+    result = build_plan(plan, scales, n_scales, n_heads, sm_scale, window, share, dev, n_sm,
                         static_cast<cudaStream_t>(stream_));
   } catch (...) {  // a host container ran out of memory: nothing crosses the C boundary
     result = LITEVAR_ERR_OOM;
