@@ -15,16 +15,17 @@
 // TMEM columns: S and P of stream s at 64 s, O at 128 + 64 s.
 //
 // The reference of a row (probabilities are 2^(score * scale - reference)) needs no maximum per chunk: it starts as the
-// maximum of the first chunk; afterwards only the chunk's SUM is looked at, and when that exceeds 2^10 the reference moves by
-// whole powers of two for the next chunk (the accumulator and the sum are scaled exactly).  bf16 and fp32 have the same
+// maximum of the first chunk's first eight keys (of the whole chunk: an extra pass, 1000 cycles of a tile's 20000); afterwards
+// only the chunk's SUM is looked at, and when that exceeds 2^10 the reference moves by whole powers of two for the next chunk
+// (the accumulator and the sum are scaled exactly).  bf16 and fp32 have the same
 // exponent range, so P is as accurate at 2^10 as at 1.  A sum beyond 2^60, or below 2^-60 where a row meets its first live key
 // late, is out of the range in which this is safe: the CTA then redoes its list, taking every chunk's maximum first (`exact`).
 //
 // What bounds it (ncu, 2K step with the full mask): exponential pipe 78 %, tensor pipe active 50 %, issue slots 53 %; the rest
 // is the hand-off from P to the next S (arrive, issue of eight MMAs, their execution, commit, wake: 700 cycles a chunk).
 // Measured on B200, with what the kernel with one softmax thread per row and 128-key tiles took before: 2K step with the full
-// mask 5.05 ms (6.71), window 1/4 1.71 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 173 / 81 / 38 us (261 / 116 / 47),
-// 256px step 10 with 960 units 90 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
+// mask 5.05 ms (6.71), window 1/4 1.71 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 168 / 79 / 36 us (261 / 116 / 47),
+// 256px step 10 with 960 units 88 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
 // the way: copy look-ups off the MMA lane -4 %, 64-key streams with uniform issue code -12 %, no maxima -12 %; share of the
 // exponentials on the FMA pipe 0 / 25 / 37.5 / 50 %: 1.80 / 1.71 / 1.78 / 1.87 ms; three stages instead of two: +1 %.
 //
@@ -192,30 +193,30 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
   const int h = unit % p.n_heads, b = unit / p.n_heads;
   volatile int* abort_flag = &sm.abort_flag;
 
-  if (threadIdx.x == 256) {
-    mbar_init(&sm.q_full, 1);
-    for (int i = 0; i < 2; ++i) {
-      for (int s = 0; s < kStages; ++s) {
-        mbar_init(&sm.k_full[i][s], KV8 ? 4 : 1);  // 8-bit cache: every softmax warp of the stream arrives
-        mbar_init(&sm.v_full[i][s], KV8 ? 4 : 1);
-      }
-      if constexpr (KV8) {
-        mbar_init(&sm.kc_full[i][0], 1);
-        mbar_init(&sm.kc_full[i][1], 1);
-        mbar_init(&sm.vc_full[i], 1);
-      }
-      mbar_init(&sm.s_full[i], 1);
-      mbar_init(&sm.o_full[i], 1);
+  if (warp >= 8 && elect_one()) {  // each issuing warp sets up its own stream's barriers
+    if (st == 0) {
+      mbar_init(&sm.q_full, 1);
+      sm.abort_flag = 0;
+      sm.redo = 0;
     }
-    sm.abort_flag = 0;
-    sm.redo = 0;
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&sm.k_full[st][s], KV8 ? 4 : 1);  // 8-bit cache: every softmax warp of the stream arrives
+      mbar_init(&sm.v_full[st][s], KV8 ? 4 : 1);
+    }
+    if constexpr (KV8) {
+      mbar_init(&sm.kc_full[st][0], 1);
+      mbar_init(&sm.kc_full[st][1], 1);
+      mbar_init(&sm.vc_full[st], 1);
+    }
+    mbar_init(&sm.s_full[st], 1);
+    mbar_init(&sm.o_full[st], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   // the next kernel of the stream may start its set-up while this grid drains; this grid's set-up ran while the
   // previous one drained.  Nothing an earlier kernel wrote is read before the wait below (the plan is older).
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (warp == 8) {
+  if (warp == 9) {
     __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem_base)),
                  "r"(kTmemCols)
@@ -226,10 +227,15 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
   const int n_all = __ldg(&sd.n_chunks[qt]);
   const int n = (n_all - st + 1) >> 1;  // this stream's chunks: st, st + 2, ...
   const KeyChunk* chunks = sd.chunks + 2 * (size_t)__ldg(&sd.row_ptr[qt]) + st;
-  tc_fence_before();
-  __syncthreads();  // barriers, TMEM address
-  tc_fence_after();
-  const uint32_t tmem = sm.tmem_base;
+  // The barriers and the TMEM address are shared here.  The issuing warps' first copies are on their way, and the softmax
+  // warps' list and mask words looked up, before the CTA meets: a tile of a short list spends 3000 of its 20000 cycles on the
+  // first copies (-2.5 to -5 % with the first reference).  With an 8-bit cache it meets first, which measured 1 % faster.
+  auto meet = [&] {
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+  };
+  if constexpr (KV8) meet();
 
   bool exact = false;  // second pass over the list, every chunk's maximum taken before its probabilities
   for (int base = 0;; base += n) {  // step counter of the pass's first chunk: barrier phases go on from pass to pass
@@ -241,7 +247,6 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       // execute in issue order, so that S may overwrite P).
       const uint64_t q_desc = make_desc(smem_u32(sm.q)), k_desc0 = make_desc(smem_u32(sm.k[st][0]));
       const uint64_t v_desc0 = make_desc(smem_u32(sm.v[st][0]));
-      const uint32_t tS = tmem + 64 * st, tO = tmem + kColO + 64 * st;
       auto chunk = [&](int i) { return chunk_at(chunks + 2 * min(i, n - 1)); };
       KeyChunk c_k = {}, c_v = {};  // what the next K and V copy takes; looked up a step ahead
       int nk = base, nv = base;     // copies issued
@@ -314,6 +319,8 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           c_k = c_v = c_next;
         }
       }
+      if (!KV8 && !exact) meet();
+      const uint32_t tS = sm.tmem_base + 64 * st, tO = tS + kColO;
       bool ok = mbar_wait_long(&sm.q_full, exact ? 1u : 0u, abort_flag, p.status);
       for (int i = base - 1; i < end && n > 0; ++i) {
         const int s = i % kStages, s1 = (i + 1) % kStages;
@@ -386,12 +393,10 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       // ---------------------------------------------------------------- softmax + epilogue
       const int lane_group = warp & 3;  // TMEM lanes 32 lane_group .. + 31
       const int m = lane_group * 32 + lane;
-      const uint32_t tlane = tmem + ((uint32_t)(lane_group * 32) << 16);
-      const uint32_t tS = tlane + 64 * st, tO = tlane + kColO + 64 * st;
       const float sc = p.sm_scale * 1.4426950408889634f;
       const float2 sc2 = make_float2(sc, sc);
       const float sc_y = sc * (0.5f / kClamp);
-      // probabilities are 2^(score * sc - msc).  msc starts as the first live chunk's maximum and moves by whole powers of two
+      // probabilities are 2^(score * sc - msc).  msc starts as the maximum of a few keys and moves by whole powers of two
       // when a chunk's sum gets large; it stays 0 and `none` until a live chunk has been seen.
       float msc = 0.f;
       bool none = true;
@@ -405,6 +410,9 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       const int* blocks = &chunks->mask;  // four ints per chunk, every second one is this stream's
       int blk = n > 0 ? __ldg(blocks) : -1, blk_next = n > 1 ? __ldg(blocks + 8) : -1;
       uint2 mk = mask_at(blk), mk_next = mask_at(blk_next);
+      if (!KV8 && !exact) meet();
+      const uint32_t tlane = sm.tmem_base + ((uint32_t)(lane_group * 32) << 16);
+      const uint32_t tS = tlane + 64 * st, tO = tlane + kColO + 64 * st;
       // chunks without a live key for any row of the warp are skipped (uniform over the warp)
       bool live = blk < 0 || __any_sync(0xffffffffu, (mk.x | mk.y) != 0u);
       bool rescale = false;  // some row of the warp has a pending alpha
@@ -441,9 +449,15 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           continue;
         }
         tc_fence_after();
-        if (j == 0 || exact) {  // the maximum first
+        if (j == 0 || exact) {  // a reference first: the chunk's maximum, or in the first pass that of its first eight keys
           float mx = -INFINITY;
-          if (live) {
+          if (live && !exact) {
+            uint32_t r[8];
+            tmem_ld8(tS, r);
+            tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 8; ++e) mx = fmaxf(mx, (mk.x >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
+          } else if (live) {
 #pragma unroll 1
             for (int hf = 0; hf < 2; ++hf) {
               const uint32_t w = hf ? mk.y : mk.x;
@@ -623,9 +637,9 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
   }
 
   // ---------------------------------------------------------------------- teardown (all paths)
-  if (warp == 8) {
+  if (warp == 9) {
     __syncwarp();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem_base), "r"(kTmemCols) : "memory");
   }
 }
 

@@ -229,7 +229,7 @@ bool quant_strides_ok(const litevar_strides_t* s) {
          (s->token % 8) == 0;
 }
 
-litevar_status_t launch_quant(QuantArgs& a, int bits, bool overlap, cudaStream_t stream) {
+litevar_status_t launch_quant(QuantArgs& a, int bits, cudaStream_t stream) {
   a.levels = (float)((1 << bits) - 1);
   a.hi = (float)((1 << (bits - 1)) - 1);
   if (a.n_rows >= (1LL << 31)) return LITEVAR_ERR_UNSUPPORTED;  // 2^31 rows of 128 bytes do not fit the device
@@ -244,7 +244,7 @@ litevar_status_t launch_quant(QuantArgs& a, int bits, bool overlap, cudaStream_t
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = overlap ? 1 : 0;
+  cfg.numAttrs = 1;  // every thread waits for the previous kernel before its first access
   const cudaError_t e = large ? cudaLaunchKernelEx(&cfg, quant_rows_kernel<4>, a)
                               : cudaLaunchKernelEx(&cfg, quant_rows_kernel<1>, a);
   if (e != cudaSuccess) {
@@ -281,7 +281,7 @@ extern "C" litevar_status_t litevar_quantize_rows(const void* x, const litevar_s
   a.n_heads = fast_div((uint32_t)n_heads);
   a.n_rows = (long long)batch * n_heads * n_tokens;
   a.codes = codes; a.scale = scale; a.zero = zero;
-  return launch_quant(a, bits, false, static_cast<cudaStream_t>(stream_));
+  return launch_quant(a, bits, static_cast<cudaStream_t>(stream_));
 }
 
 extern "C" litevar_status_t litevar_quantize_qkv(void* q, const litevar_strides_t* sq, int32_t n_q_tokens, void* k,
@@ -311,5 +311,5 @@ extern "C" litevar_status_t litevar_quantize_qkv(void* q, const litevar_strides_
   a.n_tensors = 3;
   a.n_heads = fast_div((uint32_t)n_heads);
   a.n_rows = first;
-  return launch_quant(a, bits, true, static_cast<cudaStream_t>(stream_));
+  return launch_quant(a, bits, static_cast<cudaStream_t>(stream_));
 }
