@@ -1,7 +1,8 @@
 // Tensor-core forward kernel for sm_100a: one query tile per CTA, two independent streams of key chunks.
 //
-// A CTA owns a query tile (128 queries) of one (head, batch row) and walks the live 64-key chunks of its list (the halves of
-// the plan's 128-key tiles that hold a live entry).  Two streams share the list, chunk i going to stream i % 2; each keeps its
+// A CTA owns a query tile (128 queries) of one (head, batch row) and walks the live 64-key chunks of its list (laid by the planner
+// over the tile's own live keys).  A chunk comes with the class of its two halves for every warp's 32 rows: dead halves are
+// skipped, live ones take no element mask.  Two streams share the list, chunk i going to stream i % 2; each keeps its
 // own scores, probabilities, accumulator and reference, and the two results meet at the end.  320 threads:
 //   warps 0-3, 4-7  softmax of stream 0 and 1: thread m of the group owns query slot m (TMEM lane m).  A chunk's 64 scores
 //                   come from TMEM in two halves of 32 through one rolled copy of the code: the plan's element mask, the
@@ -24,10 +25,11 @@
 // What bounds it (ncu, 2K step with the full mask): exponential pipe 78 %, tensor pipe active 50 %, issue slots 53 %; the rest
 // is the hand-off from P to the next S (arrive, issue of eight MMAs, their execution, commit, wake: 700 cycles a chunk).
 // Measured on B200, with what the kernel with one softmax thread per row and 128-key tiles took before: 2K step with the full
-// mask 5.05 ms (6.71), window 1/4 1.71 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 168 / 79 / 36 us (261 / 116 / 47),
-// 256px step 10 with 960 units 88 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
+// mask 5.05 ms (6.71), window 1/4 1.57 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 160 / 74 / 34 us (261 / 116 / 47),
+// 256px step 10 with 960 units 85 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
 // the way: copy look-ups off the MMA lane -4 %, 64-key streams with uniform issue code -12 %, no maxima -12 %; share of the
-// exponentials on the FMA pipe 0 / 25 / 37.5 / 50 %: 1.80 / 1.71 / 1.78 / 1.87 ms; three stages instead of two: +1 %.
+// exponentials on the FMA pipe 0 / 25 / 37.5 / 50 %: 1.80 / 1.71 / 1.78 / 1.87 ms; three stages instead of two: +1 %; chunks from
+// a tile's live box on and classes per half and warp (on the fixed grid, one live flag per chunk and warp: 1.69 ms) -7 %.
 //
 // Every wait on an mbarrier is bounded; when one runs out the CTA raises the plan's status word, drains its copies, frees its
 // TMEM and returns (the softmax warps still arrive for every chunk, so that the named barriers complete).  The element mask, the
@@ -136,10 +138,10 @@ __device__ __forceinline__ KeyChunk chunk_at(const KeyChunk* c) {
 __device__ __forceinline__ void load_chunk(void* dst, const CUtensorMap* raster, const CUtensorMap* patch,
                                            const KeyChunk& c, int h, int b, uint64_t* bar) {
   mbar_expect_tx(bar, kChunkBytes);
-  if (c.map_slot < 0)
-    tma_load_4d(dst, raster, 0, c.row, h, b, bar);
+  if (c.info >> 16)
+    tma_load_5d(dst, patch + ((c.info >> 16) - 1), 0, c.col, c.row, h, b, bar);
   else
-    tma_load_5d(dst, patch + c.map_slot, 0, c.col, c.row, h, b, bar);
+    tma_load_4d(dst, raster, 0, c.row, h, b, bar);
 }
 
 // One chunk of codes -> bf16 rows in the 128-byte swizzle the tensor-map copies of the bf16 path produce (16-byte piece c of row m
@@ -224,9 +226,9 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   const SetDesc sd = p.head_to_set ? p.sets[p.head_to_set[h]] : p.set0;
-  const int n_all = __ldg(&sd.n_chunks[qt]);
+  const int first = __ldg(&sd.chunk_ptr[qt]), n_all = __ldg(&sd.chunk_ptr[qt + 1]) - first;
   const int n = (n_all - st + 1) >> 1;  // this stream's chunks: st, st + 2, ...
-  const KeyChunk* chunks = sd.chunks + 2 * (size_t)__ldg(&sd.row_ptr[qt]) + st;
+  const KeyChunk* chunks = sd.chunks + first + st;
   // The barriers and the TMEM address are shared here.  The issuing warps' first copies are on their way, and the softmax
   // warps' list and mask words looked up, before the CTA meets: a tile of a short list spends 3000 of its 20000 cycles on the
   // first copies (-2.5 to -5 % with the first reference).  With an 8-bit cache it meets first, which measured 1 % faster.
@@ -403,18 +405,26 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       float alpha = 1.f;  // pending factor of the accumulator
       float2 l2a = make_float2(0.f, 0.f), l2b = make_float2(0.f, 0.f);  // row sum
       bool bad = false, ok = true;
-      const uint2* mask2 = reinterpret_cast<const uint2*>(sd.mask) + 2 * m;
-      auto mask_at = [&](int blk) {
-        return blk >= 0 ? __ldg(mask2 + (size_t)(blk >> 1) * (2 * kBlockM) + (blk & 1)) : make_uint2(~0u, ~0u);
+      // Per chunk: class of its two halves for this warp's rows (bits 0 - 1 and 2 - 3: 0 dead, 1 partial, 2 full) and the key bits
+      // of this thread's row, looked up one chunk ahead.
+      const int2* infos = reinterpret_cast<const int2*>(&chunks->info);  // {info, mask block}, every second chunk is this stream's
+      const uint2* mask_row = sd.chunk_mask + m;
+      int cls = 0, cls_next = 0;
+      auto look_up = [&](int j, int& c) {
+        uint2 bits = make_uint2(0u, 0u);
+        c = 0;
+        if (j < n) {
+          const int2 inf = __ldg(infos + 4 * j);
+          c = (inf.x >> (4 * lane_group)) & 15;
+          if (c & 5) bits = __ldg(mask_row + (size_t)inf.y * kBlockM);
+          else bits = make_uint2((c & 3) ? ~0u : 0u, (c >> 2) ? ~0u : 0u);
+        }
+        return bits;
       };
-      const int* blocks = &chunks->mask;  // four ints per chunk, every second one is this stream's
-      int blk = n > 0 ? __ldg(blocks) : -1, blk_next = n > 1 ? __ldg(blocks + 8) : -1;
-      uint2 mk = mask_at(blk), mk_next = mask_at(blk_next);
+      uint2 mk = look_up(0, cls), mk_next = look_up(1, cls_next);
       if (!KV8 && !exact) meet();
       const uint32_t tlane = sm.tmem_base + ((uint32_t)(lane_group * 32) << 16);
       const uint32_t tS = tlane + 64 * st, tO = tlane + kColO + 64 * st;
-      // chunks without a live key for any row of the warp are skipped (uniform over the warp)
-      bool live = blk < 0 || __any_sync(0xffffffffu, (mk.x | mk.y) != 0u);
       bool rescale = false;  // some row of the warp has a pending alpha
       float l_seen = 0.f;     // row sum before this chunk
       // 8-bit cache: the stream's softmax threads widen its chunks, K(i + 2) and V(i + 1) while the products after P(i) run
@@ -441,7 +451,6 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       widen_v(base);
       widen_k(base + 1);
       for (int j = 0; j < n; ++j) {
-        const bool partial = blk >= 0;
         // S(j) complete; in issue order this also means that PV(j - 1) is complete
         if (ok) ok = mbar_wait_long(&sm.s_full[st], (uint32_t)((base + j) & 1), abort_flag, p.status);
         if (!ok) {  // the issuing warp counts on every step's arrival
@@ -451,13 +460,13 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         tc_fence_after();
         if (j == 0 || exact) {  // a reference first: the chunk's maximum, or in the first pass that of its first eight keys
           float mx = -INFINITY;
-          if (live && !exact) {
+          if (cls && !exact) {
             uint32_t r[8];
             tmem_ld8(tS, r);
             tmem_wait_ld();
 #pragma unroll
             for (int e = 0; e < 8; ++e) mx = fmaxf(mx, (mk.x >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
-          } else if (live) {
+          } else if (cls) {
 #pragma unroll 1
             for (int hf = 0; hf < 2; ++hf) {
               const uint32_t w = hf ? mk.y : mk.x;
@@ -490,13 +499,13 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           }
           alpha = 1.f;
         }
-        if (live) {
 #pragma unroll 1
-          for (int hf = 0; hf < 2; ++hf) {
+        for (int hf = 0; hf < 2; ++hf) {
+          if ((cls >> (2 * hf)) & 3) {
             uint32_t r[32], pk[16];
             tmem_ld32(tS + 32 * hf, r);
             tmem_wait_ld();
-            if (partial) {  // dead scores of a partially live pair become -inf
+            if ((cls >> (2 * hf)) & 1) {  // dead scores of a partially live half become -inf
               const uint32_t w = hf ? mk.y : mk.x;
 #pragma unroll
               for (int e = 0; e < 32; ++e)
@@ -528,13 +537,12 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
               pk[(e >> 1) + 1] = kb;
             }
             tmem_st16(tS + 16 * hf, pk);  // over scores that have been read
-          }
-        } else {
-          uint32_t pk[16];
+          } else {  // no live key for any row of the warp
+            uint32_t pk[16];
 #pragma unroll
-          for (int e = 0; e < 16; ++e) pk[e] = 0u;
-          tmem_st16(tS, pk);
-          tmem_st16(tS + 16, pk);
+            for (int e = 0; e < 16; ++e) pk[e] = 0u;
+            tmem_st16(tS + 16 * hf, pk);
+          }
         }
         tmem_wait_st();  // P and, where it was rescaled, the accumulator
         tc_fence_before();
@@ -543,7 +551,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         // exceeded it, and the next chunk's masks (the words of the one after it start travelling)
         if (!exact) {
           const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y), grown = l - l_seen;
-          const bool seen = blk < 0 || (mk.x | mk.y) != 0u;  // a live key in this row
+          const bool seen = (mk.x | mk.y) != 0u;  // a live key in this row
           if (!(grown <= kMoveSum) || (none && seen)) {  // (a NaN goes this way too)
             bad |= !(grown < kRedoSum && grown > 1.f / kRedoSum);
             none = false;
@@ -559,11 +567,9 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         rescale = __any_sync(0xffffffffu, alpha != 1.f);
         widen_v(base + j + 1);
         widen_k(base + j + 2);
-        blk = blk_next;
+        cls = cls_next;
         mk = mk_next;
-        blk_next = j + 2 < n ? __ldg(blocks + 8 * (j + 2)) : -1;
-        live = blk < 0 || __any_sync(0xffffffffu, (mk.x | mk.y) != 0u);
-        mk_next = mask_at(blk_next);
+        mk_next = look_up(j + 2, cls_next);
       }
       if (!exact && __any_sync(0xffffffffu, bad) && lane == 0) sm.redo = 1;
       // the last PV product (all earlier ones are complete by issue order)

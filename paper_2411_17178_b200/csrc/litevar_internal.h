@@ -47,20 +47,27 @@ struct SmallLists {
   Pair pr[2];
 };
 
-// One 64-key half of a live pair that holds a live entry: where its K and V rows are and which mask words it has.
+// 64 keys with a live entry for some query slot of a tile, as the tensor-core kernel takes them.  The lists are laid over the live
+// keys of each query tile: 64 consecutive cache rows from a live one on, and in the patch-tiled scales 8 x 8 cells from the corner
+// of the tile's own live box on.  (Halves of the plan's 128-key tiles, on their fixed grid, are 2 to 15 % more chunks: 164 against
+// 155 a query tile at the last 2K step with window 1/4, 105 against 92 at the one before, 22.0 against 21.5 at the last of 512px.)
 struct alignas(16) KeyChunk {  // read with one 16-byte load
-  int32_t row, col;   // raster (map_slot < 0): first cache row; patch: first grid row and column of a 4 x 16 half patch
-  int32_t map_slot;   // tensor maps of the key scale (patch), -1: raster
-  int32_t mask;       // 2 * mask block + half, -1: every slot pair is live
+  int32_t row, col;   // raster: first cache row; patch: first grid row and column
+  int32_t info;       // bits 4 w + 2 h, + 1: class of keys 32 h .. + 31 for query slots 32 w .. + 31 (0 dead, 1 partial, 2 full);
+                      // bits 16 on: 1 + index of the key scale's tensor maps (patch), 0: raster
+  int32_t mask;       // block of SetDesc::chunk_mask, -1: no class is partial
 };
+constexpr int kPartialBits = 0x5555;  // of KeyChunk::info
+constexpr int kChunkSide = 8;         // of a patch chunk
 
 // Device-visible tile plan of one (step, window set).
 struct SetDesc {
   const int32_t* row_ptr;  // [n_q_tiles + 1]
   const Pair* pairs;       // [n_pairs]
   const uint4* mask;       // [n_partial][kBlockM] : 128 key bits per query slot
-  const KeyChunk* chunks;  // live halves of query tile i's pairs, from 2 * row_ptr[i] on
-  const int32_t* n_chunks; // [n_q_tiles] how many
+  const KeyChunk* chunks;      // query tile i's live chunks are [chunk_ptr[i], chunk_ptr[i + 1])
+  const int32_t* chunk_ptr;    // [n_q_tiles + 1]
+  const uint2* chunk_mask;     // [partial chunks][kBlockM] : 64 key bits per query slot
 };
 
 struct StepSet {
@@ -69,11 +76,11 @@ struct StepSet {
   int32_t* d_row_ptr = nullptr;
   Pair* d_pairs = nullptr;
   uint4* d_mask = nullptr;
-  KeyChunk* d_chunks = nullptr;   // [2 * n_pairs]
-  int32_t* d_n_chunks = nullptr;  // [n_q_tiles]
+  KeyChunk* d_chunks = nullptr;
+  int32_t* d_chunk_ptr = nullptr;  // [n_q_tiles + 1]
+  uint2* d_chunk_mask = nullptr;
   int2* d_bounds = nullptr;  // [k][s_k] {lo, hi} per key scale and query row/column (SQUARE)
-  bool first_tile_zero = false;  // every query tile lists key tile 0 first
-  int32_t* d_order = nullptr;  // [ceil(n_q_tiles / 2)] query-tile pairs, heaviest first
+  SetDesc desc() const { return SetDesc{d_row_ptr, d_pairs, d_mask, d_chunks, d_chunk_ptr, d_chunk_mask}; }
   SmallLists small = {-1, {{0, 0}, {0, 0}}};  // host copy of the tile list of a small step (n < 0: not a small step)
 };
 
@@ -96,7 +103,6 @@ struct FwdParams {
   const SetDesc* sets;          // [n_sets] for this step
   const int32_t* head_to_set;   // [H] or nullptr (all heads use set 0)
   SetDesc set0;                 // copy of sets[0]: saves the kernels one dependent load when there is one set
-  const int32_t* order;         // launch order of the query-tile pairs (heaviest first), or nullptr: natural order
   const uint16_t* q;
   const uint16_t* k;
   const uint16_t* v;
@@ -120,8 +126,6 @@ struct FwdParams {
   int32_t share_offset;         // B when the step is shared (second store at row b + B), else 0
   float sm_scale;
   int32_t* status;              // device word, set non-zero when a bounded wait expires
-  int32_t pairs_per_tile;       // average live key tiles per query tile (0: unknown); picks the kernel build
-  int32_t first_tile_zero;      // 1: every query tile's list starts with key tile 0 (its copies start at once)
   // 8-bit K/V cache (litevar_attn_forward_kv8): int8 codes [2B, H, rows, 64] with byte strides c_*, and one fp32
   // scale and zero point per row, [2B, H, rows] with strides z_sb, z_sh (rows contiguous); k and v are unused
   const int8_t* k8;
@@ -189,6 +193,11 @@ litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream
 litevar_status_t launch_forward_ws_kv8(const FwdParams& p, int n_q_tiles, cudaStream_t stream);
 
 #ifdef __CUDACC__
+// Class of 32 keys for a warp's query slots (KeyChunk::info): this slot's key bits, whether the slot is a query at all.
+__device__ __forceinline__ int key_class(uint32_t bits, bool valid) {
+  const bool any = __any_sync(0xffffffffu, bits != 0u), all = __all_sync(0xffffffffu, !valid || bits == ~0u);
+  return any ? (all ? 2 : 1) : 0;
+}
 // 8-bit cache rows (paper Section 4): 16 int8 codes of one row -> 16 bf16 values code * s + z, as two 16-byte chunks.
 // One fused multiply-add per pair and no integer conversion (that pipe is the exponential pipe): the codes are biased
 // by 128 (one XOR per four); a byte permute puts each biased code u into the second byte of the bit pattern of 2^15,

@@ -66,10 +66,10 @@ bool encode_codes(CUtensorMap* tm, const void* base, int64_t rows, int64_t heads
 }
 
 // Rank-5 map over the side x side grid of one scale inside a [batch, head, token, 64] tensor: dimensions
-// (64, column, row, head, batch); box = box_rows rows x 16 columns x 64, i.e. 16 box_rows rows of 128 B in shared memory in
-// row-major patch order.  Cells outside the grid read as zero and are not written.
+// (64, column, row, head, batch); box = box_rows rows x box_cols columns x 64, i.e. box_rows box_cols rows of 128 B in shared
+// memory in row-major order.  A copy may start at any cell.  Cells outside the grid read as zero and are not written.
 bool encode_patch(CUtensorMap* tm, const void* base, int64_t first_token, int64_t side, int64_t heads,
-                  int64_t batch, int64_t st, int64_t sh, int64_t sb, int box_rows) {
+                  int64_t batch, int64_t st, int64_t sh, int64_t sb, int box_rows, int box_cols) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) return false;
   if (heads == 1 && sh < kHeadDim) sh = st * side * side;
@@ -77,7 +77,7 @@ bool encode_patch(CUtensorMap* tm, const void* base, int64_t first_token, int64_
   const uint16_t* origin = static_cast<const uint16_t*>(base) + first_token * st;
   cuuint64_t gdim[5] = {(cuuint64_t)kHeadDim, (cuuint64_t)side, (cuuint64_t)side, (cuuint64_t)heads, (cuuint64_t)batch};
   cuuint64_t gstr[4] = {(cuuint64_t)st * 2, (cuuint64_t)(st * side) * 2, (cuuint64_t)sh * 2, (cuuint64_t)sb * 2};
-  cuuint32_t box[5] = {(cuuint32_t)kHeadDim, (cuuint32_t)kPatchCols, (cuuint32_t)box_rows, 1, 1};
+  cuuint32_t box[5] = {(cuuint32_t)kHeadDim, (cuuint32_t)box_cols, (cuuint32_t)box_rows, 1, 1};
   cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<uint16_t*>(origin), gdim, gstr, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -92,16 +92,16 @@ bool encode_tensor_maps(const FwdParams& p, tc::TensorMaps* tmp, int key_rows) {
   memset(&tm, 0, sizeof(tm));
   bool ok;
   if (p.q_patch)
-    ok = encode_patch(&tm.q, p.q, 0, p.s_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, kPatchRows);
+    ok = encode_patch(&tm.q, p.q, 0, p.s_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, kPatchRows, kPatchCols);
   else
     ok = encode_raster(&tm.q, p.q, p.n_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, kBlockM);
   ok = ok && encode_raster(&tm.kr, p.k, p.raster_len, p.n_heads, p.batch_computed, p.k_st, p.k_sh, p.k_sb, key_rows) &&
        encode_raster(&tm.vr, p.v, p.raster_len, p.n_heads, p.batch_computed, p.v_st, p.v_sh, p.v_sb, key_rows);
   for (int i = 0; ok && i < p.n_patch_scales; ++i)
     ok = encode_patch(&tm.k2[i], p.k, p.patch_off[i], p.patch_scale[i], p.n_heads, p.batch_computed, p.k_st, p.k_sh,
-                      p.k_sb, key_rows / kPatchCols) &&
+                      p.k_sb, kChunkSide, kChunkSide) &&
          encode_patch(&tm.v2[i], p.v, p.patch_off[i], p.patch_scale[i], p.n_heads, p.batch_computed, p.v_st, p.v_sh,
-                      p.v_sb, key_rows / kPatchCols);
+                      p.v_sb, kChunkSide, kChunkSide);
   return ok;
 }
 

@@ -247,7 +247,7 @@ __global__ void compact_kernel(int n_q_tiles, int n_key_tiles, const uint8_t* cl
 // ------------------------------------------------------------------ A3 pass 4: element masks of partial pairs
 __global__ void __launch_bounds__(128) mask_bits_kernel(Schedule sc, PlanGeom g, const int2* bounds,
                                                         const int32_t* radius_row, const int32_t* mask_block_of,
-                                                        uint4* mask) {
+                                                        uint4* mask, uint4* live_keys) {
   __shared__ int16_t ks_j[kBlockN], ks_r[kBlockN], ks_c[kBlockN];
   __shared__ int32_t ks_t[kBlockN];
   int kt = blockIdx.x, qt = blockIdx.y;
@@ -256,69 +256,163 @@ __global__ void __launch_bounds__(128) mask_bits_kernel(Schedule sc, PlanGeom g,
   int q;
   uint4 b = tile_row_bits(sc, g, bounds, radius_row, qt, kt, ks_j, ks_r, ks_c, ks_t, q);
   mask[(size_t)blk * kBlockM + threadIdx.x] = b;
+  // which keys of the tile some slot sees (tile_row_bits ended with a barrier)
+  __shared__ uint32_t live[4];
+  if (threadIdx.x < 4) live[threadIdx.x] = 0u;
+  __syncthreads();
+  const uint32_t w[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t o = __reduce_or_sync(0xffffffffu, w[i]);
+    if ((threadIdx.x & 31) == 0) atomicOr(&live[i], o);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) live_keys[qt * g.n_key_tiles + kt] = make_uint4(live[0], live[1], live[2], live[3]);
 }
 
-// ------------------------------------------------------------------ A3 pass 5: live 64-key halves of every live pair
-// One warp per query tile walks its pairs: a half goes on the list when some query slot has a live key in it.
-__global__ void __launch_bounds__(128) chunk_kernel(int n_q_tiles, const TileGeom* key_geom, const int32_t* row_ptr,
-                                                    const Pair* pairs, const uint4* mask, KeyChunk* chunks,
-                                                    int32_t* n_chunks) {
-  const int qt = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (qt >= n_q_tiles) return;
-  KeyChunk* out = chunks + 2 * (size_t)row_ptr[qt];
-  int count = 0;
-  for (int i = row_ptr[qt]; i < row_ptr[qt + 1]; ++i) {
-    const Pair pr = pairs[i];
-    uint32_t any[2] = {1u, 1u};
-    if (pr.mask_block >= 0) {
-      any[0] = any[1] = 0u;
+// ------------------------------------------------------------------ A3 pass 5: the chunk lists of the tensor-core kernel
+struct ChunkGeom {
+  int n_raster_tiles, n_maps;
+  int first_tile[kMaxPatchScales];  // key tile index of a patch-tiled scale's first tile
+  int side[kMaxPatchScales];
+};
+
+__device__ __forceinline__ int first_bit_from(const uint4& b, int from) {
+  const uint32_t w[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const uint4 b = mask[(size_t)pr.mask_block * kBlockM + 32 * x + lane];
-        any[0] |= b.x | b.y;
-        any[1] |= b.z | b.w;
-      }
+  for (int i = 0; i < 4; ++i) {
+    const int lo = from - 32 * i;
+    const uint32_t v = lo >= 32 ? 0u : (lo > 0 ? w[i] & (~0u << lo) : w[i]);
+    if (v) return 32 * i + __ffs(v) - 1;
+  }
+  return -1;
+}
+
+// One block per query tile; thread m works out slot m's key bits of every chunk from the masks of the tile pairs.  The first call
+// (fill = false) counts the chunks and those that need element masks, the second writes them where the scan put them.
+__global__ void __launch_bounds__(kBlockM) chunk_kernel(PlanGeom g, ChunkGeom cg, const uint8_t* cls, const int32_t* blk,
+                                                        const uint4* mask, const uint4* live_keys, bool fill,
+                                                        int32_t* chunk_ptr, int32_t* mask_ptr, KeyChunk* chunks, uint2* chunk_mask) {
+  __shared__ int warp_class[4];
+  __shared__ int box[4];  // live rows and columns of a scale: smallest row, largest row, smallest column, largest column
+  const int qt = blockIdx.x, m = threadIdx.x;
+  const size_t first = (size_t)qt * g.n_key_tiles;
+  int qr, qc;
+  const bool valid = query_slot_token(g.q_geom[qt], m, g.s_k, g.n_k, qr, qc) >= 0;
+  const uint4 ones = make_uint4(~0u, ~0u, ~0u, ~0u), zeros = make_uint4(0u, 0u, 0u, 0u);
+  auto bits_of = [&](int kt) {
+    const int c = cls[first + kt];
+    return c == 0 ? zeros : c == 2 ? ones : mask[(size_t)blk[first + kt] * kBlockM + m];
+  };
+  auto live_of = [&](int kt) {
+    const int c = cls[first + kt];
+    return c == 0 ? zeros : c == 2 ? ones : live_keys[first + kt];
+  };
+  int n = 0, n_mask = 0;
+  auto emit = [&](int row, int col, int slot, uint32_t lo, uint32_t hi) {
+    const int c = key_class(lo, valid) | key_class(hi, valid) << 2;
+    __syncthreads();
+    if ((m & 31) == 0) warp_class[m >> 5] = c;
+    __syncthreads();
+    const int info = warp_class[0] | warp_class[1] << 4 | warp_class[2] << 8 | warp_class[3] << 12;
+    if (info == 0) return;
+    const bool partial = (info & kPartialBits) != 0;
+    if (fill) {
+      const int at = mask_ptr[qt] + n_mask;
+      if (partial) chunk_mask[(size_t)at * kBlockM + m] = make_uint2(lo, hi);
+      if (m == 0) chunks[chunk_ptr[qt] + n] = KeyChunk{row, col, info | (slot + 1) << 16, partial ? at : -1};
     }
-    const TileGeom g = key_geom[pr.key_tile];
+    ++n;
+    n_mask += partial;
+  };
+  // raster prefix: 64 keys from the first live one that no chunk has yet (the fewest intervals that cover the live keys)
+  for (int kt = 0, covered = 0; kt < cg.n_raster_tiles; ++kt) {
+    const uint4 live = live_of(kt);
+    for (int at; (at = first_bit_from(live, max(covered - kt * kBlockN, 0))) >= 0; covered = kt * kBlockN + at + 64) {
+      const uint4 b0 = bits_of(kt), b1 = kt + 1 < cg.n_raster_tiles ? bits_of(kt + 1) : zeros;
+      const uint32_t w[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+      const int i = at >> 5;
+      emit(kt * kBlockN + at, 0, -1, __funnelshift_r(w[i], w[i + 1], at & 31), __funnelshift_r(w[i + 1], w[i + 2], at & 31));
+    }
+  }
+  // patch-tiled scales: 8 x 8 cells over the box of the live ones
+  for (int x = 0; x < cg.n_maps; ++x) {
+    const int n_rows = (cg.side[x] + kPatchRows - 1) / kPatchRows, n_cols = (cg.side[x] + kPatchCols - 1) / kPatchCols;
+    __syncthreads();
+    if (m < 4) box[m] = m & 1 ? -1 : 1 << 30;
+    __syncthreads();
+    for (int i = m; i < n_rows * n_cols; i += kBlockM) {
+      const uint4 live = live_of(cg.first_tile[x] + i);
+      const uint32_t w[4] = {live.x, live.y, live.z, live.w};  // two rows of 16 cells each
+      const uint32_t any = (w[0] | w[1] | w[2] | w[3]), cols = (any | any >> 16) & 0xffffu;
+      if (!any) continue;
+      const int r0 = (i / n_cols) * kPatchRows, c0 = (i % n_cols) * kPatchCols;
 #pragma unroll
-    for (int hf = 0; hf < 2; ++hf) {
-      if (__any_sync(0xffffffffu, any[hf] != 0u)) {
-        if (lane == 0) {
-          const int mk = pr.mask_block < 0 ? -1 : 2 * pr.mask_block + hf;
-          out[count] = g.scale < 0 ? KeyChunk{g.a + hf * (kBlockN / 2), 0, -1, mk}
-                                   : KeyChunk{g.a + hf * (kPatchRows / 2), g.b, g.map_slot, mk};
+      for (int r = 0; r < kPatchRows; ++r)
+        if ((w[r >> 1] >> (16 * (r & 1))) & 0xffffu) {
+          atomicMin(&box[0], r0 + r);
+          atomicMax(&box[1], r0 + r);
         }
-        ++count;
-      }
+      atomicMin(&box[2], c0 + __ffs(cols) - 1);
+      atomicMax(&box[3], c0 + 31 - __clz(cols));
     }
+    __syncthreads();
+    for (int r = box[0]; r <= box[1]; r += kChunkSide)
+      for (int c = box[2]; c <= box[3]; c += kChunkSide) {
+        // the 8 x 8 cells lie in up to 2 x 2 tiles
+        const int tr = r / kPatchRows, tc = c / kPatchCols, sh = c % kPatchCols;
+        uint32_t out[2] = {0u, 0u};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (tr + i >= n_rows) break;
+          const int kt = cg.first_tile[x] + (tr + i) * n_cols + tc;
+          const uint4 b0 = bits_of(kt), b1 = tc + 1 < n_cols ? bits_of(kt + 1) : zeros;
+          const uint32_t w0[4] = {b0.x, b0.y, b0.z, b0.w}, w1[4] = {b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+          for (int y = 0; y < kPatchRows; ++y) {  // row y of the tile is row to of the chunk
+            const int to = (tr + i) * kPatchRows + y - r, up = 16 * (y & 1);
+            if (to < 0 || to >= kChunkSide) continue;
+            const uint32_t cells = ((w0[y >> 1] >> up) & 0xffffu) | (((w1[y >> 1] >> up) & 0xffffu) << 16);
+            const uint32_t v = (cells >> sh) & 0xffu;
+            if (to < 4) out[0] |= v << (8 * to);
+            else out[1] |= v << (8 * (to - 4));
+          }
+        }
+        emit(r, c, x, out[0], out[1]);
+      }
   }
-  if (lane == 0) n_chunks[qt] = count;
+  if (!fill && m == 0) {
+    chunk_ptr[qt] = n;
+    mask_ptr[qt] = n_mask;
+  }
 }
 
-// Launch order of the CTAs of the forward kernel (one CTA = query tiles 2u and 2u+1): heaviest first, so
-// that the light corner tiles fill the tail of the grid.  Rank sort, one thread per CTA.
-__global__ void launch_order_kernel(int n_q_tiles, const int32_t* row_ptr, int32_t* order) {
-  const int n = (n_q_tiles + 1) / 2;
-  const int u = blockIdx.x * blockDim.x + threadIdx.x;
-  if (u >= n) return;
-  auto work = [&](int v) { return row_ptr[min(2 * v + 2, n_q_tiles)] - row_ptr[2 * v]; };
-  const int mine = work(u);
-  int rank = 0;
-  for (int v = 0; v < n; ++v) {
-    const int wv = work(v);
-    rank += (wv > mine) || (wv == mine && v < u);
+// One block: counts -> offsets, in place (chunk_ptr has one entry more); totals = {chunks, chunks with element masks}.
+__global__ void chunk_scan_kernel(int n_q_tiles, int32_t* chunk_ptr, int32_t* mask_ptr, int32_t* totals) {
+  extern __shared__ int32_t sh[];
+  for (int i = threadIdx.x; i < n_q_tiles; i += blockDim.x) {
+    sh[i] = chunk_ptr[i];
+    sh[n_q_tiles + i] = mask_ptr[i];
   }
-  order[rank] = u;
-}
-
-// Does every query tile list key tile 0 first?  (It does whenever the first cache rows stay live for every
-// query, as under any window of the paper: the coarsest scales are global.)  The forward kernel then starts
-// the copies of that tile before it has read anything of the plan.
-__global__ void first_tile_kernel(int n_q_tiles, const int32_t* row_ptr, const Pair* pairs, int32_t* not_zero) {
-  const int qt = blockIdx.x * blockDim.x + threadIdx.x;
-  if (qt >= n_q_tiles) return;
-  const int b = row_ptr[qt], e = row_ptr[qt + 1];
-  if (e == b || pairs[b].key_tile != 0) atomicExch(not_zero, 1);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int a = 0, b = 0;
+    for (int i = 0; i < n_q_tiles; ++i) {
+      const int na = sh[i], nb = sh[n_q_tiles + i];
+      sh[i] = a;
+      sh[n_q_tiles + i] = b;
+      a += na;
+      b += nb;
+    }
+    chunk_ptr[n_q_tiles] = a;
+    totals[0] = a;
+    totals[1] = b;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n_q_tiles; i += blockDim.x) {
+    chunk_ptr[i] = sh[i];
+    mask_ptr[i] = sh[n_q_tiles + i];
+  }
 }
 
 __global__ void empty_row_kernel(int n_k, const int32_t* row_live, int32_t* flag) {
@@ -373,14 +467,15 @@ struct Arena {
 // Scratch of one (step, window set) during planning.
 struct SetScratch {
   uint8_t* cls = nullptr;
-  int32_t *row_live = nullptr, *partial_base = nullptr, *blk = nullptr;
+  int32_t *row_live = nullptr, *partial_base = nullptr, *blk = nullptr, *chunk_mask_ptr = nullptr;
+  uint4* live_keys = nullptr;  // [candidate pairs] keys of the tile that some query slot sees
 };
 
 // Per (step, set) results the host needs: written by the planner kernels into one device array, read back once.
 struct SetTotals {
   int32_t n_pairs, n_partial, n_full, empty_row;  // count_scan_kernel / empty_row_kernel
   unsigned long long live_entries;                // classify_kernel
-  int32_t first_not_zero, pad;                    // first_tile_kernel
+  int32_t n_chunks, n_mask_chunks;                // chunk_scan_kernel
   Pair first_pairs[2];                            // the whole list of a small step (n_pairs <= 2)
 };
 
@@ -421,10 +516,10 @@ int small_mode(const litevar_plan_t* plan, const Step& st, long long units) {
   } while (0)
 
 // Everything litevar_attn_plan does after its argument checks.  Device memory: one arena for the plan (tables,
-// tile geometry, bounds, lists, launch orders; the lists sized for every candidate pair), one block for the
-// element masks (sized exactly, once the device has counted the partial pairs) and one scratch block that is
-// freed before returning.  Two synchronisations: after the counting pass (the mask block's size and the
-// empty-row check come from it) and at the end.
+// tile geometry, bounds, lists; the pair lists sized for every candidate pair), one block for the element masks
+// (sized exactly, once the device has counted the partial pairs), one for the chunk lists and their masks (the same) and one
+// scratch block that is freed before returning.  Three synchronisations: after the counting pass (the mask block's size
+// and the empty-row check come from it), after the chunks have been counted, and at the end.
 litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n_scales, int32_t n_heads, float sm_scale,
                             const litevar_window_t* window, const litevar_cfg_share_t* share, int dev, int n_sm,
                             cudaStream_t stream) {
@@ -514,14 +609,15 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
         StepSet& ss = st.sets[set];
         ss.d_bounds = plan_mem.take<int2>((size_t)(k0 + 1) * st.s_k);
         ss.d_row_ptr = plan_mem.take<int32_t>((size_t)st.n_q_tiles + 1);
-        ss.d_n_chunks = plan_mem.take<int32_t>((size_t)st.n_q_tiles);
-        ss.d_order = plan_mem.take<int32_t>((size_t)(st.n_q_tiles + 1) / 2);
+        ss.d_chunk_ptr = plan_mem.take<int32_t>((size_t)st.n_q_tiles + 1);
         ss.d_pairs = plan_mem.take<Pair>(n_cand);  // room for every candidate pair; n_pairs of them are used
         SetScratch& t = scratch[(size_t)k0 * n_sets + set];
         t.cls = tmp_mem.take<uint8_t>(n_cand);
         t.row_live = tmp_mem.take<int32_t>((size_t)st.n_k);
         t.partial_base = tmp_mem.take<int32_t>((size_t)st.n_q_tiles);
         t.blk = tmp_mem.take<int32_t>(n_cand);
+        t.chunk_mask_ptr = tmp_mem.take<int32_t>((size_t)st.n_q_tiles);
+        t.live_keys = tmp_mem.take<uint4>(n_cand);
       }
     }
   };
@@ -585,7 +681,7 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
   LV_TRY(cudaMemcpyAsync(totals.data(), d_totals, sizeof(SetTotals) * totals.size(), cudaMemcpyDeviceToHost, stream));
   LV_TRY(cudaGetLastError());
   LV_TRY(cudaStreamSynchronize(stream));
-  size_t mask_rows = 0, n_chunks = 0;
+  size_t mask_rows = 0;
   for (int k0 = 0; k0 < K; ++k0)
     for (int set = 0; set < n_sets; ++set) {
       const SetTotals& t = totals[(size_t)k0 * n_sets + set];
@@ -596,20 +692,34 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
       ss.n_full = t.n_full;
       ss.live_entries = (int64_t)t.live_entries;
       mask_rows += (size_t)t.n_partial * kBlockM;
-      n_chunks += 2 * (size_t)t.n_pairs;
     }
 
-  // ---- A3, second pass: compaction in canonical order, element masks of the partial pairs, launch order
+  // ---- A3, second pass: compaction in canonical order, element masks of the partial pairs, size of the chunk lists
   void* mask_block = nullptr;
-  static_assert(sizeof(KeyChunk) == sizeof(uint4), "the chunk lists follow the mask rows in one block");
-  LV_TRY(cudaMalloc(&mask_block, (mask_rows + n_chunks + 1) * sizeof(uint4)));
+  LV_TRY(cudaMalloc(&mask_block, (mask_rows + 1) * sizeof(uint4)));
   plan->allocations.push_back(mask_block);
   uint4* next_mask = static_cast<uint4*>(mask_block);
-  KeyChunk* next_chunk = reinterpret_cast<KeyChunk*>(next_mask + mask_rows);
+  auto run_chunk_kernel = [&](int k0, int set, bool fill) {
+    const Step& st = plan->steps[k0];
+    const StepSet& ss = st.sets[set];
+    const SetScratch& t = scratch[(size_t)k0 * n_sets + set];
+    const PlanGeom g{k0, st.s_k, st.n_k, st.L_k, st.n_key_tiles, plan->shape, st.raster_len, st.d_q_geom, st.d_key_geom};
+    ChunkGeom cg = {};
+    cg.n_raster_tiles = st.n_raster_tiles;
+    cg.n_maps = k0 + 1 - st.first_patch;
+    for (int i = 0, tile = st.n_raster_tiles; i < cg.n_maps; ++i) {
+      cg.side[i] = sc.scale[st.first_patch + i];
+      cg.first_tile[i] = tile;
+      tile += ((cg.side[i] + kPatchRows - 1) / kPatchRows) * ((cg.side[i] + kPatchCols - 1) / kPatchCols);
+    }
+    chunk_kernel<<<(unsigned)st.n_q_tiles, kBlockM, 0, stream>>>(g, cg, t.cls, t.blk, ss.d_mask, t.live_keys, fill, ss.d_chunk_ptr,
+                                                                 t.chunk_mask_ptr, ss.d_chunks, ss.d_chunk_mask);
+  };
   for (int k0 = 0; k0 < K; ++k0) {
     Step& st = plan->steps[k0];
     const PlanGeom g{k0, st.s_k, st.n_k, st.L_k, st.n_key_tiles, plan->shape, st.raster_len, st.d_q_geom, st.d_key_geom};
     const dim3 grid2((unsigned)st.n_key_tiles, (unsigned)st.n_q_tiles);
+    const int threads = st.n_q_tiles < 32 ? 32 : (st.n_q_tiles > 512 ? 512 : ((st.n_q_tiles + 31) / 32) * 32);
     for (int set = 0; set < n_sets; ++set) {
       StepSet& ss = st.sets[set];
       const SetScratch& t = scratch[(size_t)k0 * n_sets + set];
@@ -617,27 +727,48 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
       const int32_t* d_radius_row = plan->d_radius + ((size_t)set * K + k0) * K;
       ss.d_mask = next_mask;
       next_mask += (size_t)ss.n_partial * kBlockM;
-      ss.d_chunks = next_chunk;
-      next_chunk += 2 * (size_t)ss.n_pairs;
       compact_kernel<<<(unsigned)((st.n_q_tiles + 127) / 128), 128, 0, stream>>>(
           st.n_q_tiles, st.n_key_tiles, t.cls, ss.d_row_ptr, t.partial_base, ss.d_pairs, t.blk);
-      mask_bits_kernel<<<grid2, 128, 0, stream>>>(sc, g, ss.d_bounds, d_radius_row, t.blk, ss.d_mask);
-      chunk_kernel<<<(unsigned)((st.n_q_tiles + 3) / 4), 128, 0, stream>>>(st.n_q_tiles, st.d_key_geom, ss.d_row_ptr, ss.d_pairs,
-                                                                       ss.d_mask, ss.d_chunks, ss.d_n_chunks);
-      launch_order_kernel<<<(unsigned)(((st.n_q_tiles + 1) / 2 + 127) / 128), 128, 0, stream>>>(st.n_q_tiles,
-                                                                                             ss.d_row_ptr, ss.d_order);
-      first_tile_kernel<<<(unsigned)((st.n_q_tiles + 127) / 128), 128, 0, stream>>>(st.n_q_tiles, ss.d_row_ptr,
-                                                                                    ss.d_pairs, &tot->first_not_zero);
+      mask_bits_kernel<<<grid2, 128, 0, stream>>>(sc, g, ss.d_bounds, d_radius_row, t.blk, ss.d_mask, t.live_keys);
+      run_chunk_kernel(k0, set, false);
+      chunk_scan_kernel<<<1, threads, 2 * sizeof(int32_t) * st.n_q_tiles, stream>>>(st.n_q_tiles, ss.d_chunk_ptr, t.chunk_mask_ptr,
+                                                                                    &tot->n_chunks);
       if (small_step_candidate(st.n_q_tiles, st.n_key_tiles, !st.q_patch && st.first_patch == k0 + 1) &&
           ss.n_pairs >= 1 && ss.n_pairs <= 2)
         copy_first_pairs_kernel<<<1, 32, 0, stream>>>(ss.d_pairs, &tot->n_pairs, tot->first_pairs);
-      const SetDesc desc{ss.d_row_ptr, ss.d_pairs, ss.d_mask, ss.d_chunks, ss.d_n_chunks};
+    }
+  }
+  LV_TRY(cudaMemcpyAsync(totals.data(), d_totals, sizeof(SetTotals) * totals.size(), cudaMemcpyDeviceToHost, stream));
+  LV_TRY(cudaGetLastError());
+  LV_TRY(cudaStreamSynchronize(stream));
+  size_t n_chunks = 0, n_mask_chunks = 0;
+  for (const SetTotals& t : totals) {
+    n_chunks += (size_t)t.n_chunks;
+    n_mask_chunks += (size_t)t.n_mask_chunks;
+  }
+
+  // ---- the chunk lists and their masks
+  void* chunk_block = nullptr;
+  LV_TRY(cudaMalloc(&chunk_block, (n_chunks + 1) * sizeof(KeyChunk) + n_mask_chunks * kBlockM * sizeof(uint2)));
+  plan->allocations.push_back(chunk_block);
+  KeyChunk* next_chunk = static_cast<KeyChunk*>(chunk_block);
+  uint2* next_chunk_mask = reinterpret_cast<uint2*>(next_chunk + n_chunks + 1);
+  for (int k0 = 0; k0 < K; ++k0) {
+    Step& st = plan->steps[k0];
+    for (int set = 0; set < n_sets; ++set) {
+      StepSet& ss = st.sets[set];
+      const SetTotals& t = totals[(size_t)k0 * n_sets + set];
+      ss.d_chunks = next_chunk;
+      next_chunk += t.n_chunks;
+      ss.d_chunk_mask = next_chunk_mask;
+      next_chunk_mask += (size_t)t.n_mask_chunks * kBlockM;
+      run_chunk_kernel(k0, set, true);
+      const SetDesc desc = ss.desc();
       memcpy(host_at(st.d_sets + set), &desc, sizeof(desc));
     }
   }
   LV_TRY(cudaMemcpyAsync(static_cast<char*>(plan_block) + geom_end, host_fill.data() + (geom_end - geom_begin),
                          sets_end - geom_end, cudaMemcpyHostToDevice, stream));
-  LV_TRY(cudaMemcpyAsync(totals.data(), d_totals, sizeof(SetTotals) * totals.size(), cudaMemcpyDeviceToHost, stream));
   LV_TRY(cudaGetLastError());
   LV_TRY(cudaStreamSynchronize(stream));  // the scratch block is freed on return
   for (int k0 = 0; k0 < K; ++k0) {
@@ -645,7 +776,6 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
     for (int set = 0; set < n_sets; ++set) {
       const SetTotals& t = totals[(size_t)k0 * n_sets + set];
       StepSet& ss = st.sets[set];
-      ss.first_tile_zero = t.first_not_zero == 0;
       if (small_step_candidate(st.n_q_tiles, st.n_key_tiles, !st.q_patch && st.first_patch == k0 + 1) &&
           ss.n_pairs >= 1 && ss.n_pairs <= 2) {
         ss.small.n = ss.n_pairs;
@@ -738,8 +868,7 @@ static void fill_step_params(const litevar_plan_t* plan, const Step& st, int32_t
   memset(&p, 0, sizeof(p));
   p.sets = st.d_sets;
   p.head_to_set = plan->n_sets > 1 ? plan->d_head_to_set : nullptr;
-  p.set0 = SetDesc{st.sets[0].d_row_ptr, st.sets[0].d_pairs, st.sets[0].d_mask, st.sets[0].d_chunks, st.sets[0].d_n_chunks};
-  p.order = st.sets[0].d_order;
+  p.set0 = st.sets[0].desc();
   p.n_k = st.n_k;
   p.L_k = st.L_k;
   p.n_heads = plan->n_heads;
@@ -760,9 +889,6 @@ static void fill_step_params(const litevar_plan_t* plan, const Step& st, int32_t
   p.sm_scale = plan->sm_scale;
   p.status = plan->d_status;
   p.overlap_launch = 1;
-  p.first_tile_zero = st.raster_len > 0 ? 1 : 0;  // key tile 0 must be the raster tile of cache rows [0, 128)
-  for (const StepSet& ss : st.sets) p.first_tile_zero &= ss.first_tile_zero ? 1 : 0;
-  p.pairs_per_tile = (st.sets[0].n_pairs + st.n_q_tiles - 1) / st.n_q_tiles;
   p.units_per_group = units_per_l2_group(st.L_k, p.n_heads * p.batch_computed);
 }
 
@@ -940,7 +1066,7 @@ litevar_status_t litevar_plan_materialize_mask(const litevar_plan_t* plan, int32
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   size_t words = (size_t)((st.L_k + 31) / 32);
   LV_CUDA(cudaMemsetAsync(dev_bits, 0, sizeof(uint32_t) * words * st.n_k, stream));
-  SetDesc sd{ss.d_row_ptr, ss.d_pairs, ss.d_mask, ss.d_chunks, ss.d_n_chunks};
+  const SetDesc sd = ss.desc();
   PlanGeom g{step_k - 1, st.s_k, st.n_k, st.L_k, st.n_key_tiles, plan->shape, st.raster_len, st.d_q_geom, st.d_key_geom};
   materialize_kernel<<<(unsigned)st.n_q_tiles, 128, 0, stream>>>(sd, plan->sched, g, static_cast<uint32_t*>(dev_bits));
   LV_CUDA(cudaGetLastError());

@@ -22,21 +22,20 @@ namespace {
 constexpr int kStaticMaxPairs = 2048;  // candidate (query tile, key tile) pairs of one step
 constexpr int kStaticMaxDevices = 64;
 
-// Everything one step's plan needs, at fixed offsets.  Mask block c belongs to candidate pair c
-// (query tile c / n_key_tiles, key tile c % n_key_tiles), so no second compaction is needed.
+// Everything one step's plan needs, at fixed offsets.  Mask blocks 2 c and 2 c + 1 belong to the halves of
+// candidate pair c (query tile c / n_key_tiles, key tile c % n_key_tiles), so no second compaction is needed; the chunks are these
+// halves, on their fixed grid.
 struct StaticPlan {
   SetDesc set;      // read by the forward kernel through FwdParams::sets
   int32_t status;   // bounded-wait flag of the forward kernel; cleared at the start of every call
   int32_t pad[9];
-  int32_t row_ptr[kStaticMaxPairs + 1];
-  Pair pairs[kStaticMaxPairs];
-  int32_t n_chunks[kStaticMaxPairs];
+  int32_t chunk_ptr[kStaticMaxPairs + 1];
   KeyChunk chunks[2 * kStaticMaxPairs];
-  uint8_t cls[kStaticMaxPairs];
-  uint4 mask[(size_t)kStaticMaxPairs * kBlockM];
+  uint32_t cls[kStaticMaxPairs];  // KeyChunk::info of the pair's two halves
+  uint2 chunk_mask[(size_t)2 * kStaticMaxPairs * kBlockM];
 };
 
-// 4.4 MB per GPU.  In host code this name is only a handle for cudaGetSymbolAddress: it is not a device
+// 4.3 MB per GPU.  In host code this name is only a handle for cudaGetSymbolAddress: it is not a device
 // address and must never be passed to a kernel.  Device code below names it directly.
 static __device__ __align__(256) unsigned char litevar_static_scratch[sizeof(StaticPlan)];
 
@@ -49,7 +48,7 @@ __device__ __forceinline__ StaticPlan* static_plan() { return reinterpret_cast<S
 
 // One block per candidate pair: thread m owns query slot m, evaluates the window predicate of
 // paper Section 2 against the 128 key slots of the key tile, writes its 128 mask bits and the
-// class of the pair (0 dead, 1 partial, 2 full).
+// classes of the pair's two 64-key halves.
 __global__ void __launch_bounds__(kBlockM) static_classify_kernel(Schedule sc, StepArgs a) {
   __shared__ int16_t ks_j[kBlockN], ks_r[kBlockN], ks_c[kBlockN];
   __shared__ int32_t ks_t[kBlockN];
@@ -105,56 +104,52 @@ __global__ void __launch_bounds__(kBlockM) static_classify_kernel(Schedule sc, S
       if (lv) w[n >> 5] |= 1u << (n & 31);
     }
   }
-  const int cnt = __popc(w[0]) + __popc(w[1]) + __popc(w[2]) + __popc(w[3]);
-  const int any0 = __syncthreads_or((w[0] | w[1]) != 0u), any1 = __syncthreads_or((w[2] | w[3]) != 0u);
-  const int all = __syncthreads_and(!valid || cnt == kBlockN);
+  __shared__ uint32_t info;
+  if (m == 0) info = 0u;
+  __syncthreads();
+  uint32_t c = 0u;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) c |= (uint32_t)key_class(w[i], valid) << (2 * (i & 1) + 16 * (i >> 1));
+  if ((m & 31) == 0) atomicOr(&info, c << (4 * (m >> 5)));
   const int cand = qt * a.n_key_tiles + kt;
-  sp->mask[(size_t)cand * kBlockM + m] = make_uint4(w[0], w[1], w[2], w[3]);
-  if (m == 0) sp->cls[cand] = (any0 || any1) ? ((all ? 2 : 1) | (any0 ? 4 : 0) | (any1 ? 8 : 0)) : 0;
+  sp->chunk_mask[(size_t)(2 * cand) * kBlockM + m] = make_uint2(w[0], w[1]);
+  sp->chunk_mask[(size_t)(2 * cand + 1) * kBlockM + m] = make_uint2(w[2], w[3]);
+  __syncthreads();
+  if (m == 0) sp->cls[cand] = info;
 }
 
-// One block: per query tile count the live pairs, scan, write the CSR list in canonical order
-// (query tile ascending, key tile ascending), publish the descriptor and clear the status word.
+// One block: per query tile count the live chunks, scan, write the list in canonical order
+// (query tile ascending, key ascending), publish the descriptor and clear the status word.
 __global__ void static_compact_kernel(int n_q_tiles, int n_key_tiles) {
   __shared__ int32_t count[kStaticMaxPairs];
   StaticPlan* sp = static_plan();
   for (int qt = threadIdx.x; qt < n_q_tiles; qt += blockDim.x) {
     int l = 0;
-    for (int kt = 0; kt < n_key_tiles; ++kt) l += sp->cls[qt * n_key_tiles + kt] != 0;
+    for (int kt = 0; kt < n_key_tiles; ++kt) {
+      const uint32_t c = sp->cls[qt * n_key_tiles + kt];
+      l += ((c & 0xffffu) != 0u) + ((c >> 16) != 0u);
+    }
     count[qt] = l;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     int acc = 0;
     for (int qt = 0; qt < n_q_tiles; ++qt) {
-      sp->row_ptr[qt] = acc;
+      sp->chunk_ptr[qt] = acc;
       acc += count[qt];
     }
-    sp->row_ptr[n_q_tiles] = acc;
-    sp->set.row_ptr = sp->row_ptr;
-    sp->set.pairs = sp->pairs;
-    sp->set.mask = sp->mask;
-    sp->set.chunks = sp->chunks;
-    sp->set.n_chunks = sp->n_chunks;
+    sp->chunk_ptr[n_q_tiles] = acc;
+    sp->set = SetDesc{nullptr, nullptr, nullptr, sp->chunks, sp->chunk_ptr, sp->chunk_mask};
     sp->status = 0;
   }
   __syncthreads();
   for (int qt = threadIdx.x; qt < n_q_tiles; qt += blockDim.x) {
-    int o = sp->row_ptr[qt], n_chunks = 0;
-    KeyChunk* chunks = sp->chunks + 2 * o;
-    for (int kt = 0; kt < n_key_tiles; ++kt) {
-      const int cand = qt * n_key_tiles + kt;
-      const int c = sp->cls[cand];
-      if (c != 0) {
-        sp->pairs[o].key_tile = kt;
-        const bool partial = (c & 3) == 1;
-        sp->pairs[o].mask_block = partial ? cand : -1;
-        ++o;
-        for (int hf = 0; hf < 2; ++hf)
-          if (c & (4 << hf)) chunks[n_chunks++] = KeyChunk{kt * kBlockN + hf * (kBlockN / 2), 0, -1, partial ? 2 * cand + hf : -1};
+    KeyChunk* chunks = sp->chunks + sp->chunk_ptr[qt];
+    for (int kt = 0; kt < n_key_tiles; ++kt)
+      for (int hf = 0; hf < 2; ++hf) {
+        const int block = 2 * (qt * n_key_tiles + kt) + hf, info = (int)((sp->cls[block >> 1] >> (16 * hf)) & 0xffffu);
+        if (info != 0) *chunks++ = KeyChunk{kt * kBlockN + hf * (kBlockN / 2), 0, info, info & kPartialBits ? block : -1};
       }
-    }
-    sp->n_chunks[qt] = n_chunks;
   }
 }
 
@@ -260,8 +255,7 @@ extern "C" litevar_status_t litevar_attn_forward_static(
   FwdParams p;
   p.sets = &sp->set;
   p.head_to_set = nullptr;
-  p.set0 = SetDesc{sp->row_ptr, sp->pairs, sp->mask, sp->chunks, sp->n_chunks};  // device addresses inside the fixed array
-  p.order = nullptr;
+  p.set0 = SetDesc{nullptr, nullptr, nullptr, sp->chunks, sp->chunk_ptr, sp->chunk_mask};  // device addresses inside the fixed array
   p.q = static_cast<const uint16_t*>(Q);
   p.k = static_cast<const uint16_t*>(Kc);
   p.v = static_cast<const uint16_t*>(Vc);
@@ -285,9 +279,7 @@ extern "C" litevar_status_t litevar_attn_forward_static(
   p.share_offset = share_cfg ? batch_pairs : 0;
   p.sm_scale = sm_scale > 0.f ? sm_scale : 0.125f;
   p.status = &sp->status;
-  p.pairs_per_tile = 0;
   p.units_per_group = units_per_l2_group(p.L_k, p.n_heads * p.batch_computed);
-  p.first_tile_zero = 0;
   p.overlap_launch = 0;  // the plan is written by the two kernels launched just above
   return launch_forward_ws(p, a.n_q_tiles, stream);
 }

@@ -454,3 +454,26 @@ def test_row_reference_moves_and_redo(kind, tiling):
     ref = orc.attention_step(scales, 7, tab[6], Q, Kc, Vc)
     assert_close(got, ref, kind)
     plan.close()
+
+
+@pytest.mark.parametrize("shape", [binding.WINDOW_SQUARE, binding.WINDOW_BAND], ids=["square", "band"])
+@pytest.mark.parametrize("tiling", TILINGS, ids=lambda t: TNAME[t])
+@pytest.mark.parametrize("scales,radius", [((1, 3, 7, 9, 17), 0), ((1, 2, 15, 16, 23), 1), ((2, 5, 8, 16, 24), 3), ((1, 4, 25, 31, 33), 6)],
+                         ids=["r0", "r1", "r3", "r6"])
+def test_chunk_lists_off_the_tile_grid(scales, radius, tiling, shape):
+    """The tensor-core kernel's 64-key chunks start at a query tile's own live keys: boxes that straddle key tiles and grid
+    edges, narrow windows that leave gaps between the scales, band windows whose live cells fill no box; every output."""
+    lib_ready()
+    K, H, B = len(scales), 2, 1
+    tab = orc.window_table(scales, n_global_scales=0)
+    for k in range(K):
+        tab[k, :k + 1] = radius if shape == binding.WINDOW_SQUARE else [radius * s for s in scales[:k + 1]]
+    w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=95)
+    Kc, Vc = wl.make_kv(w, 0)
+    plan = binding.Plan(scales, n_heads=H, radius=tab, shape=shape, tiling=tiling)
+    for k in (K - 1, K):
+        Q = wl.make_q(w, 0, k)
+        got, _ = run_forward(plan, k, B, Q, Kc, Vc, binding.KERNEL_TCGEN05)
+        ref = orc.attention_step(scales, k, tab[k - 1], Q, Kc, Vc, band=shape == binding.WINDOW_BAND)
+        assert_close(got, ref, f"scales={scales} step {k}")
+    plan.close()
