@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) fwd_simt_kernel(FwdParams
     if (g.scale < 0) {
       q = g.a + m;
     } else {
-      const int r = g.a + m / kPatchCols, c = g.b + m % kPatchCols;
+      const int r = g.a + patch_slot_row(m), c = g.b + patch_slot_col(m);
       q = (r < p.s_k && c < p.s_k) ? r * p.s_k + c : p.n_k;
     }
   }

@@ -620,7 +620,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           if (tg.scale < 0) {
             q = tg.a + mm;
           } else {
-            const int qr = tg.a + mm / kPatchCols, qc = tg.b + mm % kPatchCols;
+            const int qr = tg.a + patch_slot_row(mm), qc = tg.b + patch_slot_col(mm);
             q = (qr < p.s_k && qc < p.s_k) ? qr * p.s_k + qc : -1;
           }
           const uint4 o4 = *reinterpret_cast<const uint4*>(slice + rl * 64 + (((ch ^ (rl >> 1)) & 3) << 4));

@@ -33,11 +33,16 @@ struct Pair {
 
 // Geometry of one query or key tile (128 slots).  Raster: scale < 0, slot m is token a + m (query tiles:
 // token of the current scale; key tiles: cache row, valid below the end of the raster prefix).  Patch:
-// scale = 0-based scale index, slot m is grid cell (a + m / kPatchCols, b + m % kPatchCols) of that scale.
+// scale = 0-based scale index; slot m of a key tile is grid cell (a + m / kPatchCols, b + m % kPatchCols) of that scale, slot m of
+// a query tile cell (a + patch_slot_row(m), b + patch_slot_col(m)).
 struct TileGeom {
   int32_t scale, a, b, map_slot;  // map_slot: index of the scale's tensor maps in the forward kernel (patch tiles)
 };
 constexpr int kPatchRows = 8, kPatchCols = 16;  // kPatchRows * kPatchCols == 128
+// Query slots 32 w .. 32 w + 31 (one warp of the tensor-core kernel) are 4 x 8 cells of the patch: their windows overlap more than
+// those of 2 x 16 cells, so that more halves of key chunks are dead for the warp (4 % of the work at the last 2K step).
+__host__ __device__ inline int patch_slot_row(int m) { return 4 * (m >> 6) + ((m >> 3) & 3); }
+__host__ __device__ inline int patch_slot_col(int m) { return 8 * ((m >> 5) & 1) + (m & 7); }
 constexpr int kMaxPatchScales = 8;              // key scales that can be tiled in 2-D patches
 
 // The whole tile list of a step with one query tile and at most two key tiles, passed to the small-step

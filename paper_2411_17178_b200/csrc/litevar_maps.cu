@@ -92,7 +92,7 @@ bool encode_tensor_maps(const FwdParams& p, tc::TensorMaps* tmp, int key_rows) {
   memset(&tm, 0, sizeof(tm));
   bool ok;
   if (p.q_patch)
-    ok = encode_patch(&tm.q, p.q, 0, p.s_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, kPatchRows, kPatchCols);
+    ok = encode_patch(&tm.q, p.q, 0, p.s_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, 4, 8);  // a warp's slots
   else
     ok = encode_raster(&tm.q, p.q, p.n_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, kBlockM);
   ok = ok && encode_raster(&tm.kr, p.k, p.raster_len, p.n_heads, p.batch_computed, p.k_st, p.k_sh, p.k_sb, key_rows) &&

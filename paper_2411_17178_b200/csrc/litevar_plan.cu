@@ -91,8 +91,8 @@ __device__ __forceinline__ int query_slot_token(const TileGeom& g, int m, int s_
     c = q - r * s_k;
     return q;
   }
-  r = g.a + m / kPatchCols;
-  c = g.b + m % kPatchCols;
+  r = g.a + patch_slot_row(m);
+  c = g.b + patch_slot_col(m);
   if (r >= s_k || c >= s_k) return -1;
   return r * s_k + c;
 }

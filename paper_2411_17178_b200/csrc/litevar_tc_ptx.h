@@ -106,7 +106,7 @@ struct TensorMaps {
   CUtensorMap k2[kMaxPatchScales], v2[kMaxPatchScales];
 };
 
-// Loads of one query / key tile according to its geometry.
+// Loads of one query tile according to its geometry (patch: four boxes of 4 x 8 cells, in slot order).
 __device__ __forceinline__ void load_q_tile(void* dst, const TensorMaps& tm, const FwdParams& p, int qt, int h, int b,
                                             uint64_t* bar) {
   if (p.q_geom == nullptr) {
@@ -117,7 +117,10 @@ __device__ __forceinline__ void load_q_tile(void* dst, const TensorMaps& tm, con
   if (g.scale < 0)
     tma_load_4d(dst, &tm.q, 0, g.a, h, b, bar);
   else
-    tma_load_5d(dst, &tm.q, 0, g.b, g.a, h, b, bar);
+#pragma unroll
+    for (int w = 0; w < 4; ++w)
+      tma_load_5d(static_cast<uint8_t*>(dst) + w * (kTileBytes / 4), &tm.q, 0, g.b + patch_slot_col(32 * w),
+                  g.a + patch_slot_row(32 * w), h, b, bar);
 }
 // Four consecutive K = 16 steps of one product in a single instruction sequence: step i reads A at
 // a_tmem + i * kAStep (TMEM columns) and B at b_desc + i * kBStep (descriptor units of 16 bytes); the first step
