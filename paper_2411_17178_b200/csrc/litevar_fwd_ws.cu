@@ -593,8 +593,12 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         tmem_ld32(tlane + kColO + 64 + 32 * st, r1);
         tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 32; ++e)
-          r[e] = __float_as_uint((w0 > 0.f ? __uint_as_float(r[e]) * w0 : 0.f) + (w1 > 0.f ? __uint_as_float(r1[e]) * w1 : 0.f));
+        for (int e = 0; e < 32; e += 2) {
+          float2 x = make_float2(__uint_as_float(r[e]) * w0, __uint_as_float(r[e + 1]) * w0);
+          if (n_all > 1) x = __ffma2_rn(make_float2(__uint_as_float(r1[e]), __uint_as_float(r1[e + 1])), make_float2(w1, w1), x);
+          r[e] = __float_as_uint(x.x);
+          r[e + 1] = __float_as_uint(x.y);
+        }
         // The warp's 32 rows x 64 B pass through its own 2 KB slice of the Q buffer (its last reader, the last score
         // product, is done: every warp of both streams has seen it through o_full), so that four neighbouring lanes store one
         // row's 64 contiguous bytes.  Chunk position XOR (row / 2) keeps both the writes and the reads free of bank conflicts.
