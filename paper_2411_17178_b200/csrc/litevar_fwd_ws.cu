@@ -600,8 +600,8 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           r[e + 1] = __float_as_uint(x.y);
         }
         // The warp's 32 rows x 64 B pass through its own 2 KB slice of the Q buffer (its last reader, the last score
-        // product, is done: every warp of both streams has seen it through o_full), so that four neighbouring lanes store one
-        // row's 64 contiguous bytes.  Chunk position XOR (row / 2) keeps both the writes and the reads free of bank conflicts.
+        // product, is done: every warp of both streams has seen it through o_full) to a tensor-map store.  Piece position XOR
+        // (row / 2) is the map's swizzle and keeps the writes free of bank conflicts.
         uint8_t* slice = sm.q + (warp << 11);
 #pragma unroll
         for (int e = 0; e < 32; e += 8) {
@@ -612,27 +612,26 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           o4.w = pack_bf16(__uint_as_float(r[e + 6]), __uint_as_float(r[e + 7]));
           *reinterpret_cast<uint4*>(slice + lane * 64 + ((((e >> 3) ^ (lane >> 1)) & 3) << 4)) = o4;
         }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
-        TileGeom tg = TileGeom{-1, qt * kBlockM, 0, 0};
-        if (p.q_geom != nullptr) tg = p.q_geom[qt];
-        uint16_t* obase = p.out + (int64_t)b * p.o_sb + (int64_t)h * p.o_sh + 32 * st;
-#pragma unroll
-        for (int it = 0; it < 4; ++it) {
-          const int rl = it * 8 + (lane >> 2), ch = lane & 3;  // row of the warp's 32, 16-byte chunk of its 64 bytes
-          const int mm = lane_group * 32 + rl;                  // query slot of that row
-          int q;                                                // its token (-1: padding slot)
-          if (tg.scale < 0) {
-            q = tg.a + mm;
+        if (lane == 0) {
+          // the slots' first token or cell; a box that starts outside the grid holds no query
+          const int bs = b + p.share_offset;
+          if (p.q_patch) {
+            const TileGeom g = p.q_geom[qt];
+            const int r0 = g.a + patch_slot_row(32 * lane_group), c0 = g.b + patch_slot_col(32 * lane_group);
+            if (r0 < p.s_k && c0 < p.s_k) {
+              tma_store_5d(&tm.o, slice, 32 * st, c0, r0, h, b);
+              if (p.share_offset > 0) tma_store_5d(&tm.o, slice, 32 * st, c0, r0, h, bs);
+            }
           } else {
-            const int qr = tg.a + patch_slot_row(mm), qc = tg.b + patch_slot_col(mm);
-            q = (qr < p.s_k && qc < p.s_k) ? qr * p.s_k + qc : -1;
+            const int q0 = qt * kBlockM + 32 * lane_group;
+            if (q0 < p.n_k) {
+              tma_store_4d(&tm.o, slice, 32 * st, q0, h, b);
+              if (p.share_offset > 0) tma_store_4d(&tm.o, slice, 32 * st, q0, h, bs);
+            }
           }
-          const uint4 o4 = *reinterpret_cast<const uint4*>(slice + rl * 64 + (((ch ^ (rl >> 1)) & 3) << 4));
-          if (q >= 0 && q < p.n_k) {
-            uint16_t* dst = obase + (int64_t)q * p.o_st + 8 * ch;
-            *reinterpret_cast<uint4*>(dst) = o4;
-            if (p.share_offset > 0) *reinterpret_cast<uint4*>(dst + (int64_t)p.share_offset * p.o_sb) = o4;
-          }
+          asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group.read 0;" ::: "memory");
         }
       }
     }

@@ -27,9 +27,10 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
-// Rank-4 map over a [batch, head, token, 64] bf16 tensor with element strides; box = box_rows tokens x 64.
+// Rank-4 map over a [batch, head, token, 64] bf16 tensor with element strides; box = box_rows tokens x box_dim elements (64, or
+// 32 with the swizzle of 64-byte rows).
 bool encode_raster(CUtensorMap* tm, const void* base, int64_t rows, int64_t heads, int64_t batch, int64_t st,
-                   int64_t sh, int64_t sb, int box_rows) {
+                   int64_t sh, int64_t sb, int box_rows, int box_dim = kHeadDim) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) return false;
   if (rows < 1) rows = 1;  // no raster tile will use this map
@@ -38,10 +39,10 @@ bool encode_raster(CUtensorMap* tm, const void* base, int64_t rows, int64_t head
   if (batch == 1 && sb < kHeadDim) sb = sh * heads;
   cuuint64_t gdim[4] = {(cuuint64_t)kHeadDim, (cuuint64_t)rows, (cuuint64_t)heads, (cuuint64_t)batch};
   cuuint64_t gstr[3] = {(cuuint64_t)st * 2, (cuuint64_t)sh * 2, (cuuint64_t)sb * 2};
-  cuuint32_t box[4] = {(cuuint32_t)kHeadDim, (cuuint32_t)box_rows, 1, 1};
+  cuuint32_t box[4] = {(cuuint32_t)box_dim, (cuuint32_t)box_rows, 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), gdim, gstr, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, box_dim == kHeadDim ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
@@ -69,7 +70,7 @@ bool encode_codes(CUtensorMap* tm, const void* base, int64_t rows, int64_t heads
 // (64, column, row, head, batch); box = box_rows rows x box_cols columns x 64, i.e. box_rows box_cols rows of 128 B in shared
 // memory in row-major order.  A copy may start at any cell.  Cells outside the grid read as zero and are not written.
 bool encode_patch(CUtensorMap* tm, const void* base, int64_t first_token, int64_t side, int64_t heads,
-                  int64_t batch, int64_t st, int64_t sh, int64_t sb, int box_rows, int box_cols) {
+                  int64_t batch, int64_t st, int64_t sh, int64_t sb, int box_rows, int box_cols, int box_dim = kHeadDim) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) return false;
   if (heads == 1 && sh < kHeadDim) sh = st * side * side;
@@ -77,12 +78,19 @@ bool encode_patch(CUtensorMap* tm, const void* base, int64_t first_token, int64_
   const uint16_t* origin = static_cast<const uint16_t*>(base) + first_token * st;
   cuuint64_t gdim[5] = {(cuuint64_t)kHeadDim, (cuuint64_t)side, (cuuint64_t)side, (cuuint64_t)heads, (cuuint64_t)batch};
   cuuint64_t gstr[4] = {(cuuint64_t)st * 2, (cuuint64_t)(st * side) * 2, (cuuint64_t)sh * 2, (cuuint64_t)sb * 2};
-  cuuint32_t box[5] = {(cuuint32_t)kHeadDim, (cuuint32_t)box_cols, (cuuint32_t)box_rows, 1, 1};
+  cuuint32_t box[5] = {(cuuint32_t)box_dim, (cuuint32_t)box_cols, (cuuint32_t)box_rows, 1, 1};
   cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<uint16_t*>(origin), gdim, gstr, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, box_dim == kHeadDim ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+
+// The output: boxes of a warp's 32 query slots x 32 columns (the two stream's warps of a slot store half a row each).
+bool encode_out(const FwdParams& p, CUtensorMap* tm) {
+  const int64_t batch = p.batch_computed + p.share_offset;
+  if (p.q_patch) return encode_patch(tm, p.out, 0, p.s_k, p.n_heads, batch, p.o_st, p.o_sh, p.o_sb, 4, 8, 32);
+  return encode_raster(tm, p.out, p.n_k, p.n_heads, batch, p.o_st, p.o_sh, p.o_sb, 32, 32);
 }
 
 }  // namespace
@@ -90,11 +98,11 @@ bool encode_patch(CUtensorMap* tm, const void* base, int64_t first_token, int64_
 bool encode_tensor_maps(const FwdParams& p, tc::TensorMaps* tmp, int key_rows) {
   tc::TensorMaps& tm = *tmp;
   memset(&tm, 0, sizeof(tm));
-  bool ok;
+  bool ok = encode_out(p, &tm.o);
   if (p.q_patch)
-    ok = encode_patch(&tm.q, p.q, 0, p.s_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, 4, 8);  // a warp's slots
+    ok = ok && encode_patch(&tm.q, p.q, 0, p.s_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, 4, 8);  // a warp's slots
   else
-    ok = encode_raster(&tm.q, p.q, p.n_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, kBlockM);
+    ok = ok && encode_raster(&tm.q, p.q, p.n_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, kBlockM);
   ok = ok && encode_raster(&tm.kr, p.k, p.raster_len, p.n_heads, p.batch_computed, p.k_st, p.k_sh, p.k_sb, key_rows) &&
        encode_raster(&tm.vr, p.v, p.raster_len, p.n_heads, p.batch_computed, p.v_st, p.v_sh, p.v_sb, key_rows);
   for (int i = 0; ok && i < p.n_patch_scales; ++i)
@@ -108,7 +116,7 @@ bool encode_tensor_maps(const FwdParams& p, tc::TensorMaps* tmp, int key_rows) {
 bool encode_code_maps(const FwdParams& p, tc::TensorMaps* tmp, int key_rows) {
   tc::TensorMaps& tm = *tmp;
   memset(&tm, 0, sizeof(tm));
-  return encode_raster(&tm.q, p.q, p.n_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, kBlockM) &&
+  return encode_out(p, &tm.o) && encode_raster(&tm.q, p.q, p.n_k, p.n_heads, p.batch_computed, p.q_st, p.q_sh, p.q_sb, kBlockM) &&
          encode_codes(&tm.kr, p.k8, p.L_k, p.n_heads, p.batch_computed, p.c_st, p.c_sh, p.c_sb, key_rows) &&
          encode_codes(&tm.vr, p.v8, p.L_k, p.n_heads, p.batch_computed, p.c_st, p.c_sh, p.c_sb, key_rows);
 }

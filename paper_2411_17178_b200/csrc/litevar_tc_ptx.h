@@ -102,9 +102,23 @@ __device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, i
 // Tensor maps of one launch.  q is rank 4 (raster query tiles) or rank 5 (patch query tiles); kr/vr
 // cover the raster prefix of the cache; k2/v2[i] cover the grid of the i-th key scale tiled in patches.
 struct TensorMaps {
+  CUtensorMap o;                   // the output: a warp's 32 query slots x 32 columns
   CUtensorMap q, kr, vr;
   CUtensorMap k2[kMaxPatchScales], v2[kMaxPatchScales];
 };
+
+// One warp's 32 output rows x 32 columns from shared memory (64-byte rows, 16-byte piece c of row m at position
+// c ^ (m / 2 % 4)); rows outside the tensor are not written.  The caller commits the group.
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, const void* src, int x, int y, int z, int w) {
+  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(map),
+               "r"(smem_u32(src)), "r"(x), "r"(y), "r"(z), "r"(w)
+               : "memory");
+}
+__device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, const void* src, int x, int y, int z, int w, int v) {
+  asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5, %6}], [%1];" ::"l"(map),
+               "r"(smem_u32(src)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(v)
+               : "memory");
+}
 
 // Loads of one query tile according to its geometry (patch: four boxes of 4 x 8 cells, in slot order).
 __device__ __forceinline__ void load_q_tile(void* dst, const TensorMaps& tm, const FwdParams& p, int qt, int h, int b,
