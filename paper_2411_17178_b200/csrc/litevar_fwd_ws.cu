@@ -12,6 +12,11 @@
 //                   complete, O += P(i) V(i) and S(i + 1) = Q K(i + 1) go out back to back; they execute in issue order, so
 //                   that S may overwrite P.  The warp runs converged and what it computes is uniform, so that descriptors
 //                   stay in uniform registers (a lane of its own: eight register moves per MMA); one elected lane issues.
+// MANY: a CTA takes several tiles in turn.  Q has two buffers; K and V copies and the first score product of the next tile go out
+// behind the last products of this one, the softmax warps look the next list up while they wait for their accumulator, and the
+// output leaves by tensor-map stores that nobody waits for until the buffer's next use.  What orders the tiles: the first
+// P V product of a tile (which overwrites the accumulator) follows the softmax warps' P, which they write after they and the
+// warp with the other stream of their rows have read both accumulators; a Q copy follows the stores of the tile that had its buffer.
 // Two CTAs per SM, so that every scheduler has four softmax warps of four streams that are in different phases.
 // TMEM columns: S and P of stream s at 64 s, O at 128 + 64 s.
 //
@@ -69,12 +74,13 @@ struct CodeStage<true> {
   uint64_t kc_full[2][2], vc_full[2];
 };
 
-template <bool KV8>
+template <bool KV8, bool MANY>
 struct WsShared : CodeStage<KV8> {
-  alignas(1024) uint8_t q[kTileBytes];  // Q; at the end the output rows pass through it
+  alignas(1024) uint8_t q[MANY ? 2 : 1][kTileBytes];  // Q; at the end of a tile the output rows pass through it
   alignas(1024) uint8_t k[2][kStages][kChunkBytes];
   alignas(1024) uint8_t v[2][kStages][kChunkBytes];
-  alignas(8) uint64_t q_full;
+  alignas(8) float2 ref[2][MANY ? kBlockM : 1];  // reference and row sum of each stream (one tile only: in its idle K stages)
+  alignas(8) uint64_t q_full[2], q_free;
   uint64_t k_full[2][kStages], v_full[2][kStages];
   uint64_t s_full[2], o_full[2];
   uint32_t tmem_base;
@@ -183,21 +189,44 @@ __device__ __forceinline__ void put_scales(float (&sz)[2][kChunkKeys], const Row
   }
 }
 
-template <bool KV8>
+template <bool KV8, bool MANY>
 __global__ void __launch_bounds__(kThreads, 2)
-fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ FwdParams p, int n_q_tiles) {
+fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ FwdParams p, int n_q_tiles, int n_items) {
+  static_assert(!(KV8 && MANY), "the code stages leave no room for a second Q buffer");
+  constexpr int kQBufs = MANY ? 2 : 1;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  WsShared<KV8>& sm = *reinterpret_cast<WsShared<KV8>*>(smem_raw);
+  WsShared<KV8, MANY>& sm = *reinterpret_cast<WsShared<KV8, MANY>*>(smem_raw);
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;  // warp-uniform
   const int st = warp < 8 ? warp >> 2 : warp - 8;  // stream
-  int qt, unit;  // grouped launch order, see cta_work
-  cta_work(p, n_q_tiles, qt, unit);
-  const int h = unit % p.n_heads, b = unit / p.n_heads;
+  // One query tile of one (head, batch row), in the grouped order of work_item, and this stream's share of its list.  A CTA
+  // takes items blockIdx.x, blockIdx.x + gridDim.x, ... (MANY; else one).
+  struct Item {
+    int qt, h, b, n_all, n;  // n: this stream's chunks st, st + 2, ...
+    const KeyChunk* chunks;  // the first of them
+    const uint2* mask;
+  };
+  auto item_at = [&](int w) {
+    Item x;
+    int unit;
+    work_item(p, n_q_tiles, w, x.qt, unit);
+    x.h = unit % p.n_heads;
+    x.b = unit / p.n_heads;
+    const SetDesc sd = p.head_to_set ? p.sets[p.head_to_set[x.h]] : p.set0;
+    const int first = __ldg(&sd.chunk_ptr[x.qt]);
+    x.n_all = __ldg(&sd.chunk_ptr[x.qt + 1]) - first;
+    x.n = (x.n_all - st + 1) >> 1;
+    x.chunks = sd.chunks + first + st;
+    x.mask = sd.chunk_mask;
+    return x;
+  };
+  const int w_step = MANY ? (int)gridDim.x : n_items;
   volatile int* abort_flag = &sm.abort_flag;
 
   if (warp >= 8 && elect_one()) {  // each issuing warp sets up its own stream's barriers
     if (st == 0) {
-      mbar_init(&sm.q_full, 1);
+      mbar_init(&sm.q_full[0], 1);
+      mbar_init(&sm.q_full[1], 1);
+      mbar_init(&sm.q_free, 8);  // every softmax warp arrives when the tile's output rows have left the buffer
       sm.abort_flag = 0;
       sm.redo = 0;
     }
@@ -225,10 +254,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  const SetDesc sd = p.head_to_set ? p.sets[p.head_to_set[h]] : p.set0;
-  const int first = __ldg(&sd.chunk_ptr[qt]), n_all = __ldg(&sd.chunk_ptr[qt + 1]) - first;
-  const int n = (n_all - st + 1) >> 1;  // this stream's chunks: st, st + 2, ...
-  const KeyChunk* chunks = sd.chunks + first + st;
+  const Item item0 = item_at(blockIdx.x);
   // The barriers and the TMEM address are shared here.  The issuing warps' first copies are on their way, and the softmax
   // warps' list and mask words looked up, before the CTA meets: a tile of a short list spends 3000 of its 20000 cycles on the
   // first copies (-2.5 to -5 % with the first reference).  With an 8-bit cache it meets first, which measured 1 % faster.
@@ -239,36 +265,83 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
   };
   if constexpr (KV8) meet();
 
-  bool exact = false;  // second pass over the list, every chunk's maximum taken before its probabilities
-  for (int base = 0;; base += n) {  // step counter of the pass's first chunk: barrier phases go on from pass to pass
-    const int end = base + n;
+  bool exact = false;  // second pass over the lists, every chunk's maximum taken before its probabilities
+  // Counters that go on from tile to tile and pass to pass, as the barriers' phases do: this stream's chunks (`base`: before the
+  // current tile), tiles, tiles in which this stream has a chunk.
+  int base = 0, tiles = 0, o_tiles = 0;
+  for (;;) {
     if (warp >= 8) {
       // ---------------------------------------------------------------- copies and MMAs of the stream.  The whole warp runs
       // this code (what it computes is uniform, so that descriptors and coordinates live in uniform registers); one
       // elected lane issues.  P(i) complete is the event to wait for: PV(i) and S(i + 1) are issued back to back (they
       // execute in issue order, so that S may overwrite P).
-      const uint64_t q_desc = make_desc(smem_u32(sm.q)), k_desc0 = make_desc(smem_u32(sm.k[st][0]));
+      const uint64_t q_desc0 = make_desc(smem_u32(sm.q[0])), k_desc0 = make_desc(smem_u32(sm.k[st][0]));
       const uint64_t v_desc0 = make_desc(smem_u32(sm.v[st][0]));
-      auto chunk = [&](int i) { return chunk_at(chunks + 2 * min(i, n - 1)); };
-      KeyChunk c_k = {}, c_v = {};  // what the next K and V copy takes; looked up a step ahead
+      // The copies run ahead of the products, into the CTA's next tile where the list ends: `at` is the tile of the next K copy,
+      // c_k its chunk, number j of it; V copies follow one step behind (c_v, of head and batch row h_v, b_v).
+      Item at = item0;
+      int at_w = blockIdx.x, j = 0;
+      KeyChunk c_k = {}, c_v = {};
+      int h_v = at.h, b_v = at.b;
       int nk = base, nv = base;     // copies issued
-      auto load_k = [&](const KeyChunk& c) {
-        if (elect_one()) load_chunk(sm.k[st][nk % kStages], &tm.kr, tm.k2, c, h, b, &sm.k_full[st][nk % kStages]);
-        ++nk;
+      auto settle = [&] {
+        while (j >= at.n) {
+          if (!MANY) {
+            at_w = n_items;
+            return;
+          }
+          at_w += w_step;
+          if (at_w >= n_items) return;
+          at = item_at(at_w);
+          j = 0;
+        }
+        c_k = chunk_at(at.chunks + 2 * j);
       };
-      auto load_v = [&](const KeyChunk& c) {
-        if (elect_one()) load_chunk(sm.v[st][nv % kStages], &tm.vr, tm.v2, c, h, b, &sm.v_full[st][nv % kStages]);
+      auto load_k = [&] {
+        if (elect_one()) load_chunk(sm.k[st][nk % kStages], &tm.kr, tm.k2, c_k, at.h, at.b, &sm.k_full[st][nk % kStages]);
+        ++nk;
+        c_v = c_k;
+        h_v = at.h;
+        b_v = at.b;
+        ++j;
+        settle();
+      };
+      auto load_v = [&] {
+        if (elect_one()) load_chunk(sm.v[st][nv % kStages], &tm.vr, tm.v2, c_v, h_v, b_v, &sm.v_full[st][nv % kStages]);
         ++nv;
+      };
+      auto chunk = [&](int i) { return chunk_at(item0.chunks + 2 * min(i, item0.n - 1)); };  // 8-bit cache (one tile)
+      int nq = tiles;  // Q copies issued (stream 0)
+      const int q_pass = nq;
+      // waits until the tile that had the buffer before has been stored (a pass starts with both buffers free)
+      auto load_q = [&](int w) {
+        bool free = true;
+        if (MANY && nq - q_pass >= kQBufs) free = mbar_wait_long(&sm.q_free, (uint32_t)((nq - kQBufs) & 1), abort_flag, p.status);
+        if (free) {
+          int qt = item0.qt, qh = item0.h, qb = item0.b;
+          if (MANY && w != (int)blockIdx.x) {
+            int unit;
+            work_item(p, n_q_tiles, w, qt, unit);
+            qh = unit % p.n_heads;
+            qb = unit / p.n_heads;
+          }
+          if (elect_one()) {
+            mbar_expect_tx(&sm.q_full[nq % kQBufs], kTileBytes);
+            load_q_tile(sm.q[nq % kQBufs], tm, p, qt, qh, qb, &sm.q_full[nq % kQBufs]);
+          }
+          ++nq;
+        }
+        return free;
       };
       // 8-bit cache: the copies bring codes, and the warp puts the rows' scales beside them (looked up a step ahead)
       RowScales rs_k = {}, rs_v = {};
       const float* scales[4] = {};
       if constexpr (KV8) {
-        const int64_t at = (int64_t)b * p.z_sb + (int64_t)h * p.z_sh;
-        scales[0] = p.k_scale + at;
-        scales[1] = p.k_zero + at;
-        scales[2] = p.v_scale + at;
-        scales[3] = p.v_zero + at;
+        const int64_t row0 = (int64_t)item0.b * p.z_sb + (int64_t)item0.h * p.z_sh;
+        scales[0] = p.k_scale + row0;
+        scales[1] = p.k_zero + row0;
+        scales[2] = p.v_scale + row0;
+        scales[3] = p.v_zero + row0;
       }
       auto load_kc = [&](const KeyChunk& c) {
         if constexpr (KV8) {
@@ -277,7 +350,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           __syncwarp();
           if (elect_one()) {
             mbar_expect_tx(&sm.kc_full[st][s], kCodeBytes);
-            tma_load_4d(sm.kc[st][s], &tm.kr, 0, c.row, h, b, &sm.kc_full[st][s]);
+            tma_load_4d(sm.kc[st][s], &tm.kr, 0, c.row, item0.h, item0.b, &sm.kc_full[st][s]);
           }
           ++nk;
         }
@@ -288,19 +361,17 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           __syncwarp();
           if (elect_one()) {
             mbar_expect_tx(&sm.vc_full[st], kCodeBytes);
-            tma_load_4d(sm.vc[st], &tm.vr, 0, c.row, h, b, &sm.vc_full[st]);
+            tma_load_4d(sm.vc[st], &tm.vr, 0, c.row, item0.h, item0.b, &sm.vc_full[st]);
           }
           ++nv;
         }
       };
-      if (n > 0) c_k = chunk(0);
       if (!exact) asm volatile("griddepcontrol.wait;" ::: "memory");
-      if (st == 0 && elect_one()) {
-        mbar_expect_tx(&sm.q_full, kTileBytes);
-        load_q_tile(sm.q, tm, p, qt, h, b, &sm.q_full);
-      }
+      bool ok = true;
+      if (st == 0) ok = load_q(blockIdx.x);
       if constexpr (KV8) {
-        if (n > 0) {
+        if (item0.n > 0) {
+          c_k = chunk(0);
           c_v = chunk(1);
           rs_k = row_scales(scales[0], scales[1], c_k.row, p.L_k, lane);
           rs_v = row_scales(scales[2], scales[3], c_k.row, p.L_k, lane);
@@ -308,74 +379,86 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           load_kc(c_k);
           load_vc(c_k);
           rs_k = rs_k1;
-          if (n > 1) load_kc(c_v);
+          if (item0.n > 1) load_kc(c_v);
           c_k = chunk(2);
           rs_k = row_scales(scales[0], scales[1], c_k.row, p.L_k, lane);
           rs_v = row_scales(scales[2], scales[3], c_v.row, p.L_k, lane);
         }
       } else {
-        for (int i = 0; i < kStages && i < n; ++i) {
-          const KeyChunk c_next = chunk(i + 1);
-          load_k(c_k);
-          load_v(c_k);
-          c_k = c_v = c_next;
+        settle();
+        for (int i = 0; i < kStages && at_w < n_items; ++i) {
+          load_k();
+          load_v();
         }
       }
+      if (MANY && st == 0 && ok && blockIdx.x + w_step < n_items) ok = load_q(blockIdx.x + w_step);
       if (!KV8 && !exact) meet();
       const uint32_t tS = sm.tmem_base + 64 * st, tO = tS + kColO;
-      bool ok = mbar_wait_long(&sm.q_full, exact ? 1u : 0u, abort_flag, p.status);
-      for (int i = base - 1; i < end && n > 0; ++i) {
-        const int s = i % kStages, s1 = (i + 1) % kStages;
-        if (ok && i + 1 < end) ok = mbar_wait_long(&sm.k_full[st][s1], (uint32_t)(((i + 1) / kStages) & 1), abort_flag, p.status);
-        if (i >= base && ok) ok = mbar_wait_long(&sm.v_full[st][s], (uint32_t)((i / kStages) & 1), abort_flag, p.status);
-        if constexpr (KV8) {  // K(i + 1) and V(i) are widened: their code buffers take K(i + 3) and V(i + 1)
-          if (ok) {
-            const KeyChunk c = c_k;
-            if (i >= base && nv < end) {
-              load_vc(c_v);
-              c_v = chunk(nv - base);
-              rs_v = row_scales(scales[2], scales[3], c_v.row, p.L_k, lane);
-            }
-            if (nk < end) {
-              load_kc(c);
-              c_k = chunk(nk - base);
-              rs_k = row_scales(scales[0], scales[1], c_k.row, p.L_k, lane);
+      int n = item0.n;
+      for (int w = blockIdx.x, x = 0;; w += w_step, ++x) {
+        int n_next = 0;
+        if (MANY && w + w_step < n_items) n_next = item_at(w + w_step).n;
+        const int end = base + n;
+        if (ok) ok = mbar_wait_long(&sm.q_full[tiles % kQBufs], (uint32_t)((tiles / kQBufs) & 1), abort_flag, p.status);
+        const uint64_t q_desc = q_desc0 + (uint64_t)((kTileBytes >> 4) * (tiles % kQBufs));
+        for (int i = base - 1; i < end && n > 0; ++i) {
+          const int s = i % kStages, s1 = (i + 1) % kStages;
+          if (ok && i + 1 < end) ok = mbar_wait_long(&sm.k_full[st][s1], (uint32_t)(((i + 1) / kStages) & 1), abort_flag, p.status);
+          if (i >= base && ok) ok = mbar_wait_long(&sm.v_full[st][s], (uint32_t)((i / kStages) & 1), abort_flag, p.status);
+          if constexpr (KV8) {  // K(i + 1) and V(i) are widened: their code buffers take K(i + 3) and V(i + 1)
+            if (ok) {
+              const KeyChunk c = c_k;
+              if (i >= base && nv < end) {
+                load_vc(c_v);
+                c_v = chunk(nv - base);
+                rs_v = row_scales(scales[2], scales[3], c_v.row, p.L_k, lane);
+              }
+              if (nk < end) {
+                load_kc(c);
+                c_k = chunk(nk - base);
+                rs_k = row_scales(scales[0], scales[1], c_k.row, p.L_k, lane);
+              }
             }
           }
-        }
-        if (i >= base) {
-          __syncwarp();
-          asm volatile("bar.sync %0, 160;" ::"r"(5 + st) : "memory");  // P(i); the softmax warps arrive even when a wait ran out
-        }
-        if (ok) {
-          tc_fence_after();
           if (i >= base) {
-            // 16 keys per step = 16 rows of 128 B = 2048 B of V and 8 packed columns of P
-            mma_ts_x4_one<8, (2048 >> 4)>(tO, tS, v_desc0 + (uint64_t)((kChunkBytes >> 4) * s), kIdescO, i > base ? 1u : 0u);
+            __syncwarp();
+            asm volatile("bar.sync %0, 160;" ::"r"(5 + st) : "memory");  // P(i); the softmax warps arrive even when a wait ran out
           }
-          if (i + 1 < end) {
-            // 16 bf16 = 32 B per step inside the swizzle rows of Q and K
-            mma_ss_x4_one<2, 2>(tS, q_desc, k_desc0 + (uint64_t)((kChunkBytes >> 4) * s1), kIdescS, 0u);
-            mma_commit_one(&sm.s_full[st]);
-          } else {
-            mma_commit_one(&sm.o_full[st]);
-          }
-          // P(i) was complete, so S(i) and PV(i - 1) are: K(i + stages) and V(i - 1 + stages) go where K(i) and V(i - 1) were
-          if constexpr (!KV8) {
-            if (i > base && nv < end) load_v(c_v);
-            if (i >= base && nk < end) {
-              load_k(c_k);
-              c_v = c_k;
-              c_k = chunk(nk - base);
+          if (ok) {
+            tc_fence_after();
+            if (i >= base) {
+              // 16 keys per step = 16 rows of 128 B = 2048 B of V and 8 packed columns of P
+              mma_ts_x4_one<8, (2048 >> 4)>(tO, tS, v_desc0 + (uint64_t)((kChunkBytes >> 4) * s), kIdescO, i > base ? 1u : 0u);
             }
+            if (i + 1 < end) {
+              // 16 bf16 = 32 B per step inside the swizzle rows of Q and K
+              mma_ss_x4_one<2, 2>(tS, q_desc, k_desc0 + (uint64_t)((kChunkBytes >> 4) * s1), kIdescS, 0u);
+              mma_commit_one(&sm.s_full[st]);
+            } else {
+              mma_commit_one(&sm.o_full[st]);
+            }
+            // P(i) was complete, so S(i) and PV(i - 1) are: K(i + stages) and V(i - 1 + stages) go where K(i) and V(i - 1) were
+            if constexpr (!KV8) {
+              if (i >= base) {
+                if (nv < nk) load_v();
+                if (at_w < n_items) load_k();
+              }
+            }
+            // the next tile's Q, once the tile before this one has left its buffer (the first two were copied at the start)
+            if (MANY && st == 0 && i == base && x > 0 && w + w_step < n_items) ok = load_q(w + w_step);
+            __syncwarp();
           }
-          __syncwarp();
         }
+        base = end;
+        n = n_next;
+        ++tiles;
+        if (!MANY || w + w_step >= n_items) break;
       }
-      if (*abort_flag || n <= 0) {  // wait (bounded) for copies still in flight before the CTA may exit
+      if (*abort_flag) {  // wait (bounded) for copies still in flight before the CTA may exit
         const unsigned long long ts = global_ns();
-        while (!mbar_try(&sm.q_full, exact ? 1u : 0u))
-          if (global_ns() - ts > kWaitLimitNs) break;
+        for (int i = nq > kQBufs ? nq - kQBufs : 0; st == 0 && i < nq; ++i)
+          while (!mbar_try(&sm.q_full[i % kQBufs], (uint32_t)((i / kQBufs) & 1)))
+            if (global_ns() - ts > kWaitLimitNs) break;
         if constexpr (KV8) {
           for (int i = nk > 2 ? nk - 2 : 0; i < nk; ++i)
             while (!mbar_try(&sm.kc_full[st][i & 1], (uint32_t)((i >> 1) & 1)))
@@ -398,17 +481,11 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       const float sc = p.sm_scale * 1.4426950408889634f;
       const float2 sc2 = make_float2(sc, sc);
       const float sc_y = sc * (0.5f / kClamp);
-      // probabilities are 2^(score * sc - msc).  msc starts as the maximum of a few keys and moves by whole powers of two
-      // when a chunk's sum gets large; it stays 0 and `none` until a live chunk has been seen.
-      float msc = 0.f;
-      bool none = true;
-      float alpha = 1.f;  // pending factor of the accumulator
-      float2 l2a = make_float2(0.f, 0.f), l2b = make_float2(0.f, 0.f);  // row sum
-      bool bad = false, ok = true;
       // Per chunk: class of its two halves for this warp's rows (bits 0 - 1 and 2 - 3: 0 dead, 1 partial, 2 full) and the key bits
       // of this thread's row, looked up one chunk ahead.
-      const int2* infos = reinterpret_cast<const int2*>(&chunks->info);  // {info, mask block}, every second chunk is this stream's
-      const uint2* mask_row = sd.chunk_mask + m;
+      int n = item0.n, n_all = item0.n_all;
+      const int2* infos = reinterpret_cast<const int2*>(&item0.chunks->info);  // {info, mask block}, every second chunk is this stream's
+      const uint2* mask_row = item0.mask + m;
       int cls = 0, cls_next = 0;
       auto look_up = [&](int j, int& c) {
         uint2 bits = make_uint2(0u, 0u);
@@ -422,199 +499,242 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         return bits;
       };
       uint2 mk = look_up(0, cls), mk_next = look_up(1, cls_next);
+      bool bad = false, ok = true;
       if (!KV8 && !exact) meet();
       const uint32_t tlane = sm.tmem_base + ((uint32_t)(lane_group * 32) << 16);
       const uint32_t tS = tlane + 64 * st, tO = tlane + kColO + 64 * st;
-      bool rescale = false;  // some row of the warp has a pending alpha
-      float l_seen = 0.f;     // row sum before this chunk
-      // 8-bit cache: the stream's softmax threads widen its chunks, K(i + 2) and V(i + 1) while the products after P(i) run
-      const int t = threadIdx.x & 127;
-      auto widen_k = [&](int i) {
-        if constexpr (KV8) {
-          if (ok && i < end && (ok = mbar_wait_long(&sm.kc_full[st][i & 1], (uint32_t)((i >> 1) & 1), abort_flag, p.status))) {
-            widen_chunk(sm.kc[st][i & 1], sm.k_sz[st][i & 1], sm.k[st][i % kStages], t);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.k_full[st][i % kStages]);
-          }
+      // the previous tile's output rows have left their buffer, which the next copy but one (the redo's next) goes to
+      auto stored = [&] {
+        if (lane == 0) {
+          asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+          if (MANY) mbar_arrive(&sm.q_free);
         }
       };
-      auto widen_v = [&](int i) {
-        if constexpr (KV8) {
-          if (ok && i < end && (ok = mbar_wait_long(&sm.vc_full[st], (uint32_t)(i & 1), abort_flag, p.status))) {
-            widen_chunk(sm.vc[st], sm.v_sz[st], sm.v[st][i % kStages], t);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sm.v_full[st][i % kStages]);
+      for (int w = blockIdx.x;; w += w_step) {
+        const int end = base + n;
+        // probabilities are 2^(score * sc - msc).  msc starts as the maximum of a few keys and moves by whole powers of two
+        // when a chunk's sum gets large; it stays 0 and `none` until a live chunk has been seen.
+        float msc = 0.f;
+        bool none = true;
+        float alpha = 1.f;  // pending factor of the accumulator
+        float2 l2a = make_float2(0.f, 0.f), l2b = make_float2(0.f, 0.f);  // row sum
+        bool rescale = false;  // some row of the warp has a pending alpha
+        float l_seen = 0.f;     // row sum before this chunk
+        // 8-bit cache: the stream's softmax threads widen its chunks, K(i + 2) and V(i + 1) while the products after P(i) run
+        const int t = threadIdx.x & 127;
+        auto widen_k = [&](int i) {
+          if constexpr (KV8) {
+            if (ok && i < end && (ok = mbar_wait_long(&sm.kc_full[st][i & 1], (uint32_t)((i >> 1) & 1), abort_flag, p.status))) {
+              widen_chunk(sm.kc[st][i & 1], sm.k_sz[st][i & 1], sm.k[st][i % kStages], t);
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&sm.k_full[st][i % kStages]);
+            }
           }
-        }
-      };
-      widen_k(base);
-      widen_v(base);
-      widen_k(base + 1);
-      for (int j = 0; j < n; ++j) {
-        // S(j) complete; in issue order this also means that PV(j - 1) is complete
-        if (ok) ok = mbar_wait_long(&sm.s_full[st], (uint32_t)((base + j) & 1), abort_flag, p.status);
-        if (!ok) {  // the issuing warp counts on every step's arrival
-          asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
-          continue;
-        }
-        tc_fence_after();
-        if (j == 0 || exact) {  // a reference first: the chunk's maximum, or in the first pass that of its first eight keys
-          float mx = -INFINITY;
-          if (cls && !exact) {
-            uint32_t r[8];
-            tmem_ld8(tS, r);
-            tmem_wait_ld();
-#pragma unroll
-            for (int e = 0; e < 8; ++e) mx = fmaxf(mx, (mk.x >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
-          } else if (cls) {
-#pragma unroll 1
-            for (int hf = 0; hf < 2; ++hf) {
-              const uint32_t w = hf ? mk.y : mk.x;
-              uint32_t r[32];
-              tmem_ld32(tS + 32 * hf, r);
+        };
+        auto widen_v = [&](int i) {
+          if constexpr (KV8) {
+            if (ok && i < end && (ok = mbar_wait_long(&sm.vc_full[st], (uint32_t)(i & 1), abort_flag, p.status))) {
+              widen_chunk(sm.vc[st], sm.v_sz[st], sm.v[st][i % kStages], t);
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&sm.v_full[st][i % kStages]);
+            }
+          }
+        };
+        widen_k(base);
+        widen_v(base);
+        widen_k(base + 1);
+        for (int j = 0; j < n; ++j) {
+          // S(j) complete; in issue order this also means that PV(j - 1) is complete
+          if (ok) ok = mbar_wait_long(&sm.s_full[st], (uint32_t)((base + j) & 1), abort_flag, p.status);
+          if (!ok) {  // the issuing warp counts on every step's arrival
+            asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
+            continue;
+          }
+          tc_fence_after();
+          if (j == 0 || exact) {  // a reference first: the chunk's maximum, or in the first pass that of its first eight keys
+            float mx = -INFINITY;
+            if (cls && !exact) {
+              uint32_t r[8];
+              tmem_ld8(tS, r);
               tmem_wait_ld();
 #pragma unroll
-              for (int e = 0; e < 32; ++e) mx = fmaxf(mx, (w >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
+              for (int e = 0; e < 8; ++e) mx = fmaxf(mx, (mk.x >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
+            } else if (cls) {
+#pragma unroll 1
+              for (int hf = 0; hf < 2; ++hf) {
+                const uint32_t w = hf ? mk.y : mk.x;
+                uint32_t r[32];
+                tmem_ld32(tS + 32 * hf, r);
+                tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 32; ++e) mx = fmaxf(mx, (w >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
+              }
+            }
+            if (mx != -INFINITY && (none || mx * sc - msc > kRescaleThreshold)) {
+              if (!none) {
+                alpha *= fast_exp2(msc - mx * sc);
+                l2a.x *= alpha; l2a.y *= alpha; l2b.x *= alpha; l2b.y *= alpha;
+              }
+              msc = mx * sc;
+              none = false;
+            }
+            rescale = __any_sync(0xffffffffu, alpha != 1.f);
+          }
+          if (rescale) {  // the accumulator follows the reference
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {
+              uint32_t o[16];
+              tmem_ld16(tO + 16 * c, o);
+              tmem_wait_ld();
+#pragma unroll
+              for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+              tmem_st16(tO + 16 * c, o);
+            }
+            alpha = 1.f;
+          }
+#pragma unroll 1
+          for (int hf = 0; hf < 2; ++hf) {
+            if ((cls >> (2 * hf)) & 3) {
+              uint32_t r[32], pk[16];
+              tmem_ld32(tS + 32 * hf, r);
+              tmem_wait_ld();
+              if ((cls >> (2 * hf)) & 1) {  // dead scores of a partially live half become -inf
+                const uint32_t w = hf ? mk.y : mk.x;
+#pragma unroll
+                for (int e = 0; e < 32; ++e)
+                  if (!((w >> e) & 1u)) r[e] = 0xff800000u;
+              }
+              // probabilities against the reference: scale and shift (packed FMAs), 2^x, row sum, bf16
+              const float2 nm2 = make_float2(-msc, -msc);
+              const float nm_y = fmaf(-msc, 0.5f / kClamp, 0.5f);
+#pragma unroll
+              for (int e = 0; e < 32; e += 4) {
+                const uint32_t* rr = r + e;
+                const float2 xa = __ffma2_rn(make_float2(__uint_as_float(rr[0]), __uint_as_float(rr[1])), sc2, nm2);
+                const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
+                // every fourth pair on the FMA pipe: the exponential pipe (16 per clock and SM) is the tighter of the two
+                float2 pb;
+                if (e & 4) {
+                  pb = exp2_fma2(make_float2(__saturatef(fmaf(__uint_as_float(rr[2]), sc_y, nm_y)),
+                                             __saturatef(fmaf(__uint_as_float(rr[3]), sc_y, nm_y))));
+                } else {
+                  const float2 xb = __ffma2_rn(make_float2(__uint_as_float(rr[2]), __uint_as_float(rr[3])), sc2, nm2);
+                  pb = make_float2(fast_exp2(xb.x), fast_exp2(xb.y));
+                }
+                // the row sum adds the probabilities as the PV product sees them (rounded to bf16): numerator and
+                // denominator of a row then agree, and a row with one dominant key reproduces that key's V exactly
+                const uint32_t ka = pack_bf16(pa.x, pa.y), kb = pack_bf16(pb.x, pb.y);
+                add_bf16_pair(l2a, ka);
+                add_bf16_pair(l2b, kb);
+                pk[(e >> 1) + 0] = ka;
+                pk[(e >> 1) + 1] = kb;
+              }
+              tmem_st16(tS + 16 * hf, pk);  // over scores that have been read
+            } else {  // no live key for any row of the warp
+              uint32_t pk[16];
+#pragma unroll
+              for (int e = 0; e < 16; ++e) pk[e] = 0u;
+              tmem_st16(tS + 16 * hf, pk);
             }
           }
-          if (mx != -INFINITY && (none || mx * sc - msc > kRescaleThreshold)) {
-            if (!none) {
-              alpha *= fast_exp2(msc - mx * sc);
-              l2a.x *= alpha; l2a.y *= alpha; l2b.x *= alpha; l2b.y *= alpha;
+          tmem_wait_st();  // P and, where it was rescaled, the accumulator
+          tc_fence_before();
+          asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
+          if (MANY && j == 0 && w != (int)blockIdx.x) stored();
+          // the rest runs while the products of the next step do: the reference, which moves for the next chunk when this one
+          // exceeded it, and the next chunk's masks (the words of the one after it start travelling)
+          if (!exact) {
+            const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y), grown = l - l_seen;
+            const bool seen = (mk.x | mk.y) != 0u;  // a live key in this row
+            if (!(grown <= kMoveSum) || (none && seen)) {  // (a NaN goes this way too)
+              bad |= !(grown < kRedoSum && grown > 1.f / kRedoSum);
+              none = false;
+              if (j + 1 < n) {
+                const int ex = (int)(__float_as_uint(grown) >> 23) - 127;  // floor(log2(grown))
+                alpha = __uint_as_float((uint32_t)(127 - ex) << 23);
+                msc += (float)ex;
+                l2a.x *= alpha; l2a.y *= alpha; l2b.x *= alpha; l2b.y *= alpha;
+              }
             }
-            msc = mx * sc;
-            none = false;
+            l_seen = (l2a.x + l2a.y) + (l2b.x + l2b.y);
           }
           rescale = __any_sync(0xffffffffu, alpha != 1.f);
+          widen_v(base + j + 1);
+          widen_k(base + j + 2);
+          cls = cls_next;
+          mk = mk_next;
+          mk_next = look_up(j + 2, cls_next);
         }
-        if (rescale) {  // the accumulator follows the reference
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
-            uint32_t o[16];
-            tmem_ld16(tO + 16 * c, o);
-            tmem_wait_ld();
-#pragma unroll
-            for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-            tmem_st16(tO + 16 * c, o);
-          }
-          alpha = 1.f;
+        const int n_here = n;
+        const bool both = n_all > 1;  // stream 1 has a chunk
+        if (MANY && n == 0 && w != (int)blockIdx.x) stored();
+        if (MANY && w + w_step < n_items) {  // the next tile's list and masks start travelling
+          const Item next = item_at(w + w_step);
+          n = next.n;
+          n_all = next.n_all;
+          infos = reinterpret_cast<const int2*>(&next.chunks->info);
+          mask_row = next.mask + m;
+          mk = look_up(0, cls);
+          mk_next = look_up(1, cls_next);
         }
-#pragma unroll 1
-        for (int hf = 0; hf < 2; ++hf) {
-          if ((cls >> (2 * hf)) & 3) {
-            uint32_t r[32], pk[16];
-            tmem_ld32(tS + 32 * hf, r);
-            tmem_wait_ld();
-            if ((cls >> (2 * hf)) & 1) {  // dead scores of a partially live half become -inf
-              const uint32_t w = hf ? mk.y : mk.x;
-#pragma unroll
-              for (int e = 0; e < 32; ++e)
-                if (!((w >> e) & 1u)) r[e] = 0xff800000u;
-            }
-            // probabilities against the reference: scale and shift (packed FMAs), 2^x, row sum, bf16
-            const float2 nm2 = make_float2(-msc, -msc);
-            const float nm_y = fmaf(-msc, 0.5f / kClamp, 0.5f);
-#pragma unroll
-            for (int e = 0; e < 32; e += 4) {
-              const uint32_t* rr = r + e;
-              const float2 xa = __ffma2_rn(make_float2(__uint_as_float(rr[0]), __uint_as_float(rr[1])), sc2, nm2);
-              const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
-              // every fourth pair on the FMA pipe: the exponential pipe (16 per clock and SM) is the tighter of the two
-              float2 pb;
-              if (e & 4) {
-                pb = exp2_fma2(make_float2(__saturatef(fmaf(__uint_as_float(rr[2]), sc_y, nm_y)),
-                                           __saturatef(fmaf(__uint_as_float(rr[3]), sc_y, nm_y))));
-              } else {
-                const float2 xb = __ffma2_rn(make_float2(__uint_as_float(rr[2]), __uint_as_float(rr[3])), sc2, nm2);
-                pb = make_float2(fast_exp2(xb.x), fast_exp2(xb.y));
-              }
-              // the row sum adds the probabilities as the PV product sees them (rounded to bf16): numerator and
-              // denominator of a row then agree, and a row with one dominant key reproduces that key's V exactly
-              const uint32_t ka = pack_bf16(pa.x, pa.y), kb = pack_bf16(pb.x, pb.y);
-              add_bf16_pair(l2a, ka);
-              add_bf16_pair(l2b, kb);
-              pk[(e >> 1) + 0] = ka;
-              pk[(e >> 1) + 1] = kb;
-            }
-            tmem_st16(tS + 16 * hf, pk);  // over scores that have been read
-          } else {  // no live key for any row of the warp
-            uint32_t pk[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) pk[e] = 0u;
-            tmem_st16(tS + 16 * hf, pk);
-          }
+        // the last PV product (all earlier ones are complete by issue order)
+        if (n_here > 0) {
+          if (ok) ok = mbar_wait_long(&sm.o_full[st], (uint32_t)(o_tiles & 1), abort_flag, p.status);
+          ++o_tiles;
         }
-        tmem_wait_st();  // P and, where it was rescaled, the accumulator
+        const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y);
+        const float own = none ? -INFINITY : msc;  // (dead keys leave traces of 2^-125 in l)
+        float2* const ref_own = MANY ? sm.ref[st] : reinterpret_cast<float2*>(sm.k[st][0]);
+        const float2* const ref_other = MANY ? sm.ref[st ^ 1] : reinterpret_cast<const float2*>(sm.k[st ^ 1][0]);
+        ref_own[m] = make_float2(own, l);
         tc_fence_before();
-        asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
-        // the rest runs while the products of the next step do: the reference, which moves for the next chunk when this one
-        // exceeded it, and the next chunk's masks (the words of the one after it start travelling)
-        if (!exact) {
-          const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y), grown = l - l_seen;
-          const bool seen = (mk.x | mk.y) != 0u;  // a live key in this row
-          if (!(grown <= kMoveSum) || (none && seen)) {  // (a NaN goes this way too)
-            bad |= !(grown < kRedoSum && grown > 1.f / kRedoSum);
-            none = false;
-            if (j + 1 < n) {
-              const int ex = (int)(__float_as_uint(grown) >> 23) - 127;  // floor(log2(grown))
-              alpha = __uint_as_float((uint32_t)(127 - ex) << 23);
-              msc += (float)ex;
-              l2a.x *= alpha; l2a.y *= alpha; l2b.x *= alpha; l2b.y *= alpha;
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + lane_group) : "memory");  // the warp with the other stream of these rows
+        tc_fence_after();
+        uint8_t* slice = sm.q[tiles % kQBufs] + (warp << 11);
+        if (ok) {
+          const float2 other = ref_other[m];
+          const float top = fmaxf(own, other.x);
+          const float f_own = fast_exp2(own - top), f_other = fast_exp2(other.x - top);
+          const float inv = 1.f / (l * f_own + other.y * f_other);
+          const float w0 = (st ? f_other : f_own) * inv, w1 = (st ? f_own : f_other) * inv;
+          // output columns [32 st, 32 st + 32) of this thread's row: both streams' accumulators, weighted (stream 1's
+          // may never have been written).
+          // The warp's 32 rows x 64 B pass through its own 2 KB slice of the Q buffer (its last reader, the last score
+          // product, is done: every warp of both streams has seen it through o_full) to a tensor-map store.  Piece position XOR
+          // (row / 2) is the map's swizzle and keeps the writes free of bank conflicts.
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            uint32_t r[16], r1[16];
+            tmem_ld16(tlane + kColO + 32 * st + 16 * c, r);
+            tmem_ld16(tlane + kColO + 64 + 32 * st + 16 * c, r1);
+            tmem_wait_ld();
+            uint32_t o[8];
+#pragma unroll
+            for (int e = 0; e < 16; e += 2) {
+              float2 x = make_float2(__uint_as_float(r[e]) * w0, __uint_as_float(r[e + 1]) * w0);
+              if (both) x = __ffma2_rn(make_float2(__uint_as_float(r1[e]), __uint_as_float(r1[e + 1])), make_float2(w1, w1), x);
+              o[e >> 1] = pack_bf16(x.x, x.y);
             }
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+              *reinterpret_cast<uint4*>(slice + lane * 64 + (((2 * c + e) ^ (lane >> 1)) & 3) * 16) =
+                  make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
           }
-          l_seen = (l2a.x + l2a.y) + (l2b.x + l2b.y);
         }
-        rescale = __any_sync(0xffffffffu, alpha != 1.f);
-        widen_v(base + j + 1);
-        widen_k(base + j + 2);
-        cls = cls_next;
-        mk = mk_next;
-        mk_next = look_up(j + 2, cls_next);
-      }
-      if (!exact && __any_sync(0xffffffffu, bad) && lane == 0) sm.redo = 1;
-      // the last PV product (all earlier ones are complete by issue order)
-      if (ok && n > 0) ok = mbar_wait_long(&sm.o_full[st], exact ? 1u : 0u, abort_flag, p.status);
-      const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y);
-      const float own = none ? -INFINITY : msc;  // (dead keys leave traces of 2^-125 in l)
-      reinterpret_cast<float2*>(sm.k[st][0])[m] = make_float2(own, l);  // the stream's stages are idle
-      tc_fence_before();
-      asm volatile("bar.sync %0, 64;" ::"r"(1 + lane_group) : "memory");  // the warp with the other stream of these rows
-      tc_fence_after();
-      if (ok && n_all > 0) {
-        const float2 other = reinterpret_cast<const float2*>(sm.k[st ^ 1][0])[m];
-        const float top = fmaxf(own, other.x);
-        const float f_own = fast_exp2(own - top), f_other = fast_exp2(other.x - top);
-        const float inv = 1.f / (l * f_own + other.y * f_other);
-        const float w0 = (st ? f_other : f_own) * inv, w1 = (st ? f_own : f_other) * inv;
-        // output columns [32 st, 32 st + 32) of this thread's row: both streams' accumulators, weighted (a stream
-        // without a live key has weight 0 and an accumulator that may never have been written)
-        uint32_t r[32], r1[32];
-        tmem_ld32(tlane + kColO + 32 * st, r);
-        tmem_ld32(tlane + kColO + 64 + 32 * st, r1);
-        tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 32; e += 2) {
-          float2 x = make_float2(__uint_as_float(r[e]) * w0, __uint_as_float(r[e + 1]) * w0);
-          if (n_all > 1) x = __ffma2_rn(make_float2(__uint_as_float(r1[e]), __uint_as_float(r1[e + 1])), make_float2(w1, w1), x);
-          r[e] = __float_as_uint(x.x);
-          r[e + 1] = __float_as_uint(x.y);
-        }
-        // The warp's 32 rows x 64 B pass through its own 2 KB slice of the Q buffer (its last reader, the last score
-        // product, is done: every warp of both streams has seen it through o_full) to a tensor-map store.  Piece position XOR
-        // (row / 2) is the map's swizzle and keeps the writes free of bank conflicts.
-        uint8_t* slice = sm.q + (warp << 11);
-#pragma unroll
-        for (int e = 0; e < 32; e += 8) {
-          uint4 o4;
-          o4.x = pack_bf16(__uint_as_float(r[e + 0]), __uint_as_float(r[e + 1]));
-          o4.y = pack_bf16(__uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
-          o4.z = pack_bf16(__uint_as_float(r[e + 4]), __uint_as_float(r[e + 5]));
-          o4.w = pack_bf16(__uint_as_float(r[e + 6]), __uint_as_float(r[e + 7]));
-          *reinterpret_cast<uint4*>(slice + lane * 64 + ((((e >> 3) ^ (lane >> 1)) & 3) << 4)) = o4;
+        if constexpr (MANY) {  // both streams' accumulators of these rows have been read: the next tile's may overwrite them
+          tc_fence_before();
+          asm volatile("bar.sync %0, 64;" ::"r"(7 + lane_group) : "memory");
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
-        if (lane == 0) {
+        if (ok && lane == 0) {
+          int qt = item0.qt, h = item0.h, b = item0.b;
+          if constexpr (MANY) {
+            int unit;
+            work_item(p, n_q_tiles, w, qt, unit);
+            h = unit % p.n_heads;
+            b = unit / p.n_heads;
+          }
           // the slots' first token or cell; a box that starts outside the grid holds no query
           const int bs = b + p.share_offset;
           if (p.q_patch) {
@@ -631,9 +751,14 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
               if (p.share_offset > 0) tma_store_4d(&tm.o, slice, 32 * st, q0, h, bs);
             }
           }
-          asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group.read 0;" ::: "memory");
+          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
+        base = end;
+        ++tiles;
+        if (!MANY || w + w_step >= n_items) break;
       }
+      stored();
+      if (!exact && __any_sync(0xffffffffu, bad) && lane == 0) sm.redo = 1;
     }
     tc_fence_before();
     __syncwarp();
@@ -641,8 +766,6 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
     tc_fence_after();
     if (exact || !*(volatile int*)&sm.redo || *abort_flag) break;
     exact = true;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // Q is copied again over the output rows
-    __syncthreads();
   }
 
   // ---------------------------------------------------------------------- teardown (all paths)
@@ -652,18 +775,19 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
   }
 }
 
-template <bool KV8>
-litevar_status_t launch_variant(const TensorMaps& tm, const FwdParams& p, int n_q_tiles, cudaStream_t stream) {
+template <bool KV8, bool MANY>
+litevar_status_t launch_variant(const TensorMaps& tm, const FwdParams& p, int n_q_tiles, int n_ctas, cudaStream_t stream) {
   static std::once_flag attr_once;
   static cudaError_t attr_err = cudaSuccess;
-  constexpr int smem_bytes = (int)sizeof(WsShared<KV8>);
+  constexpr int smem_bytes = (int)sizeof(WsShared<KV8, MANY>);
   static_assert(smem_bytes <= 115712, "two CTAs per SM");
   std::call_once(attr_once, [] {
-    attr_err = cudaFuncSetAttribute(fwd_ws_kernel<KV8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    attr_err = cudaFuncSetAttribute(fwd_ws_kernel<KV8, MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
   });
   if (attr_err != cudaSuccess) return LITEVAR_ERR_CUDA;
+  const int n_items = n_q_tiles * p.n_heads * p.batch_computed;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)n_q_tiles * (unsigned)p.n_heads * (unsigned)p.batch_computed);
+  cfg.gridDim = dim3((unsigned)(MANY ? n_ctas : n_items));
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = stream;
@@ -672,7 +796,7 @@ litevar_status_t launch_variant(const TensorMaps& tm, const FwdParams& p, int n_
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = p.overlap_launch ? 1 : 0;  // off when an earlier kernel of the stream writes what the set-up reads
-  if (cudaLaunchKernelEx(&cfg, fwd_ws_kernel<KV8>, tm, p, n_q_tiles) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, fwd_ws_kernel<KV8, MANY>, tm, p, n_q_tiles, n_items) != cudaSuccess) {
     (void)cudaGetLastError();
     return LITEVAR_ERR_CUDA;
   }
@@ -684,13 +808,22 @@ litevar_status_t launch_variant(const TensorMaps& tm, const FwdParams& p, int n_
 litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream_t stream) {
   TensorMaps tm;
   if (!encode_tensor_maps(p, &tm, kChunkKeys)) return LITEVAR_ERR_INVALID_ARG;
-  return launch_variant<false>(tm, p, n_q_tiles, stream);
+  // Short lists: a tile spends as long on its first copies, look-ups and output as on 4 to 6 chunks, and CTAs that stay overlap
+  // these with the other tiles' work.  What is lost is the balance at the end: a CTA's tiles are fixed, not dealt out.  Measured
+  // (us, one tile per CTA / staying): 10 chunks a tile at 6.5 tiles per resident CTA 83.4 / 75.3, at 2.6 37.6 / 36.9, at 1.7
+  // 25.2 / 25.7; 4 chunks at 3.2 29.0 / 24.7, at 1.6 15.3 / 15.9; 14 chunks at 4.9 73.0 / 70.2, at 2.4 39.4 / 40.0; 22 chunks
+  // at 7.8 157.3 / 155.5, at 2.9 63.6 / 65.0; 38 chunks at 1.9 66.6 / 73.4; 53 at 3.5 172 / 182; 155 at 13.8 1520 / 1680.
+  const long long items = (long long)n_q_tiles * p.n_heads * p.batch_computed, resident = 2ll * current_sm_count();
+  const int chunks = p.chunks_per_tile;
+  if (chunks > 0 && chunks <= 40 && 2 * items >= 5 * resident && 5 * items >= chunks * resident)
+    return launch_variant<false, true>(tm, p, n_q_tiles, (int)resident, stream);
+  return launch_variant<false, false>(tm, p, n_q_tiles, 0, stream);
 }
 
 litevar_status_t launch_forward_ws_kv8(const FwdParams& p, int n_q_tiles, cudaStream_t stream) {
   TensorMaps tm;
   if (!encode_code_maps(p, &tm, kChunkKeys)) return LITEVAR_ERR_INVALID_ARG;
-  return launch_variant<true>(tm, p, n_q_tiles, stream);
+  return launch_variant<true, false>(tm, p, n_q_tiles, 0, stream);
 }
 
 }  // namespace litevar

@@ -76,7 +76,7 @@ struct SetDesc {
 };
 
 struct StepSet {
-  int32_t n_pairs = 0, n_partial = 0, n_full = 0;
+  int32_t n_pairs = 0, n_partial = 0, n_full = 0, n_chunks = 0;
   int64_t live_entries = 0;
   int32_t* d_row_ptr = nullptr;
   Pair* d_pairs = nullptr;
@@ -137,6 +137,7 @@ struct FwdParams {
   const int8_t* v8;
   const float *k_scale, *k_zero, *v_scale, *v_zero;
   int64_t c_sb, c_sh, c_st, z_sb, z_sh;
+  int32_t chunks_per_tile;      // average live chunks per query tile (0: unknown); picks the tensor-core kernel's build
   int32_t units_per_group;      // launch order of the tensor-core kernels: (batch row, head) units per L2 group
   int32_t overlap_launch;       // 1: the tensor-core kernel may start its set-up before the previous kernel of the
                                 // stream has finished (the plan it reads was complete long before)

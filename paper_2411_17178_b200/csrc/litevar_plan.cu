@@ -758,6 +758,7 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
     for (int set = 0; set < n_sets; ++set) {
       StepSet& ss = st.sets[set];
       const SetTotals& t = totals[(size_t)k0 * n_sets + set];
+      ss.n_chunks = t.n_chunks;
       ss.d_chunks = next_chunk;
       next_chunk += t.n_chunks;
       ss.d_chunk_mask = next_chunk_mask;
@@ -889,6 +890,7 @@ static void fill_step_params(const litevar_plan_t* plan, const Step& st, int32_t
   p.sm_scale = plan->sm_scale;
   p.status = plan->d_status;
   p.overlap_launch = 1;
+  p.chunks_per_tile = (st.sets[0].n_chunks + st.n_q_tiles - 1) / st.n_q_tiles;
   p.units_per_group = units_per_l2_group(st.L_k, p.n_heads * p.batch_computed);
 }
 

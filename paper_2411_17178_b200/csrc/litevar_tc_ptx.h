@@ -259,16 +259,16 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return d;
 }
 
-// Launch order of the tensor-core kernels.  The (batch row, head) units are taken in groups of
-// p.units_per_group; inside a group the CTAs go query-tile pair by pair (heaviest first, the planner's order), all
+// Order of the tensor-core kernel's work items.  The (batch row, head) units are taken in groups of
+// p.units_per_group; inside a group the items go query tile by query tile, all
 // units of the group side by side.  The K/V of one group is what the CTAs resident at one time read: the host
 // sizes the group so that it fits in half of L2, and every K/V tile then comes from DRAM once per step instead of
 // once per wave of CTAs.
-__device__ __forceinline__ void cta_work(const FwdParams& p, int n_ranks, int& rank, int& unit) {
+__device__ __forceinline__ void work_item(const FwdParams& p, int n_ranks, int item, int& rank, int& unit) {
   const int n_units = p.n_heads * p.batch_computed;
   const int g_units = p.units_per_group;
-  const int group = blockIdx.x / (g_units * n_ranks);
-  const int r = blockIdx.x - group * (g_units * n_ranks);
+  const int group = item / (g_units * n_ranks);
+  const int r = item - group * (g_units * n_ranks);
   const int here = min(g_units, n_units - group * g_units);  // the last group may be smaller
   rank = r / here;
   unit = group * g_units + (r - rank * here);

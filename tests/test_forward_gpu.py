@@ -9,7 +9,7 @@ import torch
 
 from oracle import litevar_oracle as orc
 from paper_2411_17178_b200 import binding, workloads as wl
-from tests.gpu_util import assert_close, check_sampled, lib_ready, run_forward, stratified_samples
+from tests.gpu_util import REL_L2, assert_close, check_sampled, errors, lib_ready, run_forward, stratified_samples
 
 pytestmark = pytest.mark.gpu
 
@@ -476,4 +476,35 @@ def test_chunk_lists_off_the_tile_grid(scales, radius, tiling, shape):
         got, _ = run_forward(plan, k, B, Q, Kc, Vc, binding.KERNEL_TCGEN05)
         ref = orc.attention_step(scales, k, tab[k - 1], Q, Kc, Vc, band=shape == binding.WINDOW_BAND)
         assert_close(got, ref, f"scales={scales} step {k}")
+    plan.close()
+
+
+@pytest.mark.parametrize("case", ["raster", "one-chunk-tiles", "sets", "rising"])
+def test_many_tiles_per_cta(case):
+    """Enough query tiles that the tensor-core kernel's CTAs take several in turn (from 2.5 per resident CTA on): ragged tails,
+    tiles with a single chunk (one stream idle), per-head lists, sharing, and the second pass over all of a CTA's tiles."""
+    lib_ready()
+    scales = (12,) if case == "one-chunk-tiles" else (1, 2, 3, 4, 6, 9, 13)
+    B, H, K = 80 if case == "raster" else 40, 7, len(scales)  # raster: half the rows are computed
+    share = [int(case == "raster")] * K
+    tabs, head_set = [orc.window_table(scales, n_global_scales=3)], [0] * H
+    if case == "one-chunk-tiles":  # 144 queries, three key rows each: lists of three chunks and of one
+        tabs[0][0, 0] = 1
+    elif case == "sets":
+        tabs, head_set = [orc.window_table(scales, rho=r, n_global_scales=3) for r in ((1, 8), (1, 2))], [i % 2 for i in range(H)]
+    w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=96)
+    Q = wl.make_q(w, 0, K)
+    Kc, Vc = wl.make_kv(w, 0)
+    if case == "rising":
+        Kc = (Kc.float() * torch.linspace(0.2, 9, Kc.shape[2]).view(1, 1, -1, 1)).bfloat16()
+    plan = binding.Plan(scales, n_heads=H, radius=np.stack(tabs), n_sets=len(tabs), share_steps=share,
+                        head_to_set=head_set if len(tabs) > 1 else None)
+    got, _ = run_forward(plan, K, B, Q, Kc, Vc, binding.KERNEL_TCGEN05)
+    for s, t in enumerate(tabs):
+        heads = [h for h in range(H) if head_set[h] == s]
+        ref = orc.attention_step(scales, K, t[K - 1], Q[:, heads], Kc[:, heads], Vc[:, heads], share_cfg=bool(share[K - 1]))
+        # P and the output are each rounded to bf16 (2^-9 of a weight, which sum to 1, and of the result): with nine live keys
+        # a row is not an average of many values, and the error is bounded by 2^-9 max|V| twice, not by a fixed 1e-2
+        ma, rl = errors(got[:, heads], ref)
+        assert ma <= 2.0 ** -8 * float(Vc.float().abs().max()) and rl <= REL_L2, f"{case} set {s}: max-abs {ma:.3e} rel-L2 {rl:.3e}"
     plan.close()
