@@ -56,6 +56,7 @@ class _Strides(ctypes.Structure):
 
 
 _lib = None
+_host = None
 
 
 def load() -> ctypes.CDLL:
@@ -133,13 +134,26 @@ def _stream_ptr(stream) -> Optional[int]:
     return getattr(stream, "cuda_stream", stream)
 
 
-def _current_raw_stream(device_index) -> int:
-    """cudaStream_t of torch's current stream on that device, without building a Stream object."""
+def _host_module():
+    """The native Python entry (built beside the library; there is no other path)."""
+    global _host
+    if _host is None:
+        try:
+            from . import _litevar_host
+        except ImportError as e:
+            raise RuntimeError("_litevar_host.so not found or not loadable: build it with "
+                               "`python -m paper_2411_17178_b200.build` (needs a C compiler and the Python headers)") from e
+        _host = _litevar_host
+    return _host
+
+
+def _raw_stream_getter():
+    """device index -> cudaStream_t of torch's current stream on that device, without building a Stream object."""
     import torch
     try:
-        return torch._C._cuda_getCurrentRawStream(device_index if device_index is not None else torch.cuda.current_device())
+        return torch._C._cuda_getCurrentRawStream
     except AttributeError:
-        return torch.cuda.current_stream().cuda_stream
+        return lambda device_index: torch.cuda.current_stream(device_index).cuda_stream
 
 
 def _strides(t) -> _Strides:
@@ -184,13 +198,16 @@ class Plan:
                                    ctypes.byref(handle))
         _check(st, "litevar_attn_plan")
         self._h = handle
-        self._strides4 = tuple(_Strides(0, 0, 0) for _ in range(4))
-        self._strides4_ref = tuple(ctypes.byref(x) for x in self._strides4)
+        self._plan_addr = handle.value
+        self._forward_addr = ctypes.cast(lib.litevar_attn_forward, ctypes.c_void_p).value
+        self._forward = _host_module().forward
+        self._current_stream = _raw_stream_getter()
 
     def close(self) -> None:
         if getattr(self, "_h", None):
             self._lib.litevar_plan_destroy(self._h)
             self._h = None
+            self._plan_addr = 0  # a null plan is an invalid argument
 
     def __del__(self):
         try:
@@ -200,28 +217,10 @@ class Plan:
 
     # -- forward ---------------------------------------------------------------------------
     def forward(self, step_k: int, batch_pairs: int, q, k_cache, v_cache, out, stream=None) -> None:
-        """litevar_attn_forward on torch CUDA tensors (bf16, [2B, H, tokens, 64]).
-
-        The marshalling is kept short (it is most of an eager call's host time): the four stride structs live
-        in the plan and are refilled, so one plan must not be driven from several Python threads at once."""
-        sq, sk, sv, so = self._strides4
-        a = q.stride()
-        sq.batch, sq.head, sq.token = a[0], a[1], a[2]
-        b = k_cache.stride()
-        sk.batch, sk.head, sk.token = b[0], b[1], b[2]
-        c = v_cache.stride()
-        sv.batch, sv.head, sv.token = c[0], c[1], c[2]
-        d = out.stride()
-        so.batch, so.head, so.token = d[0], d[1], d[2]
-        if a[3] != 1 or b[3] != 1 or c[3] != 1 or d[3] != 1:
-            raise ValueError("expected [2B, H, tokens, 64] tensors with contiguous head_dim")
-        if stream is None:
-            stream_ptr = _current_raw_stream(q.device.index)
-        else:
-            stream_ptr = getattr(stream, "cuda_stream", stream)
-        st = self._lib.litevar_attn_forward(self._h, step_k, batch_pairs, q.data_ptr(), self._strides4_ref[0],
-                                            k_cache.data_ptr(), self._strides4_ref[1], v_cache.data_ptr(),
-                                            self._strides4_ref[2], out.data_ptr(), self._strides4_ref[3], stream_ptr)
+        """litevar_attn_forward on torch CUDA tensors (bf16, [2B, H, tokens, 64]); the marshalling is native (it is most of
+        an eager call's host time)."""
+        st = self._forward(self._forward_addr, self._plan_addr, step_k, batch_pairs, q, k_cache, v_cache, out,
+                           stream if stream is None else getattr(stream, "cuda_stream", stream), self._current_stream)
         if st != 0:
             _check(st, "litevar_attn_forward")
 
@@ -233,7 +232,7 @@ class Plan:
         assert k_scale.stride() == k_zero.stride() == v_scale.stride() == v_zero.stride() and k_scale.stride(2) == 1
         sc = _Strides(k_codes.stride(0), k_codes.stride(1), k_codes.stride(2))
         sr = _Strides(k_scale.stride(0), k_scale.stride(1), 1)
-        stream_ptr = _current_raw_stream(q.device.index) if stream is None else getattr(stream, "cuda_stream", stream)
+        stream_ptr = self._current_stream(q.get_device()) if stream is None else getattr(stream, "cuda_stream", stream)
         st = self._lib.litevar_attn_forward_kv8(
             self._h, int(step_k), int(batch_pairs), q.data_ptr(), ctypes.byref(_strides(q)), k_codes.data_ptr(),
             k_scale.data_ptr(), k_zero.data_ptr(), v_codes.data_ptr(), v_scale.data_ptr(), v_zero.data_ptr(),

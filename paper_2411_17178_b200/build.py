@@ -1,4 +1,4 @@
-"""Builds liblitevar.so (the C-ABI library) in-tree with nvcc for sm_100a.
+"""Builds liblitevar.so (the C-ABI library, nvcc, sm_100a) and _litevar_host.so (its Python entry, C compiler) in-tree.
 
     python -m paper_2411_17178_b200.build [--force] [--verbose]
 """
@@ -7,11 +7,14 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblitevar.so")
+HOST_LIB = os.path.join(HERE, "_litevar_host.so")
+HOST_SOURCE = os.path.join(CSRC, "litevar_host.c")
 SOURCES = ["litevar_plan.cu", "litevar_fwd_simt.cu", "litevar_maps.cu", "litevar_fwd_ws.cu", "litevar_fwd_small.cu", "litevar_static.cu", "litevar_calib.cu", "litevar_quant.cu"]
 HEADERS = [os.path.join(CSRC, "litevar_internal.h"), os.path.join(CSRC, "litevar_tc_ptx.h"), os.path.join(ROOT, "include", "litevar.h")]
 
@@ -23,15 +26,26 @@ def _nvcc() -> str:
     return "nvcc"
 
 
+def _stale(target: str, deps) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(d) > os.path.getmtime(target) for d in deps)
+
+
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES] + HEADERS + [os.path.abspath(__file__)]
-    return any(os.path.getmtime(d) > t for d in deps)
+    return _stale(LIB, [os.path.join(CSRC, s) for s in SOURCES] + HEADERS + [os.path.abspath(__file__)])
+
+
+def build_host(force: bool = False) -> str:
+    if force or _stale(HOST_LIB, [HOST_SOURCE, HEADERS[-1], os.path.abspath(__file__)]):
+        cmd = [os.environ.get("CC") or "gcc", "-shared", "-fPIC", "-O2", "-Wall", "-I", sysconfig.get_paths()["include"],
+               "-I", os.path.join(ROOT, "include"), HOST_SOURCE, "-o", HOST_LIB]
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError("building _litevar_host.so failed:\n" + res.stdout + res.stderr)
+    return HOST_LIB
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_host(force)
     if not force and not needs_build():
         return LIB
     cmd = [_nvcc(), "-shared", "-Xcompiler", "-fPIC", "-O3", "-std=c++17", "-lineinfo",

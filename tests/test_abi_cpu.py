@@ -73,3 +73,45 @@ def test_null_plan_calls(lib):
     assert lib.litevar_plan_step_kernel(None, 1, 1, None) == 1
     assert lib.litevar_plan_stats(None, 1, 0, None, None, None, None) == 1
     lib.litevar_plan_destroy(None)
+
+
+def test_native_forward_entry_marshals_tensors():
+    """The native Python entry hands over pointers, strides, step, pairs and stream as they are (a stand-in for the library
+    records them), takes the current stream of q's device when there is none, and refuses other layouts."""
+    build.build_host()
+    from paper_2411_17178_b200 import _litevar_host as host
+
+    class Fake:
+        def __init__(self, ptr, strides, device=3):
+            self.args = ptr, strides, device
+
+        def data_ptr(self):
+            return self.args[0]
+
+        def stride(self):
+            return self.args[1]
+
+        def get_device(self):
+            return self.args[2]
+
+    seen = []
+    P, S = ctypes.c_void_p, ctypes.POINTER(ctypes.c_int64 * 3)
+
+    @ctypes.CFUNCTYPE(ctypes.c_int, P, ctypes.c_int32, ctypes.c_int32, P, S, P, S, P, S, P, S, P)
+    def library(plan, step, pairs, q, sq, k, sk, v, sv, o, so, stream):
+        seen.append((plan, step, pairs, q, tuple(sq[0]), k, tuple(sk[0]), v, tuple(sv[0]), o, tuple(so[0]), stream))
+        return 5
+
+    addr = ctypes.cast(library, ctypes.c_void_p).value
+    t = [Fake(2 ** 47 + 16 * i, (2 ** 33 + i, 64 * i, 64, 1)) for i in range(4)]
+    want = [x for i in range(4) for x in (2 ** 47 + 16 * i, (2 ** 33 + i, 64 * i, 64))]
+    assert host.forward(addr, 2 ** 40, 7, 8, *t, 1234, None) == 5
+    assert seen[-1] == (2 ** 40, 7, 8, *want, 1234)
+    assert host.forward(addr, 0, 1, 1, *t, None, lambda device: 100 + device) == 5
+    assert seen[-1] == (None, 1, 1, *want, 103)
+    for bad in ((1, 64, 64, 2), (1, 64, 1)):
+        with pytest.raises(ValueError):
+            host.forward(addr, 1, 1, 1, *t[:3], Fake(16, bad), 1, None)
+    with pytest.raises(TypeError):
+        host.forward(addr, 1, 1, 1)
+    assert len(seen) == 2
