@@ -20,18 +20,18 @@
 // Two CTAs per SM, so that every scheduler has four softmax warps of four streams that are in different phases.
 // TMEM columns: S and P of stream s at 64 s, O at 128 + 64 s.
 //
-// The reference of a row (probabilities are 2^(score * scale - reference)) needs no maximum per chunk: it starts as the
-// maximum of the first chunk's first eight keys (of the whole chunk: an extra pass, 1000 cycles of a tile's 20000); afterwards
-// only the chunk's SUM is looked at, and when that exceeds 2^10 the reference moves by whole powers of two for the next chunk
-// (the accumulator and the sum are scaled exactly).  bf16 and fp32 have the same
-// exponent range, so P is as accurate at 2^10 as at 1.  A sum beyond 2^60, or below 2^-60 where a row meets its first live key
-// late, is out of the range in which this is safe: the CTA then redoes its list, taking every chunk's maximum first (`exact`).
+// The reference of a row (probabilities are 2^(score * scale - reference)) is the maximum of the first chunk's first eight keys
+// and stays (0 where none of them is live): bf16 and fp32 have the same exponent range, so P, its sum and the accumulator are as
+// accurate at 2^90 as at 1, and a tile's rows need neither a maximum per chunk nor a rescaled accumulator.  At the end a row whose
+// sum left [2^-96, 2^96] sends the CTA through its lists again, with every chunk's maximum taken first (`exact`).  (A reference
+// that followed the chunk sums by powers of two from 2^10 on, tested at every chunk: 2 to 3 % slower, 512px step 10 155.6 us
+// against 151.)
 //
 // What bounds it (ncu, 2K step with the full mask): exponential pipe 78 %, tensor pipe active 50 %, issue slots 53 %; the rest
 // is the hand-off from P to the next S (arrive, issue of eight MMAs, their execution, commit, wake: 700 cycles a chunk).
 // Measured on B200, with what the kernel with one softmax thread per row and 128-key tiles took before: 2K step with the full
-// mask 5.05 ms (6.71), window 1/4 1.57 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 160 / 74 / 34 us (261 / 116 / 47),
-// 256px step 10 with 960 units 85 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
+// mask 5.05 ms (6.71), window 1/4 1.49 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 151 / 68 / 31 us (261 / 116 / 47),
+// 256px step 10 with 960 units 74 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
 // the way: copy look-ups off the MMA lane -4 %, 64-key streams with uniform issue code -12 %, no maxima -12 %; share of the
 // exponentials on the FMA pipe 0 / 25 / 37.5 / 50 %: 1.80 / 1.71 / 1.78 / 1.87 ms; three stages instead of two: +1 %; chunks from
 // a tile's live box on and classes per half and warp (on the fixed grid, one live flag per chunk and warp: 1.69 ms) -7 %.
@@ -57,8 +57,7 @@ constexpr int kStages = 2;                // K ring and V ring of a stream
 constexpr int kThreads = 320;             // two streams of four softmax warps, one issuing warp each
 constexpr uint32_t kTmemCols = 256, kColO = 128;  // S (and P over it) of stream s at 64 s, O at 128 + 64 s
 
-constexpr float kMoveSum = 1024.f;        // a chunk whose probabilities sum to more moves the row's reference
-constexpr float kRedoSum = 1152921504606846976.f;  // 2^60: beyond it the reference was too far off
+constexpr float kRange = 79228162514264337593543950336.f;  // 2^96: a row sum beyond it, or below its inverse, redoes the list
 
 // 8-bit cache build: the codes of a chunk (64 rows of 64 bytes, as the tensor-map copy delivers them, no swizzle) and its rows'
 // scales and shifted zero points, on their way into the bf16 stages (empty in the bf16 build).
@@ -512,14 +511,11 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       };
       for (int w = blockIdx.x;; w += w_step) {
         const int end = base + n;
-        // probabilities are 2^(score * sc - msc).  msc starts as the maximum of a few keys and moves by whole powers of two
-        // when a chunk's sum gets large; it stays 0 and `none` until a live chunk has been seen.
+        // probabilities are 2^(score * sc - msc); `none` until msc has been set from a live key
         float msc = 0.f;
         bool none = true;
-        float alpha = 1.f;  // pending factor of the accumulator
         float2 l2a = make_float2(0.f, 0.f), l2b = make_float2(0.f, 0.f);  // row sum
-        bool rescale = false;  // some row of the warp has a pending alpha
-        float l_seen = 0.f;     // row sum before this chunk
+        uint32_t seen = 0u;  // not 0: this row has had a live key
         // 8-bit cache: the stream's softmax threads widen its chunks, K(i + 2) and V(i + 1) while the products after P(i) run
         const int t = threadIdx.x & 127;
         auto widen_k = [&](int i) {
@@ -570,27 +566,26 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
                 for (int e = 0; e < 32; ++e) mx = fmaxf(mx, (w >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
               }
             }
+            float alpha = 1.f;
             if (mx != -INFINITY && (none || mx * sc - msc > kRescaleThreshold)) {
               if (!none) {
-                alpha *= fast_exp2(msc - mx * sc);
+                alpha = fast_exp2(msc - mx * sc);
                 l2a.x *= alpha; l2a.y *= alpha; l2b.x *= alpha; l2b.y *= alpha;
               }
               msc = mx * sc;
               none = false;
             }
-            rescale = __any_sync(0xffffffffu, alpha != 1.f);
-          }
-          if (rescale) {  // the accumulator follows the reference
+            if (exact && __any_sync(0xffffffffu, alpha != 1.f)) {  // the accumulator follows the reference
 #pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
-              uint32_t o[16];
-              tmem_ld16(tO + 16 * c, o);
-              tmem_wait_ld();
+              for (int c = 0; c < 4; ++c) {
+                uint32_t o[16];
+                tmem_ld16(tO + 16 * c, o);
+                tmem_wait_ld();
 #pragma unroll
-              for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-              tmem_st16(tO + 16 * c, o);
+                for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                tmem_st16(tO + 16 * c, o);
+              }
             }
-            alpha = 1.f;
           }
 #pragma unroll 1
           for (int hf = 0; hf < 2; ++hf) {
@@ -641,24 +636,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           tc_fence_before();
           asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
           if (MANY && j == 0 && w != (int)blockIdx.x) stored();
-          // the rest runs while the products of the next step do: the reference, which moves for the next chunk when this one
-          // exceeded it, and the next chunk's masks (the words of the one after it start travelling)
-          if (!exact) {
-            const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y), grown = l - l_seen;
-            const bool seen = (mk.x | mk.y) != 0u;  // a live key in this row
-            if (!(grown <= kMoveSum) || (none && seen)) {  // (a NaN goes this way too)
-              bad |= !(grown < kRedoSum && grown > 1.f / kRedoSum);
-              none = false;
-              if (j + 1 < n) {
-                const int ex = (int)(__float_as_uint(grown) >> 23) - 127;  // floor(log2(grown))
-                alpha = __uint_as_float((uint32_t)(127 - ex) << 23);
-                msc += (float)ex;
-                l2a.x *= alpha; l2a.y *= alpha; l2b.x *= alpha; l2b.y *= alpha;
-              }
-            }
-            l_seen = (l2a.x + l2a.y) + (l2b.x + l2b.y);
-          }
-          rescale = __any_sync(0xffffffffu, alpha != 1.f);
+          seen |= mk.x | mk.y;
           widen_v(base + j + 1);
           widen_k(base + j + 2);
           cls = cls_next;
@@ -683,7 +661,8 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           ++o_tiles;
         }
         const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y);
-        const float own = none ? -INFINITY : msc;  // (dead keys leave traces of 2^-125 in l)
+        bad |= !exact && seen && !(l < kRange && l > 1.f / kRange);  // (a NaN goes this way too)
+        const float own = seen ? msc : -INFINITY;  // (dead keys leave traces of 2^-125 in l)
         float2* const ref_own = MANY ? sm.ref[st] : reinterpret_cast<float2*>(sm.k[st][0]);
         const float2* const ref_other = MANY ? sm.ref[st ^ 1] : reinterpret_cast<const float2*>(sm.k[st ^ 1][0]);
         ref_own[m] = make_float2(own, l);
