@@ -6,7 +6,7 @@
 // own scores, probabilities, accumulator and reference, and the two results meet at the end.  320 threads:
 //   warps 0-3, 4-7  softmax of stream 0 and 1: thread m of the group owns query slot m (TMEM lane m).  A chunk's 64 scores
 //                   come from TMEM in two halves of 32 through one rolled copy of the code: the plan's element mask, the
-//                   probabilities (every fourth pair of exponentials on the FMA pipe by a cubic, the rest on the exponential
+//                   probabilities (about a quarter of the exponentials on the FMA pipe by a cubic, the rest on the exponential
 //                   pipe), their sum, and P (packed bf16) over the scores that have been read.
 //   warps 8, 9      the stream's copies (K and V chunks by tensor-map copies into rings of two stages) and MMAs: once P(i) is
 //                   complete, O += P(i) V(i) and S(i + 1) = Q K(i + 1) go out back to back; they execute in issue order, so
@@ -30,10 +30,9 @@
 // What bounds it (ncu, 2K step with the full mask): exponential pipe 78 %, tensor pipe active 50 %, issue slots 53 %; the rest
 // is the hand-off from P to the next S (arrive, issue of eight MMAs, their execution, commit, wake: 700 cycles a chunk).
 // Measured on B200, with what the kernel with one softmax thread per row and 128-key tiles took before: 2K step with the full
-// mask 5.05 ms (6.71), window 1/4 1.49 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 151 / 68 / 31 us (261 / 116 / 47),
+// mask 5.05 ms (6.71), window 1/4 1.45 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 151 / 68 / 31 us (261 / 116 / 47),
 // 256px step 10 with 960 units 74 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
-// the way: copy look-ups off the MMA lane -4 %, 64-key streams with uniform issue code -12 %, no maxima -12 %; share of the
-// exponentials on the FMA pipe 0 / 25 / 37.5 / 50 %: 1.80 / 1.71 / 1.78 / 1.87 ms; three stages instead of two: +1 %; chunks from
+// the way: copy look-ups off the MMA lane -4 %, 64-key streams with uniform issue code -12 %, no maxima -12 %; three stages instead of two: +1 %; chunks from
 // a tile's live box on and classes per half and warp (on the fixed grid, one live flag per chunk and warp: 1.69 ms) -7 %.
 //
 // Every wait on an mbarrier is bounded; when one runs out the CTA raises the plan's status word, drains its copies, frees its
@@ -107,6 +106,15 @@ __device__ __forceinline__ float2 exp2_fma2(float2 y) {
   z = __ffma2_rn(z, f, make_float2(0.9999280571937561f, 0.9999280571937561f));
   return make_float2(__uint_as_float(__float_as_uint(z.x) + (__float_as_uint(t.x) << 23)),
                      __uint_as_float(__float_as_uint(z.y) + (__float_as_uint(t.y) << 23)));
+}
+
+// Which of a half's 16 pairs of exponentials take the FMA pipe (second pair of every four keys e .. e + 3): five with one tile per
+// CTA, four on short lists with several, three beside the widening of an 8-bit cache, whose arithmetic is on that pipe too.
+// Measured for 3 / 4 / 5 / 6 pairs: 2K step 14 1484 / 1488 / 1451 / 1494 us; 512px step 10 153.6 / 153.3 / 153.8 / 154.4 us; the same
+// with an 8-bit cache 227.9 / 229.6 / 233.6 / 237 us.
+template <bool KV8, bool MANY>
+__device__ __forceinline__ constexpr bool on_fma_pipe(int e) {
+  return KV8 ? (e & 4) != 0 && e != 28 : MANY ? (e & 4) != 0 : (e & 4) != 0 || e == 16;
 }
 
 // acc += the two bf16 halves of a packed pair: fp32 additions that take a bf16 operand as it is (no unpacking)
@@ -607,9 +615,9 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
                 const uint32_t* rr = r + e;
                 const float2 xa = __ffma2_rn(make_float2(__uint_as_float(rr[0]), __uint_as_float(rr[1])), sc2, nm2);
                 const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
-                // every fourth pair on the FMA pipe: the exponential pipe (16 per clock and SM) is the tighter of the two
+                // some pairs on the FMA pipe: the exponential pipe (16 per clock and SM) is the tighter of the two
                 float2 pb;
-                if (e & 4) {
+                if (on_fma_pipe<KV8, MANY>(e)) {
                   pb = exp2_fma2(make_float2(__saturatef(fmaf(__uint_as_float(rr[2]), sc_y, nm_y)),
                                              __saturatef(fmaf(__uint_as_float(rr[3]), sc_y, nm_y))));
                 } else {
