@@ -23,8 +23,8 @@
 // pass at memory speed) and the histogram pass reads one or a few summed maps instead of all of them.  The histogram pass costs
 // about 3.5 times what reading its input costs, so this pays from two maps on; it takes fp32 sums of at most
 // kMaxSumMaps maps and a scratch buffer of at most kScratchBytes (a single 2K map, 2.2 GB, goes to the histogram directly).
-// Measured on B200: 64 maps of the last 512px step (587 MB): the call 338 -> 169 us; 1280 maps of the last 256px step
-// (891 MB): see below.
+// Measured on B200: 64 maps of the last 512px step (587 MB; sums 94 us, histogram 20 us): the call 338 -> 147 us; 1280 maps of the
+// last 256px step (891 MB): 391 -> 222 us.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -46,9 +46,12 @@ constexpr int kMaxSumMaps = 256;               // maps added up in fp32
 constexpr size_t kScratchBytes = 32u << 20;    // summed maps of one call, at most
 
 // out[g][i] = sum of maps m in [g * per_group, (g + 1) * per_group) of maps[m][i].  A thread owns kSumPerThread entries, a block's
-// width apart (coalesced whatever the alignment of a map), and has kSumPerThread * kSumUnroll loads in flight.
+// width apart (coalesced whatever the alignment of a map), and has kSumPerThread * kSumUnroll loads in flight.  Clears the
+// histogram on the way, and lets the histogram pass be launched while the last blocks run (it waits for them).
 __global__ void __launch_bounds__(kSumThreads) sum_maps_kernel(const float* __restrict__ maps, int64_t n, int64_t n_maps,
-                                                               int64_t per_group, float* __restrict__ out) {
+                                                               int64_t per_group, float* __restrict__ out, double* hist) {
+  if (blockIdx.y == 0)
+    for (int i = blockIdx.x * kSumThreads + threadIdx.x; i < kMaxScales * kMaxDist; i += gridDim.x * kSumThreads) hist[i] = 0.0;
   const int64_t first = (int64_t)blockIdx.x * (kSumThreads * kSumPerThread) + threadIdx.x;
   const int64_t m0 = blockIdx.y * per_group, m1 = min(n_maps, m0 + per_group);
   float acc[kSumPerThread] = {};
@@ -79,6 +82,7 @@ __global__ void __launch_bounds__(kSumThreads) sum_maps_kernel(const float* __re
 #pragma unroll
   for (int e = 0; e < kSumPerThread; ++e)
     if (first + e * kSumThreads < n) out[blockIdx.y * n + first + e * kSumThreads] = acc[e];
+  asm volatile("griddepcontrol.launch_dependents;");
 }
 
 // Stream-ordered pool of the calibration scratch, one per device, made on first use.  It keeps at most one call's scratch
@@ -171,6 +175,7 @@ calib_hist_kernel(Schedule sc, int k0, int first_part, int s_max, const float* _
   const int warp_global = blockIdx.x * kCalibWarps + warp;
   const int n_warps = gridDim.x * kCalibWarps;
   const int flush_every = max(1, kCalibFlushRows / rows_per_batch);
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the summed maps and the cleared histogram
 
   for (int j = first_part + blockIdx.y; j <= k0; j += gridDim.y) {  // few rows: the parts go to blocks of their own
     const int s_j = sc.scale[j];
@@ -329,7 +334,7 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
     float* summed = reinterpret_cast<float*>(scratch + hist_bytes);
     const long long per_block = kSumThreads * kSumPerThread;
     sum_maps_kernel<<<dim3((unsigned)((map_len + per_block - 1) / per_block), (unsigned)groups), kSumThreads, 0, stream>>>(
-        maps, map_len, n_maps, per_group, summed);
+        maps, map_len, n_maps, per_group, summed, d_hist);
     if (cudaGetLastError() != cudaSuccess) st = LITEVAR_ERR_CUDA;
     maps = summed;
     n_maps = groups;
@@ -343,7 +348,7 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
   if (blocks_per_sm > 32 / kCalibWarps) blocks_per_sm = 32 / kCalibWarps;
   if (blocks_per_sm < 1) blocks_per_sm = 1;
   const long long n_warps = (long long)n_sm * blocks_per_sm * kCalibWarps;
-  if (st != LITEVAR_OK || cudaMemsetAsync(d_hist, 0, hist_bytes, stream) != cudaSuccess ||
+  if (st != LITEVAR_OK || (groups == 0 && cudaMemsetAsync(d_hist, 0, hist_bytes, stream) != cudaSuccess) ||
       cudaFuncSetAttribute(calib_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     st = LITEVAR_ERR_CUDA;
   for (long long first = 0; first < rows && st == LITEVAR_OK; first += kCalibMaxRows) {
@@ -364,9 +369,19 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
     long long blocks = (n_batches + kCalibWarps - 1) / kCalibWarps;
     if (blocks > (long long)n_sm * blocks_per_sm) blocks = (long long)n_sm * blocks_per_sm;
     const unsigned parts = (unsigned)(k0 + 1 - first_part);
-    calib_hist_kernel<<<dim3((unsigned)blocks, n_batches <= 2 * n_warps ? parts : 1u), kCalibWarps * 32, smem, stream>>>(
-        sc, k0, first_part, s_max, maps + first * L_k, n_rows, (int)(first % n_k), rows_per_batch, d_hist);
-    if (cudaGetLastError() != cudaSuccess) st = LITEVAR_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks, n_batches <= 2 * n_warps ? parts : 1u);
+    cfg.blockDim = dim3(kCalibWarps * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = groups > 0 && first == 0 ? 1 : 0;  // behind sum_maps_kernel
+    if (cudaLaunchKernelEx(&cfg, calib_hist_kernel, sc, k0, first_part, s_max, maps + first * L_k, n_rows, (int)(first % n_k),
+                           rows_per_batch, d_hist) != cudaSuccess)
+      st = LITEVAR_ERR_CUDA;
   }
   if (st == LITEVAR_OK && (cudaMemcpyAsync(hist.data(), d_hist, sizeof(double) * kMaxDist * (size_t)step_k, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
                            cudaStreamSynchronize(stream) != cudaSuccess))
