@@ -154,9 +154,9 @@ litevar_status_t litevar_attn_forward(const litevar_plan_t* plan, int32_t step_k
  *   Kcodes, Vcodes   device int8 [2B, H, >= L_k, 64]; strides `scodes` in bytes (= elements), each a multiple of 16,
  *                    token stride >= 64, base pointers 16-byte aligned
  *   Kscale, Kzero, Vscale, Vzero   device fp32 [2B, H, >= L_k]; strides `srow` in elements, token stride must be 1
- * Small steps run the small-step kernel, which widens the prefix while it stages it; the others run the
- * two-threads-per-row tcgen05 kernel: tensor-map copies bring the codes of a tile into the stage, three warps widen
- * them in place.  The plan must use raster tiles at this step (LITEVAR_TILING_RASTER, or AUTO at grid sides below
+ * Small steps run the small-step kernel, which widens the prefix while it stages it; the others run the tcgen05
+ * kernel: tensor-map copies bring the codes of a 64-key chunk, the softmax warps widen them into the bf16 stages
+ * while the products run.  The plan must use raster tiles at this step (LITEVAR_TILING_RASTER, or AUTO at grid sides below
  * 48): else UNSUPPORTED.
  * Asynchronous, allocates nothing.  Errors: INVALID_ARG (before any launch), UNSUPPORTED, CUDA.
  */
@@ -219,8 +219,9 @@ litevar_status_t litevar_attn_forward_static(const int32_t* scales, int32_t n_sc
  *   radius   host out [n_scales]: -1 for parts j <= n_global_scales and for j > step_k, else the radius;
  *            a row of this kind is what litevar_window_t.radius takes
  *   ratio    host out [n_scales][256] or NULL: R_w for w = 0 .. s_j - 1 (1 elsewhere)
- *   stream   the kernel runs there; the call synchronises the stream and allocates 32 KB of scratch
- * One pass over the maps (the kernel is bound by reading them once).
+ *   stream   the kernel runs there; the call synchronises the stream; its scratch (32 KB, and up to 32 MB
+ *            where several maps are added up first) comes from a pool of the library that keeps it between calls
+ * One pass over the maps (the call is bound by reading them once).
  * Errors: INVALID_ARG, OOM, CUDA.
  */
 litevar_status_t litevar_calibrate_windows(const int32_t* scales, int32_t n_scales, int32_t step_k,

@@ -1,4 +1,4 @@
-// Tensor-core forward kernel for sm_100a: one query tile per CTA, two independent streams of key chunks.
+// Tensor-core forward kernel for sm_100a: a query tile per CTA at a time, two independent streams of key chunks.
 //
 // A CTA owns a query tile (128 queries) of one (head, batch row) and walks the live 64-key chunks of its list (laid by the planner
 // over the tile's own live keys).  A chunk comes with the class of its two halves for every warp's 32 rows: dead halves are
@@ -85,7 +85,8 @@ struct WsShared : CodeStage<KV8> {
   int abort_flag, redo;
 };
 
-// Instruction descriptors (kind::f16): D fp32, A/B bf16, M = 128, N = 64; see the field list in the other kernel.
+// Instruction descriptors (kind::f16).  Fields: D type at bit 4 (1: fp32), A and B type at bits 7 and 10 (1: bf16), B transposed
+// (MN-major, as V lies in shared memory) at bit 16, N / 8 at bit 17, M / 16 at bit 24.
 constexpr uint32_t kIdescS = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kChunkKeys >> 3) << 17) |
                              ((uint32_t)(kBlockM >> 4) << 24);
 constexpr uint32_t kIdescO = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(kHeadDim >> 3) << 17) |

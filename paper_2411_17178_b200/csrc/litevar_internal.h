@@ -15,7 +15,6 @@ constexpr int kMaxScale = 256;
 constexpr int kHeadDim = 64;
 constexpr int kBlockM = 128;  // query slots per tile
 constexpr int kBlockN = 128;  // key slots per tile
-constexpr int kMaskWordsPerRow = kBlockN / 32;
 
 // Schedule of one plan, passed to kernels by value (paper Section 2: n_k = s_k^2, off_j, L_k).
 struct Schedule {
@@ -103,7 +102,7 @@ struct Step {
   SetDesc* d_sets = nullptr;  // [n_sets]
 };
 
-// Arguments of one forward launch, common to both kernels.
+// Arguments of one forward launch, common to the kernels.
 struct FwdParams {
   const SetDesc* sets;          // [n_sets] for this step
   const int32_t* head_to_set;   // [H] or nullptr (all heads use set 0)
@@ -143,7 +142,6 @@ struct FwdParams {
                                 // stream has finished (the plan it reads was complete long before)
 };
 
-// SM count of the current device, looked up once per device (the attribute query costs a microsecond).
 // L2 size of the current device in bytes, looked up once per device.
 inline long long current_l2_bytes() {
   static long long cached[64] = {};
@@ -158,6 +156,7 @@ inline long long current_l2_bytes() {
   return n;
 }
 
+// SM count of the current device, looked up once per device (the attribute query costs a microsecond).
 inline int current_sm_count() {
   static int cached[64] = {};
   int dev = 0;

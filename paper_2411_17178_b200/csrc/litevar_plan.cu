@@ -3,8 +3,9 @@
 // The planner turns the window definition of the paper's Section 2 (one window per part of the
 // step-k attention map, the first parts global) into, per step, a CSR list of live
 // (query tile, key tile) pairs plus a 128x128-bit element mask for every partially live pair.
-// Everything that depends on the mask geometry happens here; the attention kernels only walk
-// the list and apply the bit masks, so they are independent of the window shape.
+// From
+// these come the 64-key chunk lists that the tensor-core kernel walks.  Everything that depends on the mask geometry happens here;
+// the attention kernels only walk a list and apply the bit masks, so they are independent of the window shape.
 #include <cuda_runtime.h>
 
 #include <cstdio>

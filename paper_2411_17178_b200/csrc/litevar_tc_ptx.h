@@ -1,6 +1,6 @@
 // Device-side building blocks of the tensor-core forward kernels (sm_100a): mbarrier, TMA, tcgen05 and TMEM
-// wrappers in inline PTX, the shared-memory and instruction descriptors, the tensor maps of one launch and the
-// walk over the union of two live key-tile lists.  Included by the forward kernels only.
+// wrappers in inline PTX, the shared-memory descriptor, the tensor maps of one launch and the order of its work
+// items.  Included by the tensor-core forward kernel and the host code that encodes its maps.
 #pragma once
 
 #include <cuda.h>
@@ -53,7 +53,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // Bounded wait of a pipeline's role.  Returns false when another role gave up or the time limit passed; the caller then falls
-// through to the common teardown. the polls carry a suspend-time hint (1 ms), so that a waiting
+// through to the common teardown.  The polls carry a suspend-time hint (1 ms), so that a waiting
 // warp leaves its issue slots to the others (measured on the 2K step: 2.5 % against polls without the hint, although a poll
 // takes 112 cycles instead of 74), and the clock is the SM's cycle counter (the global timer costs hundreds of cycles
 // per read).  The limit is 2^32 cycles, two seconds or more at any clock the part runs at.
@@ -123,18 +123,15 @@ __device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, const void*
 // Loads of one query tile according to its geometry (patch: four boxes of 4 x 8 cells, in slot order).
 __device__ __forceinline__ void load_q_tile(void* dst, const TensorMaps& tm, const FwdParams& p, int qt, int h, int b,
                                             uint64_t* bar) {
-  if (p.q_geom == nullptr) {
+  if (!p.q_patch) {
     tma_load_4d(dst, &tm.q, 0, qt * kBlockM, h, b, bar);
     return;
   }
   const TileGeom g = p.q_geom[qt];
-  if (g.scale < 0)
-    tma_load_4d(dst, &tm.q, 0, g.a, h, b, bar);
-  else
 #pragma unroll
-    for (int w = 0; w < 4; ++w)
-      tma_load_5d(static_cast<uint8_t*>(dst) + w * (kTileBytes / 4), &tm.q, 0, g.b + patch_slot_col(32 * w),
-                  g.a + patch_slot_row(32 * w), h, b, bar);
+  for (int w = 0; w < 4; ++w)
+    tma_load_5d(static_cast<uint8_t*>(dst) + w * (kTileBytes / 4), &tm.q, 0, g.b + patch_slot_col(32 * w),
+                g.a + patch_slot_row(32 * w), h, b, bar);
 }
 // Four consecutive K = 16 steps of one product in a single instruction sequence: step i reads A at
 // a_tmem + i * kAStep (TMEM columns) and B at b_desc + i * kBStep (descriptor units of 16 bytes); the first step
@@ -201,17 +198,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
       : "r"(taddr)
       : "memory");
 }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
-        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
-        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
-      : "memory");
-}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
@@ -228,11 +214,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
-}
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
 }
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -252,11 +233,6 @@ __device__ __forceinline__ float fast_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
 }
 
 // Order of the tensor-core kernel's work items.  The (batch row, head) units are taken in groups of

@@ -46,6 +46,21 @@ def test_calibration_matches_oracle(scales, k, peaked):
     plan.close()
 
 
+@pytest.mark.parametrize("n_maps", [1, 2, 5, 258])
+@pytest.mark.parametrize("scales,k", [((1, 2, 3, 4, 5), 5), ((1, 2, 3, 4, 6, 9), 6), ((1, 2, 3, 9, 11), 5)])
+def test_calibration_sums_maps_first(scales, k, n_maps):
+    """Maps are added up entry by entry in groups before the histogram pass (not a single one): groups that do not divide the
+    number of maps, more than one fp32 sum's worth (256), map lengths off the summing block's 1024 entries."""
+    lib_ready()
+    maps = dyadic_maps(scales, k, n_maps, 7 * k + n_maps, peaked=True)
+    dev = torch.tensor(maps, dtype=torch.float32, device="cuda")
+    rad, ratio = binding.calibrate_windows(scales, k, dev, 0.8, want_ratio=True)
+    assert rad.tolist() == orc.calibrate_radius(scales, k, maps, 0.8).tolist()
+    for j in range(4, k + 1):
+        for w in range(scales[j - 1]):
+            assert ratio[j - 1, w] == pytest.approx(orc.window_ratio(scales, k, j, w, maps), rel=1e-12, abs=1e-15)
+
+
 def test_calibration_many_rows_per_warp():
     """More (map, query) rows than resident warps: batches of several rows, several batch waves, and query
     indices that wrap around from one map to the next inside a batch."""

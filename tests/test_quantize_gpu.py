@@ -42,6 +42,28 @@ def test_quantiser_matches_oracle_bit_for_bit(shape, kind):
     _check_against_oracle(x, 8, binding.quantize_rows(x, 8, want_codes=True))
 
 
+@pytest.mark.parametrize("shape", [(31, 33, 1027, 64), (1, 3, 349526, 64), (7, 30, 4994, 64)])
+@pytest.mark.parametrize("bits", [8, 3])
+def test_quantiser_of_many_rows(shape, bits):
+    """From 2^20 rows on a thread group takes four rows in turn: token counts that are no multiple of four (groups straddle
+    heads and batch rows) and a last group that is not full; a strided view behaves as its copy."""
+    lib_ready()
+    x = _rows(shape, 17 + bits, "offset").cuda()
+    assert x.numel() // 64 >= 1 << 20
+    got = binding.quantize_rows(x, bits, want_codes=True)
+    # rows are independent: below 2^20 rows the one-row path, which the tests above pin to the oracle, gives the same bits
+    flat = x.view(1, 1, -1, 64)
+    n = flat.shape[2]
+    for a in range(0, n, 500_000):
+        b = min(n, a + 500_000)
+        part = binding.quantize_rows(flat[:, :, a:b].contiguous(), bits, want_codes=True)
+        for whole, p, w in zip(got, part, (64, 64, 1, 1)):
+            assert torch.equal(whole.reshape(-1, w)[a:b], p.reshape(-1, w))
+    # and the ends of the range against the oracle itself
+    for sl in (slice(0, 37), slice(n - 37, n)):
+        _check_against_oracle(flat[:, :, sl], bits, tuple(t.reshape(1, 1, n, *t.shape[3:])[:, :, sl] for t in got))
+
+
 @pytest.mark.parametrize("bits", [2, 4, 6])
 def test_quantiser_other_bit_widths(bits):
     lib_ready()
