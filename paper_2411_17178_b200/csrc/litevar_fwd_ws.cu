@@ -27,8 +27,9 @@
 // that followed the chunk sums by powers of two from 2^10 on, tested at every chunk: 2 to 3 % slower, 512px step 10 155.6 us
 // against 151.)
 //
-// What bounds it (ncu, 2K step with the full mask): exponential pipe 78 %, tensor pipe active 50 %, issue slots 53 %; the rest
-// is the hand-off from P to the next S (arrive, issue of eight MMAs, their execution, commit, wake: 700 cycles a chunk).
+// What bounds it (ncu, 2K step, full mask / window 1/4): issue slots 72 / 69 % busy, exponential pipe 61 / 51 %, tensor pipe active
+// 44 / 41 %; 6.5 instructions a score.  The rest is the hand-off from P to the next S (arrive, issue of eight MMAs, their
+// execution, commit, wake: 700 cycles a chunk), which the four streams of an SM cover for one another.
 // Measured on B200, with what the kernel with one softmax thread per row and 128-key tiles took before: 2K step with the full
 // mask 5.05 ms (6.71), window 1/4 1.45 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 151 / 68 / 31 us (261 / 116 / 47),
 // 256px step 10 with 960 units 74 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
