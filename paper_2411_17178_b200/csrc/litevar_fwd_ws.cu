@@ -681,8 +681,10 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         tc_fence_after();
         uint8_t* slice = sm.q[tiles % kQBufs] + (warp << 11);
         if (ok) {
+          // Weights against the larger of the two masses 2^reference * sum.  (Against the larger reference they are wrong: a stream
+          // without a live key among its first eight has reference 0, however far below the other's mass its own lies.)
           const float2 other = ref_other[m];
-          const float top = fmaxf(own, other.x);
+          const float top = fmaxf(own + fast_log2(l), other.x + fast_log2(other.y));
           const float f_own = fast_exp2(own - top), f_other = fast_exp2(other.x - top);
           const float inv = 1.f / (l * f_own + other.y * f_other);
           const float w0 = (st ? f_other : f_own) * inv, w1 = (st ? f_own : f_other) * inv;

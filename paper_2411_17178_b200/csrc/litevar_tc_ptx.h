@@ -235,6 +235,12 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
+__device__ __forceinline__ float fast_log2(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // Order of the tensor-core kernel's work items.  The (batch row, head) units are taken in groups of
 // p.units_per_group; inside a group the items go query tile by query tile, all
 // units of the group side by side.  The K/V of one group is what the CTAs resident at one time read: the host

@@ -22,6 +22,8 @@ TC_KERNELS = (binding.KERNEL_TCGEN05, binding.KERNEL_TCGEN05_WS)
 
 TILINGS = [binding.TILING_RASTER, binding.TILING_PATCH]
 TNAME = {binding.TILING_RASTER: "raster", binding.TILING_PATCH: "patch"}
+# builds of the tcgen05 kernel with the tilings they take (an 8-bit cache: raster only)
+BUILDS = [(b, t) for b in ("one-tile", "many-tiles", "8-bit") for t in TILINGS if (b, t) != ("8-bit", binding.TILING_PATCH)]
 
 
 @pytest.mark.parametrize("tiling", TILINGS, ids=lambda t: TNAME[t])
@@ -507,4 +509,40 @@ def test_many_tiles_per_cta(case):
         # a row is not an average of many values, and the error is bounded by 2^-9 max|V| twice, not by a fixed 1e-2
         ma, rl = errors(got[:, heads], ref)
         assert ma <= 2.0 ** -8 * float(Vc.float().abs().max()) and rl <= REL_L2, f"{case} set {s}: max-abs {ma:.3e} rel-L2 {rl:.3e}"
+    plan.close()
+
+
+@pytest.mark.parametrize("case", ["first", "second"])
+@pytest.mark.parametrize("build,tiling", BUILDS, ids=lambda x: TNAME.get(x, x))
+def test_streams_with_far_references(build, tiling, case):
+    """One key stream's reference is taken from keys far below the others (logits of -92 against -40), the other stream has no
+    live key among its first eight and reference 0: both sums are in range, and the stream with the small reference holds most
+    of the weight.  `case` says which stream that is."""
+    lib_ready()
+    H, B = (8, 32) if build == "many-tiles" else (2, 1)
+    if case == "first":         # cache rows 0 to 7 are global: the first keys of the first chunk of every tile
+        scales, low = (1, 2, 3, 4, 6, 9, 13), list(range(8))
+        tab = orc.window_table(scales)
+    else:                       # second chunk: raster rows 64 on; patches: columns 8 on of the 12 x 12 grid, for the last query column
+        scales, low = (12, 16), [8, 9, 10, 11] + list(range(64, 72))
+        tab = orc.full_table(scales)
+        tab[1] = 3, 9
+    K, n, L = len(scales), scales[-1] ** 2, sum(s * s for s in scales)
+    logits = torch.full((L,), -40.0)
+    logits[low] = -92.0
+    w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=97)
+    Q = torch.ones(2 * B, H, n, 64).bfloat16()
+    Kc = (logits / 8).view(1, 1, L, 1).expand(2 * B, H, L, 64).bfloat16()    # q . k / 8 = logit, exactly
+    Vc = wl.make_kv(w, 0)[1]
+    plan = binding.Plan(scales, n_heads=H, radius=tab, tiling=tiling)
+    if build == "8-bit":
+        (K8, *kq), (V8, *vq) = (binding.quantize_rows(t.cuda(), want_codes=True) for t in (Kc, Vc))
+        out = torch.full(Q.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+        plan.forward_kv8(K, B, Q.cuda(), *kq, *vq, out)
+        got, Kc, Vc = out.double().cpu().numpy(), K8.cpu(), V8.cpu()
+    else:
+        got, _ = run_forward(plan, K, B, Q, Kc, Vc, binding.KERNEL_TCGEN05)
+    for b in {0, B, 2 * B - 1}:
+        ref = orc.attention_step(scales, K, tab[K - 1], Q[b:b + 1], Kc[b:b + 1], Vc[b:b + 1])
+        assert_close(got[b:b + 1], ref, f"batch row {b}")
     plan.close()
