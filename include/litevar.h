@@ -127,6 +127,7 @@ litevar_status_t litevar_attn_plan(const int32_t* scales, int32_t n_scales, int3
  *   Q, out       device bf16 [2B, H, n_k, 64] with the given strides
  *   Kcache,Vcache device bf16 [2B, H, >= L_k, 64]; only rows [0, L_k) are read
  *   strides      in elements; each a multiple of 8; base pointers 16-byte aligned
+ *                out may be Q itself (same pointer and strides); it must not overlap Q, K or V in another way
  *   stream       cudaStream_t; the call is asynchronous, allocates nothing, synchronises nothing
  *
  * At a shared step the kernel runs for rows [0,B) only, never reads rows [B,2B) of Q/K/V,

@@ -23,7 +23,8 @@
 // The reference of a row (probabilities are 2^(score * scale - reference)) is the maximum of the first chunk's first eight keys
 // and stays (0 where none of them is live): bf16 and fp32 have the same exponent range, so P, its sum and the accumulator are as
 // accurate at 2^90 as at 1, and a tile's rows need neither a maximum per chunk nor a rescaled accumulator.  At the end a row whose
-// sum left [2^-96, 2^96] sends the CTA through its lists again, with every chunk's maximum taken first (`exact`).  (A reference
+// sum left [2^-96, 2^96] sends the CTA through its lists again, with every chunk's maximum taken first (`exact`), for the 32 rows
+// of a warp that it belongs to, which are stored then.  (A reference
 // that followed the chunk sums by powers of two from 2^10 on, tested at every chunk: 2 to 3 % slower, 512px step 10 155.6 us
 // against 151.)
 //
@@ -39,6 +40,7 @@
 // Every wait on an mbarrier is bounded; when one runs out the CTA raises the plan's status word, drains its copies, frees its
 // TMEM and returns (the softmax warps still arrive for every chunk, so that the named barriers complete).  The element mask, the
 // lists and CFG sharing (second store at batch row b + B) are those of the plan (paper Sections 2 and 3).
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 
@@ -57,6 +59,7 @@ constexpr int kStages = 2;                // K ring and V ring of a stream
 constexpr int kThreads = 320;             // two streams of four softmax warps, one issuing warp each
 constexpr uint32_t kTmemCols = 256, kColO = 128;  // S (and P over it) of stream s at 64 s, O at 128 + 64 s
 
+constexpr int kMaxTiles = 1024;  // of a CTA that takes several (MANY)
 constexpr float kRange = 79228162514264337593543950336.f;  // 2^96: a row sum beyond it, or below its inverse, redoes the list
 
 // 8-bit cache build: the codes of a chunk (64 rows of 64 bytes, as the tensor-map copy delivers them, no swizzle) and its rows'
@@ -82,6 +85,8 @@ struct WsShared : CodeStage<KV8> {
   alignas(8) uint64_t q_full[2], q_free;
   uint64_t k_full[2][kStages], v_full[2][kStages];
   uint64_t s_full[2], o_full[2];
+  uint32_t held[4][MANY ? kMaxTiles / 32 : 1];  // bit x: the 32 rows of the CTA's tile x are left to the second pass
+  int out_of_range[4][2];  // 1 + the last even and odd tile with such rows (a warp is at most one tile ahead of its partner)
   uint32_t tmem_base;
   int abort_flag, redo;
 };
@@ -253,6 +258,8 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (threadIdx.x < 4 * (sizeof(sm.held[0]) / sizeof(uint32_t))) (&sm.held[0][0])[threadIdx.x] = 0u;
+  if (threadIdx.x < 8) (&sm.out_of_range[0][0])[threadIdx.x] = 0;
   // the next kernel of the stream may start its set-up while this grid drains; this grid's set-up ran while the
   // previous one drained.  Nothing an earlier kernel wrote is read before the wait below (the plan is older).
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -512,14 +519,14 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       if (!KV8 && !exact) meet();
       const uint32_t tlane = sm.tmem_base + ((uint32_t)(lane_group * 32) << 16);
       const uint32_t tS = tlane + 64 * st, tO = tlane + kColO + 64 * st;
-      // the previous tile's output rows have left their buffer, which the next copy but one (the redo's next) goes to
+      // the previous tile's output rows have left their buffer, which the next copy but one (the second pass's next) goes to
       auto stored = [&] {
         if (lane == 0) {
           asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
           if (MANY) mbar_arrive(&sm.q_free);
         }
       };
-      for (int w = blockIdx.x;; w += w_step) {
+      for (int w = blockIdx.x, x = 0;; w += w_step, ++x) {
         const int end = base + n;
         // probabilities are 2^(score * sc - msc); `none` until msc has been set from a live key
         float msc = 0.f;
@@ -671,7 +678,10 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           ++o_tiles;
         }
         const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y);
-        bad |= !exact && seen && !(l < kRange && l > 1.f / kRange);  // (a NaN goes this way too)
+        if (!exact && seen && !(l < kRange && l > 1.f / kRange)) {  // (a NaN goes this way too)
+          bad = true;
+          sm.out_of_range[lane_group][x & 1] = x + 1;
+        }
         const float own = seen ? msc : -INFINITY;  // (dead keys leave traces of 2^-125 in l)
         float2* const ref_own = MANY ? sm.ref[st] : reinterpret_cast<float2*>(sm.k[st][0]);
         const float2* const ref_other = MANY ? sm.ref[st ^ 1] : reinterpret_cast<const float2*>(sm.k[st ^ 1][0]);
@@ -718,7 +728,19 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
+        // 32 rows one of which is out of range in either stream are not stored, and the second pass stores these rows only: every
+        // row is stored once (two bulk stores to one address have no order), and a row of Q that the second pass reads has not been
+        // overwritten where the output takes Q's place.
         if (ok && lane == 0) {
+          bool store;
+          if constexpr (MANY) {
+            store = exact ? (sm.held[lane_group][x >> 5] >> (x & 31)) & 1u : *(volatile int*)&sm.out_of_range[lane_group][x & 1] != x + 1;
+            if (!exact && !store && st == 0) {
+              sm.held[lane_group][x >> 5] |= 1u << (x & 31);
+            }
+          } else {
+            store = exact == (*(volatile int*)&sm.out_of_range[lane_group][0] != 0);
+          }
           int qt = item0.qt, h = item0.h, b = item0.b;
           if constexpr (MANY) {
             int unit;
@@ -731,13 +753,13 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           if (p.q_patch) {
             const TileGeom g = p.q_geom[qt];
             const int r0 = g.a + patch_slot_row(32 * lane_group), c0 = g.b + patch_slot_col(32 * lane_group);
-            if (r0 < p.s_k && c0 < p.s_k) {
+            if (store && r0 < p.s_k && c0 < p.s_k) {
               tma_store_5d(&tm.o, slice, 32 * st, c0, r0, h, b);
               if (p.share_offset > 0) tma_store_5d(&tm.o, slice, 32 * st, c0, r0, h, bs);
             }
           } else {
             const int q0 = qt * kBlockM + 32 * lane_group;
-            if (q0 < p.n_k) {
+            if (store && q0 < p.n_k) {
               tma_store_4d(&tm.o, slice, 32 * st, q0, h, b);
               if (p.share_offset > 0) tma_store_4d(&tm.o, slice, 32 * st, q0, h, bs);
             }
@@ -807,7 +829,7 @@ litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream
   const long long items = (long long)n_q_tiles * p.n_heads * p.batch_computed, resident = 2ll * current_sm_count();
   const int chunks = p.chunks_per_tile;
   if (chunks > 0 && chunks <= 40 && 2 * items >= 5 * resident && 5 * items >= chunks * resident)
-    return launch_variant<false, true>(tm, p, n_q_tiles, (int)resident, stream);
+    return launch_variant<false, true>(tm, p, n_q_tiles, (int)std::max(resident, (items + kMaxTiles - 1) / kMaxTiles), stream);
   return launch_variant<false, false>(tm, p, n_q_tiles, 0, stream);
 }
 

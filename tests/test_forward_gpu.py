@@ -9,7 +9,7 @@ import torch
 
 from oracle import litevar_oracle as orc
 from paper_2411_17178_b200 import binding, workloads as wl
-from tests.gpu_util import REL_L2, assert_close, check_sampled, errors, lib_ready, run_forward, stratified_samples
+from tests.gpu_util import MAX_ABS, REL_L2, assert_close, check_sampled, errors, lib_ready, run_forward, stratified_samples
 
 pytestmark = pytest.mark.gpu
 
@@ -545,4 +545,44 @@ def test_streams_with_far_references(build, tiling, case):
     for b in {0, B, 2 * B - 1}:
         ref = orc.attention_step(scales, K, tab[K - 1], Q[b:b + 1], Kc[b:b + 1], Vc[b:b + 1])
         assert_close(got[b:b + 1], ref, f"batch row {b}")
+    plan.close()
+
+
+@pytest.mark.parametrize("build,tiling", BUILDS, ids=lambda x: TNAME.get(x, x))
+def test_output_in_place_of_q_with_a_second_pass(build, tiling):
+    """`out` may be Q itself.  Two keys with scores in the thousands send rows to the second pass, which reads Q again: the
+    result has the bits of a call with an output of its own, which agrees with the oracle."""
+    lib_ready()
+    scales, K = (1, 2, 3, 4, 6, 9, 13), 7
+    H, B = (7, 40) if build == "many-tiles" else (2, 1)
+    w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=94)
+    Q = wl.make_q(w, 0, K)
+    Kc, Vc = wl.make_kv(w, 0)
+    L = Kc.shape[2]
+    Kc[:, :, L - 40] *= 300
+    Kc[:, :, 150] *= -250
+    plan = binding.Plan(scales, n_heads=H, tiling=tiling)
+    plan.set_kernel(binding.KERNEL_TCGEN05)
+    k, v = Kc.cuda(), Vc.cuda()
+    if build == "8-bit":
+        (k, *kq), (v, *vq) = (binding.quantize_rows(t, want_codes=True) for t in (k, v))
+
+    def call(q, out):
+        if build == "8-bit":
+            plan.forward_kv8(K, B, q, *kq, *vq, out)
+        else:
+            plan.forward(K, B, q, k, v, out)
+        return out
+
+    apart = call(Q.cuda(), torch.full(Q.shape, float("nan"), dtype=torch.bfloat16, device="cuda"))
+    q = Q.cuda()
+    assert torch.equal(call(q, q).view(torch.int16), apart.view(torch.int16))
+    row = orc.window_table(scales)[K - 1]
+    for b in {0, 2 * B - 1}:
+        ref = orc.attention_step(scales, K, row, Q[b:b + 1], k[b:b + 1].cpu(), v[b:b + 1].cpu())
+        ma, rl = errors(apart[b:b + 1].double().cpu().numpy(), ref)
+        # a row with one dominant key is that key's V, which the 8-bit build widens to within one bf16 unit of the dequantised
+        # row (product and sum are rounded together): 2^-7 of its magnitude on top of the parity tolerance
+        bound = MAX_ABS + (2.0 ** -7 * float(v.float().abs().max()) if build == "8-bit" else 0.0)
+        assert ma <= bound and rl <= REL_L2, f"batch row {b}: max-abs {ma:.3e} rel-L2 {rl:.3e}"
     plan.close()
