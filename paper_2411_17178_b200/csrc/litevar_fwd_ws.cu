@@ -98,15 +98,16 @@ constexpr uint32_t kIdescS = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kC
 constexpr uint32_t kIdescO = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(kHeadDim >> 3) << 17) |
                              ((uint32_t)(kBlockM >> 4) << 24);
 
-// 2^x on the FMA pipe for x = score * scale - reference clamped to [-125, 125]: the caller's multiply-add saturates
-// y = (x + 125) / 250 to [0, 1] (dead keys, -inf, give 0).  x = n + f with n = round(x) and f in [-1/2, 1/2]; 2^f by a cubic
-// fitted to it (relative error 7.5e-5, far inside the bf16 rounding of P), 2^n by adding n to the exponent field.
-constexpr float kClamp = 125.f;
+// 2^x on the FMA pipe for x = score * scale - reference clamped to [-125, 100]: the caller's multiply-add saturates
+// y = (100 - x) / 225 to [0, 1].  Dead keys (-inf) give 1 and 2^-125; a NaN saturates to 0 and gives 2^100, which takes the row's
+// sum out of range.  x = n + f with n = round(x) and f in [-1/2, 1/2]; 2^f by a cubic fitted to it (relative error 7.5e-5, far
+// inside the bf16 rounding of P), 2^n by adding n to the exponent field.
+constexpr float kClampHigh = 100.f, kClampSpan = 225.f;
 __device__ __forceinline__ float2 exp2_fma2(float2 y) {
-  const float2 range = make_float2(2.f * kClamp, 2.f * kClamp);
-  const float2 t = __ffma2_rn(y, range, make_float2(12582912.f - kClamp, 12582912.f - kClamp));  // n in the low mantissa bits
-  const float2 m = __fadd2_rn(make_float2(12582912.f - kClamp, 12582912.f - kClamp), make_float2(-t.x, -t.y));  // -n - 125
-  const float2 f = __ffma2_rn(y, range, m);
+  const float2 span = make_float2(-kClampSpan, -kClampSpan);
+  const float2 t = __ffma2_rn(y, span, make_float2(12582912.f + kClampHigh, 12582912.f + kClampHigh));  // n in the low mantissa bits
+  const float2 m = __fadd2_rn(make_float2(12582912.f + kClampHigh, 12582912.f + kClampHigh), make_float2(-t.x, -t.y));  // 100 - n
+  const float2 f = __ffma2_rn(y, span, m);
   float2 z = __ffma2_rn(make_float2(0.05517153441905975f, 0.05517153441905975f), f,
                         make_float2(0.2426111102104187f, 0.2426111102104187f));
   z = __ffma2_rn(z, f, make_float2(0.6932610273361206f, 0.6932610273361206f));
@@ -496,7 +497,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       const int m = lane_group * 32 + lane;
       const float sc = p.sm_scale * 1.4426950408889634f;
       const float2 sc2 = make_float2(sc, sc);
-      const float sc_y = sc * (0.5f / kClamp);
+      const float sc_y = -sc / kClampSpan;
       // Per chunk: class of its two halves for this warp's rows (bits 0 - 1 and 2 - 3: 0 dead, 1 partial, 2 full) and the key bits
       // of this thread's row, looked up one chunk ahead.
       int n = item0.n, n_all = item0.n_all;
@@ -618,7 +619,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
               }
               // probabilities against the reference: scale and shift (packed FMAs), 2^x, row sum, bf16
               const float2 nm2 = make_float2(-msc, -msc);
-              const float nm_y = fmaf(-msc, 0.5f / kClamp, 0.5f);
+              const float nm_y = fmaf(msc, 1.f / kClampSpan, kClampHigh / kClampSpan);
 #pragma unroll
               for (int e = 0; e < 32; e += 4) {
                 const uint32_t* rr = r + e;
@@ -677,12 +678,15 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           if (ok) ok = mbar_wait_long(&sm.o_full[st], (uint32_t)(o_tiles & 1), abort_flag, p.status);
           ++o_tiles;
         }
-        const float l = (l2a.x + l2a.y) + (l2b.x + l2b.y);
+        float l = (l2a.x + l2a.y) + (l2b.x + l2b.y);
         if (!exact && seen && !(l < kRange && l > 1.f / kRange)) {  // (a NaN goes this way too)
           bad = true;
           sm.out_of_range[lane_group][x & 1] = x + 1;
         }
-        const float own = seen ? msc : -INFINITY;  // (dead keys leave traces of 2^-125 in l)
+        // Against exact maxima a sum is at most 2^8 times the number of keys: a larger one is a score of +inf or NaN.
+        if (exact && seen && !(l < kRange)) l = NAN;
+        // (dead keys leave traces of 2^-125 in l; in the second pass a stream without a reference has scores of -inf only)
+        const float own = seen && !(exact && none) ? msc : -INFINITY;
         float2* const ref_own = MANY ? sm.ref[st] : reinterpret_cast<float2*>(sm.k[st][0]);
         const float2* const ref_other = MANY ? sm.ref[st ^ 1] : reinterpret_cast<const float2*>(sm.k[st ^ 1][0]);
         ref_own[m] = make_float2(own, l);

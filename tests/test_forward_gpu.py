@@ -586,3 +586,44 @@ def test_output_in_place_of_q_with_a_second_pass(build, tiling):
         bound = MAX_ABS + (2.0 ** -7 * float(v.float().abs().max()) if build == "8-bit" else 0.0)
         assert ma <= bound and rl <= REL_L2, f"batch row {b}: max-abs {ma:.3e} rel-L2 {rl:.3e}"
     plan.close()
+
+
+@pytest.mark.parametrize("value", ["nan", "inf", "-inf", "all -inf"])
+@pytest.mark.parametrize("build,tiling", BUILDS, ids=lambda x: TNAME.get(x, x))
+def test_non_finite_scores(build, tiling, value):
+    """One key of every head has a score of NaN, +inf or -inf, at another place of its chunk in each of 64 heads: the rows that
+    attend to it are NaN (-inf: the key has weight 0), the others are untouched.  All scores -inf: NaN rows."""
+    lib_ready()
+    scales, K, H = (1, 2, 3, 4, 6, 9, 13), 7, 64
+    B = 4 if build == "many-tiles" else 1
+    w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=98)
+    Q = wl.make_q(w, 0, K).float().abs().add(0.125).bfloat16()     # positive: q . (inf, inf, ...) = inf
+    Kc, Vc = wl.make_kv(w, 0)
+    L = Kc.shape[2]
+    k, v = Kc.cuda(), Vc.cuda()
+    if build == "8-bit":
+        (k, *kq), (v, *vq) = (binding.quantize_rows(t, want_codes=True) for t in (k, v))
+    bad = float(value.split()[-1])
+    at = [slice(0, L)] * 4 if value == "all -inf" else list(range(L - 100, L - 100 + H))
+    for h, t in enumerate(at):
+        k[:, h, t] = bad
+        if build == "8-bit":
+            kq[1][:, h, t], kq[2][:, h, t] = 0.0, bad
+    plan = binding.Plan(scales, n_heads=H, tiling=tiling)
+    plan.set_kernel(binding.KERNEL_TCGEN05)
+    out = torch.zeros(Q.shape, dtype=torch.bfloat16, device="cuda")
+    if build == "8-bit":
+        plan.forward_kv8(K, B, Q.cuda(), *kq, *vq, out)
+    else:
+        plan.forward(K, B, Q.cuda(), k, v, out)
+    assert plan.poll() == 0
+    b = 2 * B - 1
+    live = torch.from_numpy(orc.mask(scales, K, orc.window_table(scales)[K - 1]))
+    s = 0.125 * Q[b].double() @ k[b].double().cpu().transpose(-1, -2)
+    p = torch.softmax(s.masked_fill(~live, float("-inf")), -1)
+    ref, got = (p @ v[b].double().cpu()).numpy(), out[b].double().cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    finite = ~np.isnan(ref)
+    assert finite.any() and (finite.all() == (value == "-inf"))
+    assert_close(got[finite], ref[finite], value)
+    plan.close()
