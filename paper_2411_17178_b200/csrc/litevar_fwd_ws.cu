@@ -21,11 +21,10 @@
 // TMEM columns: S and P of stream s at 64 s, O at 128 + 64 s.
 //
 // The reference of a row (probabilities are 2^(score * scale - reference)) is the maximum of the first chunk's first eight keys
-// and stays (0 where none of them is live): bf16 and fp32 have the same exponent range, so P, its sum and the accumulator are as
-// accurate at 2^90 as at 1, and a tile's rows need neither a maximum per chunk nor a rescaled accumulator.  At the end a row whose
-// sum left [2^-96, 2^96] sends the CTA through its lists again, with every chunk's maximum taken first (`exact`), for the 32 rows
-// of a warp that it belongs to, which are stored then.  (A reference
-// that followed the chunk sums by powers of two from 2^10 on, tested at every chunk: 2 to 3 % slower, 512px step 10 155.6 us
+// and stays (0 where none of them is live): bf16 and fp32 have the same exponent range, so P and its sum are as accurate at 2^90 as
+// at 1, and a tile's rows need neither a maximum per chunk nor a rescaled accumulator.  At the end a row whose sum or output is
+// out of range (kRange, kSmall) sends the CTA through its lists again, with every chunk's maximum taken first (`exact`), for the 32
+// rows of a warp that it belongs to, which are stored then.  (A reference that followed the chunk sums by powers of two from 2^10 on, tested at every chunk: 2 to 3 % slower, 512px step 10 155.6 us
 // against 151.)
 //
 // What bounds it (ncu, 2K step, full mask / window 1/4): issue slots 72 / 69 % busy, exponential pipe 61 / 51 %, tensor pipe active
@@ -60,7 +59,12 @@ constexpr int kThreads = 320;             // two streams of four softmax warps, 
 constexpr uint32_t kTmemCols = 256, kColO = 128;  // S (and P over it) of stream s at 64 s, O at 128 + 64 s
 
 constexpr int kMaxTiles = 1024;  // of a CTA that takes several (MANY)
-constexpr float kRange = 79228162514264337593543950336.f;  // 2^96: a row sum beyond it, or below its inverse, redoes the list
+// A row sum of the first pass outside (2^-64, 2^96) goes to the second pass.  (The lower end keeps the traces of dead keys, 2^-125
+// each, 2^-48 below a sum over any number of keys.)
+constexpr float kRange = 79228162514264337593543950336.f, kRangeLow = 5.42101086242752217e-20f;
+// So does a row of output that is not finite (sums of P V overflow before those of P), or so small beside its weight, where that is
+// above 1, that products P V may have been subnormal (2^-126 each, 2^14 of them).
+constexpr float kSmall = 7.88860905221011805e-31f;  // 2^-100
 
 // 8-bit cache build: the codes of a chunk (64 rows of 64 bytes, as the tensor-map copy delivers them, no swizzle) and its rows'
 // scales and shifted zero points, on their way into the bf16 stages (empty in the bf16 build).
@@ -679,7 +683,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           ++o_tiles;
         }
         float l = (l2a.x + l2a.y) + (l2b.x + l2b.y);
-        if (!exact && seen && !(l < kRange && l > 1.f / kRange)) {  // (a NaN goes this way too)
+        if (__builtin_expect(!exact && seen && !(l < kRange && l > kRangeLow), 0)) {  // (a NaN goes this way too)
           bad = true;
           sm.out_of_range[lane_group][x & 1] = x + 1;
         }
@@ -707,6 +711,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           // The warp's 32 rows x 64 B pass through its own 2 KB slice of the Q buffer (its last reader, the last score
           // product, is done: every warp of both streams has seen it through o_full) to a tensor-map store.  Piece position XOR
           // (row / 2) is the map's swizzle and keeps the writes free of bank conflicts.
+          float largest = 0.f;
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             uint32_t r[16], r1[16];
@@ -719,17 +724,23 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
               float2 x = make_float2(__uint_as_float(r[e]) * w0, __uint_as_float(r[e + 1]) * w0);
               if (both) x = __ffma2_rn(make_float2(__uint_as_float(r1[e]), __uint_as_float(r1[e + 1])), make_float2(w1, w1), x);
               o[e >> 1] = pack_bf16(x.x, x.y);
+              asm("max.NaN.f32 %0, %0, %1, %2;" : "+f"(largest) : "f"(fabsf(x.x)), "f"(fabsf(x.y)));
             }
 #pragma unroll
             for (int e = 0; e < 2; ++e)
               *reinterpret_cast<uint4*>(slice + lane * 64 + (((2 * c + e) ^ (lane >> 1)) & 3) * 16) =
                   make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
           }
+          const float weight = fmaxf(w0, w1);
+          if (__builtin_expect(!exact && top > -INFINITY && !(largest < INFINITY && (weight <= 1.f || largest > weight * kSmall)), 0)) {
+            bad = true;
+            sm.out_of_range[lane_group][x & 1] = x + 1;
+          }
         }
-        if constexpr (MANY) {  // both streams' accumulators of these rows have been read: the next tile's may overwrite them
-          tc_fence_before();
-          asm volatile("bar.sync %0, 64;" ::"r"(7 + lane_group) : "memory");
-        }
+        // the pair of warps agrees on what is out of range; both streams' accumulators of these rows have been read, so that the
+        // next tile's may overwrite them
+        tc_fence_before();
+        asm volatile("bar.sync %0, 64;" ::"r"(7 + lane_group) : "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         // 32 rows one of which is out of range in either stream are not stored, and the second pass stores these rows only: every

@@ -627,3 +627,33 @@ def test_non_finite_scores(build, tiling, value):
     assert finite.any() and (finite.all() == (value == "-inf"))
     assert_close(got[finite], ref[finite], value)
     plan.close()
+
+
+@pytest.mark.parametrize("logits,magnitude", [((-30.0, 30.0), 1e30), ((-30.0, 30.0), 1e12), ((-40.0, -40.0), 1e-30), ((-43.0, -43.0), 1e-14)])
+@pytest.mark.parametrize("build,tiling", BUILDS, ids=lambda x: TNAME.get(x, x))
+def test_values_of_any_magnitude(build, tiling, logits, magnitude):
+    """Row sums near the ends of the first pass's range (logits of the first eight cache rows and of the others) times values
+    that are large or small: the products of P and V leave the fp32 range where P and its sum do not."""
+    lib_ready()
+    scales, K = (1, 2, 3, 4, 6, 9, 13), 7
+    H, B = (8, 32) if build == "many-tiles" else (2, 1)
+    L = sum(s * s for s in scales)
+    lg = torch.full((L,), logits[1])
+    lg[:8] = logits[0]
+    w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=97)
+    Q = torch.ones(2 * B, H, 169, 64).bfloat16()
+    Kc = (lg / 8).view(1, 1, L, 1).expand(2 * B, H, L, 64).bfloat16()       # q . k / 8 = logit
+    Vc = (wl.make_kv(w, 0)[1].float() * magnitude).bfloat16()
+    plan = binding.Plan(scales, n_heads=H, tiling=tiling)
+    if build == "8-bit":
+        (K8, *kq), (V8, *vq) = (binding.quantize_rows(t.cuda(), want_codes=True) for t in (Kc, Vc))
+        out = torch.full(Q.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+        plan.forward_kv8(K, B, Q.cuda(), *kq, *vq, out)
+        got, Kc, Vc = out.double().cpu().numpy(), K8.cpu(), V8.cpu()
+    else:
+        got, _ = run_forward(plan, K, B, Q, Kc, Vc, binding.KERNEL_TCGEN05)
+    row = orc.window_table(scales)[K - 1]
+    for b in {0, 2 * B - 1}:
+        ref = orc.attention_step(scales, K, row, Q[b:b + 1], Kc[b:b + 1], Vc[b:b + 1])
+        assert_close(got[b:b + 1] / magnitude, ref / magnitude, f"batch row {b}")
+    plan.close()
