@@ -68,6 +68,11 @@ __device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
   asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
   return d;
 }
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float d;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
 __device__ __forceinline__ float lo_bf16(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float hi_bf16(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
 
@@ -150,9 +155,11 @@ __global__ void __launch_bounds__(kQuantThreads, 4) quant_rows_kernel(const __gr
       if ((part & (R - 1)) == g) mine = top[g];
     const float mx = lo_bf16(mine), mn = -hi_bf16(mine);
     const float s = __fdiv_rn(__fsub_rn(mx, mn), a.levels);
-    const float r = __fdiv_rn(1.f, s > 0.f ? s : 1.f);
+    // no step (s = 0, or a row of NaN): estimates of 0, or NaN where x - z is not finite
+    const float s1 = s > 0.f ? s : INFINITY;
+    const float r = __fdiv_rn(1.f, s1);
     const float z = __fmul_rn(__fadd_rn(mx, mn), 0.5f);
-    const float lo = __fsub_rn(__fadd_rn(__fdiv_rn(__fsub_rn(mn, z), s > 0.f ? s : 1.f), kMagic), kMagic);
+    const float lo = __fsub_rn(__fadd_rn(__fdiv_rn(__fsub_rn(mn, z), s1), kMagic), kMagic);
     const unsigned row = group * R + (part & (R - 1));
     if (part < R && row < (unsigned)a.n_rows && (R > 1 || ti[0] == 0)) {
       if (a.scale != nullptr) a.scale[row] = s;
@@ -179,9 +186,9 @@ __global__ void __launch_bounds__(kQuantThreads, 4) quant_rows_kernel(const __gr
     // stays near 2^(B-1) here), subtracting it again gives it as a float.  The estimate y = (x - z) * (1 / s) is within
     // |y| * 2^-23 < 2^-15.9 of the true quotient and the correctly rounded quotient within 2^-17 of it, so an
     // estimate farther than 2^-14 from a half-integer rounds as the IEEE quotient does; a thread with an estimate
-    // closer than that redoes its eight values with the division.  So does every thread of a row whose step is so
-    // small that its reciprocal is not a normal number.  (s = 0: x = z for every element, code 0.)  What has the minimum's
-    // difference x - z has its code, and what is above the largest code ends there.
+    // closer than that, or that is NaN, redoes its eight values with the division.  So does every thread of a row whose step is so
+    // small that its reciprocal is not a normal number.  What has the minimum's difference x - z has its code, and what is above
+    // the largest code ends there.
     const float d_min = __fsub_rn(-hi_bf16(top[g]), z), lo = lo_row[g];
     float2 t[4];  // 1.5 * 2^23 + code
     float far = 0.f;
@@ -189,20 +196,26 @@ __global__ void __launch_bounds__(kQuantThreads, 4) quant_rows_kernel(const __gr
     for (int i = 0; i < 4; ++i) {
       const float2 dz = __fadd2_rn(make_float2(lo_bf16(u[i]), hi_bf16(u[i])), nz2);
       float2 y = __fmul2_rn(dz, r2);
-      y = make_float2(fminf(dz.x == d_min ? lo : y.x, a.hi), fminf(dz.y == d_min ? lo : y.y, a.hi));
+      y = make_float2(min_nan(dz.x == d_min ? lo : y.x, a.hi), min_nan(dz.y == d_min ? lo : y.y, a.hi));
       t[i] = __fadd2_rn(y, magic2);
       const float2 n = __fadd2_rn(t[i], nmagic2);
       const float2 d = __fadd2_rn(y, make_float2(-n.x, -n.y));
-      asm("max.f32 %0, %0, %1, %2;" : "+f"(far) : "f"(fabsf(d.x)), "f"(fabsf(d.y)));
+      asm("max.NaN.f32 %0, %0, %1, %2;" : "+f"(far) : "f"(fabsf(d.x)), "f"(fabsf(d.y)));
     }
-    if (far > 0.5f - 0.00006103515625f || !((s > 0.f ? s : 1.f) > 1e-30f)) {  // rare (one thread-row in a thousand)
+    if (!(far <= 0.5f - 0.00006103515625f) || !((s > 0.f ? s : 1.f) > 1e-30f)) {  // rare (one thread-row in a thousand)
       const float s1 = s > 0.f ? s : 1.f;
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         t[i] = make_float2(__fadd_rn(fminf(__fdiv_rn(__fsub_rn(lo_bf16(u[i]), z), s1), a.hi), kMagic),
                            __fadd_rn(fminf(__fdiv_rn(__fsub_rn(hi_bf16(u[i]), z), s1), a.hi), kMagic));
+      if (far != far) {  // a NaN takes the lowest code, a row without a step 0
+        const float top_code = s > 0.f ? a.hi : 0.f, low_code = s > 0.f ? -1.f - a.hi : 0.f;
+        auto code = [&](float x) { return __fadd_rn(fminf(fmaxf(__fdiv_rn(__fsub_rn(x, z), s1), low_code), top_code), kMagic); };
+#pragma unroll
+        for (int i = 0; i < 4; ++i) t[i] = make_float2(code(lo_bf16(u[i])), code(hi_bf16(u[i])));
+      }
     }
-    // (-(2^B - 1) / 2 rounds to -2^(B-1) at the lowest: no lower clamp)
+    // (the fast way needs no lower clamp: -(2^B - 1) / 2 rounds to -2^(B-1) at the lowest)
     uint32_t packed[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {

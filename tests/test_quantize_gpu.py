@@ -64,6 +64,35 @@ def test_quantiser_of_many_rows(shape, bits):
         _check_against_oracle(flat[:, :, sl], bits, tuple(t.reshape(1, 1, n, *t.shape[3:])[:, :, sl] for t in got))
 
 
+@pytest.mark.parametrize("n_rows", [8, 1 << 20], ids=["one-row-groups", "four-row-groups"])
+@pytest.mark.parametrize("bits", [8, 3])
+def test_quantiser_rows_that_are_not_finite(bits, n_rows):
+    """A NaN is left out of the row's maximum and minimum and has the lowest code; where an infinity is in the row every code is
+    the lowest (0 times infinity); a row whose maximum and minimum are equal, or all NaN, has code 0; steps and zero points that
+    overflow have no dequantised value but what code * s + z gives."""
+    lib_ready()
+    inf, nan, low = float("inf"), float("nan"), -(1 << (bits - 1))
+    plain = _rows((1, 1, 8, 64), 23, "normal")[0, 0]
+    x = plain.clone()
+    x[0, 3], x[0, 60] = nan, nan
+    plain[0, 3] = plain[0, 60] = plain[0, 4]     # row 0 without its NaNs: a value that is there anyway
+    x[1, 5], x[2, 7] = inf, -inf
+    x[3] = nan
+    x[4], x[5] = 3e38, -3e38                      # max + min overflows: zero point +-inf
+    x[6, 0], x[6, 1] = 3e38, -3e38                # max - min overflows: step inf
+    c, s, z, deq = orc.quantize_rows(plain.float().numpy(), bits)
+    c[0, [3, 60]] = low
+    deq[0, [3, 60]] = orc.round_to_bf16(np.float32(low) * s[0] + z[0])
+    c[1:3], c[3:7] = low, 0
+    deq[1], deq[2], deq[3], deq[4], deq[5], deq[6] = nan, -inf, nan, inf, -inf, nan
+    s[1:7, 0] = inf, inf, nan, 0, 0, inf
+    z[1:7, 0] = inf, -inf, nan, inf, -inf, 0
+    got = binding.quantize_rows(x.repeat(n_rows // 8, 1).view(1, 1, n_rows, 64).cuda(), bits, want_codes=True)
+    for g, ref in zip(got, (deq, c, s[:, 0], z[:, 0])):
+        g = g[0, 0].float().cpu().numpy()
+        assert np.array_equal(g, np.tile(ref, (n_rows // 8,) + (1,) * (ref.ndim - 1)).astype(np.float32), equal_nan=True)
+
+
 @pytest.mark.parametrize("bits", [2, 4, 6])
 def test_quantiser_other_bit_widths(bits):
     lib_ready()
