@@ -44,21 +44,20 @@ __device__ __forceinline__ uint32_t div_by(uint32_t n, const FastDiv& f) {
   return (uint32_t)(((uint64_t)n * f.mul) >> f.shift);
 }
 
-// One tensor of a launch: rows [first_row, first_row + batch * n_heads * n_tokens) of the launch's row space.
+// One tensor of a launch: its rows go to the groups of eight threads from first_group on.
 struct QuantTensor {
   const uint16_t* x;
   uint16_t* dq;  // nullptr: no dequantised output
   int64_t x_sb, x_sh, x_st, d_sb, d_sh, d_st;
   FastDiv n_tokens;
-  long long first_row;
+  uint32_t n_rows, first_group;
 };
 struct QuantArgs {
   QuantTensor t[3];
   int32_t n_tensors;
   FastDiv n_heads;
-  long long n_rows;
   float levels, hi;
-  int8_t* codes;  // outputs of the first tensor only
+  int8_t* codes;  // (one tensor only)
   float* scale;
   float* zero;
 };
@@ -76,45 +75,38 @@ __device__ __forceinline__ float min_nan(float a, float b) {
 __device__ __forceinline__ float lo_bf16(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float hi_bf16(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
 
-// kQuantRowsPerGroup rows per 8-thread group: that many 16-byte loads in flight per thread.  Four for large
-// tensors (bandwidth), one for the few rows of a single step (more threads, shorter latency chain).
-template <int kQuantRowsPerGroup>
+// R rows per 8-thread group: that many 16-byte loads in flight per thread (launch_quant has the rule).  MANY: several tensors,
+// which have no outputs but the dequantised rows (one tensor: its addresses are read from fixed places).
+template <int R, bool MANY>
 __global__ void __launch_bounds__(kQuantThreads, 4) quant_rows_kernel(const __grid_constant__ QuantArgs a) {
   // the rows were written by earlier work of the stream; a launch with programmatic serialisation starts early
   asm volatile("griddepcontrol.launch_dependents;");
-  constexpr int R = kQuantRowsPerGroup;
   constexpr float kMagic = 12582912.f;  // 1.5 * 2^23: a float in [2^23, 2^24) holds an integer in its low mantissa bits
   const int part = threadIdx.x & 7;  // 16-byte column of the row
-  // rows [R * group, R * group + R) per eight threads, no loop: the grid covers the rows (fewer than 2^31,
-  // checked on the host).  Slots past the last row redo the last row and store nothing, so that every lane
-  // joins the shuffles.
+  // R consecutive rows of a tensor per eight threads, no loop: the grid covers the rows (fewer than 2^31, checked on the
+  // host).  Slots past a tensor's last row redo that row and store nothing, so that every lane joins the shuffles.
   const unsigned group = blockIdx.x * (unsigned)(kQuantThreads / 8) + (threadIdx.x >> 3);
-  int ti[R];
+  int ti = 0;
+  if (MANY && group >= a.t[1].first_group) ti = group >= a.t[2].first_group ? 2 : 1;
+  const QuantTensor& tn = a.t[ti];
+  const unsigned first = (group - (MANY ? tn.first_group : 0u)) * R;
   int64_t x_off[R], d_off[R];
   uint4 raw[R];
   {
-    const unsigned row0 = min(group * R, (unsigned)a.n_rows - 1u);
-    int ti0 = 0;
-    if (R == 1) {  // (launches of several tensors take one row per group)
-      if (a.n_tensors > 1 && row0 >= (unsigned)a.t[1].first_row) ti0 = 1;
-      if (a.n_tensors > 2 && row0 >= (unsigned)a.t[2].first_row) ti0 = 2;
-    }
-    const QuantTensor& tn = a.t[ti0];
-    const unsigned local = row0 - (unsigned)tn.first_row;
-    const unsigned bh = div_by(local, tn.n_tokens);
-    unsigned t = local - bh * tn.n_tokens.d;
+    const unsigned row0 = min(first, tn.n_rows - 1u);
+    const unsigned bh = div_by(row0, tn.n_tokens);
+    unsigned t = row0 - bh * tn.n_tokens.d;
     unsigned b = div_by(bh, a.n_heads);
     unsigned h = bh - b * a.n_heads.d;
     const bool one_head = t + R <= tn.n_tokens.d;  // the group's rows are tokens of one head (all of them exist)
 #pragma unroll
     for (int g = 0; g < R; ++g) {
-      ti[g] = ti0;
       if (g > 0 && one_head) {
         x_off[g] = x_off[0] + g * tn.x_st;
         d_off[g] = d_off[0] + g * tn.d_st;
         continue;
       }
-      if (g > 0 && group * R + g < (unsigned)a.n_rows && ++t == tn.n_tokens.d) {
+      if (g > 0 && first + g < tn.n_rows && ++t == tn.n_tokens.d) {
         t = 0;
         if (++h == a.n_heads.d) {
           h = 0;
@@ -127,7 +119,7 @@ __global__ void __launch_bounds__(kQuantThreads, 4) quant_rows_kernel(const __gr
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll
-  for (int g = 0; g < R; ++g) raw[g] = *reinterpret_cast<const uint4*>(a.t[ti[g]].x + x_off[g]);
+  for (int g = 0; g < R; ++g) raw[g] = *reinterpret_cast<const uint4*>(tn.x + x_off[g]);
 
   // the row's maximum and minimum: packed bf16 maxima of x and -x (exact), then (max, -min) as one pair through three
   // shuffles; the eight threads of a row are adjacent lanes
@@ -160,8 +152,8 @@ __global__ void __launch_bounds__(kQuantThreads, 4) quant_rows_kernel(const __gr
     const float r = __fdiv_rn(1.f, s1);
     const float z = __fmul_rn(__fadd_rn(mx, mn), 0.5f);
     const float lo = __fsub_rn(__fadd_rn(__fdiv_rn(__fsub_rn(mn, z), s1), kMagic), kMagic);
-    const unsigned row = group * R + (part & (R - 1));
-    if (part < R && row < (unsigned)a.n_rows && (R > 1 || ti[0] == 0)) {
+    const unsigned row = first + (part & (R - 1));
+    if (!MANY && part < R && row < tn.n_rows) {
       if (a.scale != nullptr) a.scale[row] = s;
       if (a.zero != nullptr) a.zero[row] = z;
     }
@@ -176,8 +168,7 @@ __global__ void __launch_bounds__(kQuantThreads, 4) quant_rows_kernel(const __gr
   }
 #pragma unroll
   for (int g = 0; g < R; ++g) {
-    const QuantTensor& tn = a.t[ti[g]];
-    const bool valid = group * R + g < (unsigned)a.n_rows;
+    const bool valid = first + g < tn.n_rows;
     const uint32_t u[4] = {raw[g].x, raw[g].y, raw[g].z, raw[g].w};
     const float s = s_row[g], r = r_row[g], z = z_row[g];
     const float2 nz2 = make_float2(-z, -z), r2 = make_float2(r, r);
@@ -226,13 +217,13 @@ __global__ void __launch_bounds__(kQuantThreads, 4) quant_rows_kernel(const __gr
     }
     if (valid && tn.dq != nullptr)
       *reinterpret_cast<uint4*>(tn.dq + d_off[g]) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-    if (valid && ti[g] == 0 && a.codes != nullptr) {
+    if (!MANY && valid && a.codes != nullptr) {
       uint32_t w[2];
 #pragma unroll
       for (int i = 0; i < 2; ++i)  // the low bytes of four codes
         w[i] = __byte_perm(__byte_perm(__float_as_uint(t[2 * i].x), __float_as_uint(t[2 * i].y), 0x0040),
                            __byte_perm(__float_as_uint(t[2 * i + 1].x), __float_as_uint(t[2 * i + 1].y), 0x0040), 0x5410);
-      *reinterpret_cast<uint2*>(a.codes + (size_t)(group * R + g) * kHeadDim + part * 8) = make_uint2(w[0], w[1]);
+      *reinterpret_cast<uint2*>(a.codes + (size_t)(first + g) * kHeadDim + part * 8) = make_uint2(w[0], w[1]);
     }
   }
 }
@@ -242,13 +233,21 @@ bool quant_strides_ok(const litevar_strides_t* s) {
          (s->token % 8) == 0;
 }
 
-litevar_status_t launch_quant(QuantArgs& a, int bits, cudaStream_t stream) {
+litevar_status_t launch_quant(QuantArgs& a, long long rows, int bits, cudaStream_t stream) {
   a.levels = (float)((1 << bits) - 1);
   a.hi = (float)((1 << (bits - 1)) - 1);
-  if (a.n_rows >= (1LL << 31)) return LITEVAR_ERR_UNSUPPORTED;  // 2^31 rows of 128 bytes do not fit the device
-  const bool large = a.n_tensors == 1 && a.n_rows >= (1LL << 20);
-  const long long rows_per_block = (kQuantThreads / 8) * (large ? 4 : 1);
-  const long long blocks = (a.n_rows + rows_per_block - 1) / rows_per_block;
+  if (rows >= (1LL << 31)) return LITEVAR_ERR_UNSUPPORTED;  // 2^31 rows of 128 bytes do not fit the device
+  // One row per group: more threads and a shorter chain; four: more loads in flight and the row's divisions shared.  Measured (us,
+  // one / four): one tensor, 2^15 rows 3.97 / 6.09, 2^16 6.30 / 6.51, 2^17 11.0 / 10.3, 2^18 20.6 / 18.4, 2^21 167 / 136; three
+  // tensors, 76 800 rows 7.71 / 7.98, 196 608 16.4 / 15.2, 1.5 million 117 / 98.
+  const bool large = rows >= (3LL << 15);
+  const int per_group = large ? 4 : 1;
+  long long groups = 0;
+  for (int i = 0; i < a.n_tensors; ++i) {
+    a.t[i].first_group = (uint32_t)groups;
+    groups += (a.t[i].n_rows + per_group - 1) / per_group;
+  }
+  const long long blocks = (groups + kQuantThreads / 8 - 1) / (kQuantThreads / 8);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)blocks);
   cfg.blockDim = dim3(kQuantThreads);
@@ -258,8 +257,9 @@ litevar_status_t launch_quant(QuantArgs& a, int bits, cudaStream_t stream) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;  // every thread waits for the previous kernel before its first access
-  const cudaError_t e = large ? cudaLaunchKernelEx(&cfg, quant_rows_kernel<4>, a)
-                              : cudaLaunchKernelEx(&cfg, quant_rows_kernel<1>, a);
+  const bool many = a.n_tensors > 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, large ? (many ? quant_rows_kernel<4, true> : quant_rows_kernel<4, false>)
+                                                       : (many ? quant_rows_kernel<1, true> : quant_rows_kernel<1, false>), a);
   if (e != cudaSuccess) {
     (void)cudaGetLastError();
     return LITEVAR_ERR_CUDA;
@@ -289,12 +289,12 @@ extern "C" litevar_status_t litevar_quantize_rows(const void* x, const litevar_s
   a.t[0].x_sb = sx->batch; a.t[0].x_sh = sx->head; a.t[0].x_st = sx->token;
   if (x_dq) { a.t[0].d_sb = sdq->batch; a.t[0].d_sh = sdq->head; a.t[0].d_st = sdq->token; }
   a.t[0].n_tokens = fast_div((uint32_t)n_tokens);
-  a.t[0].first_row = 0;
   a.n_tensors = 1;
   a.n_heads = fast_div((uint32_t)n_heads);
-  a.n_rows = (long long)batch * n_heads * n_tokens;
+  const long long rows = (long long)batch * n_heads * n_tokens;
+  a.t[0].n_rows = (uint32_t)rows;
   a.codes = codes; a.scale = scale; a.zero = zero;
-  return launch_quant(a, bits, static_cast<cudaStream_t>(stream_));
+  return launch_quant(a, rows, bits, static_cast<cudaStream_t>(stream_));
 }
 
 extern "C" litevar_status_t litevar_quantize_qkv(void* q, const litevar_strides_t* sq, int32_t n_q_tokens, void* k,
@@ -310,7 +310,7 @@ extern "C" litevar_status_t litevar_quantize_qkv(void* q, const litevar_strides_
   void* ptr[3] = {q, k, v};
   const litevar_strides_t* st[3] = {sq, sk, sv};
   const int32_t tokens[3] = {n_q_tokens, n_kv_tokens, n_kv_tokens};
-  long long first = 0;
+  long long rows = 0;
   for (int i = 0; i < 3; ++i) {
     a.t[i].x = static_cast<const uint16_t*>(ptr[i]);
     a.t[i].dq = static_cast<uint16_t*>(ptr[i]);
@@ -318,11 +318,11 @@ extern "C" litevar_status_t litevar_quantize_qkv(void* q, const litevar_strides_
     a.t[i].x_sh = a.t[i].d_sh = st[i]->head;
     a.t[i].x_st = a.t[i].d_st = st[i]->token;
     a.t[i].n_tokens = fast_div((uint32_t)tokens[i]);
-    a.t[i].first_row = first;
-    first += (long long)batch * n_heads * tokens[i];
+    const long long n = (long long)batch * n_heads * tokens[i];
+    a.t[i].n_rows = (uint32_t)n;
+    rows += n;
   }
   a.n_tensors = 3;
   a.n_heads = fast_div((uint32_t)n_heads);
-  a.n_rows = first;
-  return launch_quant(a, bits, static_cast<cudaStream_t>(stream_));
+  return launch_quant(a, rows, bits, static_cast<cudaStream_t>(stream_));
 }

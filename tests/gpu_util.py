@@ -80,3 +80,21 @@ def check_sampled(out, ref, samples, what):
     got = out.double().cpu().numpy() if hasattr(out, "double") else out
     g = np.stack([got[b, h, q] for b, h, q in samples])
     return assert_close(g, ref, what)
+
+
+def captured_grids(calls):
+    """Grid sizes of the kernels that `calls` launches, from a CUDA graph it is captured in (and not run)."""
+    from cuda.bindings import driver as cu
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        calls()
+    raw = cu.CUgraph(init_value=graph.raw_cuda_graph())
+    _, _, n = cu.cuGraphGetNodes(raw, 0)
+    err, nodes, _ = cu.cuGraphGetNodes(raw, n)
+    grids = []
+    for node in nodes[:n]:
+        if cu.cuGraphNodeGetType(node)[1] == cu.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            err, params = cu.cuGraphKernelNodeGetParams(node)
+            assert err == cu.CUresult.CUDA_SUCCESS
+            grids.append(params.gridDimX)
+    return grids

@@ -9,7 +9,7 @@ import torch
 
 from oracle import litevar_oracle as orc
 from paper_2411_17178_b200 import binding, workloads as wl
-from tests.gpu_util import assert_close, errors, lib_ready
+from tests.gpu_util import assert_close, captured_grids, errors, lib_ready
 
 pytestmark = pytest.mark.gpu
 
@@ -45,20 +45,24 @@ def test_quantiser_matches_oracle_bit_for_bit(shape, kind):
 @pytest.mark.parametrize("shape", [(31, 33, 1027, 64), (1, 3, 349526, 64), (7, 30, 4994, 64)])
 @pytest.mark.parametrize("bits", [8, 3])
 def test_quantiser_of_many_rows(shape, bits):
-    """From 2^20 rows on a thread group takes four rows in turn: token counts that are no multiple of four (groups straddle
+    """A thread group takes four rows in turn (from 98304 rows on): token counts that are no multiple of four (groups straddle
     heads and batch rows) and a last group that is not full; a strided view behaves as its copy."""
     lib_ready()
     x = _rows(shape, 17 + bits, "offset").cuda()
     assert x.numel() // 64 >= 1 << 20
     got = binding.quantize_rows(x, bits, want_codes=True)
-    # rows are independent: below 2^20 rows the one-row path, which the tests above pin to the oracle, gives the same bits
+    # rows are independent: the one-row path of fewer rows, which the tests above pin to the oracle, gives the same bits
     flat = x.view(1, 1, -1, 64)
     n = flat.shape[2]
-    for a in range(0, n, 500_000):
-        b = min(n, a + 500_000)
+    for a in range(0, n, 90_000):
+        b = min(n, a + 90_000)
         part = binding.quantize_rows(flat[:, :, a:b].contiguous(), bits, want_codes=True)
         for whole, p, w in zip(got, part, (64, 64, 1, 1)):
             assert torch.equal(whole.reshape(-1, w)[a:b], p.reshape(-1, w))
+    # token-major storage
+    got_t = binding.quantize_rows(x.transpose(1, 2).contiguous().transpose(1, 2), bits, want_codes=True)
+    for whole, strided in zip(got, got_t):
+        assert torch.equal(whole, strided)
     # and the ends of the range against the oracle itself
     for sl in (slice(0, 37), slice(n - 37, n)):
         _check_against_oracle(flat[:, :, sl], bits, tuple(t.reshape(1, 1, n, *t.shape[3:])[:, :, sl] for t in got))
@@ -91,6 +95,25 @@ def test_quantiser_rows_that_are_not_finite(bits, n_rows):
     for g, ref in zip(got, (deq, c, s[:, 0], z[:, 0])):
         g = g[0, 0].float().cpu().numpy()
         assert np.array_equal(g, np.tile(ref, (n_rows // 8,) + (1,) * (ref.ndim - 1)).astype(np.float32), equal_nan=True)
+
+
+@pytest.mark.parametrize("n_q,n_kv", [(18, 29), (577, 601), (1, 1999), (18724, 1)])
+def test_quantise_qkv_takes_four_rows_per_group(n_q, n_kv):
+    """The three tensors of one launch, from 98304 rows on four rows per group and below it one: token counts that are no multiple of
+    four, so that groups straddle heads and a tensor ends within one; the bits of one launch per tensor."""
+    lib_ready()
+    B, H = 5, 7
+    q, k, v = (_rows((B, H, n, 64), 31 + i, "offset").cuda() for i, n in enumerate((n_q, n_kv + 3, n_kv + 3)))
+    want = [binding.quantize_rows(t, 8) for t in (q, k[:, :, 3:], v[:, :, 3:])]
+    head = [t[:, :, :3].clone() for t in (k, v)]
+    per_group = 4 if B * H * (n_q + 2 * n_kv) >= 3 << 15 else 1
+    groups = sum(-(-B * H * n // per_group) for n in (n_q, n_kv, n_kv))
+    assert captured_grids(lambda: binding.quantize_qkv(q, k[:, :, 3:], v[:, :, 3:])) == [-(-groups // 32)]
+    binding.quantize_qkv(q, k[:, :, 3:], v[:, :, 3:])
+    for got, ref in zip((q, k[:, :, 3:], v[:, :, 3:]), want):
+        assert torch.equal(got.view(torch.int16), ref.view(torch.int16))
+    for got, ref in zip((k, v), head):      # the rows in front are not touched
+        assert torch.equal(got[:, :, :3].view(torch.int16), ref.view(torch.int16))
 
 
 @pytest.mark.parametrize("bits", [2, 4, 6])
