@@ -322,8 +322,17 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
     }
   }
   char* scratch = nullptr;
-  if (cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), hist_bytes + (size_t)(groups * map_len) * sizeof(float), pool,
-                              stream) != cudaSuccess) {
+  auto allocate = [&] {
+    return cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), hist_bytes + (size_t)(groups * map_len) * sizeof(float), pool,
+                                   stream);
+  };
+  cudaError_t got = allocate();
+  if (got == cudaErrorMemoryAllocation && groups > 0) {  // no room for the summed maps: straight to the histogram
+    (void)cudaGetLastError();
+    groups = 0;
+    got = allocate();
+  }
+  if (got != cudaSuccess) {
     (void)cudaGetLastError();
     return LITEVAR_ERR_OOM;
   }

@@ -3,6 +3,10 @@
 Most cases use maps that are non-negative multiples of 1/1024: every partial sum is then exact in fp64 in any
 order and the integer decision "smallest radius whose window mass reaches R_0 of the part's mass" must agree
 exactly.  One case uses real softmax rows, where the kernel's fp32 bins round: see the bound there."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -12,6 +16,7 @@ from paper_2411_17178_b200 import binding, workloads as wl
 from tests.gpu_util import lib_ready
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def dyadic_maps(scales, k, n_maps, seed, peaked=False):
@@ -59,6 +64,52 @@ def test_calibration_sums_maps_first(scales, k, n_maps):
     for j in range(4, k + 1):
         for w in range(scales[j - 1]):
             assert ratio[j - 1, w] == pytest.approx(orc.window_ratio(scales, k, j, w, maps), rel=1e-12, abs=1e-15)
+
+
+FAKE_MALLOC = """
+#define _GNU_SOURCE
+#include <dlfcn.h>
+#include <stdio.h>
+#include <stdlib.h>
+int cudaMallocFromPoolAsync(void** p, size_t n, void* pool, void* stream) {
+  static int (*real)(void**, size_t, void*, void*);
+  if (!real) real = (int (*)(void**, size_t, void*, void*))dlsym(dlopen("libcudart.so.12", RTLD_LAZY | RTLD_NOLOAD), "cudaMallocFromPoolAsync");
+  const char* limit = getenv("FAKE_MALLOC_LIMIT");
+  fprintf(stderr, "asked for %zu\\n", n);
+  return limit && n > strtoull(limit, 0, 10) ? 2 /* cudaErrorMemoryAllocation */ : real(p, n, pool, stream);
+}
+"""
+
+
+def test_calibration_without_room_for_summed_maps(tmp_path):
+    """Where the scratch for the summed maps cannot be had, the maps go to the histogram one by one; where that of the histogram
+    cannot either, the call says so.  A stand-in for the allocation call, in a process of its own, refuses what is above a limit."""
+    lib_ready()
+    (tmp_path / "fake.c").write_text(FAKE_MALLOC)
+    fake = str(tmp_path / "fake.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-O1", str(tmp_path / "fake.c"), "-o", fake, "-ldl"], check=True)
+    script = """
+import os, numpy as np, torch
+from paper_2411_17178_b200 import binding
+scales, k = (1, 2, 3, 4, 12), 5
+n, L = 144, 174
+maps = (torch.randint(0, 64, (4, n, L), generator=torch.Generator().manual_seed(3)).float() / 1024).cuda()
+call = lambda: binding.calibrate_windows(scales, k, maps, 0.8, want_ratio=True)
+want = call()
+os.putenv("FAKE_MALLOC_LIMIT", "40000")
+got = call()
+assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+os.putenv("FAKE_MALLOC_LIMIT", "1000")
+try:
+    call()
+except binding.LitevarError as e:
+    print("status", e.status)
+"""
+    res = subprocess.run([sys.executable, "-c", script], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                         env=dict(os.environ, LD_PRELOAD=fake))
+    assert res.returncode == 0 and res.stdout.strip() == "status 5", res.stdout + res.stderr[-3000:]
+    asked = [int(x.split()[-1]) for x in res.stderr.splitlines() if x.startswith("asked for")]
+    assert asked[0] == asked[1] > 100_000 and asked[2] == 32768     # summed, refused, the histogram's alone
 
 
 def test_calibration_many_rows_per_warp():
