@@ -220,8 +220,9 @@ litevar_status_t litevar_attn_forward_static(const int32_t* scales, int32_t n_sc
  *   radius   host out [n_scales]: -1 for parts j <= n_global_scales and for j > step_k, else the radius;
  *            a row of this kind is what litevar_window_t.radius takes
  *   ratio    host out [n_scales][256] or NULL: R_w for w = 0 .. s_j - 1 (1 elsewhere)
- *   stream   the kernel runs there; the call synchronises the stream; its scratch (32 KB, and up to 32 MB
- *            where several maps are added up first) comes from a pool of the library that keeps it between calls
+ *   stream   the kernel runs there; the call synchronises the stream; its scratch (32 KB, and up to 64 MB
+ *            where several maps are added up first, in fp64) comes from a pool of the library that keeps it between
+ *            calls; maps are not added up where that much cannot be had
  * One pass over the maps (the call is bound by reading them once).
  * Errors: INVALID_ARG, OOM, CUDA.
  */

@@ -8,7 +8,7 @@
 // running sum over d then gives the window mass for every w.  The pass is bound by reading the maps once.
 //
 // A warp owns batches of consecutive (map, query) rows and walks them once per part, so that it needs
-// histogram bins for one part at a time: bins[distance][lane] in shared memory (fp32), private to the lane,
+// histogram bins for one part at a time: bins[distance][lane] in shared memory (fp32; fp64 for summed maps), private to the lane,
 // updated with plain loads and stores.  After at most 256 rows the bins are summed over the lanes in fp64 and
 // added to the global histogram with one fp64 add per non-empty bin.
 //   Parts of up to 256 keys: a lane reads flat key positions t = 32 * chunk + lane, so every lane of a load is
@@ -21,10 +21,12 @@
 //
 // The distance of an entry does not depend on the map, so several maps are added up entry by entry first (sum_maps_kernel, a
 // pass at memory speed) and the histogram pass reads one or a few summed maps instead of all of them.  The histogram pass costs
-// about 3.5 times what reading its input costs, so this pays from two maps on; it takes fp32 sums of at most
-// kMaxSumMaps maps and a scratch buffer of at most kScratchBytes (a single 2K map, 2.2 GB, goes to the histogram directly).
-// Measured on B200: 64 maps of the last 512px step (587 MB; sums 94 us, histogram 20 us): the call 338 -> 147 us; 1280 maps of the
-// last 256px step (891 MB): 391 -> 222 us.
+// about 3.5 times what reading its input costs, so this pays from two maps on.  The sums and their histogram are fp64: rounded to
+// fp32, a sum over all maps weighs in every entry, where the maps' own histograms average their roundings (error of R_w with fp32
+// sums 1.0e-9 to 2.2e-9 rms, 0.8e-10 to 4.0e-10 map by map).  Scratch of at most kScratchBytes (a single 2K map, 2.2 GB, goes to
+// the histogram directly, and so do all maps where the scratch cannot be had).
+// Measured on B200 (whole calls, us, maps one by one / summed): 64 maps of the last 512px step (587 MB) 338 / 161; 1280 maps of the
+// last 256px step (891 MB) 391 / 225; with fp32 sums and bins 158 and 218.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -42,19 +44,18 @@ constexpr int kMaxDist = kMaxScale;   // distances 0 .. s_j - 1
 constexpr int kCalibFlushRows = 256;  // rows a lane's fp32 bins take in before they are flushed
 constexpr int kCalibMaxRows = 1 << 30;  // (map, query) rows of one launch
 constexpr int kSumThreads = 256, kSumPerThread = 4, kSumUnroll = 4;
-constexpr int kMaxSumMaps = 256;               // maps added up in fp32
-constexpr size_t kScratchBytes = 32u << 20;    // summed maps of one call, at most
+constexpr size_t kScratchBytes = 64u << 20;    // summed maps of one call, at most
 
 // out[g][i] = sum of maps m in [g * per_group, (g + 1) * per_group) of maps[m][i].  A thread owns kSumPerThread entries, a block's
 // width apart (coalesced whatever the alignment of a map), and has kSumPerThread * kSumUnroll loads in flight.  Clears the
 // histogram on the way, and lets the histogram pass be launched while the last blocks run (it waits for them).
 __global__ void __launch_bounds__(kSumThreads) sum_maps_kernel(const float* __restrict__ maps, int64_t n, int64_t n_maps,
-                                                               int64_t per_group, float* __restrict__ out, double* hist) {
+                                                               int64_t per_group, double* __restrict__ out, double* hist) {
   if (blockIdx.y == 0)
     for (int i = blockIdx.x * kSumThreads + threadIdx.x; i < kMaxScales * kMaxDist; i += gridDim.x * kSumThreads) hist[i] = 0.0;
   const int64_t first = (int64_t)blockIdx.x * (kSumThreads * kSumPerThread) + threadIdx.x;
   const int64_t m0 = blockIdx.y * per_group, m1 = min(n_maps, m0 + per_group);
-  float acc[kSumPerThread] = {};
+  double acc[kSumPerThread] = {};
   const float* src = maps + m0 * n + first;
   if (first + (kSumPerThread - 1) * kSumThreads < n) {
     int64_t m = m0;
@@ -121,33 +122,32 @@ struct ScratchPools {
 };
 
 // Wide part (more than 256 keys) of one query row: NC 32-column chunks per key row, 16 loads in flight per round.
-template <int NC>
-__device__ __forceinline__ void calib_wide_row(float* bins, int lane, const float* __restrict__ part, int s_j, int cr,
-                                               int cc) {
+template <int NC, typename T>
+__device__ __forceinline__ void calib_wide_row(T* bins, int lane, const T* __restrict__ part, int s_j, int cr, int cc) {
   constexpr int KR = 16 / NC;
   int dc[NC];
-  float outer[NC];
+  T outer[NC];
   bool cv[NC];
 #pragma unroll
   for (int u = 0; u < NC; ++u) {
     const int kc = lane + 32 * u;
     cv[u] = kc < s_j;
     dc[u] = abs(kc - cc);
-    outer[u] = 0.f;
+    outer[u] = 0;
   }
   for (int kr0 = 0; kr0 < s_j; kr0 += KR) {
-    float a[KR][NC];
+    T a[KR][NC];
 #pragma unroll
     for (int v = 0; v < KR; ++v)
 #pragma unroll
       for (int u = 0; u < NC; ++u)
-        a[v][u] = (cv[u] && kr0 + v < s_j) ? __ldg(part + (kr0 + v) * s_j + lane + 32 * u) : 0.f;
+        a[v][u] = (cv[u] && kr0 + v < s_j) ? __ldg(part + (kr0 + v) * s_j + lane + 32 * u) : T(0);
 #pragma unroll
     for (int v = 0; v < KR; ++v) {
       const int kr = kr0 + v;
       if (kr < s_j) {
         const int dr = abs(kr - cr);
-        float inner = 0.f;
+        T inner = 0;
 #pragma unroll
         for (int u = 0; u < NC; ++u) {
           if (dc[u] < dr) inner += a[v][u]; else outer[u] += a[v][u];
@@ -161,19 +161,22 @@ __device__ __forceinline__ void calib_wide_row(float* bins, int lane, const floa
     if (cv[u]) bins[(dc[u] << 5) + lane] += outer[u];
 }
 
-__global__ void __launch_bounds__(kCalibWarps * 32, 32 / kCalibWarps)
-calib_hist_kernel(Schedule sc, int k0, int first_part, int s_max, const float* __restrict__ maps, int n_rows_total,
+// T: float for maps (fp32 bins, at most kCalibFlushRows rows each), double for summed maps (nothing is rounded to fp32 again).
+template <typename T>
+__global__ void __launch_bounds__(kCalibWarps * 32, sizeof(T) == 4 ? 32 / kCalibWarps : 16 / kCalibWarps)
+calib_hist_kernel(Schedule sc, int k0, int first_part, int s_max, const T* __restrict__ maps, int n_rows_total,
                   int q_first /* query index of row 0 */, int rows_per_batch,
                   double* __restrict__ hist /* [kMaxScales][kMaxDist] */) {
-  extern __shared__ float sh[];  // [kCalibWarps][s_max][32]
+  extern __shared__ __align__(8) uint8_t sh[];  // T [warps][s_max][32]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* bins = sh + (size_t)warp * s_max * 32;
+  const int n_block_warps = blockDim.x >> 5;
+  T* bins = reinterpret_cast<T*>(sh) + (size_t)warp * s_max * 32;
   const int s_k = sc.scale[k0];
   const int n_k = s_k * s_k;
   const int L_k = sc.off[k0 + 1];
   const int n_batches = (n_rows_total + rows_per_batch - 1) / rows_per_batch;
-  const int warp_global = blockIdx.x * kCalibWarps + warp;
-  const int n_warps = gridDim.x * kCalibWarps;
+  const int warp_global = blockIdx.x * n_block_warps + warp;
+  const int n_warps = gridDim.x * n_block_warps;
   const int flush_every = max(1, kCalibFlushRows / rows_per_batch);
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the summed maps and the cleared histogram
 
@@ -185,7 +188,7 @@ calib_hist_kernel(Schedule sc, int k0, int first_part, int s_max, const float* _
     const int r_t0 = lane / s_j, c_t0 = lane - r_t0 * s_j;
     const int off_j = sc.off[j];
     double* hist_j = hist + (size_t)j * kMaxDist;
-    for (int d = 0; d < s_j; ++d) bins[(d << 5) + lane] = 0.f;
+    for (int d = 0; d < s_j; ++d) bins[(d << 5) + lane] = 0;
     int pending = 0;
     for (int batch = warp_global; batch < n_batches; batch += n_warps) {
       const int row0 = batch * rows_per_batch;
@@ -197,7 +200,7 @@ calib_hist_kernel(Schedule sc, int k0, int first_part, int s_max, const float* _
         const int r = (int)q / s_k, c = (int)q - r * s_k;
         pk = (((2 * r + 1) * s_j) / (2 * s_k)) | ((((2 * c + 1) * s_j) / (2 * s_k)) << 16);
       }
-      const float* src = maps + (size_t)row0 * L_k + off_j;
+      const T* src = maps + (size_t)row0 * L_k + off_j;
       if (n_chunks <= 8) {
         for (int i0 = 0; i0 < nb; i0 += 8) {
           int cr[8], cc[8];
@@ -208,13 +211,13 @@ calib_hist_kernel(Schedule sc, int k0, int first_part, int s_max, const float* _
             cc[u] = p >> 16;
           }
           const int ng = nb - i0;
-          const float* grp = src + (size_t)i0 * L_k + lane;
+          const T* grp = src + (size_t)i0 * L_k + lane;
           int r_t = r_t0, c_t = c_t0;
           for (int ch = 0; ch < n_chunks; ++ch) {
             const bool tv = (ch << 5) + lane < n_j;
-            float a[8];
+            T a[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) a[u] = (tv && u < ng) ? __ldg(grp + (size_t)u * L_k + (ch << 5)) : 0.f;
+            for (int u = 0; u < 8; ++u) a[u] = (tv && u < ng) ? __ldg(grp + (size_t)u * L_k + (ch << 5)) : T(0);
             if (tv) {
               // rows past the end of the batch carry zeros into a valid bin
 #pragma unroll
@@ -234,7 +237,7 @@ calib_hist_kernel(Schedule sc, int k0, int first_part, int s_max, const float* _
         for (int i = 0; i < nb; ++i) {
           const int p = __shfl_sync(0xffffffffu, pk, i);
           const int cr = p & 0xffff, cc = p >> 16;
-          const float* part = src + (size_t)i * L_k;
+          const T* part = src + (size_t)i * L_k;
           switch (nc) {
             case 1: calib_wide_row<1>(bins, lane, part, s_j, cr, cc); break;
             case 2: calib_wide_row<2>(bins, lane, part, s_j, cr, cc); break;
@@ -258,7 +261,7 @@ calib_hist_kernel(Schedule sc, int k0, int first_part, int s_max, const float* _
           }
         }
         __syncwarp();
-        for (int d = 0; d < s_j; ++d) bins[(d << 5) + lane] = 0.f;
+        for (int d = 0; d < s_j; ++d) bins[(d << 5) + lane] = 0;
       }
     }
     __syncwarp();
@@ -307,14 +310,13 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
     return LITEVAR_ERR_CUDA;
   }
   (void)cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-  // groups of maps that are added up: as many as fill the chip with threads, no more maps in one than kMaxSumMaps
+  // groups of maps that are added up: as many as fill the chip with threads
   long long groups = 0, per_group = 0;
-  if (n_maps > 1 && map_len <= (long long)(kScratchBytes / sizeof(float))) {
+  if (n_maps > 1 && map_len <= (long long)(kScratchBytes / sizeof(double))) {
     const long long threads = (map_len + kSumPerThread - 1) / kSumPerThread;
     groups = (2048ll * n_sm + threads - 1) / threads;
-    if (groups < (n_maps + kMaxSumMaps - 1) / kMaxSumMaps) groups = (n_maps + kMaxSumMaps - 1) / kMaxSumMaps;
     if (groups > (n_maps + 3) / 4) groups = (n_maps + 3) / 4;
-    const long long room = (long long)(kScratchBytes / sizeof(float)) / map_len;
+    const long long room = (long long)(kScratchBytes / sizeof(double)) / map_len;
     if (groups > room || groups > 65535) groups = 0;  // too much for the scratch: straight to the histogram
     if (groups > 0) {
       per_group = (n_maps + groups - 1) / groups;
@@ -323,7 +325,7 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
   }
   char* scratch = nullptr;
   auto allocate = [&] {
-    return cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), hist_bytes + (size_t)(groups * map_len) * sizeof(float), pool,
+    return cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), hist_bytes + (size_t)(groups * map_len) * sizeof(double), pool,
                                    stream);
   };
   cudaError_t got = allocate();
@@ -339,26 +341,29 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
   double* d_hist = reinterpret_cast<double*>(scratch);
   litevar_status_t st = LITEVAR_OK;
   std::vector<double> hist((size_t)kMaxScales * kMaxDist);
+  double* summed = nullptr;
   if (groups > 0) {
-    float* summed = reinterpret_cast<float*>(scratch + hist_bytes);
+    summed = reinterpret_cast<double*>(scratch + hist_bytes);
     const long long per_block = kSumThreads * kSumPerThread;
     sum_maps_kernel<<<dim3((unsigned)((map_len + per_block - 1) / per_block), (unsigned)groups), kSumThreads, 0, stream>>>(
         maps, map_len, n_maps, per_group, summed, d_hist);
     if (cudaGetLastError() != cudaSuccess) st = LITEVAR_ERR_CUDA;
-    maps = summed;
     n_maps = groups;
   }
   const long long rows = (long long)n_maps * n_k;
   int s_max = 1;
   for (int j = first_part; j <= k0; ++j) s_max = scales[j] > s_max ? scales[j] : s_max;
-  const size_t smem = sizeof(float) * 32 * (size_t)s_max * kCalibWarps;
-  // resident warps: up to 32 per SM, fewer where the bins of the widest part need the shared memory
+  const size_t warp_smem = (groups > 0 ? sizeof(double) : sizeof(float)) * 32 * (size_t)s_max;
+  const int block_warps = warp_smem * kCalibWarps > (200u << 10) ? kCalibWarps / 2 : kCalibWarps;  // (fp64 bins, 200 distances and more)
+  const size_t smem = warp_smem * block_warps;
+  // resident warps: up to 32 per SM (16 with fp64 bins), fewer where the bins of the widest part need the shared memory
   int blocks_per_sm = (int)((200u << 10) / (smem + 1024));
-  if (blocks_per_sm > 32 / kCalibWarps) blocks_per_sm = 32 / kCalibWarps;
+  if (blocks_per_sm > (groups > 0 ? 16 : 32) / kCalibWarps) blocks_per_sm = (groups > 0 ? 16 : 32) / kCalibWarps;
   if (blocks_per_sm < 1) blocks_per_sm = 1;
-  const long long n_warps = (long long)n_sm * blocks_per_sm * kCalibWarps;
+  const long long n_warps = (long long)n_sm * blocks_per_sm * block_warps;
   if (st != LITEVAR_OK || (groups == 0 && cudaMemsetAsync(d_hist, 0, hist_bytes, stream) != cudaSuccess) ||
-      cudaFuncSetAttribute(calib_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      (groups > 0 ? cudaFuncSetAttribute(calib_hist_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                  : cudaFuncSetAttribute(calib_hist_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
     st = LITEVAR_ERR_CUDA;
   for (long long first = 0; first < rows && st == LITEVAR_OK; first += kCalibMaxRows) {
     const int n_rows = (int)(rows - first < kCalibMaxRows ? rows - first : kCalibMaxRows);
@@ -375,12 +380,12 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
       }
     }
     const long long n_batches = ((long long)n_rows + rows_per_batch - 1) / rows_per_batch;
-    long long blocks = (n_batches + kCalibWarps - 1) / kCalibWarps;
+    long long blocks = (n_batches + block_warps - 1) / block_warps;
     if (blocks > (long long)n_sm * blocks_per_sm) blocks = (long long)n_sm * blocks_per_sm;
     const unsigned parts = (unsigned)(k0 + 1 - first_part);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks, n_batches <= 2 * n_warps ? parts : 1u);
-    cfg.blockDim = dim3(kCalibWarps * 32);
+    cfg.blockDim = dim3((unsigned)block_warps * 32);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
@@ -388,8 +393,13 @@ extern "C" litevar_status_t litevar_calibrate_windows(const int32_t* scales, int
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = groups > 0 && first == 0 ? 1 : 0;  // behind sum_maps_kernel
-    if (cudaLaunchKernelEx(&cfg, calib_hist_kernel, sc, k0, first_part, s_max, maps + first * L_k, n_rows, (int)(first % n_k),
-                           rows_per_batch, d_hist) != cudaSuccess)
+    const int q_first = (int)(first % n_k);
+    const cudaError_t e =
+        groups > 0 ? cudaLaunchKernelEx(&cfg, calib_hist_kernel<double>, sc, k0, first_part, s_max,
+                                        static_cast<const double*>(summed + first * L_k), n_rows, q_first, rows_per_batch, d_hist)
+                   : cudaLaunchKernelEx(&cfg, calib_hist_kernel<float>, sc, k0, first_part, s_max, maps + first * L_k, n_rows,
+                                        q_first, rows_per_batch, d_hist);
+    if (e != cudaSuccess)
       st = LITEVAR_ERR_CUDA;
   }
   if (st == LITEVAR_OK && (cudaMemcpyAsync(hist.data(), d_hist, sizeof(double) * kMaxDist * (size_t)step_k, cudaMemcpyDeviceToHost, stream) != cudaSuccess ||

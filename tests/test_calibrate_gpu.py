@@ -66,6 +66,22 @@ def test_calibration_sums_maps_first(scales, k, n_maps):
             assert ratio[j - 1, w] == pytest.approx(orc.window_ratio(scales, k, j, w, maps), rel=1e-12, abs=1e-15)
 
 
+@pytest.mark.parametrize("n_maps", [2, 7, 300])
+@pytest.mark.parametrize("scales,k", [((1, 2, 3, 4, 6, 9), 6), ((1, 2, 3, 20, 24), 5), ((1, 2, 3, 225, 4), 5)])
+def test_calibration_of_softmax_maps_is_summed_in_fp64(scales, k, n_maps):
+    """Values that are no short binary fractions: sums over maps and over the windows are fp64 (2^-53 of an addend at most, fewer
+    than 2^24 addends of one sign), small and wide parts, and a part too wide for four warps' bins in shared memory."""
+    lib_ready()
+    n, L = orc.map_shape(scales, k)
+    maps = torch.softmax(2 * torch.randn(n_maps, n, L, generator=torch.Generator().manual_seed(k + n_maps)), -1)
+    rad, ratio = binding.calibrate_windows(scales, k, maps.cuda(), 0.9, want_ratio=True)
+    total = maps.double().sum(0, keepdim=True).numpy()
+    assert rad.tolist() == orc.calibrate_radius(scales, k, total, 0.9).tolist()
+    for j in range(4, k + 1):
+        for w in sorted({0, 1, 2, scales[j - 1] // 3, scales[j - 1] - 1} & set(range(scales[j - 1]))):
+            assert ratio[j - 1, w] == pytest.approx(orc.window_ratio(scales, k, j, w, total), rel=2.0 ** -29, abs=0.0)
+
+
 FAKE_MALLOC = """
 #define _GNU_SOURCE
 #include <dlfcn.h>
