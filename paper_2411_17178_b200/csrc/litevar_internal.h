@@ -95,6 +95,7 @@ struct Step {
   int32_t first_patch = 0;    // key scales with 0-based index >= first_patch are tiled in patches (== step count: none)
   int32_t raster_len = 0;     // cache rows [0, raster_len) are covered by raster key tiles
   int32_t n_raster_tiles = 0;
+  int32_t chunks_per_tile = 0;  // average live chunks per query tile over the heads, whichever window sets they use
   litevar::TileGeom* d_q_geom = nullptr;    // [n_q_tiles]
   litevar::TileGeom* d_key_geom = nullptr;  // [n_key_tiles]
   std::vector<litevar::TileGeom> q_geom, key_geom;  // host copies

@@ -785,6 +785,10 @@ litevar_status_t build_plan(litevar_plan* plan, const int32_t* scales, int32_t n
         ss.small.pr[1] = t.first_pairs[1];
       }
     }
+    long long chunks = 0;
+    for (int h = 0; h < n_heads; ++h) chunks += st.sets[plan->head_to_set.empty() ? 0 : plan->head_to_set[h]].n_chunks;
+    const long long tiles = (long long)st.n_q_tiles * n_heads;
+    st.chunks_per_tile = (int32_t)((chunks + tiles - 1) / tiles);
   }
   return LITEVAR_OK;
 }
@@ -891,7 +895,7 @@ static void fill_step_params(const litevar_plan_t* plan, const Step& st, int32_t
   p.sm_scale = plan->sm_scale;
   p.status = plan->d_status;
   p.overlap_launch = 1;
-  p.chunks_per_tile = (st.sets[0].n_chunks + st.n_q_tiles - 1) / st.n_q_tiles;
+  p.chunks_per_tile = st.chunks_per_tile;
   p.units_per_group = units_per_l2_group(st.L_k, p.n_heads * p.batch_computed);
 }
 

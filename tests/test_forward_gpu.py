@@ -9,7 +9,7 @@ import torch
 
 from oracle import litevar_oracle as orc
 from paper_2411_17178_b200 import binding, workloads as wl
-from tests.gpu_util import MAX_ABS, REL_L2, assert_close, check_sampled, errors, lib_ready, run_forward, stratified_samples
+from tests.gpu_util import MAX_ABS, REL_L2, assert_close, captured_grids, check_sampled, errors, lib_ready, run_forward, stratified_samples
 
 pytestmark = pytest.mark.gpu
 
@@ -656,4 +656,23 @@ def test_values_of_any_magnitude(build, tiling, logits, magnitude):
     for b in {0, 2 * B - 1}:
         ref = orc.attention_step(scales, K, row, Q[b:b + 1], Kc[b:b + 1], Vc[b:b + 1])
         assert_close(got[b:b + 1] / magnitude, ref / magnitude, f"batch row {b}")
+    plan.close()
+
+
+@pytest.mark.parametrize("wide_heads", [7, 1])
+@pytest.mark.parametrize("wide_set", [0, 1])
+def test_build_follows_the_lists_of_all_heads(wide_set, wide_heads):
+    """Whether CTAs take several tiles depends on the average list over the heads, not on the order of the window sets: 48 x 48
+    patch tiles with long lists (everything live, 71 chunks and more) and short ones (window 1/8)."""
+    lib_ready()
+    scales, K, H, B = (1, 2, 3, 4, 6, 9, 13, 18, 24, 32, 48), 11, 8, 12
+    wide, narrow = orc.full_table(scales), orc.window_table(scales, rho=(1, 8))
+    tabs = [wide, narrow] if wide_set == 0 else [narrow, wide]
+    plan = binding.Plan(scales, n_heads=H, radius=np.stack(tabs), n_sets=2,
+                        head_to_set=[wide_set if h < wide_heads else 1 - wide_set for h in range(H)])
+    q = torch.zeros(2 * B, H, 48 * 48, 64, dtype=torch.bfloat16, device="cuda")
+    kv = torch.zeros(2 * B, H, sum(s * s for s in scales), 64, dtype=torch.bfloat16, device="cuda")
+    tiles = 6 * 3 * H * 2 * B
+    ctas = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert captured_grids(lambda: plan.forward(K, B, q, kv, kv, q)) == [tiles if wide_heads == 7 else ctas]
     plan.close()
