@@ -134,6 +134,12 @@ def _stream_ptr(stream) -> Optional[int]:
     return getattr(stream, "cuda_stream", stream)
 
 
+def _stream_int(stream) -> int:
+    """The stream as a number, from what a ctypes void* argument takes: a torch stream, a number, a c_void_p, ..."""
+    stream = getattr(stream, "cuda_stream", stream)
+    return stream if type(stream) is int else ctypes.cast(stream, ctypes.c_void_p).value or 0
+
+
 def _host_module():
     """The native Python entry (built beside the library; there is no other path)."""
     global _host
@@ -220,7 +226,7 @@ class Plan:
         """litevar_attn_forward on torch CUDA tensors (bf16, [2B, H, tokens, 64]); the marshalling is native (it is most of
         an eager call's host time)."""
         st = self._forward(self._forward_addr, self._plan_addr, step_k, batch_pairs, q, k_cache, v_cache, out,
-                           stream if stream is None else getattr(stream, "cuda_stream", stream), self._current_stream)
+                           stream if stream is None else _stream_int(stream), self._current_stream)
         if st != 0:
             _check(st, "litevar_attn_forward")
 

@@ -109,6 +109,18 @@ def test_native_forward_entry_marshals_tensors():
     assert seen[-1] == (2 ** 40, 7, 8, *want, 1234)
     assert host.forward(addr, 0, 1, 1, *t, None, lambda device: 100 + device) == 5
     assert seen[-1] == (None, 1, 1, *want, 103)
+    # a stream in every form that a ctypes void* argument takes; a null stream is not "no stream"
+    plan = object.__new__(binding.Plan)
+    plan._h = None
+    plan._forward, plan._forward_addr, plan._plan_addr, plan._current_stream = host.forward, addr, 1, lambda device: 77
+
+    class TorchStream:
+        cuda_stream = 4321
+
+    for stream, value in ((None, 77), (0, None), (55, 55), (ctypes.c_void_p(56), 56), (ctypes.c_void_p(0), None), (TorchStream(), 4321)):
+        with pytest.raises(binding.LitevarError):   # the stand-in's status is 5
+            plan.forward(7, 8, *t, stream=stream)
+        assert seen.pop()[-1] == value
     for bad in ((1, 64, 64, 2), (1, 64, 1)):
         with pytest.raises(ValueError):
             host.forward(addr, 1, 1, 1, *t[:3], Fake(16, bad), 1, None)
