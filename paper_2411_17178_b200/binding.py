@@ -147,7 +147,7 @@ def _host_module():
         try:
             from . import _litevar_host
         except ImportError as e:
-            raise RuntimeError("_litevar_host.so not found or not loadable: build it with "
+            raise RuntimeError("_litevar_host not found or not loadable in this interpreter: build it with "
                                "`python -m paper_2411_17178_b200.build` (needs a C compiler and the Python headers)") from e
         _host = _litevar_host
     return _host

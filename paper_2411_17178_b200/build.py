@@ -1,4 +1,4 @@
-"""Builds liblitevar.so (the C-ABI library, nvcc, sm_100a) and _litevar_host.so (its Python entry, C compiler) in-tree.
+"""Builds liblitevar.so (the C-ABI library, nvcc, sm_100a) and _litevar_host.*.so (its Python entry, C compiler) in-tree.
 
     python -m paper_2411_17178_b200.build [--force] [--verbose]
 """
@@ -13,7 +13,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblitevar.so")
-HOST_LIB = os.path.join(HERE, "_litevar_host.so")
+HOST_LIB = os.path.join(HERE, "_litevar_host" + sysconfig.get_config_var("EXT_SUFFIX"))  # of this interpreter
 HOST_SOURCE = os.path.join(CSRC, "litevar_host.c")
 SOURCES = ["litevar_plan.cu", "litevar_fwd_simt.cu", "litevar_maps.cu", "litevar_fwd_ws.cu", "litevar_fwd_small.cu", "litevar_static.cu", "litevar_calib.cu", "litevar_quant.cu"]
 HEADERS = [os.path.join(CSRC, "litevar_internal.h"), os.path.join(CSRC, "litevar_tc_ptx.h"), os.path.join(ROOT, "include", "litevar.h")]

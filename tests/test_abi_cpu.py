@@ -3,6 +3,8 @@ and argument validation that happens before any device work returns the document
 import ctypes
 import os
 import re
+import sys
+import sysconfig
 
 import pytest
 
@@ -73,6 +75,13 @@ def test_null_plan_calls(lib):
     assert lib.litevar_plan_step_kernel(None, 1, 1, None) == 1
     assert lib.litevar_plan_stats(None, 1, 0, None, None, None, None) == 1
     lib.litevar_plan_destroy(None)
+
+
+def test_native_entry_is_this_interpreters():
+    """The native entry carries the interpreter's tag: another Python version does not take it for its own and builds one."""
+    suffix = sysconfig.get_config_var("EXT_SUFFIX")
+    assert os.path.basename(build.build_host()) == "_litevar_host" + suffix and sys.implementation.cache_tag in suffix
+    assert os.path.samefile(binding._host_module().__file__, build.HOST_LIB)
 
 
 def test_native_forward_entry_marshals_tensors():
