@@ -13,7 +13,8 @@ from tests.gpu_util import MAX_ABS, REL_L2, assert_close, captured_grids, check_
 
 pytestmark = pytest.mark.gpu
 
-# AUTO is what callers get: the small-step kernel where a step fits it, one of the two tcgen05 kernels elsewhere
+# AUTO is what callers get: the small-step kernel where a step fits it, the tcgen05 kernel elsewhere (TCGEN05 and TCGEN05_WS name
+# its short and its long lists)
 KERNELS = [binding.KERNEL_SIMT, binding.KERNEL_TCGEN05, binding.KERNEL_TCGEN05_WS, binding.KERNEL_AUTO]
 KNAME = {binding.KERNEL_SIMT: "simt", binding.KERNEL_TCGEN05: "tcgen05", binding.KERNEL_TCGEN05_WS: "tcgen05-row",
          binding.KERNEL_AUTO: "auto"}
@@ -96,7 +97,7 @@ def test_config4_final_steps_sampled(tiling):
         smp = stratified_samples(plan, k, 2 * B, w.n_heads, w.scales[k - 1], 20 if tiling == binding.TILING_AUTO else 8, rng)
         total += len(smp)
         ref = orc.attention_sampled(w.scales, k, tab[k - 1], Q, Kc, Vc, smp, share_cfg=True)
-        # the default tiling with the kernel AUTO picks and with both tcgen05 kernels; patch tiles with both
+        # the default tiling with the kernel AUTO picks and with the tcgen05 kernel; patch tiles with the latter
         for kernel in ((binding.KERNEL_AUTO,) if tiling == binding.TILING_AUTO else ()) + TC_KERNELS:
             got, out = run_forward(plan, k, B, Q, Kc, Vc, kernel)
             check_sampled(got, ref, smp, f"config 4 step {k} {KNAME[kernel]}")
@@ -124,7 +125,7 @@ def test_config5_sampled(rho, tiling):
     smp = stratified_samples(plan, 14, 2, w.n_heads, 128, 128 if tiling == binding.TILING_AUTO else 8, rng)
     assert tiling != binding.TILING_AUTO or len(smp) >= 4096
     ref = orc.attention_sampled(w.scales, 14, tab[13], Q, Kc, Vc, smp)
-    # what AUTO launches for the 2K step (the kernel with a softmax thread per query row), then the other kernel
+    # what AUTO reports for the 2K step (long lists), then the kernel named by its other constant
     assert plan.step_kernel(14, 1) == binding.KERNEL_TCGEN05_WS
     for kernel in (binding.KERNEL_AUTO, binding.KERNEL_TCGEN05):
         got, _ = run_forward(plan, 14, 1, Q, Kc, Vc, kernel)
@@ -359,16 +360,15 @@ def test_bench_launch_configuration_sampled(cfg, steps, per_unit):
 
 
 def _expected_tc(plan, k):
-    """The tcgen05 kernel AUTO picks for a step that is not a small one: the kernel with a softmax thread per
-    query row from eight live key tiles per query tile on."""
+    """What AUTO reports for a step that is not a small one: long lists from eight live key tiles per query tile on."""
     nq, _, npairs = plan.tile_counts(k)
     return binding.KERNEL_TCGEN05_WS if -(-npairs // nq) >= 8 else binding.KERNEL_TCGEN05
 
 
 def test_step_kernel_selection():
     """AUTO runs the small-step kernel on steps with one query tile, at most two raster key tiles and little
-    work, whatever the batch; a tcgen05 kernel elsewhere (the row kernel on long tile lists); forcing a kernel or
-    patch tiles overrides it."""
+    work, whatever the batch; the tcgen05 kernel elsewhere (with a constant of its own on long tile lists); forcing a
+    kernel or patch tiles overrides it."""
     lib_ready()
     S, T, R, M = binding.KERNEL_SIMT, binding.KERNEL_TCGEN05, binding.KERNEL_TCGEN05_WS, binding.KERNEL_SMALL
     plan = binding.Plan(wl.SCALES_256, n_heads=2)
@@ -430,8 +430,8 @@ def test_small_step_kernel_shape_extremes(scales, n_global, share):
 @pytest.mark.parametrize("kind", ["late-huge", "rising", "all-low"])
 @pytest.mark.parametrize("tiling", TILINGS, ids=lambda t: TNAME[t])
 def test_row_reference_moves_and_redo(kind, tiling):
-    """The tcgen05 kernel's reference of a row moves by a chunk's sum, and the list is redone when a score is out of
-    its range: scores that rise from chunk to chunk by less than 2^60, a late key far above everything before it, and rows
+    """The tcgen05 kernel's reference of a row is taken from its first keys and stays, and the list is redone where the row's sum
+    leaves the range: scores that rise from chunk to chunk by up to 2^50, a late key far above everything before it, and rows
     whose first live key comes late with every score far below 0."""
     lib_ready()
     scales, H, B = (1, 2, 3, 4, 6, 9, 13), 2, 1
@@ -481,27 +481,38 @@ def test_chunk_lists_off_the_tile_grid(scales, radius, tiling, shape):
     plan.close()
 
 
-@pytest.mark.parametrize("case", ["raster", "one-chunk-tiles", "sets", "rising"])
-def test_many_tiles_per_cta(case):
-    """Enough query tiles that the tensor-core kernel's CTAs take several in turn (from 2.5 per resident CTA on): ragged tails,
-    tiles with a single chunk (one stream idle), per-head lists, sharing, and the second pass over all of a CTA's tiles."""
+@pytest.mark.parametrize("case", ["shared", "one-chunk-tiles", "sets", "second-pass"])
+@pytest.mark.parametrize("tiling", TILINGS, ids=lambda t: TNAME[t])
+def test_many_tiles_per_cta(case, tiling):
+    """Enough query tiles that the tensor-core kernel's CTAs take several in turn (from 2.5 per resident CTA on, three or four each
+    here): ragged tails, tiles with a single chunk (one stream idle), per-head lists, sharing, and the second pass over all of a
+    CTA's tiles."""
     lib_ready()
     scales = (12,) if case == "one-chunk-tiles" else (1, 2, 3, 4, 6, 9, 13)
-    B, H, K = 80 if case == "raster" else 40, 7, len(scales)  # raster: half the rows are computed
-    share = [int(case == "raster")] * K
+    B, H, K = 80 if case == "shared" else 40, 7, len(scales)  # shared: half the rows are computed
+    share = [int(case == "shared")] * K
     tabs, head_set = [orc.window_table(scales, n_global_scales=3)], [0] * H
-    if case == "one-chunk-tiles":  # 144 queries, three key rows each: lists of three chunks and of one
+    if case == "one-chunk-tiles":  # 144 queries, three key rows each: lists of three chunks and of one (raster)
         tabs[0][0, 0] = 1
     elif case == "sets":
         tabs, head_set = [orc.window_table(scales, rho=r, n_global_scales=3) for r in ((1, 8), (1, 2))], [i % 2 for i in range(H)]
     w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=96)
     Q = wl.make_q(w, 0, K)
     Kc, Vc = wl.make_kv(w, 0)
-    if case == "rising":
-        Kc = (Kc.float() * torch.linspace(0.2, 9, Kc.shape[2]).view(1, 1, -1, 1)).bfloat16()
-    plan = binding.Plan(scales, n_heads=H, radius=np.stack(tabs), n_sets=len(tabs), share_steps=share,
+    if case == "second-pass":
+        # cache rows 0 to 7, the first keys of every tile's first chunk in either tiling, have logits near -80; all others, among
+        # them rows 8 to 13 of the same chunk, which every query sees, near +10: more than 2^96 apart for every row
+        Q = (1 + 0.02 * Q.float()).bfloat16()
+        Kc = (10 / 8 + 0.1 * Kc.float()).bfloat16()
+        Kc[:, :, :8] = -80 / 8
+        s = (Q[0].double() @ Kc[0].double().transpose(-1, -2)) / (8 * np.log(2))
+        assert float((s[:, :, 8:14].amax(-1) - s[:, :, :8].amax(-1)).min()) > 97
+    plan = binding.Plan(scales, n_heads=H, radius=np.stack(tabs), n_sets=len(tabs), share_steps=share, tiling=tiling,
                         head_to_set=head_set if len(tabs) > 1 else None)
-    got, _ = run_forward(plan, K, B, Q, Kc, Vc, binding.KERNEL_TCGEN05)
+    got, out = run_forward(plan, K, B, Q, Kc, Vc, binding.KERNEL_TCGEN05)
+    q, k, v = Q.cuda(), Kc.cuda(), Vc.cuda()
+    ctas = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert captured_grids(lambda: plan.forward(K, B, q, k, v, out)) == [ctas]
     for s, t in enumerate(tabs):
         heads = [h for h in range(H) if head_set[h] == s]
         ref = orc.attention_step(scales, K, t[K - 1], Q[:, heads], Kc[:, heads], Vc[:, heads], share_cfg=bool(share[K - 1]))
