@@ -175,7 +175,7 @@ litevar_status_t litevar_attn_forward_kv8(const litevar_plan_t* plan, int32_t st
  * litevar_attn_plan keeps its tile lists in memory it gets from cudaMalloc.  A caller that may not
  * allocate (it runs inside a fixed device-memory budget, it is a plug-in that must stay away from its
  * host's allocator, or it is reached at a point where allocation is forbidden) uses this call instead:
- * it builds the tile plan of step_k on the device inside a fixed 4.4 MB array that is part of the
+ * it builds the tile plan of step_k on the device inside a fixed 4.3 MB array that is part of the
  * library image, then runs the same tensor-core forward kernel on it.  It calls no cudaMalloc, no
  * cudaFree and no allocating library routine; it launches three kernels on `stream` and returns
  * without synchronising.

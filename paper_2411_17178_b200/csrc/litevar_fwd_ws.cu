@@ -6,8 +6,8 @@
 // own scores, probabilities, accumulator and reference, and the two results meet at the end.  320 threads:
 //   warps 0-3, 4-7  softmax of stream 0 and 1: thread m of the group owns query slot m (TMEM lane m).  A chunk's 64 scores
 //                   come from TMEM in two halves of 32 through one rolled copy of the code: the plan's element mask, the
-//                   probabilities (about a quarter of the exponentials on the FMA pipe by a cubic, the rest on the exponential
-//                   pipe), their sum, and P (packed bf16) over the scores that have been read.
+//                   probabilities (19 to 31 % of the exponentials, by build, on the FMA pipe by a cubic, the rest on the
+//                   exponential pipe), their sum, and P (packed bf16) over the scores that have been read.
 //   warps 8, 9      the stream's copies (K and V chunks by tensor-map copies into rings of two stages) and MMAs: once P(i) is
 //                   complete, O += P(i) V(i) and S(i + 1) = Q K(i + 1) go out back to back; they execute in issue order, so
 //                   that S may overwrite P.  The warp runs converged and what it computes is uniform, so that descriptors
@@ -24,15 +24,16 @@
 // and stays (0 where none of them is live): bf16 and fp32 have the same exponent range, so P and its sum are as accurate at 2^90 as
 // at 1, and a tile's rows need neither a maximum per chunk nor a rescaled accumulator.  At the end a row whose sum or output is
 // out of range (kRange, kSmall) sends the CTA through its lists again, with every chunk's maximum taken first (`exact`), for the 32
-// rows of a warp that it belongs to, which are stored then.  (A reference that followed the chunk sums by powers of two from 2^10 on, tested at every chunk: 2 to 3 % slower, 512px step 10 155.6 us
-// against 151.)
+// rows of a warp that it belongs to, which are stored then.  The look at the output and the agreement of the two warps of a row on
+// it take 1 % of the 2K step and 2 % of a launch with one tile per CTA (0.2 us).  (A reference that followed the chunk sums by powers
+// of two from 2^10 on, tested at every chunk: 2 to 3 % slower, 512px step 10 155.6 us against 151.)
 //
-// What bounds it (ncu, 2K step, full mask / window 1/4): issue slots 72 / 69 % busy, exponential pipe 61 / 51 %, tensor pipe active
+// What bounds it (ncu, 2K step, full mask / window 1/4): issue slots some 70 % busy, exponential pipe 60 / 50 %, tensor pipe active
 // 44 / 41 %; 6.5 instructions a score.  The rest is the hand-off from P to the next S (arrive, issue of eight MMAs, their
 // execution, commit, wake: 700 cycles a chunk), which the four streams of an SM cover for one another.
 // Measured on B200, with what the kernel with one softmax thread per row and 128-key tiles took before: 2K step with the full
-// mask 5.05 ms (6.71), window 1/4 1.45 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 151 / 68 / 31 us (261 / 116 / 47),
-// 256px step 10 with 960 units 74 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
+// mask 4.94 ms (6.71), window 1/4 1.48 ms (2.65), 512px steps 10 / 9 / 8 with 288 units 151 / 69 / 30 us (261 / 116 / 47),
+// 256px step 10 with 960 units 75 us (117 on the kernel with two threads per row, which this one also replaces).  Steps on
 // the way: copy look-ups off the MMA lane -4 %, 64-key streams with uniform issue code -12 %, no maxima -12 %; three stages instead of two: +1 %; chunks from
 // a tile's live box on and classes per half and warp (on the fixed grid, one live flag per chunk and warp: 1.69 ms) -7 %.
 //

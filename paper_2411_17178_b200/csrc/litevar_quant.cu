@@ -7,14 +7,13 @@
 // take the IEEE division.
 //
 // In a generation the rows of a step are quantised once, when they are appended to the K/V cache (and Q as it
-// is produced); the attention kernels then read the dequantised bf16 rows unchanged.  The pass is bound by
-// reading and writing each row once: eight threads share a row (16 bytes each) and take up to four rows at a
-// time (four loads in flight), the row's maximum and minimum come from three shuffles, every thread codes and
+// is produced); the attention kernels then read the dequantised bf16 rows unchanged.  A row is read
+// and written once: eight threads share it (16 bytes each) and take up to four rows at a time (four loads in flight), the row's maximum and minimum come from three shuffles, every thread codes and
 // rebuilds its own eight values.  It may run in place.
 //
-// Bound by instruction issue (ncu: 76 % of the slots, 4.6 TB/s).  A [64, 30, 680, 64] cache with codes (428 MB moved): 135 us
-// before, 92 us now: maxima on packed bf16 pairs and three shuffles a row instead of six, the row's divisions shared among the
-// threads of a row, index divisions by multiplication, and the code of a row's minimum (a tie by construction, which sent
+// Bound by instruction issue (ncu, a [64, 30, 680, 64] cache without codes: 77 % of the slots).  That cache with codes (428 MB
+// moved) takes 92 us, 4.6 TB/s; it took 135 before: maxima on packed bf16 pairs and three shuffles a row instead of six, the row's
+// divisions shared among the threads of a row, index divisions by multiplication, and the code of a row's minimum (a tie by construction, which sent
 // every warp through the IEEE divisions of the slow path) decided once per row.
 //
 // The integer decision is taken in fp32 with one IEEE operation at a time (no contraction into fused
@@ -44,7 +43,7 @@ __device__ __forceinline__ uint32_t div_by(uint32_t n, const FastDiv& f) {
   return (uint32_t)(((uint64_t)n * f.mul) >> f.shift);
 }
 
-// One tensor of a launch: its rows go to the groups of eight threads from first_group on.
+// One tensor of a launch; its rows go to the groups of eight threads from first_group on.
 struct QuantTensor {
   const uint16_t* x;
   uint16_t* dq;  // nullptr: no dequantised output
