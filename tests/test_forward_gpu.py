@@ -670,6 +670,44 @@ def test_values_of_any_magnitude(build, tiling, logits, magnitude):
     plan.close()
 
 
+@pytest.mark.parametrize("scales", [(8,), (1, 2, 3, 4, 5, 6, 8, 10, 13), (1, 2, 3, 4, 6, 9, 13, 18, 24)], ids=["one-chunk", "raster", "long"])
+@pytest.mark.parametrize("build,tiling", BUILDS, ids=lambda x: TNAME.get(x, x))
+def test_values_of_one_give_rows_of_one(build, tiling, scales):
+    """The row sums are the same products as the output's (P times a block of ones behind V): with V = 1 everywhere a row is 1 to the
+    bit, whatever the scores, in lists of one chunk to 16 (every stage of the V ring), ragged ends and partly dead chunks."""
+    lib_ready()
+    K, n, L = len(scales), scales[-1] ** 2, sum(s * s for s in scales)
+    H, B = (8, -(-740 // (16 * -(-n // 128)))) if build == "many-tiles" else (3, 1)
+    w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=89)
+    Q, Kc = wl.make_q(w, 0, K).cuda(), wl.make_kv(w, 0)[0].cuda()
+    one = torch.ones_like(Kc)
+    plan = binding.Plan(scales, n_heads=H, rho=(1, 8), tiling=tiling)
+    plan.set_kernel(binding.KERNEL_TCGEN05)
+    out = torch.full_like(Q, float("nan"))
+    if build == "8-bit":
+        (K8, *kq), (V8, *vq) = (binding.quantize_rows(t, want_codes=True) for t in (Kc, one))
+        plan.forward_kv8(K, B, Q, *kq, *vq, out)
+    else:
+        plan.forward(K, B, Q, Kc, one, out)
+    assert plan.poll() == 0
+    assert bool((out == 1).all())
+    plan.close()
+
+
+@pytest.mark.parametrize("pairs,many", [(32, True), (1, False)])
+def test_short_raster_lists_share_ctas(pairs, many):
+    """256px step 10 (10 chunks a tile) with enough tiles, and with too few; 512px step 10 (22) takes a CTA per tile at any size."""
+    lib_ready()
+    ctas = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    for scales, short in ((wl.SCALES_256, True), (wl.SCALES_512, False)):
+        H, n, L = 15, scales[-1] ** 2, sum(s * s for s in scales)
+        q = torch.zeros(2 * pairs, H, n, 64, dtype=torch.bfloat16, device="cuda")
+        kv = torch.zeros(2 * pairs, H, L, 64, dtype=torch.bfloat16, device="cuda")
+        plan = binding.Plan(scales, n_heads=H)
+        assert captured_grids(lambda: plan.forward(10, pairs, q, kv, kv, q)) == [ctas if many and short else n // 128 * H * 2 * pairs]
+        plan.close()
+
+
 @pytest.mark.parametrize("wide_heads", [7, 1])
 @pytest.mark.parametrize("wide_set", [0, 1])
 def test_build_follows_the_lists_of_all_heads(wide_set, wide_heads):
