@@ -254,6 +254,10 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
     x.mask = sd.chunk_mask;
     return x;
   };
+  // Loop bounds that come from memory, marked as the same in all lanes: the issuing warps' counters and descriptors stay in uniform
+  // registers (thousand cycles without / with it: several tiles per CTA, 256px steps 8 / 9 / 10 with 960 units 50.4 / 50.1, 100.7 /
+  // 99.6, 134.0 / 131.0; 8-bit cache, last 512px step 417.5 / 414.5).  In the other build they do anyway, and the loop got slower.
+  auto uniform = [](int v) { return MANY || KV8 ? __shfl_sync(0xffffffffu, v, 0) : v; };
   const int w_step = MANY ? (int)gridDim.x : n_items;
   const int n_tiles = MANY ? (n_items - (int)blockIdx.x + w_step - 1) / w_step : 1;  // of this CTA
   volatile int* abort_flag = &sm.abort_flag;
@@ -319,7 +323,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
   // with a P V product.
   int base = 0, tiles = 0, o_tiles = 0;
   for (;;) {
-    const int sweeps = exact ? 2 : 1, n_lists = n_tiles * sweeps;
+    const int sweeps = uniform(exact ? 2 : 1), n_lists = n_tiles * sweeps;
     if (warp == 9) {
       // ---------------------------------------------------------------- copies of K and V.  The whole warp runs this code (what it
       // computes is uniform); one elected lane issues.  S(g) complete frees the stage of K(g) and, in issue order, that of
@@ -494,7 +498,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         const int x = exact ? list >> 1 : list, i_q = tiles + x;
         const bool maxima = exact && !(list & 1);
         int n_next = n;
-        if (MANY && !maxima && x + 1 < n_tiles) n_next = item_at((int)blockIdx.x + (x + 1) * w_step).n;
+        if (MANY && !maxima && x + 1 < n_tiles) n_next = uniform(item_at((int)blockIdx.x + (x + 1) * w_step).n);
         const int end = base + n;
         if (ok) ok = mbar_wait_long(&sm.q_full[i_q % kQBufs], (uint32_t)((i_q / kQBufs) & 1), abort_flag, p.status);
         // Q to TMEM (32 packed columns): a score product that reads both operands from shared memory waits for the 6 KB of a step.
@@ -818,7 +822,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
     __syncwarp();
     __syncthreads();
     tc_fence_after();
-    if (exact || !*(volatile int*)&sm.redo || *abort_flag) break;
+    if (uniform(exact || !*(volatile int*)&sm.redo || *abort_flag)) break;
     exact = true;
   }
 
