@@ -14,7 +14,7 @@
 //                   issues.
 //   warp 9          K and V chunks by tensor-map copies into rings of four stages.
 // The row sums are 16 more columns of O: the products take 16 columns of V from a block of ones behind the stages (the leading byte
-// offset of V's descriptor).  A sum by additions is one instruction a score (64 of the 346 that a warp issues per chunk now, all
+// offset of V's descriptor).  A sum by additions is one instruction a score (64, beside the 360 that a warp issues per chunk now, all
 // included).  Q is a TMEM operand: a step of S = Q K with both operands in shared memory waits for their 6 KB (50 cycles, 32 with Q in
 // TMEM), and the two CTAs of an SM share that.
 // MANY: a CTA takes several tiles in turn.  Q has two buffers; K and V copies of the next tile go out behind the last ones of this
@@ -32,7 +32,7 @@
 // whose sum or output is out of range (kRange, kSmall) sends the CTA through its lists again (`exact`), each list twice: once for
 // the rows' maxima, then against them, for the 32 rows of a warp that it belongs to, which are stored then.
 //
-// What bounds it (ncu, 2K step, full mask): issue slots 72 % busy, exponential pipe 64 %, tensor pipe active 56 %; 5.4 instructions a
+// What bounds it (ncu, 2K step, full mask): issue slots 72 % busy, exponential pipe 64 %, tensor pipe active 56 %; 5.6 instructions a
 // score.  (More warps do not help: three streams of softmax warps, or three score buffers so that none waits for its next scores,
 // took as long as before with the sums still added by instructions.)  Measured on B200, in thousand cycles of a launch, with one accumulator and
 // sums of its own per stream / shared accumulator and sums by products / and Q in TMEM / and six pairs of a half's 16 on the FMA pipe:
