@@ -25,10 +25,14 @@
 // Two CTAs per SM, so that every scheduler has four softmax warps of four streams that are in different phases.
 // TMEM columns: S and P of stream s at 64 s, O at 128, the row sums at 192, Q at 208.
 //
-// The reference of a row (probabilities are 2^(score * scale - reference)) is the maximum of the first chunk's first eight keys
+// The reference of a row (probabilities are 2^(score * scale - reference)) is the maximum of the first chunk's first 32 keys
 // and stays (0 where none of them is live): bf16 and fp32 have the same exponent range, so P and its sum are as accurate at 2^90 as
-// at 1, and a tile's rows need neither a maximum per chunk nor a rescaled accumulator.  The stream with the first chunk hands it to
-// the other one (which is then a little behind: both streams at the same point of a chunk are 4 to 5 % slower).  At the end a row
+// at 1, and a tile's rows need neither a maximum per chunk nor a rescaled accumulator.  The key it is taken from has a probability of
+// 1, without rounding, and the larger its weight the more that is worth: error against fp64 (relative L2, N(0, 1) inputs; with the
+// maximum of eight keys / of 32 / with two accumulators and a maximum of eight keys for each) 256px step 8 2.306e-3 / 2.282e-3 /
+// 2.293e-3, 256px step 10 2.291 / 2.273 / 2.281, 512px step 10 2.324 / 2.316 / 2.322.  The stream with the first chunk hands the
+// reference to the other one (which is then a little behind: both streams at the same point of a chunk are 4 to 5 % slower), in front
+// of the loop over the chunks: as a case inside it, a loop of 22 chunks took 1 % longer even with eight keys.  At the end a row
 // whose sum or output is out of range (kRange, kSmall) sends the CTA through its lists again (`exact`), each list twice: once for
 // the rows' maxima, then against them, for the 32 rows of a warp that it belongs to, which are stored then.
 //
@@ -61,6 +65,7 @@ constexpr int kSumCols = 16;              // of the accumulator, behind O: P tim
 constexpr int kThreads = 320;             // two streams of four softmax warps, one warp for the MMAs, one for the copies
 constexpr uint32_t kTmemCols = 256, kColO = 128, kColQ = kColO + kHeadDim + kSumCols;  // S (and P over it) of stream s at 64 s, then O and the row sums, then Q
 
+constexpr int kRefKeys = 32;      // of a tile's first chunk, whose maximum is a row's reference
 constexpr unsigned kIdleNs = 200;  // (50 or 500: the same)
 constexpr int kMaxTiles = 1024;  // of a CTA that takes several (MANY)
 // A row sum of the first pass outside (2^-64, 2^96) goes to the second pass.  (The lower end keeps the traces of dead keys, 2^-125
@@ -609,6 +614,11 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       int qt = item0.qt, h = item0.h, b = item0.b;
       float msc = 0.f;      // probabilities are 2^(score * sc - msc)
       float top = 0.f;      // second pass: the row's maximum
+      // S(i) complete; in issue order this also means that PV(i - 2) is complete
+      auto wait_scores = [&](int i) {
+        if (ok) ok = mbar_wait_long(&sm.s_full[st], (uint32_t)((i >> 1) & 1), abort_flag, p.status);
+        if (ok) tc_fence_after();
+      };
       for (int list = 0; list < n_lists; ++list) {
         const int x = exact ? list >> 1 : list;
         const bool maxima = exact && !(list & 1);
@@ -624,30 +634,40 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           box_live = r0 < p.s_k && c0 < p.s_k;
           row_live = r0 + (lane >> 3) < p.s_k && c0 + (lane & 7) < p.s_k;
         }
-        for (; g < end; g += 2) {
-          // S(g) complete; in issue order this also means that PV(g - 2) is complete
-          if (ok) ok = mbar_wait_long(&sm.s_full[st], (uint32_t)((g >> 1) & 1), abort_flag, p.status);
-          if (ok) tc_fence_after();
-          if (!exact && g - base < 2) {  // this stream's first chunk of the tile (the warps meet here whether a wait ran out or not)
-            if (g == base) {             // the tile's first: the rows' references
-              float mx = -INFINITY;
-              if (ok && cls) {
-                uint32_t r[8];
-                tmem_ld8(tS, r);
-                tmem_wait_ld();
+        if (g < end) wait_scores(g);
+        if (!exact && g < end) {  // (the warps meet here whether a wait ran out or not)
+          if (g == base) {        // the tile's first chunk: the rows' references
+            float mx = -INFINITY;
+            if (ok && (cls & 3)) {
+              uint32_t r[kRefKeys];
+              tmem_ld32(tS, r);
+              tmem_wait_ld();
+              if (cls & 1) {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) mx = fmaxf(mx, (mk.x >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
+                for (int e = 0; e < kRefKeys; ++e)
+                  if (!((mk.x >> e) & 1u)) r[e] = 0xff800000u;
               }
-              msc = mx != -INFINITY ? mx * sc : 0.f;
-              if (n > 1) {
-                sm.ref[m] = msc;
-                asm volatile("bar.arrive %0, 64;" ::"r"(12 + lane_group) : "memory");
-              }
-            } else {
-              asm volatile("bar.sync %0, 64;" ::"r"(12 + lane_group) : "memory");
-              msc = sm.ref[m];
+              float top4[4];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) top4[i] = fmaxf(__uint_as_float(r[i]), __uint_as_float(r[4 + i]));
+#pragma unroll
+              for (int e = 8; e < kRefKeys; e += 8)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                  asm("max.f32 %0, %0, %1, %2;" : "+f"(top4[i]) : "f"(__uint_as_float(r[e + i])), "f"(__uint_as_float(r[e + 4 + i])));
+              mx = fmaxf(fmaxf(top4[0], top4[1]), fmaxf(top4[2], top4[3]));
             }
+            msc = mx != -INFINITY ? mx * sc : 0.f;
+            if (n > 1) {
+              sm.ref[m] = msc;
+              asm volatile("bar.arrive %0, 64;" ::"r"(12 + lane_group) : "memory");
+            }
+          } else {
+            asm volatile("bar.sync %0, 64;" ::"r"(12 + lane_group) : "memory");
+            msc = sm.ref[m];
           }
+        }
+        for (; g < end; g += 2) {
           if (ok) {
             if (maxima && cls) {
 #pragma unroll 1
@@ -712,6 +732,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           cls = cls_next;
           mk = mk_next;
           mk_next = look_up(g + 4 - base, cls_next);
+          if (g + 2 < end) wait_scores(g + 2);
         }
         if (MANY && idle && x > 0 && maxima == exact) stored();
         const int n_here = n, h_here = h, b_here = b;

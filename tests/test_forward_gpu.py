@@ -430,7 +430,7 @@ def test_small_step_kernel_shape_extremes(scales, n_global, share):
 @pytest.mark.parametrize("kind", ["late-huge", "rising", "all-low"])
 @pytest.mark.parametrize("tiling", TILINGS, ids=lambda t: TNAME[t])
 def test_row_reference_moves_and_redo(kind, tiling):
-    """The tcgen05 kernel's reference of a row is taken from its first keys and stays, and the list is redone where the row's sum
+    """The tcgen05 kernel's reference of a row is taken from its first 32 keys and stays, and the list is redone where the row's sum
     leaves the range: scores that rise from chunk to chunk by up to 2^50, a late key far above everything before it, and rows
     whose first live key comes late with every score far below 0."""
     lib_ready()
@@ -500,13 +500,13 @@ def test_many_tiles_per_cta(case, tiling):
     Q = wl.make_q(w, 0, K)
     Kc, Vc = wl.make_kv(w, 0)
     if case == "second-pass":
-        # cache rows 0 to 7, the first keys of every tile's first chunk in either tiling, have logits near -80; all others, among
-        # them rows 8 to 13 of the same chunk, which every query sees, near +10: more than 2^96 apart for every row
+        # cache rows 0 to 31, the first keys of every tile's first chunk in either tiling, have logits near -80, all others near
+        # +10: more than 2^96 apart for every row
         Q = (1 + 0.02 * Q.float()).bfloat16()
         Kc = (10 / 8 + 0.1 * Kc.float()).bfloat16()
-        Kc[:, :, :8] = -80 / 8
+        Kc[:, :, :32] = -80 / 8
         s = (Q[0].double() @ Kc[0].double().transpose(-1, -2)) / (8 * np.log(2))
-        assert float((s[:, :, 8:14].amax(-1) - s[:, :, :8].amax(-1)).min()) > 97
+        assert float((s[:, :, 32:].amin(-1) - s[:, :, :32].amax(-1)).min()) > 97
     plan = binding.Plan(scales, n_heads=H, radius=np.stack(tabs), n_sets=len(tabs), share_steps=share, tiling=tiling,
                         head_to_set=head_set if len(tabs) > 1 else None)
     got, out = run_forward(plan, K, B, Q, Kc, Vc, binding.KERNEL_TCGEN05)
@@ -643,14 +643,14 @@ def test_non_finite_scores(build, tiling, value):
 @pytest.mark.parametrize("logits,magnitude", [((-30.0, 30.0), 1e30), ((-30.0, 30.0), 1e12), ((-40.0, -40.0), 1e-30), ((-43.0, -43.0), 1e-14)])
 @pytest.mark.parametrize("build,tiling", BUILDS, ids=lambda x: TNAME.get(x, x))
 def test_values_of_any_magnitude(build, tiling, logits, magnitude):
-    """Row sums near the ends of the first pass's range (logits of the first eight cache rows and of the others) times values
+    """Row sums near the ends of the first pass's range (logits of the first 32 cache rows and of the others) times values
     that are large or small: the products of P and V leave the fp32 range where P and its sum do not."""
     lib_ready()
     scales, K = (1, 2, 3, 4, 6, 9, 13), 7
     H, B = (8, 32) if build == "many-tiles" else (2, 1)
     L = sum(s * s for s in scales)
     lg = torch.full((L,), logits[1])
-    lg[:8] = logits[0]
+    lg[:32] = logits[0]
     w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=97)
     Q = torch.ones(2 * B, H, 169, 64).bfloat16()
     Kc = (lg / 8).view(1, 1, L, 1).expand(2 * B, H, L, 64).bfloat16()       # q . k / 8 = logit
@@ -691,6 +691,34 @@ def test_values_of_one_give_rows_of_one(build, tiling, scales):
         plan.forward(K, B, Q, Kc, one, out)
     assert plan.poll() == 0
     assert bool((out == 1).all())
+    plan.close()
+
+
+@pytest.mark.parametrize("step,pairs", [(8, 16), (10, 16), (10, 1)], ids=["four-chunks", "ten-chunks", "one-tile-per-cta"])
+def test_rounding_error_of_short_lists(step, pairs):
+    """P is rounded to bf16 against the row's reference, whose own key is exact.  The error against fp64 is no larger than that of two
+    separate halves of the list (every other 64-key chunk), each against the maximum of its first eight keys."""
+    lib_ready()
+    H, n, L = 16, wl.SCALES_256[step - 1] ** 2, sum(s * s for s in wl.SCALES_256[:step])
+    plan = binding.Plan(wl.SCALES_256, n_heads=H, radius=orc.full_table(wl.SCALES_256))
+    plan.set_kernel(binding.KERNEL_TCGEN05)
+    stream = torch.arange(L, device="cuda") // 64 % 2
+    error = torch.zeros(2, dtype=torch.float64, device="cuda")
+    gen = torch.Generator(device="cuda")
+    for seed in range(16 // pairs):
+        gen.manual_seed(seed)
+        q, k, v = (torch.randn((2 * pairs, H, t, 64), device="cuda", generator=gen).bfloat16() for t in (n, L, L))
+        out = torch.empty_like(q)
+        plan.forward(step, pairs, q, k, v, out)
+        s = q.double() @ k.double().mT * (0.125 / np.log(2))
+        v = v.double()
+        ref = torch.softmax(s * np.log(2), -1) @ v
+        top = torch.stack([s[..., :8].amax(-1), s[..., 64:72].amax(-1)], -1)[..., stream]
+        p = torch.exp2(s - top).bfloat16().double() * torch.exp2(top)
+        halves = ((p @ v) / p.sum(-1, keepdim=True)).bfloat16()
+        error += torch.stack([(x.double() - ref).square().sum() for x in (out, halves)])
+    assert plan.poll() == 0
+    assert error[0] <= error[1], (error / ref.square().sum() / (16 // pairs)).sqrt().tolist()
     plan.close()
 
 
