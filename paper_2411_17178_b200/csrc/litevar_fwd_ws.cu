@@ -13,9 +13,12 @@
 //                   that descriptors stay in uniform registers (a lane of its own: eight register moves per MMA); one elected lane
 //                   issues.
 //   warp 9          K and V chunks by tensor-map copies into rings of four stages.
-// The row sums are 16 more columns of O: the products take 16 columns of V from a block of ones behind the stages (the leading byte
-// offset of V's descriptor).  A sum by additions is one instruction a score (64, beside the 360 that a warp issues per chunk now, all
-// included).  Q is a TMEM operand: a step of S = Q K with both operands in shared memory waits for their 6 KB (50 cycles, 32 with Q in
+// The row sums are 16 more columns of O: the products take 16 columns of V from a block behind the stages (the leading byte offset of
+// V's descriptor) that is 1 where key and column agree modulo 4, and a sum is four of them added up.  (A product shifts its addends
+// to the largest exponent and cuts them off there: with ones everywhere 16 addends a step lose up to a bit of the sum each, always
+// in the same direction.  Over the 34240 keys of the last 2K step, keys three times as sharp, outputs were too large by 1.0e-4; with
+// four addends a step by 1.5e-5, with one too small by 1.9e-5, with sums by additions too small by 1.5e-5.  Time: the same.)  A sum
+// by additions is one instruction a score (64, beside the 360 that a warp issues per chunk now, all included).  Q is a TMEM operand: a step of S = Q K with both operands in shared memory waits for their 6 KB (50 cycles, 32 with Q in
 // TMEM), and the two CTAs of an SM share that.
 // MANY: a CTA takes several tiles in turn.  Q has two buffers; K and V copies of the next tile go out behind the last ones of this
 // one, the softmax warps look the next list up while they wait for their accumulator, and the
@@ -61,7 +64,7 @@ namespace {
 constexpr int kChunkKeys = kBlockN / 2;
 constexpr uint32_t kChunkBytes = kChunkKeys * kHeadDim * 2;
 constexpr int kStages = 4;                // K ring and V ring; chunk g of the CTA is in stage g % kStages
-constexpr int kSumCols = 16;              // of the accumulator, behind O: P times a block of ones
+constexpr int kSumCols = 16;              // of the accumulator, behind O: row sums over the keys that agree with the column modulo 4
 constexpr int kThreads = 320;             // two streams of four softmax warps, one warp for the MMAs, one for the copies
 constexpr uint32_t kTmemCols = 256, kColO = 128, kColQ = kColO + kHeadDim + kSumCols;  // S (and P over it) of stream s at 64 s, then O and the row sums, then Q
 
@@ -94,7 +97,7 @@ struct WsShared : CodeStage<KV8> {
   alignas(1024) uint8_t q[MANY ? 2 : 1][kTileBytes];  // Q; at the end of a tile the output rows pass through it
   alignas(1024) uint8_t k[kStages][kChunkBytes];
   alignas(1024) uint8_t v[kStages][kChunkBytes];
-  alignas(1024) uint8_t ones[16 * kHeadDim * 2];  // bf16 ones: 16 keys, the part of V that gives the row sums
+  alignas(1024) uint8_t ones[16 * kHeadDim * 2];  // 16 keys of the part of V that gives the row sums
   float ref[kBlockM];     // the rows' references, from the stream with the tile's first chunk to the other
   float top[2][kBlockM];  // second pass: the rows' maxima over the keys of each stream
   alignas(8) uint64_t q_full[2], q_free;
@@ -184,9 +187,12 @@ __device__ __forceinline__ bool mbar_wait_idle(uint64_t* bar, uint32_t parity, v
   } while (!mbar_try(bar, parity));
   return true;
 }
-// one fp32 column of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t& r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
+// four fp32 columns of this thread's TMEM lane
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr)
+               : "memory");
 }
 // Where a chunk's 64 rows are (`map`: 0 raster, else 1 + the patch-tiled key scale's map).
 struct ChunkAt {
@@ -299,7 +305,9 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
   if (threadIdx.x < 4 * (sizeof(sm.held[0]) / sizeof(uint32_t))) (&sm.held[0][0])[threadIdx.x] = 0u;
   if (threadIdx.x < 8) (&sm.out_of_range[0][0])[threadIdx.x] = 0;
   if (threadIdx.x < sizeof(sm.ones) / 16) {
-    reinterpret_cast<uint4*>(sm.ones)[threadIdx.x] = make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
+    // key threadIdx.x / 8: bf16 ones in every fourth column (all 16-byte pieces of a row are the same, wherever the swizzle puts them)
+    const uint32_t one = threadIdx.x & 8 ? 0x3f800000u : 0x3f80u, low = threadIdx.x & 16 ? 0u : one, high = threadIdx.x & 16 ? one : 0u;
+    reinterpret_cast<uint4*>(sm.ones)[threadIdx.x] = make_uint4(low, high, low, high);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the tensor pipe reads them
   }
   // the next kernel of the stream may start its set-up while this grid drains; this grid's set-up ran while the
@@ -468,7 +476,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       // stay in uniform registers); one elected lane issues.  P(g) complete is the event to wait for: O += P(g) V(g) and S(g + 2)
       // go out back to back (they execute in issue order, so that S may overwrite P).
       const uint64_t q_desc0 = make_desc(smem_u32(sm.q[0])), k_desc0 = make_desc(smem_u32(sm.k[0]));
-      // V: 64 columns in the stage, the 16 behind them (leading byte offset) in the block of ones
+      // V: 64 columns in the stage, the 16 behind them (leading byte offset) in the block of sm.ones
       const uint32_t ones_at = (smem_u32(sm.ones) - smem_u32(sm.v[0])) >> 4;
       const uint64_t v_desc0 = (make_desc(smem_u32(sm.v[0])) & ~(0x3fffull << 16)) | ((uint64_t)ones_at << 16);
       int nq = 0;  // Q copies issued in this pass
@@ -524,7 +532,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           if (ok) {
             tc_fence_after();
             if (g >= base && !maxima) {
-              // 16 keys per step = 16 rows of 128 B = 2048 B of V (the block of ones stays) and 8 packed columns of P
+              // 16 keys per step = 16 rows of 128 B = 2048 B of V (the block for the sums stays) and 8 packed columns of P
               mma_ts_x4_one<8, (2048 >> 4) - ((2048 >> 4) << 16)>(tO, tS + 64 * (g & 1), v_desc0 + (uint64_t)((kChunkBytes >> 4) * s) - ((uint64_t)((kChunkBytes >> 4) * s) << 16),
                                                                   kIdescO, g > base ? 1u : 0u);
               if (g + 1 == end) mma_commit_one(&sm.o_full);
@@ -766,13 +774,13 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         uint8_t* slice = sm.q[tiles % kQBufs] + (warp << 11);
         if (ok) {
           tc_fence_after();
-          // Row sum: P times ones, as the P V product sees P (rounded to bf16): numerator and denominator of a row agree, and a row
+          // Row sum: over P as the P V product sees it (rounded to bf16), so that numerator and denominator of a row agree, and a row
           // with one dominant key reproduces that key's V exactly.
-          uint32_t r[32], r_sum;
-          tmem_ld1(tlane + kColO + kHeadDim, r_sum);
+          uint32_t r[32], sums[4];
+          tmem_ld4(tlane + kColO + kHeadDim, sums);
           tmem_ld32(tlane + kColO + 32 * st, r);
           tmem_wait_ld();
-          float l = __uint_as_float(r_sum);
+          float l = (__uint_as_float(sums[0]) + __uint_as_float(sums[1])) + (__uint_as_float(sums[2]) + __uint_as_float(sums[3]));
           if (__builtin_expect(!exact && row_live && !(l < kRange && l > kRangeLow), 0)) {  // (a NaN goes this way too)
             bad = true;
             sm.out_of_range[lane_group][x & 1] = x + 1;
