@@ -47,7 +47,7 @@
 // (with one tile per CTA 281) / 271 / 267; last 256px step with 128 units 31.0 / 28.5 / 28.1 / 27.9.
 //
 // Every wait on an mbarrier is bounded; when one runs out the CTA raises the plan's status word, drains its copies, frees its
-// TMEM and returns (the softmax warps still arrive for every chunk, so that the named barriers complete).  The element mask, the
+// TMEM and returns (the softmax warps still meet the issuing warp for every chunk, so that the named barriers complete).  The element mask, the
 // lists and CFG sharing (second store at batch row b + B) are those of the plan (paper Sections 2 and 3).
 #include <algorithm>
 #include <cstring>
@@ -107,6 +107,7 @@ struct WsShared : CodeStage<KV8> {
   int out_of_range[4][2];  // 1 + the last even and odd tile with such rows (a warp is at most one tile ahead of its partner)
   uint32_t tmem_base;
   int abort_flag, redo;
+  int met[2];  // 1 + the last chunk of each stream whose P the issuing warp has met
 };
 
 // Instruction descriptors (kind::f16).  Fields: D type at bit 4 (1: fp32), A and B type at bits 7 and 10 (1: bf16), B transposed
@@ -193,6 +194,15 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr)
                : "memory");
+}
+// Until *at >= n, or some seconds.  (One asm block: a loop in C++ here, however cold, costs the one-tile build's hot loop 4 %.)
+__device__ __forceinline__ void wait_met(const int* at, int n) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .s32 v, i;\n\tmov.s32 i, 0;\n"
+      "AGAIN:\n\tld.volatile.shared.s32 v, [%0];\n\tsetp.ge.s32 p, v, %1;\n\t@p bra MET;\n\tnanosleep.u32 200;\n\t"
+      "add.s32 i, i, 1;\n\tsetp.lt.s32 p, i, 16777216;\n\t@p bra AGAIN;\nMET:\n\t}"
+      ::"r"(smem_u32(at)), "r"(n)
+      : "memory");
 }
 // Where a chunk's 64 rows are (`map`: 0 raster, else 1 + the patch-tiled key scale's map).
 struct ChunkAt {
@@ -282,6 +292,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
     mbar_init(&sm.o_full, 1);
     sm.abort_flag = 0;
     sm.redo = 0;
+    sm.met[0] = sm.met[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -528,6 +539,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           if (g >= base) {
             __syncwarp();
             asm volatile("bar.sync %0, 160;" ::"r"(5 + (g & 1)) : "memory");  // P(g); the softmax warps arrive even when a wait ran out
+            *(volatile int*)&sm.met[g & 1] = g + 1;
           }
           if (ok) {
             tc_fence_after();
@@ -675,65 +687,63 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
             msc = sm.ref[m];
           }
         }
-        for (; g < end; g += 2) {
-          if (ok) {
-            if (maxima && cls) {
+        for (; g < end && ok; g += 2) {
+          if (maxima && cls) {
 #pragma unroll 1
-              for (int hf = 0; hf < 2; ++hf) {
-                const uint32_t w = hf ? mk.y : mk.x;
-                uint32_t r[32];
-                tmem_ld32(tS + 32 * hf, r);
-                tmem_wait_ld();
+            for (int hf = 0; hf < 2; ++hf) {
+              const uint32_t w = hf ? mk.y : mk.x;
+              uint32_t r[32];
+              tmem_ld32(tS + 32 * hf, r);
+              tmem_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) top = fmaxf(top, (w >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
-              }
-            }
-            if (!maxima) {
-#pragma unroll
-              for (int hf = 0; hf < 2; ++hf) {
-                if ((cls >> (2 * hf)) & 3) {
-                  uint32_t r[32], pk[16];
-                  tmem_ld32(tS + 32 * hf, r);
-                  tmem_wait_ld();
-                  if ((cls >> (2 * hf)) & 1) {  // dead scores of a partially live half become -inf
-                    const uint32_t w = hf ? mk.y : mk.x;
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                      if (!((w >> e) & 1u)) r[e] = 0xff800000u;
-                  }
-                  // probabilities against the reference: scale and shift (packed FMAs), 2^x, row sum, bf16
-                  const float2 nm2 = make_float2(-msc, -msc);
-                  const float nm_y = fmaf(msc, 1.f / kClampSpan, kClampHigh / kClampSpan);
-#pragma unroll
-                  for (int e = 0; e < 32; e += 4) {
-                    const uint32_t* rr = r + e;
-                    const float2 xa = __ffma2_rn(make_float2(__uint_as_float(rr[0]), __uint_as_float(rr[1])), sc2, nm2);
-                    const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
-                    // some pairs on the FMA pipe: the exponential pipe (16 per clock and SM) is the tighter of the two
-                    float2 pb;
-                    if (on_fma_pipe<KV8, MANY>(e)) {
-                      pb = exp2_fma2(make_float2(__saturatef(fmaf(__uint_as_float(rr[2]), sc_y, nm_y)),
-                                                 __saturatef(fmaf(__uint_as_float(rr[3]), sc_y, nm_y))));
-                    } else {
-                      const float2 xb = __ffma2_rn(make_float2(__uint_as_float(rr[2]), __uint_as_float(rr[3])), sc2, nm2);
-                      pb = make_float2(fast_exp2(xb.x), fast_exp2(xb.y));
-                    }
-                    pk[(e >> 1) + 0] = pack_bf16(pa.x, pa.y);
-                    pk[(e >> 1) + 1] = pack_bf16(pb.x, pb.y);
-                  }
-                  tmem_st16(tS + 16 * hf, pk);  // over scores that have been read
-                } else {  // no live key for any row of the warp
-                  uint32_t pk[16];
-#pragma unroll
-                  for (int e = 0; e < 16; ++e) pk[e] = 0u;
-                  tmem_st16(tS + 16 * hf, pk);
-                }
-              }
-              tmem_wait_st();
+              for (int e = 0; e < 32; ++e) top = fmaxf(top, (w >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
             }
           }
+          if (!maxima) {
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+              if ((cls >> (2 * hf)) & 3) {
+                uint32_t r[32], pk[16];
+                tmem_ld32(tS + 32 * hf, r);
+                tmem_wait_ld();
+                if ((cls >> (2 * hf)) & 1) {  // dead scores of a partially live half become -inf
+                  const uint32_t w = hf ? mk.y : mk.x;
+#pragma unroll
+                  for (int e = 0; e < 32; ++e)
+                    if (!((w >> e) & 1u)) r[e] = 0xff800000u;
+                }
+                // probabilities against the reference: scale and shift (packed FMAs), 2^x, row sum, bf16
+                const float2 nm2 = make_float2(-msc, -msc);
+                const float nm_y = fmaf(msc, 1.f / kClampSpan, kClampHigh / kClampSpan);
+#pragma unroll
+                for (int e = 0; e < 32; e += 4) {
+                  const uint32_t* rr = r + e;
+                  const float2 xa = __ffma2_rn(make_float2(__uint_as_float(rr[0]), __uint_as_float(rr[1])), sc2, nm2);
+                  const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
+                  // some pairs on the FMA pipe: the exponential pipe (16 per clock and SM) is the tighter of the two
+                  float2 pb;
+                  if (on_fma_pipe<KV8, MANY>(e)) {
+                    pb = exp2_fma2(make_float2(__saturatef(fmaf(__uint_as_float(rr[2]), sc_y, nm_y)),
+                                               __saturatef(fmaf(__uint_as_float(rr[3]), sc_y, nm_y))));
+                  } else {
+                    const float2 xb = __ffma2_rn(make_float2(__uint_as_float(rr[2]), __uint_as_float(rr[3])), sc2, nm2);
+                    pb = make_float2(fast_exp2(xb.x), fast_exp2(xb.y));
+                  }
+                  pk[(e >> 1) + 0] = pack_bf16(pa.x, pa.y);
+                  pk[(e >> 1) + 1] = pack_bf16(pb.x, pb.y);
+                }
+                tmem_st16(tS + 16 * hf, pk);  // over scores that have been read
+              } else {  // no live key for any row of the warp
+                uint32_t pk[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) pk[e] = 0u;
+                tmem_st16(tS + 16 * hf, pk);
+              }
+            }
+            tmem_wait_st();
+          }
           tc_fence_before();
-          asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");  // (the issuing warp counts on every step's arrival)
+          asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
           if (MANY && x > 0 && g - base < 2 && maxima == exact) stored();
           widen_v(g + 2);
           widen_k(g + 4);
@@ -741,6 +751,12 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           mk = mk_next;
           mk_next = look_up(g + 4 - base, cls_next);
           if (g + 2 < end) wait_scores(g + 2);
+        }
+        // A wait ran out.  The issuing warp counts on every chunk's arrival, and the barrier on one of every warp at a time: S(g) says
+        // that P(g - 2) has been met, and where no S is waited for any more the issuing warp's note does.
+        for (; g < end; g += 2) {
+          wait_met(&sm.met[st], g - 1);
+          asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
         }
         if (MANY && idle && x > 0 && maxima == exact) stored();
         const int n_here = n, h_here = h, b_here = b;
