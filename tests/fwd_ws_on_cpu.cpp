@@ -20,7 +20,7 @@ using std::min;
 using Clock = std::chrono::steady_clock;
 using CUtensorMap = int;
 
-constexpr auto kWait = std::chrono::milliseconds(60), kLate = std::chrono::milliseconds(180), kHang = std::chrono::seconds(10);
+constexpr std::chrono::milliseconds kWait{60}, kLate{180}, kHang{10000};
 
 struct Hang {};
 struct Cta {
