@@ -70,6 +70,7 @@ constexpr uint32_t kTmemCols = 256, kColO = 128, kColQ = kColO + kHeadDim + kSum
 
 constexpr int kRefKeys = 32;      // of a tile's first chunk, whose maximum is a row's reference
 constexpr unsigned kIdleNs = 200;  // (50 or 500: the same)
+constexpr int kPolls = 1 << 23;    // of kIdleNs and more: two seconds
 constexpr int kMaxTiles = 1024;  // of a CTA that takes several (MANY)
 // A row sum of the first pass outside (2^-64, 2^96) goes to the second pass.  (The lower end keeps the traces of dead keys, 2^-125
 // each, 2^-48 below a sum over any number of keys.)
@@ -102,7 +103,7 @@ struct WsShared : CodeStage<KV8> {
   float top[2][kBlockM];  // second pass: the rows' maxima over the keys of each stream
   alignas(8) uint64_t q_full[2], q_free;
   uint64_t k_full[kStages], k_free[kStages], v_full[kStages];
-  uint64_t s_full[2], o_full;
+  uint64_t s_full[2], o_full, drained;
   uint32_t held[4][MANY ? kMaxTiles / 32 : 1];  // bit x: the 32 rows of the CTA's tile x are left to the second pass
   int out_of_range[4][2];  // 1 + the last even and odd tile with such rows (a warp is at most one tile ahead of its partner)
   uint32_t tmem_base;
@@ -290,6 +291,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
     mbar_init(&sm.s_full[0], 1);
     mbar_init(&sm.s_full[1], 1);
     mbar_init(&sm.o_full, 1);
+    mbar_init(&sm.drained, 1);
     sm.abort_flag = 0;
     sm.redo = 0;
     sm.met[0] = sm.met[1] = 0;
@@ -464,23 +466,17 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         }
       }
       base = nk;
-      if (*abort_flag) {  // wait (bounded) for copies still in flight before the CTA may exit
-        const unsigned long long ts = global_ns();
-        if constexpr (KV8) {
-          for (int i = nk > kStages ? nk - kStages : 0; i < nk; ++i)
-            while (!mbar_try(&sm.kc_full[i & 1][(i >> 1) & 1], (uint32_t)((i >> 2) & 1)))
-              if (global_ns() - ts > kWaitLimitNs) break;
-          for (int i = nv > 2 ? nv - 2 : 0; i < nv; ++i)
-            while (!mbar_try(&sm.vc_full[i & 1], (uint32_t)((i >> 1) & 1)))
-              if (global_ns() - ts > kWaitLimitNs) break;
-        } else {
-          for (int i = nk > kStages ? nk - kStages : 0; i < nk; ++i)
-            while (!mbar_try(&sm.k_full[i % kStages], (uint32_t)((i / kStages) & 1)))
-              if (global_ns() - ts > kWaitLimitNs) break;
-          for (int i = nv > kStages ? nv - kStages : 0; i < nv; ++i)
-            while (!mbar_try(&sm.v_full[i % kStages], (uint32_t)((i / kStages) & 1)))
-              if (global_ns() - ts > kWaitLimitNs) break;
-        }
+      // Wait (bounded) for the last copies, whose wait in another warp may run out after this one is done.
+      int polls = kPolls;
+      auto landed = [&](uint64_t* bar, int phase) {
+        while (!mbar_try(bar, (uint32_t)(phase & 1)) && --polls > 0) __nanosleep(kIdleNs);
+      };
+      if constexpr (KV8) {
+        for (int i = nk > kStages ? nk - kStages : 0; i < nk; ++i) landed(&sm.kc_full[i & 1][(i >> 1) & 1], i >> 2);
+        for (int i = nv > 2 ? nv - 2 : 0; i < nv; ++i) landed(&sm.vc_full[i & 1], i >> 1);
+      } else {
+        for (int i = nk > kStages ? nk - kStages : 0; i < nk; ++i) landed(&sm.k_full[i % kStages], i / kStages);
+        for (int i = nv > kStages ? nv - kStages : 0; i < nv; ++i) landed(&sm.v_full[i % kStages], i / kStages);
       }
     } else if (warp == 8) {
       // ---------------------------------------------------------------- Q and the MMAs.  The whole warp runs this code (descriptors
@@ -872,6 +868,13 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
   }
 
   // ---------------------------------------------------------------------- teardown (all paths)
+  if (*abort_flag) {  // products may be in flight, which read the stages and write TMEM
+    if (warp == 8) {
+      mma_commit_one(&sm.drained);
+      for (int polls = kPolls; !mbar_try(&sm.drained, 0u) && --polls > 0;) __nanosleep(kIdleNs);
+    }
+    __syncthreads();
+  }
   if (warp == 4) {
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sm.tmem_base), "r"(kTmemCols) : "memory");

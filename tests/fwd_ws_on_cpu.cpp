@@ -1,6 +1,7 @@
 // The roles of the tensor-core forward kernel on CPU threads, one per warp: barriers, copies and products stand for themselves only
-// (no numbers are computed).  A copy arrives late, past the limit of the waits; the CTA must then come to its end on every warp.
-// Built by tests/test_forward_roles_cpu.py, which puts the kernel's own text into fwd_ws_kernel.inc.
+// (no numbers are computed).  A copy arrives late, past the limit of the waits; the CTA must then come to its end on every
+// warp, with no copy and no product in flight.  // Built by tests/test_forward_roles_cpu.py, which puts the kernel's own
+// text into fwd_ws_kernel.inc.
 #include <bit>
 #include <chrono>
 #include <cmath>
@@ -139,7 +140,7 @@ inline void wait_met(const int* at, int n) {
 }
 inline void mma_commit_one(uint64_t* bar) {
   std::lock_guard<std::mutex> lock(cta->mutex);
-  cta->products.push_back({bar, Clock::now()});
+  cta->products.push_back({bar, Clock::now() + std::chrono::milliseconds(cta->late < 0 ? 0 : 2)});
 }
 inline void bar_meet(int id, int n, bool wait) {
   std::unique_lock<std::mutex> lock(cta->mutex);
@@ -157,6 +158,7 @@ inline void bar_sync(int id, int n) { bar_meet(id, n, true); }
 inline void bar_arrive(int id, int n) { bar_meet(id, n, false); }
 inline void __syncthreads() { bar_sync(0, 320); }
 inline void __syncwarp() {}
+inline void __nanosleep(unsigned ns) { std::this_thread::sleep_for(std::chrono::nanoseconds(ns)); }
 template <class T>
 T __shfl_sync(unsigned, T v, int) { return v; }
 inline bool __any_sync(unsigned, bool v) { return v; }
@@ -230,17 +232,19 @@ int run(const std::vector<int>& chunks, bool second_pass, int late) {
       }
     });
   for (auto& w : warps) w.join();
+  int in_flight;
   {
     std::lock_guard<std::mutex> lock(c.mutex);
+    in_flight = (int)(c.copies.size() + c.products.size());
     c.done = true;
   }
   engine.join();
   free(c.smem);
-  const bool bad = c.hung || c.status != (late >= 0);
+  const bool bad = c.hung || in_flight || c.status != (late >= 0);
   if (bad) {
     printf("KV8 %d MANY %d second pass %d copy %d late, lists", KV8, MANY, second_pass, late);
     for (int n : chunks) printf(" %d", n);
-    printf(": %sstatus %d\n", c.hung ? "hangs, " : "", c.status);
+    printf(": %s%d copies or products in flight, status %d\n", c.hung ? "hangs, " : "", in_flight, c.status);
   }
   return bad ? -1 : c.copies_seen;
 }

@@ -42,6 +42,6 @@ def roles(tmp_path_factory):
 @pytest.mark.parametrize("second_pass", [False, True], ids=["first-pass", "second-pass"])
 @pytest.mark.parametrize("kind", ["one-tile", "many-tiles", "8-bit"])
 def test_a_late_copy_ends_the_cta(roles, kind, second_pass):
-    """Every warp returns, and the status word is raised."""
+    """Every warp returns, the status word is raised, and no copy or product is in flight."""
     res = subprocess.run([roles, kind] + ["second"] * second_pass, capture_output=True, text=True, timeout=300)
     assert res.returncode == 0, res.stdout
