@@ -34,8 +34,11 @@
 // 1, without rounding, and the larger its weight the more that is worth: error against fp64 (relative L2, N(0, 1) inputs; with the
 // maximum of eight keys / of 32 / with two accumulators and a maximum of eight keys for each) 256px step 8 2.306e-3 / 2.282e-3 /
 // 2.293e-3, 256px step 10 2.291 / 2.273 / 2.281, 512px step 10 2.324 / 2.316 / 2.322.  The stream with the first chunk hands the
-// reference to the other one (which is then a little behind: both streams at the same point of a chunk are 4 to 5 % slower), in front
-// of the loop over the chunks: as a case inside it, a loop of 22 chunks took 1 % longer even with eight keys.  At the end a row
+// reference to the other one (which is then a little behind: both streams at the same point of a chunk are 4 to 5 % slower).  Each
+// stream's first chunk is a copy of the loop's body in front of it, so that its scores are loaded and masked once: as a case inside
+// the loop (with eight keys) / as a load of its own in front of it / as a copy, 256px steps 8, 9 and 10 with 960 units take 24.9 /
+// 25.4 / 25.0, 54.4 / 55.4 / 54.4 and 74.4 / 75.1 / 73.9 us, step 9 with 480 30.5 / 31.5 / 30.6, last 512px step 143.0 / 142.8 / 141.0,
+// with an 8-bit cache 222.9 / 220.6 / 219.8, 2K step 12 150.9 / 149.9 / 149.0.  At the end a row
 // whose sum or output is out of range (kRange, kSmall) sends the CTA through its lists again (`exact`), each list twice: once for
 // the rows' maxima, then against them, for the 32 rows of a warp that it belongs to, which are stored then.
 //
@@ -68,7 +71,6 @@ constexpr int kSumCols = 16;              // of the accumulator, behind O: row s
 constexpr int kThreads = 320;             // two streams of four softmax warps, one warp for the MMAs, one for the copies
 constexpr uint32_t kTmemCols = 256, kColO = 128, kColQ = kColO + kHeadDim + kSumCols;  // S (and P over it) of stream s at 64 s, then O and the row sums, then Q
 
-constexpr int kRefKeys = 32;      // of a tile's first chunk, whose maximum is a row's reference
 constexpr unsigned kIdleNs = 200;  // (50 or 500: the same)
 constexpr int kPolls = 1 << 23;    // of kIdleNs and more: two seconds
 constexpr int kMaxTiles = 1024;  // of a CTA that takes several (MANY)
@@ -195,6 +197,18 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr)
                : "memory");
+}
+// Largest of 32 scores (dead ones: -inf), four chains of three-way maxima.
+__device__ __forceinline__ float largest_score(const uint32_t* r) {
+  float top[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) top[i] = fmaxf(__uint_as_float(r[i]), __uint_as_float(r[4 + i]));
+#pragma unroll
+  for (int e = 8; e < 32; e += 8)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      asm("max.f32 %0, %0, %1, %2;" : "+f"(top[i]) : "f"(__uint_as_float(r[e + i])), "f"(__uint_as_float(r[e + 4 + i])));
+  return fmaxf(fmaxf(top[0], top[1]), fmaxf(top[2], top[3]));
 }
 // Until *at >= n, or some seconds.  (One asm block: a loop in C++ here, however cold, costs the one-tile build's hot loop 4 %.)
 __device__ __forceinline__ void wait_met(const int* at, int n) {
@@ -635,6 +649,71 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         if (ok) ok = mbar_wait_long(&sm.s_full[st], (uint32_t)((i >> 1) & 1), abort_flag, p.status);
         if (ok) tc_fence_after();
       };
+      auto load_scores = [&](int hf, uint32_t* r) {
+        tmem_ld32(tS + 32 * hf, r);
+        tmem_wait_ld();
+        if ((cls >> (2 * hf)) & 1) {  // dead scores of a partially live half become -inf
+          const uint32_t w = hf ? mk.y : mk.x;
+#pragma unroll
+          for (int e = 0; e < 32; ++e)
+            if (!((w >> e) & 1u)) r[e] = 0xff800000u;
+        }
+      };
+      // probabilities against the reference: scale and shift (packed FMAs), 2^x, bf16, over scores that have been read
+      auto store_probabilities = [&](int hf, const uint32_t* r) {
+        uint32_t pk[16];
+        const float2 nm2 = make_float2(-msc, -msc);
+        const float nm_y = fmaf(msc, 1.f / kClampSpan, kClampHigh / kClampSpan);
+#pragma unroll
+        for (int e = 0; e < 32; e += 4) {
+          const uint32_t* rr = r + e;
+          const float2 xa = __ffma2_rn(make_float2(__uint_as_float(rr[0]), __uint_as_float(rr[1])), sc2, nm2);
+          const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
+          // some pairs on the FMA pipe: the exponential pipe (16 per clock and SM) is the tighter of the two
+          float2 pb;
+          if (on_fma_pipe<KV8, MANY>(e)) {
+            pb = exp2_fma2(make_float2(__saturatef(fmaf(__uint_as_float(rr[2]), sc_y, nm_y)),
+                                       __saturatef(fmaf(__uint_as_float(rr[3]), sc_y, nm_y))));
+          } else {
+            const float2 xb = __ffma2_rn(make_float2(__uint_as_float(rr[2]), __uint_as_float(rr[3])), sc2, nm2);
+            pb = make_float2(fast_exp2(xb.x), fast_exp2(xb.y));
+          }
+          pk[(e >> 1) + 0] = pack_bf16(pa.x, pa.y);
+          pk[(e >> 1) + 1] = pack_bf16(pb.x, pb.y);
+        }
+        tmem_st16(tS + 16 * hf, pk);
+      };
+      auto store_zeros = [&](int hf) {
+        uint32_t pk[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) pk[e] = 0u;
+        tmem_st16(tS + 16 * hf, pk);
+      };
+      // The row's reference, from the stream with the tile's first chunk (`mx`: the maximum of its first 32 live scores) to the other.
+      auto hand_over = [&](float mx) {
+        if (g == base) {
+          msc = mx != -INFINITY ? mx * sc : 0.f;
+          if (n > 1) {
+            sm.ref[m] = msc;
+            asm volatile("bar.arrive %0, 64;" ::"r"(12 + lane_group) : "memory");
+          }
+        } else {
+          asm volatile("bar.sync %0, 64;" ::"r"(12 + lane_group) : "memory");
+          msc = sm.ref[m];
+        }
+      };
+      // P(g) is complete, or of S(g) the maxima: the issuing warp is told, and this warp goes on to its next chunk.
+      auto chunk_done = [&](int x, int end, bool first_list) {
+        tc_fence_before();
+        asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
+        if (MANY && x > 0 && g - base < 2 && first_list) stored();
+        widen_v(g + 2);
+        widen_k(g + 4);
+        cls = cls_next;
+        mk = mk_next;
+        mk_next = look_up(g + 4 - base, cls_next);
+        if (g + 2 < end) wait_scores(g + 2);
+      };
       for (int list = 0; list < n_lists; ++list) {
         const int x = exact ? list >> 1 : list;
         const bool maxima = exact && !(list & 1);
@@ -651,102 +730,53 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
           row_live = r0 + (lane >> 3) < p.s_k && c0 + (lane & 7) < p.s_k;
         }
         if (g < end) wait_scores(g);
-        if (!exact && g < end) {  // (the warps meet here whether a wait ran out or not)
-          if (g == base) {        // the tile's first chunk: the rows' references
-            float mx = -INFINITY;
-            if (ok && (cls & 3)) {
-              uint32_t r[kRefKeys];
-              tmem_ld32(tS, r);
-              tmem_wait_ld();
-              if (cls & 1) {
-#pragma unroll
-                for (int e = 0; e < kRefKeys; ++e)
-                  if (!((mk.x >> e) & 1u)) r[e] = 0xff800000u;
-              }
-              float top4[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) top4[i] = fmaxf(__uint_as_float(r[i]), __uint_as_float(r[4 + i]));
-#pragma unroll
-              for (int e = 8; e < kRefKeys; e += 8)
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                  asm("max.f32 %0, %0, %1, %2;" : "+f"(top4[i]) : "f"(__uint_as_float(r[e + i])), "f"(__uint_as_float(r[e + 4 + i])));
-              mx = fmaxf(fmaxf(top4[0], top4[1]), fmaxf(top4[2], top4[3]));
+        if (!exact && g < end) {  // the stream's first chunk, with the rows' references (the warps meet here whether a wait ran out or not)
+          if (ok) {
+            uint32_t r[32];
+            if (cls & 3) {
+              load_scores(0, r);
+              hand_over(g == base ? largest_score(r) : 0.f);
+              store_probabilities(0, r);
+            } else {
+              hand_over(-INFINITY);
+              store_zeros(0);
             }
-            msc = mx != -INFINITY ? mx * sc : 0.f;
-            if (n > 1) {
-              sm.ref[m] = msc;
-              asm volatile("bar.arrive %0, 64;" ::"r"(12 + lane_group) : "memory");
+            if (cls >> 2) {
+              load_scores(1, r);
+              store_probabilities(1, r);
+            } else {
+              store_zeros(1);
             }
+            tmem_wait_st();
+            chunk_done(x, end, true);
+            g += 2;
           } else {
-            asm volatile("bar.sync %0, 64;" ::"r"(12 + lane_group) : "memory");
-            msc = sm.ref[m];
+            hand_over(-INFINITY);
           }
         }
         for (; g < end && ok; g += 2) {
-          if (maxima && cls) {
+          if (maxima) {  // second pass: the list once for the rows' maxima
 #pragma unroll 1
-            for (int hf = 0; hf < 2; ++hf) {
-              const uint32_t w = hf ? mk.y : mk.x;
-              uint32_t r[32];
-              tmem_ld32(tS + 32 * hf, r);
-              tmem_wait_ld();
-#pragma unroll
-              for (int e = 0; e < 32; ++e) top = fmaxf(top, (w >> e) & 1u ? __uint_as_float(r[e]) : -INFINITY);
-            }
-          }
-          if (!maxima) {
+            for (int hf = 0; hf < 2; ++hf)
+              if ((cls >> (2 * hf)) & 3) {
+                uint32_t r[32];
+                load_scores(hf, r);
+                top = fmaxf(top, largest_score(r));
+              }
+          } else {
 #pragma unroll
             for (int hf = 0; hf < 2; ++hf) {
               if ((cls >> (2 * hf)) & 3) {
-                uint32_t r[32], pk[16];
-                tmem_ld32(tS + 32 * hf, r);
-                tmem_wait_ld();
-                if ((cls >> (2 * hf)) & 1) {  // dead scores of a partially live half become -inf
-                  const uint32_t w = hf ? mk.y : mk.x;
-#pragma unroll
-                  for (int e = 0; e < 32; ++e)
-                    if (!((w >> e) & 1u)) r[e] = 0xff800000u;
-                }
-                // probabilities against the reference: scale and shift (packed FMAs), 2^x, row sum, bf16
-                const float2 nm2 = make_float2(-msc, -msc);
-                const float nm_y = fmaf(msc, 1.f / kClampSpan, kClampHigh / kClampSpan);
-#pragma unroll
-                for (int e = 0; e < 32; e += 4) {
-                  const uint32_t* rr = r + e;
-                  const float2 xa = __ffma2_rn(make_float2(__uint_as_float(rr[0]), __uint_as_float(rr[1])), sc2, nm2);
-                  const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
-                  // some pairs on the FMA pipe: the exponential pipe (16 per clock and SM) is the tighter of the two
-                  float2 pb;
-                  if (on_fma_pipe<KV8, MANY>(e)) {
-                    pb = exp2_fma2(make_float2(__saturatef(fmaf(__uint_as_float(rr[2]), sc_y, nm_y)),
-                                               __saturatef(fmaf(__uint_as_float(rr[3]), sc_y, nm_y))));
-                  } else {
-                    const float2 xb = __ffma2_rn(make_float2(__uint_as_float(rr[2]), __uint_as_float(rr[3])), sc2, nm2);
-                    pb = make_float2(fast_exp2(xb.x), fast_exp2(xb.y));
-                  }
-                  pk[(e >> 1) + 0] = pack_bf16(pa.x, pa.y);
-                  pk[(e >> 1) + 1] = pack_bf16(pb.x, pb.y);
-                }
-                tmem_st16(tS + 16 * hf, pk);  // over scores that have been read
+                uint32_t r[32];
+                load_scores(hf, r);
+                store_probabilities(hf, r);
               } else {  // no live key for any row of the warp
-                uint32_t pk[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e) pk[e] = 0u;
-                tmem_st16(tS + 16 * hf, pk);
+                store_zeros(hf);
               }
             }
             tmem_wait_st();
           }
-          tc_fence_before();
-          asm volatile("bar.arrive %0, 160;" ::"r"(5 + st) : "memory");
-          if (MANY && x > 0 && g - base < 2 && maxima == exact) stored();
-          widen_v(g + 2);
-          widen_k(g + 4);
-          cls = cls_next;
-          mk = mk_next;
-          mk_next = look_up(g + 4 - base, cls_next);
-          if (g + 2 < end) wait_scores(g + 2);
+          chunk_done(x, end, maxima);
         }
         // A wait ran out.  The issuing warp counts on every chunk's arrival, and the barrier on one of every warp at a time: S(g) says
         // that P(g - 2) has been met, and where no S is waited for any more the issuing warp's note does.

@@ -168,6 +168,7 @@ inline float __uint_as_float(uint32_t v) { return std::bit_cast<float>(v); }
 inline float __saturatef(float x) { return x; }
 inline float2 __ffma2_rn(float2 a, float2, float2) { return a; }
 inline float2 __fmul2_rn(float2 a, float2) { return a; }
+inline float largest_score(const uint32_t*) { return 0.f; }
 inline float2 exp2_fma2(float2 x) { return x; }
 inline float fast_exp2(float x) { return x; }
 inline uint32_t pack_bf16(float, float) { return 0; }
