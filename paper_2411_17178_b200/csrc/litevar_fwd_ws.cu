@@ -565,12 +565,14 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
               mma_commit_one(&sm.s_full[g & 1]);
               if (!KV8) mma_commit_one(&sm.k_free[s2]);
             }
-            // the next tile's Q, once the tile before this one has left its buffer (the first two were copied at the start)
-            if (MANY && g == base && x > 0 && nq == x + 1 && nq < n_tiles) ok = load_q();
+            // The next tile's Q, once the tile before this one has left its buffer (the first two were copied at the start).  Both
+            // streams' warps see to that behind their first chunk: a wait behind the first chunk of one held up the product of the
+            // other (256px step 8 with 960 units 25.0 us, 24.2 behind the second).
+            if (MANY && g > base && x > 0 && nq == x + 1 && nq < n_tiles) ok = load_q();
             __syncwarp();
           }
         }
-        if (MANY && ok && x > 0 && nq == x + 1 && nq < n_tiles) ok = load_q();  // (no chunk at all)
+        if (MANY && ok && x > 0 && nq == x + 1 && nq < n_tiles) ok = load_q();  // (less than two chunks)
         base = end;
         n = n_next;
       }
