@@ -950,11 +950,13 @@ litevar_status_t launch_forward_ws(const FwdParams& p, int n_q_tiles, cudaStream
   // these with the other tiles' work.  What is lost is the balance at the end: a CTA's tiles are fixed, not dealt out.  Measured
   // (thousand cycles, one tile per CTA / staying): 4 chunks at 3.2 tiles per resident CTA 56.2 / 50.6, 6 at 3.2 63.7 / 60.0, at 6.5
   // 113.7 / 100.5, 10 at 3.2 81.4 / 80.6, at 6.5 144.3 / 133.5, 8 at 2.9 60.8 / 60.9, at 5.8 117.1 / 113.1, at 1.5 38.2 / 38.9; 14
-  // at 4.9 125.4 / 133.0, at 9.7 236.9 / 244.0; 22 at 7.8 267 / 291, at 15.6 523 / 544; patch tiles of a 48 x 48 step at 11.7 with window 1/4, 1/8, 1/16: 571 / 670, 385 / 433, 304 / 330.  (Patch tiles with window
-  // sets of their own per head keep the line at 40 chunks on average that all launches had.)
+  // at 4.9 125.4 / 133.0, at 9.7 236.9 / 244.0; 22 at 7.8 267 / 291, at 15.6 523 / 544; patch tiles of a 48 x 48 step at 11.7 with
+  // window 1/4, 1/8, 1/16: 571 / 670, 385 / 433, 304 / 330.  Sets of their own per head make no difference, the average over the
+  // heads counts (us, the same step): all keys for one head in eight and 1/8 for the others 263 / 322, 1/4 and 1/8 262 / 313, 1/8 and
+  // 1/16 189 / 215, 1/16 and 1/48 155 / 163.
   const long long items = (long long)n_q_tiles * p.n_heads * p.batch_computed, resident = 2ll * current_sm_count();
   const int chunks = p.chunks_per_tile;
-  if (chunks > 0 && chunks <= (p.q_patch && p.head_to_set ? 40 : 12) && 2 * items >= 5 * resident && 5 * items >= chunks * resident)
+  if (chunks > 0 && chunks <= 12 && 2 * items >= 5 * resident && 5 * items >= chunks * resident)
     return launch_variant<false, true>(tm, p, n_q_tiles, (int)std::max(resident, (items + kMaxTiles - 1) / kMaxTiles), stream);
   return launch_variant<false, false>(tm, p, n_q_tiles, 0, stream);
 }

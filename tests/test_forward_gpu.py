@@ -758,17 +758,38 @@ def test_short_raster_lists_share_ctas(pairs, many):
 @pytest.mark.parametrize("wide_heads", [7, 1])
 @pytest.mark.parametrize("wide_set", [0, 1])
 def test_build_follows_the_lists_of_all_heads(wide_set, wide_heads):
-    """Whether CTAs take several tiles depends on the average list over the heads, not on the order of the window sets: 48 x 48
-    patch tiles with long lists (everything live, 71 chunks and more) and short ones (window 1/8)."""
+    """Whether CTAs take several tiles depends on the average list over the heads, not on the order of the window sets: 24 x 24
+    raster tiles with long lists (everything live, 22 chunks) and short ones (window 1/16), on average above or below the line at 12."""
     lib_ready()
-    scales, K, H, B = (1, 2, 3, 4, 6, 9, 13, 18, 24, 32, 48), 11, 8, 12
-    wide, narrow = orc.full_table(scales), orc.window_table(scales, rho=(1, 8))
+    scales, H, B = (1, 2, 3, 4, 6, 9, 13, 18, 24), 8, 12
+    K = len(scales)
+    wide, narrow = orc.full_table(scales), orc.window_table(scales, rho=(1, 16))
     tabs = [wide, narrow] if wide_set == 0 else [narrow, wide]
-    plan = binding.Plan(scales, n_heads=H, radius=np.stack(tabs), n_sets=2,
-                        head_to_set=[wide_set if h < wide_heads else 1 - wide_set for h in range(H)])
+    head_set = [wide_set if h < wide_heads else 1 - wide_set for h in range(H)]
+    plan = binding.Plan(scales, n_heads=H, radius=np.stack(tabs), n_sets=2, head_to_set=head_set)
+    w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=88)
+    Q = wl.make_q(w, 0, K)
+    Kc, Vc = wl.make_kv(w, 0)
+    q, k, v = Q.cuda(), Kc.cuda(), Vc.cuda()
+    out = torch.empty_like(q)
+    ctas = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert captured_grids(lambda: plan.forward(K, B, q, k, v, out)) == [5 * H * 2 * B if wide_heads == 7 else ctas]
+    plan.forward(K, B, q, k, v, out)
+    assert plan.poll() == 0
+    b = 2 * B - 1
+    for h in (0, H - 1):
+        ref = orc.attention_step(scales, K, tabs[head_set[h]][K - 1], Q[b:, h:h + 1], Kc[b:, h:h + 1], Vc[b:, h:h + 1])
+        assert_close(out[b:, h:h + 1].double().cpu().numpy(), ref, f"head {h}")
+    plan.close()
+
+
+def test_head_sets_follow_the_line_of_one_set():
+    """48 x 48 patch tiles with window sets per head, 25 chunks on average: one tile per CTA, as with one set of such lists."""
+    lib_ready()
+    scales, H, B = (1, 2, 3, 4, 6, 9, 13, 18, 24, 32, 48), 8, 12
+    tabs = np.stack([orc.window_table(scales, rho=(1, 4)), orc.window_table(scales, rho=(1, 8))])
     q = torch.zeros(2 * B, H, 48 * 48, 64, dtype=torch.bfloat16, device="cuda")
     kv = torch.zeros(2 * B, H, sum(s * s for s in scales), 64, dtype=torch.bfloat16, device="cuda")
-    tiles = 6 * 3 * H * 2 * B
-    ctas = 2 * torch.cuda.get_device_properties(0).multi_processor_count
-    assert captured_grids(lambda: plan.forward(K, B, q, kv, kv, q)) == [tiles if wide_heads == 7 else ctas]
-    plan.close()
+    for plan in (binding.Plan(scales, n_heads=H, radius=tabs, n_sets=2, head_to_set=[0, 1] * 4), binding.Plan(scales, n_heads=H, radius=tabs[0])):
+        assert captured_grids(lambda: plan.forward(11, B, q, kv, kv, q)) == [6 * 3 * H * 2 * B]
+        plan.close()
