@@ -620,7 +620,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         }
       };
       // 8-bit cache: the stream's softmax threads widen its chunks, V(g) before they hand P(g) over and K(g + 4) after it
-      const int t = threadIdx.x & 127, pass_end = base + item0.n * sweeps;
+      const int t = threadIdx.x & 127, pass_end = base + item0.n * sweeps, v_from = pass_end - item0.n;  // (the walk for the maxima needs no V)
       auto widen_k = [&](int i) {
         if constexpr (KV8) {
           if (ok && i < pass_end &&
@@ -634,7 +634,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
       auto widen_v = [&](int i) {
         if constexpr (KV8) {
           if (ok && i < pass_end && (ok = mbar_wait_long(&sm.vc_full[st], (uint32_t)((i >> 1) & 1), abort_flag, p.status))) {
-            widen_chunk(sm.vc[st], sm.v_sz[st], sm.v[i % kStages], t);
+            if (i >= v_from) widen_chunk(sm.vc[st], sm.v_sz[st], sm.v[i % kStages], t);
             __syncwarp();
             if (lane == 0) mbar_arrive(&sm.vc_free[st]);
           }
