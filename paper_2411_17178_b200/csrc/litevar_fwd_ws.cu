@@ -18,8 +18,9 @@
 // to the largest exponent and cuts them off there: with ones everywhere 16 addends a step lose up to a bit of the sum each, always
 // in the same direction.  Over the 34240 keys of the last 2K step, keys three times as sharp, outputs were too large by 1.0e-4; with
 // four addends a step by 1.5e-5, with one too small by 1.9e-5, with sums by additions too small by 1.5e-5.  Time: the same.)  A sum
-// by additions is one instruction a score (64, beside the 360 that a warp issues per chunk now, all included).  Q is a TMEM operand: a step of S = Q K with both operands in shared memory waits for their 6 KB (50 cycles, 32 with Q in
-// TMEM), and the two CTAs of an SM share that.
+// by additions is one instruction a score (64, beside the 360 that a warp issues per chunk now, all included).
+// Q is a TMEM operand: a step of S = Q K with both operands in shared memory waits for their 6 KB (50 cycles, 32 with Q in TMEM), and
+// the two CTAs of an SM share that.
 // MANY: a CTA takes several tiles in turn.  Q has two buffers; K and V copies of the next tile go out behind the last ones of this
 // one, the softmax warps look the next list up while they wait for their accumulator, and the
 // output leaves by tensor-map stores that nobody waits for until the buffer's next use.  What orders the tiles: the first
@@ -44,14 +45,17 @@
 //
 // What bounds it (ncu, 2K step, full mask): issue slots 72 % busy, exponential pipe 64 %, tensor pipe active 56 %; 5.6 instructions a
 // score.  (More warps do not help: three streams of softmax warps, or three score buffers so that none waits for its next scores,
-// took as long as before with the sums still added by instructions.)  Measured on B200, in thousand cycles of a launch, with one accumulator and
-// sums of its own per stream / shared accumulator and sums by products / and Q in TMEM / and six pairs of a half's 16 on the FMA pipe:
-// 2K step with the full mask 8840 / 8100 / 7720 / 7500, window 1/4 2710 / 2540 / 2455 / 2400; last 512px step, 288 units 285 / 292
-// (with one tile per CTA 281) / 271 / 267; last 256px step with 128 units 31.0 / 28.5 / 28.1 / 27.9.
+// took as long as before with the sums still added by instructions.)  Measured on B200, in thousand cycles of a launch, with one
+// accumulator and sums of its own per stream / shared accumulator and sums by products / and Q in TMEM / and six pairs of a half's
+// 16 on the FMA pipe: 2K step with the full mask 8840 / 8100 / 7720 / 7500, window 1/4 2710 / 2540 / 2455 / 2400; last 512px step,
+// 288 units 285 / 292 (with one tile per CTA 281) / 271 / 267; last 256px step with 128 units 31.0 / 28.5 / 28.1 / 27.9.  All rows out
+// of range, so that every list is walked three times: 2K step, window 1/4, 1365 -> 3660 to 3730 us, last 256px step with 960 units
+// 84 -> 200, last 512px step on an 8-bit cache 229 -> 573.
 //
-// Every wait on an mbarrier is bounded; when one runs out the CTA raises the plan's status word, drains its copies, frees its
-// TMEM and returns (the softmax warps still meet the issuing warp for every chunk, so that the named barriers complete).  The element mask, the
-// lists and CFG sharing (second store at batch row b + B) are those of the plan (paper Sections 2 and 3).
+// Every wait on an mbarrier is bounded; when one runs out the CTA raises the plan's status word, waits for its copies and products
+// in flight, frees its TMEM and returns (the softmax warps still meet the issuing warp for every chunk, so that the named barriers
+// complete).  The element mask, the lists and CFG sharing (second store at batch row b + B) are those of the plan (paper
+// Sections 2 and 3).
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -69,17 +73,20 @@ constexpr uint32_t kChunkBytes = kChunkKeys * kHeadDim * 2;
 constexpr int kStages = 4;                // K ring and V ring; chunk g of the CTA is in stage g % kStages
 constexpr int kSumCols = 16;              // of the accumulator, behind O: row sums over the keys that agree with the column modulo 4
 constexpr int kThreads = 320;             // two streams of four softmax warps, one warp for the MMAs, one for the copies
-constexpr uint32_t kTmemCols = 256, kColO = 128, kColQ = kColO + kHeadDim + kSumCols;  // S (and P over it) of stream s at 64 s, then O and the row sums, then Q
+// TMEM columns: S (and P over it) of stream s at 64 s, then O and the row sums, then Q
+constexpr uint32_t kTmemCols = 256, kColO = 128, kColQ = kColO + kHeadDim + kSumCols;
 
 constexpr unsigned kIdleNs = 200;  // (50 or 500: the same)
 constexpr int kPolls = 1 << 23;    // of kIdleNs and more: two seconds
 constexpr int kMaxTiles = 1024;  // of a CTA that takes several (MANY)
 // A row sum of the first pass outside (2^-64, 2^96) goes to the second pass.  (The lower end keeps the traces of dead keys, 2^-125
-// each, 2^-48 below a sum over any number of keys.)
+// each, below 2^-41 of a sum over the longest list there is, kMaxScales * kMaxScale^2 = 2^20 keys in one accumulator; 2^-46 over the
+// 34240 of the last 2K step.)
 constexpr float kRange = 79228162514264337593543950336.f, kRangeLow = 5.42101086242752217e-20f;
 // So does a row of output that is not finite (sums of P V overflow before those of P), or so small beside its weight, where that is
-// above 1, that products P V may have been subnormal (2^-126 each, 2^14 of them).
-constexpr float kSmall = 7.88860905221011805e-31f;  // 2^-100
+// above 1, that products P V may have been subnormal (2^-126 each, 2^20 of them: 2^-12 of the smallest output that is kept).
+constexpr float kSmall = 5.04870979341447553e-29f;  // 2^-94
+static_assert((long long)kMaxScales * kMaxScale * kMaxScale <= 1 << 20, "keys of a list, in kRangeLow and kSmall");
 
 // 8-bit cache build: the codes of a chunk (64 rows of 64 bytes, as the tensor-map copy delivers them, no swizzle) and its rows'
 // scales and zero points, on their way into the bf16 stages (empty in the bf16 build).  Chunk g is number g / 2 of stream g % 2.
@@ -142,7 +149,8 @@ __device__ __forceinline__ float2 exp2_fma2(float2 y) {
 // per CTA, two with several on short lists (where the widest tiles are partly masked and the arithmetic is not what a tile waits for),
 // three beside the widening of an 8-bit cache, whose arithmetic is on that pipe too.  Measured for 3 / 4 / 5 / 6 / 7 pairs, thousand
 // cycles: 2K step 14 2470 / 2455 / 2436 / 2401 / 2426, with the full mask 7800 / 7720 / 7630 / 7500 / 7580; several tiles per CTA, last
-// 256px step with 960 units, for 2 / 4 / 5 pairs: 131.8 / 132.6 / 135.5; 8-bit cache, last 512px step, for 3 / 4 / 5 449 / 457 / 460.
+// 256px step with 960 units, for 2 / 4 / 5 pairs: 131.8 / 132.6 / 135.5; 8-bit cache, last 512px step, for 3 / 4 / 5 449 / 457 / 460
+// (with scales put beside the codes by instructions; 414 with asynchronous copies of them).
 template <bool KV8, bool MANY>
 __device__ __forceinline__ constexpr bool on_fma_pipe(int e) {
   return KV8 ? (e & 4) != 0 && e != 28 : MANY ? e == 4 || e == 20 : (e & 4) != 0 || (e & 15) == 0;
@@ -315,8 +323,10 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
   if (warp == 9 && elect_one()) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&sm.k_full[s], KV8 ? 4 : 1);  // 8-bit cache: every softmax warp of the stream arrives
-      mbar_init(&sm.k_free[s], 1);
-      mbar_init(&sm.v_full[s], 1);
+      if constexpr (!KV8) {
+        mbar_init(&sm.k_free[s], 1);
+        mbar_init(&sm.v_full[s], 1);
+      }
     }
     if constexpr (KV8) {
       for (int s = 0; s < 2; ++s) {
@@ -555,8 +565,9 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
             tc_fence_after();
             if (g >= base && !maxima) {
               // 16 keys per step = 16 rows of 128 B = 2048 B of V (the block for the sums stays) and 8 packed columns of P
-              mma_ts_x4_one<8, (2048 >> 4) - ((2048 >> 4) << 16)>(tO, tS + 64 * (g & 1), v_desc0 + (uint64_t)((kChunkBytes >> 4) * s) - ((uint64_t)((kChunkBytes >> 4) * s) << 16),
-                                                                  kIdescO, g > base ? 1u : 0u);
+              const uint64_t stage = (uint64_t)((kChunkBytes >> 4) * s);
+              mma_ts_x4_one<8, (2048 >> 4) - ((2048 >> 4) << 16)>(tO, tS + 64 * (g & 1), v_desc0 + stage - (stage << 16), kIdescO,
+                                                                  g > base ? 1u : 0u);
               if (g + 1 == end) mma_commit_one(&sm.o_full);
             }
             if (g + 2 < end) {
@@ -620,7 +631,7 @@ fwd_ws_kernel(const __grid_constant__ TensorMaps tm, const __grid_constant__ Fwd
         }
       };
       // 8-bit cache: the stream's softmax threads widen its chunks, V(g) before they hand P(g) over and K(g + 4) after it
-      const int t = threadIdx.x & 127, pass_end = base + item0.n * sweeps, v_from = pass_end - item0.n;  // (the walk for the maxima needs no V)
+      const int t = threadIdx.x & 127, pass_end = base + item0.n * sweeps, v_from = pass_end - item0.n;  // (maxima: no V)
       auto widen_k = [&](int i) {
         if constexpr (KV8) {
           if (ok && i < pass_end &&
