@@ -523,39 +523,43 @@ def test_many_tiles_per_cta(case, tiling):
     plan.close()
 
 
-@pytest.mark.parametrize("case", ["first", "second"])
+@pytest.mark.parametrize("scales", [(8,), (1, 2, 3, 4, 5, 6), (1, 2, 3, 4, 5, 6, 8), (1, 2, 3, 4, 5, 6, 8, 10, 13)],
+                         ids=["1-chunk", "2-chunks", "3-chunks", "7-chunks"])
 @pytest.mark.parametrize("build,tiling", BUILDS, ids=lambda x: TNAME.get(x, x))
-def test_streams_with_far_references(build, tiling, case):
-    """One key stream's reference is taken from keys far below the others (logits of -92 against -40), the other stream has no
-    live key among its first eight and reference 0: both sums are in range, and the stream with the small reference holds most
-    of the weight.  `case` says which stream that is."""
+def test_reference_of_every_row_reaches_both_streams(build, tiling, scales):
+    """The stream with a tile's first chunk hands the rows' references to the other one, tile after tile.  All keys of a row have the
+    same logit, which differs from row to row and tile to tile by up to 2^40: chunks taken against another row's or an earlier
+    tile's reference would have a weight of their own, with sums that stay in the first pass's range."""
     lib_ready()
-    H, B = (8, 32) if build == "many-tiles" else (2, 1)
-    if case == "first":         # cache rows 0 to 7 are global: the first keys of the first chunk of every tile
-        scales, low = (1, 2, 3, 4, 6, 9, 13), list(range(8))
-        tab = orc.window_table(scales)
-    else:                       # second chunk: raster rows 64 on; patches: columns 8 on of the 12 x 12 grid, for the last query column
-        scales, low = (12, 16), [8, 9, 10, 11] + list(range(64, 72))
-        tab = orc.full_table(scales)
-        tab[1] = 3, 9
     K, n, L = len(scales), scales[-1] ** 2, sum(s * s for s in scales)
-    logits = torch.full((L,), -40.0)
-    logits[low] = -92.0
+    H, B = (8, -(-740 // (16 * -(-n // 128)))) if build == "many-tiles" else (3, 1)
     w = wl.small_workload(scales, n_heads=H, batch_pairs=B, index=97)
-    Q = torch.ones(2 * B, H, n, 64).bfloat16()
-    Kc = (logits / 8).view(1, 1, L, 1).expand(2 * B, H, L, 64).bfloat16()    # q . k / 8 = logit, exactly
+    logit = torch.randint(-28, 29, (2 * B, H, n, 1), generator=torch.Generator().manual_seed(3)) / 2
+    Q = logit.expand(2 * B, H, n, 64).bfloat16()
+    Kc = torch.full((2 * B, H, L, 64), 0.125).bfloat16()     # q . k / 8 = logit, exactly
     Vc = wl.make_kv(w, 0)[1]
-    plan = binding.Plan(scales, n_heads=H, radius=tab, tiling=tiling)
+    tab = orc.window_table(scales)
+    plan = binding.Plan(scales, n_heads=H, tiling=tiling)
+    plan.set_kernel(binding.KERNEL_TCGEN05)
+    q, k, v = Q.cuda(), Kc.cuda(), Vc.cuda()
+    out = torch.full(Q.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
     if build == "8-bit":
-        (K8, *kq), (V8, *vq) = (binding.quantize_rows(t.cuda(), want_codes=True) for t in (Kc, Vc))
-        out = torch.full(Q.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
-        plan.forward_kv8(K, B, Q.cuda(), *kq, *vq, out)
-        got, Kc, Vc = out.double().cpu().numpy(), K8.cpu(), V8.cpu()
+        (k, *kq), (v, *vq) = (binding.quantize_rows(t, want_codes=True) for t in (k, v))
+        plan.forward_kv8(K, B, q, *kq, *vq, out)
+        Kc, Vc = k.cpu(), v.cpu()
     else:
-        got, _ = run_forward(plan, K, B, Q, Kc, Vc, binding.KERNEL_TCGEN05)
+        plan.forward(K, B, q, k, v, out)
+    if build == "many-tiles":
+        ctas = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+        assert captured_grids(lambda: plan.forward(K, B, q, k, v, out)) == [ctas]
+    assert plan.poll() == 0
+    got = out.double().cpu().numpy()
     for b in {0, B, 2 * B - 1}:
         ref = orc.attention_step(scales, K, tab[K - 1], Q[b:b + 1], Kc[b:b + 1], Vc[b:b + 1])
-        assert_close(got[b:b + 1], ref, f"batch row {b}")
+        ma, rl = errors(got[b:b + 1], ref)
+        # equal probabilities are exact; the output is rounded to bf16 (2^-9 of its size), 8-bit rows once more
+        bound = 2.0 ** -8 * float(Vc.float().abs().max())
+        assert ma <= bound and rl <= REL_L2, f"batch row {b}: max-abs {ma:.3e} rel-L2 {rl:.3e}"
     plan.close()
 
 
