@@ -18,7 +18,7 @@
 // to the largest exponent and cuts them off there: with ones everywhere 16 addends a step lose up to a bit of the sum each, always
 // in the same direction.  Over the 34240 keys of the last 2K step, keys three times as sharp, outputs were too large by 1.0e-4; with
 // four addends a step by 1.5e-5, with one too small by 1.9e-5, with sums by additions too small by 1.5e-5.  Time: the same.)  A sum
-// by additions is one instruction a score (64, beside the 360 that a warp issues per chunk now, all included).
+// by additions is one instruction a score (64, beside the 346 that a warp issues per chunk now, all included).
 // Q is a TMEM operand: a step of S = Q K with both operands in shared memory waits for their 6 KB (50 cycles, 32 with Q in TMEM), and
 // the two CTAs of an SM share that.
 // MANY: a CTA takes several tiles in turn.  Q has two buffers; K and V copies of the next tile go out behind the last ones of this
@@ -43,7 +43,7 @@
 // whose sum or output is out of range (kRange, kSmall) sends the CTA through its lists again (`exact`), each list twice: once for
 // the rows' maxima, then against them, for the 32 rows of a warp that it belongs to, which are stored then.
 //
-// What bounds it (ncu, 2K step, full mask): issue slots 72 % busy, exponential pipe 64 %, tensor pipe active 56 %; 5.6 instructions a
+// What bounds it (ncu, 2K step, full mask): issue slots 70 % busy, exponential pipe 65 %, tensor pipe active 58 %; 5.4 instructions a
 // score.  (More warps do not help: three streams of softmax warps, or three score buffers so that none waits for its next scores,
 // took as long as before with the sums still added by instructions.)  Measured on B200, in thousand cycles of a launch, with one
 // accumulator and sums of its own per stream / shared accumulator and sums by products / and Q in TMEM / and six pairs of a half's
